@@ -20,8 +20,10 @@
 // over short runs before they are added in double.
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <vector>
 
+#include "circuit_passes.cuh"
 #include "common.cuh"
 
 namespace qc {
@@ -178,113 +180,410 @@ __device__ __forceinline__ double block_reduce(double v) {
 }
 
 // ------------------------------------------------------------ forward ----
+// What a pass's operators are on one batch element, prepared once per call
+// in FP64 by k_prep (the sines and cosines of GB300's slow FP64 pipe stay out
+// of the tile kernels).
+//
+// A rotation is applied without its factor: RY as b0 = a0 + t a1,
+// b1 = a1 - t a0 with t = s/c when |s| <= |c|, else b0 = t a0 + a1,
+// b1 = t a1 - a0 with t = c/s (RX likewise with i t), two multiply-adds an
+// amplitude and component instead of a 2x2 product; the factors c or s of all
+// of a pass's operators go into its one phase per amplitude.
+enum OpMode { OM_RY0, OM_RY1, OM_RX0, OM_RX1, OM_RZ, OM_H };
 template <typename R>
-__global__ void __launch_bounds__(ADJ_T) k_fwd_gate(typename CT<R>::V2* __restrict__ psi, int n, GateDev g,
-                                                    const double* __restrict__ theta, int64_t stride) {
-  using IO = AmpIO<R>;
-  const int b = blockIdx.y;
-  typename CT<R>::V2* s = psi + ((uint64_t)b << n);
-  const double th = (g.kind <= QC_G_RZ) ? theta[(int64_t)b * stride + g.param] : 0.0;
-  const Mat2<R> U = block_matrix<R>(g.kind, th);
-  const uint64_t np = (g.kind == QC_G_CNOT) ? (1ull << (n - 2)) : (1ull << (n - 1));
-  for (uint64_t p = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; p < np; p += (uint64_t)gridDim.x * blockDim.x) {
-    uint64_t i1;
-    const uint64_t i0 = gate_pair(g, p, i1);
-    Cx<R> a0 = IO::ld(s + i0), a1 = IO::ld(s + i1);
-    apply_any<R>(g.kind, U, a0, a1);
-    IO::st(s + i0, a0);
-    IO::st(s + i1, a1);
-  }
+struct OpRec {
+  R t, u;
+  int mode;
+};
+// tab: phase of a thread's lane bits [0, 32), its warp bits [32, 48), of the
+// register bits [48, 56); the phase times the pass's factor is their product.
+template <typename R>
+struct PassRec {
+  typename CT<R>::V2 tab[56];
+  OpRec<R> op[TP_MAXOP];
+};
+
+// 1 / sqrt(1 + t^2) as an unevaluated sum (the rounded root and its first
+// correction): the product of a pass's factors is then good to one rounding,
+// so the state's norm does not drift by it.
+__device__ __forceinline__ double2 inv_norm(double t) {
+  const double s = fma(t, t, 1.0), sl = fma(t, t, 1.0 - s), r = 1.0 / sqrt(s);
+  const double q = s * r, ql = fma(s, r, -q);
+  const double res = fma(-q, r, 1.0) - ql * r - sl * r * r;  // 1 - (1 + t^2) r^2
+  return make_double2(r, 0.5 * r * res);
 }
 
-// Two rotations on one qubit, ga then gb: one pass with M = U_b U_a.
+// Per pass and batch element (grid.x, grid.y).  dir = +1: the operators as
+// they are, the phase in the last round; -1: their inverses, the phase in the
+// first round.
 template <typename R>
-__global__ void __launch_bounds__(ADJ_T) k_fwd_rot2(typename CT<R>::V2* __restrict__ psi, int n, GateDev ga,
-                                                    GateDev gb, const double* __restrict__ theta, int64_t stride) {
-  using IO = AmpIO<R>;
-  const int b = blockIdx.y;
-  typename CT<R>::V2* s = psi + ((uint64_t)b << n);
-  const Mat2<R> M = block_matrix<R>(ga.kind, theta[(int64_t)b * stride + ga.param], gb.kind,
-                                    theta[(int64_t)b * stride + gb.param]);
-  const int q = ga.q0;
-  const uint64_t np = 1ull << (n - 1);
-  for (uint64_t p = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; p < np; p += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t i0 = insert0(p, q), i1 = i0 | (1ull << q);
-    Cx<R> a0 = IO::ld(s + i0), a1 = IO::ld(s + i1);
-    apply2<R, MK_GENERAL>(M, a0, a1);
-    IO::st(s + i0, a0);
-    IO::st(s + i1, a1);
-  }
-}
-
-// The same pass for complex64 with 16-byte accesses: an item is two
-// neighbouring pairs (q >= 1: amplitudes i0, i0+1 and i0 + 2^q, i0 + 2^q + 1)
-// or one pair (q = 0: amplitudes 2v, 2v+1 in one vector); four items per
-// trip on three blocks per SM (eight-byte loads, one pair per trip, streamed
-// the 64-state batch at 0.78 of copy bandwidth on GB300).
-constexpr int FWD_UNR = 4;
-__device__ __forceinline__ void rot_v(const Mat2<float>& M, float4& A, float4& B) {
-  Cx<float> a0 = cmake(A.x, A.y), c0 = cmake(A.z, A.w), a1 = cmake(B.x, B.y), c1 = cmake(B.z, B.w);
-  apply2<float, MK_GENERAL>(M, a0, a1);
-  apply2<float, MK_GENERAL>(M, c0, c1);
-  A = make_float4(a0.re, a0.im, c0.re, c0.im);
-  B = make_float4(a1.re, a1.im, c1.re, c1.im);
-}
-__global__ void __launch_bounds__(ADJ_T, 4) k_fwd_rot2_c64(float2* __restrict__ psi, int n, GateDev ga, GateDev gb,
-                                                           const double* __restrict__ theta, int64_t stride) {
-  const int b = blockIdx.y;
-  float2* s = psi + ((uint64_t)b << n);
-  const Mat2<float> M = block_matrix<float>(ga.kind, theta[(int64_t)b * stride + ga.param], gb.kind,
-                                            theta[(int64_t)b * stride + gb.param]);
-  const int q = ga.q0;
-  const uint64_t G = (uint64_t)gridDim.x * blockDim.x;
-  uint64_t v = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (q == 0) {
-    float4* w = reinterpret_cast<float4*>(s);
-    const uint64_t items = 1ull << (n - 1);
-    for (; v + (FWD_UNR - 1) * G < items; v += FWD_UNR * G) {
-      float4 A[FWD_UNR];
-#pragma unroll
-      for (int u = 0; u < FWD_UNR; ++u) A[u] = w[v + u * G];
-#pragma unroll
-      for (int u = 0; u < FWD_UNR; ++u) {
-        Cx<float> a0 = cmake(A[u].x, A[u].y), a1 = cmake(A[u].z, A[u].w);
-        apply2<float, MK_GENERAL>(M, a0, a1);
-        w[v + u * G] = make_float4(a0.re, a0.im, a1.re, a1.im);
+__global__ void __launch_bounds__(128) k_prep(const TilePass* __restrict__ passes, PassRec<R>* __restrict__ recs, int B,
+                                              const double* __restrict__ theta, int64_t stride, int dir) {
+  __shared__ double2 ph[TP_MAXK + 3];  // e^{-i dir theta / 2}
+  __shared__ double2 fac[TP_MAXOP];  // factor as an unevaluated sum
+  const TilePass& P = passes[blockIdx.x];
+  const int b = blockIdx.y, tid = threadIdx.x;
+  PassRec<R>& rec = recs[(int64_t)blockIdx.x * B + b];
+  const double* th = theta + (int64_t)b * stride;
+  if (tid < P.nop) {
+    const TileOp o = P.op[tid];
+    OpRec<R> r{};
+    double2 f = make_double2(1.0, 0.0);
+    if (o.ka == QC_G_H) {
+      r.mode = OM_H;
+      f = inv_norm(1.0);
+    } else {
+      double s, c;
+      sincos(-0.5 * dir * th[o.pa], &s, &c);  // b0 = c a0 + s a1 undoes RY(theta)
+      if (o.ka == QC_G_RZ) {
+        r.mode = OM_RZ;
+        r.t = (R)c;
+        r.u = (R)s;
+      } else {
+        const bool small = fabs(s) <= fabs(c);
+        r.mode = (o.ka == QC_G_RY ? OM_RY0 : OM_RX0) + (small ? 0 : 1);
+        r.t = (R)(small ? s / c : c / s);
+        f = inv_norm((double)r.t);  // of the t in use: the operator is unitary to rounding
+        if ((small ? c : s) < 0.0) f = make_double2(-f.x, -f.y);
       }
     }
-    for (; v < items; v += G) {
-      const float4 A = w[v];
-      Cx<float> a0 = cmake(A.x, A.y), a1 = cmake(A.z, A.w);
-      apply2<float, MK_GENERAL>(M, a0, a1);
-      w[v] = make_float4(a0.re, a0.im, a1.re, a1.im);
-    }
-    return;
+    rec.op[tid] = r;
+    fac[tid] = f;
+  } else if (tid >= 64 && tid < 64 + P.kt) {
+    const int p = tid - 64;
+    double s = 0.0, c = 1.0;
+    if (P.dp[p] >= 0) sincos(-0.5 * dir * th[P.dp[p]], &s, &c);
+    ph[p] = make_double2(c, s);
   }
-  const uint64_t items = 1ull << (n - 2), st = 1ull << q;
-  for (; v + (FWD_UNR - 1) * G < items; v += FWD_UNR * G) {
-    uint64_t i0[FWD_UNR];
-    float4 A[FWD_UNR], B[FWD_UNR];
+  __syncthreads();
+  if (tid < 56) {
+    const TileRound& rd = P.rd[dir > 0 ? P.nround - 1 : 0];
+    constexpr int rb = 3;
+    double re = 1.0, im = 0.0;
+    // thread bit i is the i-th tile position outside the round's registers
+    int i = 0;
+    for (int p = 0; p < P.kt; ++p) {
+      int reg = -1;
+      for (int x = 0; x < rb; ++x)
+        if (rd.r[x] == p) reg = x;
+      int bit;
+      bool mine;
+      if (reg >= 0) {
+        mine = tid >= 48;
+        bit = (tid - 48) >> reg;
+      } else {
+        mine = i < 5 ? tid < 32 : (tid >= 32 && tid < 48);
+        bit = i < 5 ? tid >> i : (tid - 32) >> (i - 5);
+        ++i;
+      }
+      if (!mine || P.dp[p] < 0) continue;
+      const double c = ph[p].x, s = (bit & 1) ? -ph[p].y : ph[p].y;
+      const double nr = re * c - im * s;
+      im = re * s + im * c;
+      re = nr;
+    }
+    // products of rounded phases: back to modulus 1, then the factor
+    const double m = 0.5 * (fma(re, re, -1.0) + im * im);
+    re = fma(-m, re, re);
+    im = fma(-m, im, im);
+    if (tid >= 48) {
+      double h = 1.0, l = 0.0;
+      for (int k = 0; k < P.nop; ++k) {
+        const double p = h * fac[k].x;
+        l = fma(h, fac[k].x, -p) + fma(h, fac[k].y, l * fac[k].x);
+        h = p;
+      }
+      re = fma(re, l, re * h);
+      im = fma(im, l, im * h);
+    }
+    rec.tab[tid] = CT<R>::make((R)re, (R)im);
+  }
+}
+
+// The merged operators of the complex64 forward passes as 2x2 matrices.
+__global__ void __launch_bounds__(64) k_prep_mats(const TilePass* __restrict__ passes, Mat2<float>* __restrict__ mats, int B,
+                                                  const double* __restrict__ theta, int64_t stride) {
+  const TilePass& P = passes[blockIdx.x];
+  const int b = blockIdx.y;
+  if ((int)threadIdx.x >= P.nop) return;
+  const TileOp o = P.op[threadIdx.x];
+  const double* th = theta + (int64_t)b * stride;
+  Mat2<double> M = gate_matrix<double>(o.ka, o.pa >= 0 ? th[o.pa] : 0.0);
+  if (o.kb >= 0) {
+    const Mat2<double> A = M, Bm = gate_matrix<double>(o.kb, th[o.pb]);
+    for (int r = 0; r < 2; ++r)
+      for (int c = 0; c < 2; ++c) M.m[2 * r + c] = cmul2(Bm.m[2 * r], A.m[c], Bm.m[2 * r + 1], A.m[2 + c]);
+  }
+  Mat2<float> F;
+  for (int k = 0; k < 4; ++k) F.m[k] = cmake<float>((float)M.m[k].re, (float)M.m[k].im);
+  mats[((int64_t)blockIdx.x * B + b) * TP_MAXOP + threadIdx.x] = F;
+}
+
+// One operator on a thread's 2^RB amplitudes along register bit BIT.
+template <int MODE, int BIT, int RB, typename R>
+__device__ __forceinline__ void op_mode(const R t, const R u, Cx<R>* v) {
 #pragma unroll
-    for (int u = 0; u < FWD_UNR; ++u) {
-      i0[u] = insert0(2 * (v + u * G), q);
-      A[u] = *reinterpret_cast<const float4*>(s + i0[u]);
-      B[u] = *reinterpret_cast<const float4*>(s + (i0[u] | st));
+  for (int m = 0; m < (1 << (RB - 1)); ++m) {
+    const int j0 = ((m >> BIT) << (BIT + 1)) | (m & ((1 << BIT) - 1)), j1 = j0 | (1 << BIT);
+    const Cx<R> a = v[j0], c = v[j1];
+    if (MODE == OM_RY0) {  // a + t c, c - t a
+      v[j0] = cmake<R>(fma(t, c.re, a.re), fma(t, c.im, a.im));
+      v[j1] = cmake<R>(fma(-t, a.re, c.re), fma(-t, a.im, c.im));
+    } else if (MODE == OM_RY1) {  // t a + c, t c - a
+      v[j0] = cmake<R>(fma(t, a.re, c.re), fma(t, a.im, c.im));
+      v[j1] = cmake<R>(fma(t, c.re, -a.re), fma(t, c.im, -a.im));
+    } else if (MODE == OM_RX0) {  // a + i t c, c + i t a
+      v[j0] = cmake<R>(fma(-t, c.im, a.re), fma(t, c.re, a.im));
+      v[j1] = cmake<R>(fma(-t, a.im, c.re), fma(t, a.re, c.im));
+    } else if (MODE == OM_RX1) {  // t a + i c, t c + i a
+      v[j0] = cmake<R>(fma(t, a.re, -c.im), fma(t, a.im, c.re));
+      v[j1] = cmake<R>(fma(t, c.re, -a.im), fma(t, c.im, a.re));
+    } else if (MODE == OM_RZ) {  // (t + i u) a, (t - i u) c
+      v[j0] = cmake<R>(fma(-u, a.im, t * a.re), fma(u, a.re, t * a.im));
+      v[j1] = cmake<R>(fma(u, c.im, t * c.re), fma(-u, c.re, t * c.im));
+    } else {  // a + c, a - c
+      v[j0] = cmake<R>(a.re + c.re, a.im + c.im);
+      v[j1] = cmake<R>(a.re - c.re, a.im - c.im);
     }
+  }
+}
+template <int BIT, int RB, typename R>
+__device__ __forceinline__ void op_bit(const OpRec<R>& o, Cx<R>* v) {
+  switch (o.mode) {
+    case OM_RY0: op_mode<OM_RY0, BIT, RB>(o.t, o.u, v); break;
+    case OM_RY1: op_mode<OM_RY1, BIT, RB>(o.t, o.u, v); break;
+    case OM_RX0: op_mode<OM_RX0, BIT, RB>(o.t, o.u, v); break;
+    case OM_RX1: op_mode<OM_RX1, BIT, RB>(o.t, o.u, v); break;
+    case OM_RZ: op_mode<OM_RZ, BIT, RB>(o.t, o.u, v); break;
+    default: op_mode<OM_H, BIT, RB>(o.t, o.u, v); break;
+  }
+}
+template <int BIT, int RB>
+__device__ __forceinline__ void mat_bit(const Mat2<float>& M, Cx<float>* v) {
 #pragma unroll
-    for (int u = 0; u < FWD_UNR; ++u) {
-      rot_v(M, A[u], B[u]);
-      *reinterpret_cast<float4*>(s + i0[u]) = A[u];
-      *reinterpret_cast<float4*>(s + (i0[u] | st)) = B[u];
+  for (int m = 0; m < (1 << (RB - 1)); ++m) {
+    const int j0 = ((m >> BIT) << (BIT + 1)) | (m & ((1 << BIT) - 1));
+    apply2<float, MK_GENERAL>(M, v[j0], v[j0 | (1 << BIT)]);
+  }
+}
+
+template <typename V2>
+__device__ __forceinline__ V2* sm_at(V2* sm, int byte) {
+  return reinterpret_cast<V2*>(reinterpret_cast<unsigned char*>(sm) + byte);
+}
+
+// The register rounds of a pass on the tile in `sm`, each closed by a barrier.
+template <typename R> struct Fwd;
+template <> struct Fwd<float> {
+  static constexpr int RB = 4, VE = 2;
+  using Ops = Mat2<float>;
+};
+template <> struct Fwd<double> {
+  static constexpr int RB = 3, VE = 1;
+  using Ops = PassRec<double>;
+};
+
+template <typename R>
+__device__ __forceinline__ void fwd_rounds(const TilePass& P, typename CT<R>::V2* sm, const typename Fwd<R>::Ops* ops) {
+  constexpr int RB = Fwd<R>::RB, NA = 1 << RB;
+  const int tid = threadIdx.x;
+  const bool active = tid < (1 << (P.kt - RB));
+#pragma unroll 1
+  for (int r = 0; r < P.nround; ++r) {
+    const TileRound& rd = P.rd[r];
+    if (active) {
+      const int base = tp_round_base<R, RB>(rd);
+      int bas[RB];
+#pragma unroll
+      for (int x = 0; x < RB; ++x) bas[x] = rd.bas[x];
+      Cx<R> v[NA];
+#pragma unroll
+      for (int j = 0; j < NA; ++j) v[j] = AmpIO<R>::ld(sm_at(sm, tp_round_at<RB>(base, bas, j)));
+#pragma unroll 1
+      for (int k = rd.op0; k < rd.op1; ++k) {
+        if constexpr (sizeof(R) == 4) {
+          const Mat2<float> M = ops[k];
+          switch (P.op[k].bit) {
+            case 0: mat_bit<0, RB>(M, v); break;
+            case 1: mat_bit<1, RB>(M, v); break;
+            case 2: mat_bit<2, RB>(M, v); break;
+            default: mat_bit<3, RB>(M, v); break;
+          }
+        } else {
+          const OpRec<R> o = ops->op[k];
+          switch (P.op[k].bit) {
+            case 0: op_bit<0, RB, R>(o, v); break;
+            case 1: op_bit<1, RB, R>(o, v); break;
+            default: op_bit<2, RB, R>(o, v); break;
+          }
+        }
+      }
+      if constexpr (sizeof(R) == 8) {
+        if (r == P.nround - 1 && (P.has_diag || P.nop)) {
+          const auto A = ops->tab[tid & 31], Bw = ops->tab[32 + (tid >> 5)];
+          const Cx<R> d = cmul(cmake<R>(A.x, A.y), cmake<R>(Bw.x, Bw.y));
+#pragma unroll
+          for (int j = 0; j < NA; ++j) {
+            const auto J = ops->tab[48 + j];
+            v[j] = cmul(v[j], cmul(d, cmake<R>(J.x, J.y)));
+          }
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < NA; ++j) AmpIO<R>::st(sm_at(sm, tp_round_at<RB>(base, bas, j)), v[j]);
+    }
+    __syncthreads();
+  }
+}
+
+// 16-byte vectors of a tile (TileShare), to and from shared memory at byte
+// offsets i0 and i1 of their amplitudes.
+template <typename R> struct Vec;
+template <> struct Vec<float> {
+  using T = float4;
+  __device__ static void to_sm(float2* sm, int i0, int i1, const float4& v) {
+    *sm_at(sm, i0) = make_float2(v.x, v.y);
+    *sm_at(sm, i1) = make_float2(v.z, v.w);
+  }
+  __device__ static float4 from_sm(float2* sm, int i0, int i1) {
+    const float2 a = *sm_at(sm, i0), b = *sm_at(sm, i1);
+    return make_float4(a.x, a.y, b.x, b.y);
+  }
+  // al: the state starts on a 16-byte boundary (8 bytes suffice for the caller)
+  __device__ static float4 ld(const float2* g, bool al) {
+    if (al) return *reinterpret_cast<const float4*>(g);
+    const float2 a = g[0], b = g[1];
+    return make_float4(a.x, a.y, b.x, b.y);
+  }
+  __device__ static void st(float2* g, const float4& v, bool al) {
+    if (al) {
+      *reinterpret_cast<float4*>(g) = v;
+    } else {
+      g[0] = make_float2(v.x, v.y);
+      g[1] = make_float2(v.z, v.w);
     }
   }
-  for (; v < items; v += G) {
-    const uint64_t i0 = insert0(2 * v, q);
-    float4 A = *reinterpret_cast<const float4*>(s + i0), B = *reinterpret_cast<const float4*>(s + (i0 | st));
-    rot_v(M, A, B);
-    *reinterpret_cast<float4*>(s + i0) = A;
-    *reinterpret_cast<float4*>(s + (i0 | st)) = B;
+  __device__ static float4 zero() { return make_float4(0.f, 0.f, 0.f, 0.f); }
+  __device__ static float4 one() { return make_float4(1.f, 0.f, 0.f, 0.f); }
+};
+template <> struct Vec<double> {
+  using T = double2;
+  __device__ static void to_sm(double2* sm, int i0, int, const double2& v) { *sm_at(sm, i0) = v; }
+  __device__ static double2 from_sm(double2* sm, int i0, int) { return *sm_at(sm, i0); }
+  __device__ static double2 ld(const double2* g, bool) { return *g; }
+  __device__ static void st(double2* g, const double2& v, bool) { *g = v; }
+  __device__ static double2 zero() { return make_double2(0.0, 0.0); }
+  __device__ static double2 one() { return make_double2(1.0, 0.0); }
+};
+
+constexpr int FWD_T = 512, FWD_LV = 3, FWD_NV = 1 << FWD_LV;  // threads of a full tile, vectors of each
+
+// One pass over the batch: tile blockIdx.x of state blockIdx.y (first: the
+// state is |0..0>, nothing is read).
+template <typename R>
+__global__ void __launch_bounds__(FWD_T, 2) k_fwd_tile(typename CT<R>::V2* __restrict__ psi, int n,
+                                                       const __grid_constant__ TilePass P,
+                                                       const typename Fwd<R>::Ops* __restrict__ recs, int nrec, int first) {
+  using V2 = typename CT<R>::V2;
+  using V = typename Vec<R>::T;
+  extern __shared__ __align__(16) unsigned char dynsm[];
+  V2* sm = reinterpret_cast<V2*>(dynsm);
+  auto* ops = reinterpret_cast<typename Fwd<R>::Ops*>(dynsm + (sizeof(V2) << P.kt));
+  const int tid = threadIdx.x, T = blockDim.x;
+  const uint64_t base = tp_tile_base(P, blockIdx.x);
+  V2* g = psi + ((uint64_t)blockIdx.y << n) + base;
+  const bool al = (reinterpret_cast<uintptr_t>(psi) & 15) == 0;
+  {  // this element's operators
+    const int words = (int)(sizeof(typename Fwd<R>::Ops) * nrec / 16);
+    const uint4* src = reinterpret_cast<const uint4*>(recs + (size_t)blockIdx.y * nrec);
+    for (int i = tid; i < words; i += T) reinterpret_cast<uint4*>(ops)[i] = src[i];
   }
+  TileShare<R, FWD_LV> sh;
+  sh.init(P, T);
+  V v[FWD_NV];
+#pragma unroll
+  for (int u = 0; u < FWD_NV; ++u) {
+    if (first) v[u] = (tid + u == 0 && base == 0) ? Vec<R>::one() : Vec<R>::zero();
+    else v[u] = Vec<R>::ld(g + sh.g(u), al);
+  }
+#pragma unroll
+  for (int u = 0; u < FWD_NV; ++u) Vec<R>::to_sm(sm, sh.a(u), sh.a(u) ^ tp_at<R>(1), v[u]);
+  __syncthreads();
+  fwd_rounds<R>(P, sm, ops);
+  const int cst = tp_cst(P, base);
+#pragma unroll
+  for (int u = 0; u < FWD_NV; ++u) {
+    const int s = sh.s(u) ^ cst;
+    Vec<R>::st(g + sh.g(u), Vec<R>::from_sm(sm, s, s ^ sh.s1), al);
+  }
+}
+
+// The whole circuit of states that fit one tile: one block a state, all
+// passes in shared memory, one store at the end.
+template <typename R>
+__global__ void __launch_bounds__(FWD_T, 2) k_fwd_whole(typename CT<R>::V2* __restrict__ psi, int n,
+                                                        const TilePass* __restrict__ passes, int npass,
+                                                        const typename Fwd<R>::Ops* __restrict__ recs, int nrec, int B) {
+  using V2 = typename CT<R>::V2;
+  using V = typename Vec<R>::T;
+  constexpr int VE = Fwd<R>::VE;
+  extern __shared__ __align__(16) unsigned char dynsm[];
+  __shared__ TilePass P;
+  const int tid = threadIdx.x, T = blockDim.x, kt = passes[0].kt, ne = 1 << n, b = blockIdx.x;
+  V2* sm = reinterpret_cast<V2*>(dynsm);
+  auto* ops = reinterpret_cast<typename Fwd<R>::Ops*>(dynsm + (sizeof(V2) << kt));
+  for (int e = tid; e < (1 << kt); e += T) sm[tp_swz<R>(e)] = CT<R>::make((R)(e == 0), (R)0);
+  V v[FWD_NV];
+#pragma unroll 1
+  for (int k = 0; k < npass; ++k) {
+    static_assert(sizeof(TilePass) % 4 == 0, "copied in words");
+    for (int i = tid; i < (int)sizeof(TilePass) / 4; i += T)
+      reinterpret_cast<uint32_t*>(&P)[i] = reinterpret_cast<const uint32_t*>(passes + k)[i];
+    const int words = (int)(sizeof(typename Fwd<R>::Ops) * nrec / 16);
+    const uint4* src = reinterpret_cast<const uint4*>(recs + ((size_t)k * B + b) * nrec);
+    for (int i = tid; i < words; i += T) reinterpret_cast<uint4*>(ops)[i] = src[i];
+    __syncthreads();
+    fwd_rounds<R>(P, sm, ops);
+    // P, through registers (the last pass's goes with the store)
+    TileShare<R, FWD_LV> sh;
+    sh.init(P, T);
+#pragma unroll
+    for (int u = 0; u < FWD_NV; ++u)
+      if ((tid + T * u) * VE < (1 << kt)) v[u] = Vec<R>::from_sm(sm, sh.s(u), sh.s(u) ^ sh.s1);
+    __syncthreads();
+    if (k + 1 < npass) {
+#pragma unroll
+      for (int u = 0; u < FWD_NV; ++u)
+        if ((tid + T * u) * VE < (1 << kt)) Vec<R>::to_sm(sm, sh.a(u), sh.a(u) ^ tp_at<R>(1), v[u]);
+    }
+  }
+  V2* g = psi + ((uint64_t)b << n);
+  const bool al = (reinterpret_cast<uintptr_t>(psi) & 15) == 0;
+#pragma unroll
+  for (int u = 0; u < FWD_NV; ++u) {
+    const int e = (tid + T * u) * VE;
+    if (e < ne) Vec<R>::st(g + e, v[u], al);
+  }
+}
+
+// Host data to the device by value of a kernel parameter: no host buffer has
+// to outlive the call, and a captured graph carries the data itself.
+struct Blob {
+  uint4 d[512];
+};
+__global__ void k_put(const __grid_constant__ Blob blob, uint4* __restrict__ dst, int words) {
+  for (int i = threadIdx.x; i < words; i += blockDim.x) dst[i] = blob.d[i];
+}
+// Returns the launches made.  bytes is rounded up to 16: dst has that room.
+static int put_bytes(void* dst, const void* src, size_t bytes, cudaStream_t st) {
+  int nk = 0;
+  for (size_t o = 0; o < bytes; o += sizeof(Blob), ++nk) {
+    Blob blob;
+    const size_t m = std::min(sizeof(Blob), bytes - o);
+    memcpy(blob.d, reinterpret_cast<const char*>(src) + o, m);
+    k_put<<<1, 256, 0, st>>>(blob, reinterpret_cast<uint4*>(reinterpret_cast<char*>(dst) + o), (int)((m + 15) / 16));
+  }
+  return nk;
 }
 
 // CNOT ring CNOT(0,1) .. CNOT(n-2,n-1), CNOT(n-1,0) as a basis permutation
@@ -550,7 +849,7 @@ static unsigned gx_for(int n, int B) {
   const uint64_t pairs = 1ull << (n - 1);
   uint64_t gx = (pairs + ADJ_T - 1) / ADJ_T;
   const int res = std::min(resident_blocks((const void*)k_bwd_rot2<R>, ADJ_T, 0),
-                           resident_blocks((const void*)k_fwd_gate<R>, ADJ_T, 0));
+                           resident_blocks((const void*)k_bwd_gate<R>, ADJ_T, 0));
   const uint64_t cap = std::max<uint64_t>(1, (uint64_t)sm_count() * res / (uint64_t)B);
   gx = std::min<uint64_t>(gx, std::min<uint64_t>(cap, ADJ_GX_MAX));
   return (unsigned)std::max<uint64_t>(gx, 1);
@@ -564,36 +863,72 @@ struct Bufs {
   typename CT<R>::V2* spare;
 };
 
-// Forward passes; the result is in bufs.psi (which may be the workspace).
+// Passes of a forward sweep on the device, with room for the operators of as
+// many batch elements at a time as fit PREP_BYTES.
+constexpr size_t PREP_BYTES = 64u << 20;
 template <typename R>
-static int forward_passes(const std::vector<AdjOp>& ops, int n, int B, const double* theta, int64_t stride,
-                          Bufs<R>& bf, cudaStream_t st) {
-  const dim3 grid(gx_for<R>(n, B), B);
-  // complex64 rotation pairs: three blocks per SM over the whole batch
-  const uint64_t vitems = n >= 2 ? (1ull << (n - 2)) : 1ull;
-  const unsigned gxv = (unsigned)std::max<uint64_t>(
-      1, std::min<uint64_t>((vitems + FWD_UNR * ADJ_T - 1) / (FWD_UNR * ADJ_T), 3ull * sm_count() / (uint64_t)B));
-  const uint64_t tot = (uint64_t)B << n;
-  k_zero_state_batch<R><<<grid_for(tot, ADJ_T, 8), ADJ_T, 0, st>>>(bf.psi, n, B);
-  int nk = 1;
-  for (const AdjOp& op : ops) {
-    if (op.kind == AOP_RING) {
-      k_ring<R><<<grid, ADJ_T, 0, st>>>(bf.psi, bf.spare, n, 0);
-      std::swap(bf.psi, bf.spare);
-    } else if (op.kind == AOP_ROT2) {
-      if constexpr (sizeof(R) == 4) {
-        if (n >= 2) {
-          k_fwd_rot2_c64<<<dim3(gxv, B), ADJ_T, 0, st>>>(reinterpret_cast<float2*>(bf.psi), n, op.a, op.b, theta,
-                                                         stride);
-          ++nk;
-          continue;
-        }
-      }
-      k_fwd_rot2<R><<<grid, ADJ_T, 0, st>>>(bf.psi, n, op.a, op.b, theta, stride);
-    } else {
-      k_fwd_gate<R><<<grid, ADJ_T, 0, st>>>(bf.psi, n, op.a, theta, stride);
-    }
+struct FwdPlan {
+  std::vector<TilePass> passes;
+  TilePass* dpass = nullptr;
+  typename Fwd<R>::Ops* recs = nullptr;
+  int chunk = 0;  // batch elements at a time
+  static constexpr int nrec = sizeof(R) == 4 ? TP_MAXOP : 1;
+};
+
+template <typename R>
+static cudaError_t fwd_plan(FwdPlan<R>& F, const qc_gate* gates, int ng, int n, int B, cudaStream_t st) {
+  const TileCfg cfg = sizeof(R) == 4 ? TileCfg{13, 4, 4, true, false} : TileCfg{12, 3, 3, false, false};
+  F.passes = build_passes<R>(gates, ng, n, cfg);
+  if (F.passes.empty()) return cudaSuccess;
+  const size_t per = F.passes.size() * F.nrec * sizeof(typename Fwd<R>::Ops);
+  F.chunk = (int)std::max<size_t>(1, std::min<size_t>(B, PREP_BYTES / per));
+  cudaError_t e = cudaMallocAsync((void**)&F.dpass, (F.passes.size() * sizeof(TilePass) + 15) / 16 * 16, st);
+  if (e == cudaSuccess) e = cudaMallocAsync((void**)&F.recs, per * F.chunk, st);
+  if (e != cudaSuccess && F.dpass) cudaFreeAsync(F.dpass, st);
+  return e;
+}
+template <typename R>
+static void fwd_plan_free(FwdPlan<R>& F, cudaStream_t st) {
+  if (F.dpass) cudaFreeAsync(F.dpass, st);
+  if (F.recs) cudaFreeAsync(F.recs, st);
+}
+
+template <typename K>
+static void allow_smem(K kernel, size_t bytes) {
+  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+// psi_b = U_G .. U_1 |0..0>; returns the launches made.
+template <typename R>
+static int forward_passes(const FwdPlan<R>& F, int n, int B, const double* theta, int64_t stride,
+                          typename CT<R>::V2* psi, cudaStream_t st) {
+  if (F.passes.empty()) {
+    k_zero_state_batch<R><<<grid_for((int64_t)B << n, ADJ_T, 8), ADJ_T, 0, st>>>(psi, n, B);
+    return 1;
+  }
+  const int np = (int)F.passes.size();
+  int nk = put_bytes(F.dpass, F.passes.data(), np * sizeof(TilePass), st);
+  const int kt = F.passes[0].kt, T = std::max(32, 1 << (kt - Fwd<R>::RB));
+  const size_t smem = (sizeof(typename CT<R>::V2) << kt) + sizeof(typename Fwd<R>::Ops) * F.nrec;
+  allow_smem(k_fwd_tile<R>, smem);
+  allow_smem(k_fwd_whole<R>, smem);
+  for (int b0 = 0; b0 < B; b0 += F.chunk) {
+    const int nb = std::min(F.chunk, B - b0);
+    const double* th = theta + (int64_t)b0 * stride;
+    typename CT<R>::V2* s = psi + ((uint64_t)b0 << n);
+    if constexpr (sizeof(R) == 4)
+      k_prep_mats<<<dim3(np, nb), 64, 0, st>>>(F.dpass, F.recs, nb, th, stride);
+    else
+      k_prep<R><<<dim3(np, nb), 128, 0, st>>>(F.dpass, F.recs, nb, th, stride, 1);
     ++nk;
+    if (n <= kt) {
+      k_fwd_whole<R><<<nb, T, smem, st>>>(s, n, F.dpass, np, F.recs, F.nrec, nb);
+      ++nk;
+    } else {
+      for (int k = 0; k < np; ++k, ++nk)
+        k_fwd_tile<R><<<dim3(1u << (n - kt), nb), T, smem, st>>>(s, n, F.passes[k], F.recs + (size_t)k * nb * F.nrec,
+                                                                 F.nrec, k == 0);
+    }
   }
   return nk;
 }
@@ -607,20 +942,11 @@ static bool has_ring(const std::vector<AdjOp>& ops) {
 template <typename R>
 static qc_status forward_impl(int n, int B, const qc_gate* gates, int n_gates, const double* theta,
                               int64_t stride, void* psi, cudaStream_t st) {
-  using V2 = typename CT<R>::V2;
-  const std::vector<AdjOp> ops = compile_ops(gates, n_gates, n);
-  const size_t bytes = ((size_t)B << n) * sizeof(V2);
-  V2* ws = nullptr;
-  if (has_ring(ops)) {
-    cudaError_t e = cudaMallocAsync((void**)&ws, bytes, st);
-    if (e != cudaSuccess) return cuda_fail(e, "forward workspace");
-  }
-  Bufs<R> bf{reinterpret_cast<V2*>(psi), nullptr, ws};
-  int nk = forward_passes<R>(ops, n, B, theta, stride, bf, st);
-  if (bf.psi != reinterpret_cast<V2*>(psi)) {
-    cudaMemcpyAsync(psi, bf.psi, bytes, cudaMemcpyDeviceToDevice, st);
-  }
-  if (ws) cudaFreeAsync(ws, st);
+  FwdPlan<R> F;
+  const cudaError_t e = fwd_plan(F, gates, n_gates, n, B, st);
+  if (e != cudaSuccess) return cuda_fail(e, "forward workspace");
+  const int nk = forward_passes<R>(F, n, B, theta, stride, reinterpret_cast<typename CT<R>::V2*>(psi), st);
+  fwd_plan_free(F, st);
   return check_launch("circuit forward", nk);
 }
 
@@ -640,12 +966,15 @@ static qc_status adjoint_impl(int n, int B, const qc_gate* gates, int n_gates, c
   cudaError_t e = cudaMallocAsync((void**)&dT, sizeof(TermsDev), st);
   if (e == cudaSuccess) e = cudaMallocAsync((void**)&part, sizeof(double) * 2 * (size_t)gx * B, st);
   if (e == cudaSuccess && has_ring(ops)) e = cudaMallocAsync((void**)&ws, bytes, st);
+  FwdPlan<R> F;
+  if (e == cudaSuccess) e = fwd_plan(F, gates, n_gates, n, B, st);
   TermsDev* hT = nullptr;
   if (e == cudaSuccess) e = cudaMallocHost((void**)&hT, sizeof(TermsDev));
   if (e != cudaSuccess) {
     if (dT) cudaFreeAsync(dT, st);
     if (part) cudaFreeAsync(part, st);
     if (ws) cudaFreeAsync(ws, st);
+    fwd_plan_free(F, st);
     return cuda_fail(e, "adjoint workspace");
   }
   double* part_b = part + (size_t)gx * B;
@@ -661,11 +990,7 @@ static qc_status adjoint_impl(int n, int B, const qc_gate* gates, int n_gates, c
   if (e != cudaSuccess) s = cuda_fail(e, "adjoint setup");
   if (!s) {
     Bufs<R> bf{reinterpret_cast<V2*>(psi), reinterpret_cast<V2*>(lam), ws};
-    // the forward pass may rotate psi into the workspace; lam stays put
-    Bufs<R> fb{bf.psi, nullptr, bf.spare};
-    int nk = forward_passes<R>(ops, n, B, theta, stride, fb, st);
-    bf.psi = fb.psi;
-    bf.spare = fb.spare;
+    int nk = forward_passes<R>(F, n, B, theta, stride, bf.psi, st);
     k_apply_h<R><<<grid, ADJ_T, 0, st>>>(bf.psi, bf.lam, n, dT);
     k_energy<R><<<grid, ADJ_T, 0, st>>>(bf.psi, bf.lam, n, part);
     k_final_batch<<<B, ADJ_T, 0, st>>>(part, gx, energy, 1, 0);
@@ -699,6 +1024,7 @@ static qc_status adjoint_impl(int n, int B, const qc_gate* gates, int n_gates, c
   cudaFreeAsync(dT, st);
   cudaFreeAsync(part, st);
   if (ws) cudaFreeAsync(ws, st);
+  fwd_plan_free(F, st);
   if (!s && e != cudaSuccess) s = cuda_fail(e, "adjoint");
   return s;
 }
