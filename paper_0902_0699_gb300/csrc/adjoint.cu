@@ -1,18 +1,15 @@
 // Parameterised circuits on a batch of states and the adjoint gradient of
 // E = <psi|H|psi> (not part of the QCMPI paper).
 //
-// The gate list is first compiled into passes: two consecutive rotations on
-// the same qubit become one pass, and a full CNOT ring CNOT(0,1), CNOT(1,2),
-// .., CNOT(n-1,0) -- a permutation of basis indices (prefix parity) --
-// becomes one gather pass; any other gate is a pass of its own.  Batch
-// element b is grid.y, so each block builds its element's matrices once.
+// The gate list is compiled into passes over shared-memory tiles
+// (circuit_passes.cuh).
 //
 // Forward: psi_b = U_G .. U_1 |0..0>.  Backward: lambda = H psi (one gather
 // pass over the Pauli terms), E = Re <psi|lambda>, then the passes are
-// walked in reverse; a rotation pass reads psi_j and lambda_j, accumulates
-// Im <lambda_j|P_j|psi_j> -- the derivative of U_j = exp(-i theta P_j / 2)
-// gives dE/dtheta_j = 2 Re <lambda_j|(-i/2) P_j|psi_j> = Im <lambda_j|P_j|psi_j>
-// -- and applies U_j^dagger to both.  No intermediate state is stored: psi
+// walked in reverse; a rotation accumulates Im <lambda_j|P_j|psi_j> -- the
+// derivative of U_j = exp(-i theta P_j / 2) gives
+// dE/dtheta_j = 2 Re <lambda_j|(-i/2) P_j|psi_j> = Im <lambda_j|P_j|psi_j>
+// -- and U_j^dagger is applied to both.  No intermediate state is stored: psi
 // is uncomputed instead of checkpointed.
 //
 // Accumulation is FP64: complex128 with FMA in double; complex64 products
@@ -30,10 +27,6 @@ namespace qc {
 
 #define ADJ_T 256
 #define ADJ_GX_MAX 256
-
-struct GateDev {
-  int kind, q0, q1, param;
-};
 
 // Rotation matrices exp(-i theta P / 2) for P = X, Y, Z; H.
 template <typename R>
@@ -68,52 +61,6 @@ __device__ __forceinline__ Mat2<R> gate_matrix(int kind, double theta) {
   return U;
 }
 
-// The block's matrix for (kind, theta), or the product U_b U_a of two: one
-// thread evaluates the FP64 sines and cosines (costly on GB300's FP64 pipe)
-// and the block reads the result from shared memory.
-template <typename R>
-__device__ __forceinline__ Mat2<R> block_matrix(int ka, double tha, int kb = -1, double thb = 0.0) {
-  __shared__ Mat2<double> sh;
-  if (threadIdx.x == 0) {
-    const Mat2<double> A = gate_matrix<double>(ka, tha);
-    if (kb < 0) {
-      sh = A;
-    } else {
-      const Mat2<double> Bm = gate_matrix<double>(kb, thb);
-      for (int r = 0; r < 2; ++r)
-        for (int c = 0; c < 2; ++c) sh.m[2 * r + c] = cmul2(Bm.m[2 * r], A.m[c], Bm.m[2 * r + 1], A.m[2 + c]);
-    }
-  }
-  __syncthreads();
-  Mat2<R> U;
-  for (int k = 0; k < 4; ++k) U.m[k] = cmake<R>((R)sh.m[k].re, (R)sh.m[k].im);
-  __syncthreads();  // sh may be rewritten by a second call in the same kernel
-  return U;
-}
-
-template <typename R>
-__device__ __forceinline__ void apply_any(int kind, const Mat2<R>& U, Cx<R>& a0, Cx<R>& a1) {
-  if (kind == QC_G_RY) apply2<R, MK_REAL>(U, a0, a1);
-  else if (kind == QC_G_RZ) apply2<R, MK_DIAG>(U, a0, a1);
-  else if (kind == QC_G_H) apply2<R, MK_HAD>(U, a0, a1);
-  else if (kind == QC_G_CNOT) apply2<R, MK_SWAPX>(U, a0, a1);
-  else apply2<R, MK_GENERAL>(U, a0, a1);
-}
-
-// Pair enumeration of one gate: 1q gates insert a zero at q0; CNOT inserts
-// zeros at both qubits and sets the control bit.
-__device__ __forceinline__ uint64_t gate_pair(const GateDev& g, uint64_t p, uint64_t& partner) {
-  if (g.kind == QC_G_CNOT) {
-    const int lo = min(g.q0, g.q1), hi = max(g.q0, g.q1);
-    const uint64_t i0 = insert0(insert0(p, lo), hi) | (1ull << g.q0);
-    partner = i0 | (1ull << g.q1);
-    return i0;
-  }
-  const uint64_t i0 = insert0(p, g.q0);
-  partner = i0 | (1ull << g.q0);
-  return i0;
-}
-
 // ----------------------------------------------------- accumulators ------
 template <typename R> struct Acc;
 template <> struct Acc<double> {
@@ -122,6 +69,10 @@ template <> struct Acc<double> {
   __device__ void sub(double x, double y) { a = fma(-x, y, a); }
   __device__ void flush() {}
   __device__ double value() const { return a; }
+  __device__ void merge(const Acc& o) { a += o.a; }
+  __device__ void merge_neg(const Acc& o) { a -= o.a; }
+  __device__ void into(double& z) const { z += a; }
+  __device__ bool finite() const { return isfinite(a); }
 };
 // complex64: products exact as float pairs (two-product), summed as a float
 // pair with two-sum (relative error ~ terms * 2^-48), converted to double
@@ -148,24 +99,22 @@ template <> struct Acc<float> {
     s = c = 0.f;
   }
   __device__ double value() const { return a; }
-};
-
-// Accumulate Im <l|P|p> over one pair for the generator P of a rotation.
-template <typename R>
-__device__ __forceinline__ void acc_generator(Acc<R>& acc, int kind, const Cx<R>& p0, const Cx<R>& p1,
-                                              const Cx<R>& l0, const Cx<R>& l1) {
-  // Im(conj(a) b) = a.re b.im - a.im b.re
-  if (kind == QC_G_RZ) {  // Z: conj(l0) p0 - conj(l1) p1
-    acc.add(l0.re, p0.im); acc.sub(l0.im, p0.re);
-    acc.sub(l1.re, p1.im); acc.add(l1.im, p1.re);
-  } else if (kind == QC_G_RX) {  // X: conj(l0) p1 + conj(l1) p0
-    acc.add(l0.re, p1.im); acc.sub(l0.im, p1.re);
-    acc.add(l1.re, p0.im); acc.sub(l1.im, p0.re);
-  } else {  // Y: conj(l0)(-i p1) + conj(l1)(i p0); Im(conj(a)(-i b)) = -Re(conj(a) b)
-    acc.sub(l0.re, p1.re); acc.sub(l0.im, p1.im);
-    acc.add(l1.re, p0.re); acc.add(l1.im, p0.im);
+  __device__ void merge(const Acc& o) { put(o.s, o.c); }
+  __device__ void merge_neg(const Acc& o) { put(-o.s, -o.c); }
+  __device__ void into(float2& z) const {
+    Acc t;
+    t.s = z.x;
+    t.c = z.y;
+    t.put(s, c);
+    z = make_float2(t.s, t.c);
   }
-}
+  __device__ bool finite() const { return isfinite(s); }
+  // (s + c) 2^k rounded to an integer (k may exceed a float's range of exponents)
+  __device__ long long fixed(int k) const {
+    const float f0 = __int_as_float((127 + k / 2) << 23), f1 = __int_as_float((127 + k - k / 2) << 23);
+    return __float2ll_rn(s * f0 * f1) + __float2ll_rn(c * f0 * f1);
+  }
+};
 
 __device__ __forceinline__ double block_reduce(double v) {
   __shared__ double sh[32];
@@ -194,6 +143,8 @@ template <typename R>
 struct OpRec {
   R t, u;
   int mode;
+  int eq;    // backward: the sum's value is f times the one accumulated, eq = floor(log2 f)
+  double f;
 };
 // tab: phase of a thread's lane bits [0, 32), its warp bits [32, 48), of the
 // register bits [48, 56); the phase times the pass's factor is their product.
@@ -256,6 +207,13 @@ __global__ void __launch_bounds__(128) k_prep(const TilePass* __restrict__ passe
     ph[p] = make_double2(c, s);
   }
   __syncthreads();
+  if (dir < 0 && tid < P.nop) {  // operator `tid` still has the factors from itself on in psi and in lambda
+    double f = 1.0;
+    for (int k = tid; k < P.nop; ++k) f *= fac[k].x;
+    f = 1.0 / (f * f);
+    rec.op[tid].f = f;
+    rec.op[tid].eq = ilogb(f);
+  }
   if (tid < 56) {
     const TileRound& rd = P.rd[dir > 0 ? P.nround - 1 : 0];
     constexpr int rb = 3;
@@ -586,41 +544,6 @@ static int put_bytes(void* dst, const void* src, size_t bytes, cudaStream_t st) 
   return nk;
 }
 
-// CNOT ring CNOT(0,1) .. CNOT(n-2,n-1), CNOT(n-1,0) as a basis permutation
-// j -> A(j): A(j)_k = j_0 ^ .. ^ j_k for k >= 1 and A(j)_0 = j_1 ^ .. ^ j_{n-1}.
-__device__ __forceinline__ uint64_t ring_fwd(uint64_t x, int n) {
-  const uint64_t mask = (n >= 64) ? ~0ull : ((1ull << n) - 1ull);
-  uint64_t p = x;
-  p ^= (p << 1) & mask;
-  p ^= (p << 2) & mask;
-  p ^= (p << 4) & mask;
-  p ^= (p << 8) & mask;
-  p ^= (p << 16) & mask;
-  p ^= (p << 32) & mask;
-  const uint64_t top = (p >> (n - 1)) & 1ull;
-  return (p & ~1ull) | (top ^ (x & 1ull));
-}
-// inverse: x_k = y_k ^ y_{k-1} (k >= 1), x_0 = y_0, then bits 0 and 1 take y_{n-1}
-__device__ __forceinline__ uint64_t ring_inv(uint64_t y, int n) {
-  const uint64_t mask = (n >= 64) ? ~0ull : ((1ull << n) - 1ull);
-  uint64_t x = (y ^ (y << 1)) & mask;
-  if ((y >> (n - 1)) & 1ull) x ^= 3ull;
-  return x;
-}
-
-// out[j] = in[src(j)] for every batch element; forward: the ring maps
-// psi'[A(x)] = psi[x], so out[y] = in[A^{-1}(y)]; inverse: out[x] = in[A(x)].
-template <typename R>
-__global__ void __launch_bounds__(ADJ_T) k_ring(const typename CT<R>::V2* __restrict__ in,
-                                                typename CT<R>::V2* __restrict__ out, int n, int inverse) {
-  const int b = blockIdx.y;
-  const typename CT<R>::V2* s = in + ((uint64_t)b << n);
-  typename CT<R>::V2* d = out + ((uint64_t)b << n);
-  const uint64_t N = 1ull << n;
-  for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j < N; j += (uint64_t)gridDim.x * blockDim.x)
-    d[j] = s[inverse ? ring_fwd(j, n) : ring_inv(j, n)];
-}
-
 template <typename R>
 __global__ void k_zero_state_batch(typename CT<R>::V2* __restrict__ psi, int n, int B) {
   const uint64_t N = 1ull << n, tot = N * (uint64_t)B;
@@ -639,79 +562,378 @@ __global__ void k_final_batch(const double* __restrict__ part, int gx, double* _
 }
 
 // ------------------------------------------------------------ backward ---
-// One gate: accumulate Im <lam|P|psi> (rotations), apply U^dagger to both.
-template <typename R>
-__global__ void __launch_bounds__(ADJ_T) k_bwd_gate(typename CT<R>::V2* __restrict__ psi,
-                                                    typename CT<R>::V2* __restrict__ lam, int n, GateDev g,
-                                                    const double* __restrict__ theta, int64_t stride,
-                                                    double* __restrict__ part) {
-  using IO = AmpIO<R>;
-  const int b = blockIdx.y;
-  typename CT<R>::V2* s = psi + ((uint64_t)b << n);
-  typename CT<R>::V2* l = lam + ((uint64_t)b << n);
-  const bool rot = g.kind <= QC_G_RZ;
-  const double th = rot ? -theta[(int64_t)b * stride + g.param] : 0.0;  // U^dagger
-  const Mat2<R> U = block_matrix<R>(g.kind, th);
-  const uint64_t np = (g.kind == QC_G_CNOT) ? (1ull << (n - 2)) : (1ull << (n - 1));
-  Acc<R> acc;
-  for (uint64_t p = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; p < np; p += (uint64_t)gridDim.x * blockDim.x) {
-    uint64_t i1;
-    const uint64_t i0 = gate_pair(g, p, i1);
-    Cx<R> p0 = IO::ld(s + i0), p1 = IO::ld(s + i1);
-    Cx<R> l0 = IO::ld(l + i0), l1 = IO::ld(l + i1);
-    if (rot) acc_generator<R>(acc, g.kind, p0, p1, l0, l1);
-    apply_any<R>(g.kind, U, p0, p1);
-    apply_any<R>(g.kind, U, l0, l1);
-    IO::st(s + i0, p0);
-    IO::st(s + i1, p1);
-    IO::st(l + i0, l0);
-    IO::st(l + i1, l1);
-  }
-  if (rot) {
-    acc.flush();
-    const double t = block_reduce(acc.value());
-    if (threadIdx.x == 0) part[(int64_t)b * gridDim.x + blockIdx.x] = t;
+// A pass of the backward sweep undoes P (address map of the tile's load),
+// then D, then the operators of S last to first, on psi and lambda together.
+// The derivative of each rotation is taken where its own qubit has been
+// undone up to it: what other qubits' operators did meanwhile is unitary and
+// commutes with the generator, so it does not change Im <lambda|P|psi>.
+//
+//  - The derivatives of all of D's RZ come from one product
+//    w_j = Im(conj(lambda_j) psi_j) per amplitude and its signed sums: over a
+//    thread's register bits on the spot, over its other tile bits when the
+//    block is done (the sign is the thread's).
+//  - Those of S (RX, RY, inner RZ) are four products a pair.
+//
+// Sums: complex64 products exact as float pairs, a thread's pairs in float
+// pairs (Acc), then 64-bit fixed point; complex128 in FP64 per thread, then
+// two 64-bit words of fixed point.  Every sum is bounded by ||psi|| ||lambda||
+// <= sum_k |c_k|, which sets the point (accumulated integers do not depend on
+// the order of the blocks).
+template <typename R> struct Bwd;
+template <> struct Bwd<float> {
+  static constexpr int KT = 12, C0 = 4, T = 512, LV = 2, VE = 2;
+  using Z = float2;  // a thread's running sum
+};
+template <> struct Bwd<double> {
+  static constexpr int KT = 11, C0 = 3, T = 256, LV = 3, VE = 1;
+  using Z = double;
+};
+constexpr int BWD_SLOTS = TP_MAXOP + TP_MAXK + 3;  // sums of a pass: operators, then tile positions of D
+
+// Im <l|P|p> over the pairs of register bit BIT for a rotation's generator.
+template <int BIT, typename R>
+__device__ __forceinline__ void grad_bit(Acc<R>& acc, int mode, const Cx<R>* p, const Cx<R>* l) {
+  // Im(conj(a) b) = a.re b.im - a.im b.re
+#pragma unroll
+  for (int m = 0; m < 4; ++m) {
+    const int j0 = ((m >> BIT) << (BIT + 1)) | (m & ((1 << BIT) - 1)), j1 = j0 | (1 << BIT);
+    if (mode == OM_RZ) {  // Z: conj(l0) p0 - conj(l1) p1
+      acc.add(l[j0].re, p[j0].im); acc.sub(l[j0].im, p[j0].re);
+      acc.sub(l[j1].re, p[j1].im); acc.add(l[j1].im, p[j1].re);
+    } else if (mode == OM_RX0 || mode == OM_RX1) {  // X: conj(l0) p1 + conj(l1) p0
+      acc.add(l[j0].re, p[j1].im); acc.sub(l[j0].im, p[j1].re);
+      acc.add(l[j1].re, p[j0].im); acc.sub(l[j1].im, p[j0].re);
+    } else {  // Y: conj(l0)(-i p1) + conj(l1)(i p0); Im(conj(a)(-i b)) = -Re(conj(a) b)
+      acc.sub(l[j0].re, p[j1].re); acc.sub(l[j0].im, p[j1].im);
+      acc.add(l[j1].re, p[j0].re); acc.add(l[j1].im, p[j0].im);
+    }
   }
 }
 
-// Two rotations ga then gb (forward order) on one qubit, walked backwards:
-// gradient of gb, undo gb, gradient of ga, undo ga -- one pass.
+// value * 2^k, k up to twice an exponent's range
+__device__ __forceinline__ double scale2(double v, int k) { return ldexp(ldexp(v, k / 2), k - k / 2); }
+
+// Sum of a 64-bit integer over the warp (in every lane); |sum| < 2^57.
+__device__ __forceinline__ long long warp_sum(long long v) {
+  const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)(v & 0x3ffffff));
+  const int hi = __reduce_add_sync(0xffffffffu, (int)(v >> 26));
+  return ((long long)hi << 26) + (long long)lo;
+}
+
+// A block's sums: shared memory behind the two tiles.
+//   complex64: z[4][T] float pairs, y[nwarp][nop] integers
+//   complex128: z[4][T], y[nop][T] doubles
 template <typename R>
-__global__ void __launch_bounds__(ADJ_T) k_bwd_rot2(typename CT<R>::V2* __restrict__ psi,
-                                                    typename CT<R>::V2* __restrict__ lam, int n, GateDev ga,
-                                                    GateDev gb, const double* __restrict__ theta, int64_t stride,
-                                                    double* __restrict__ part_a, double* __restrict__ part_b) {
-  using IO = AmpIO<R>;
-  const int b = blockIdx.y;
-  typename CT<R>::V2* s = psi + ((uint64_t)b << n);
-  typename CT<R>::V2* l = lam + ((uint64_t)b << n);
-  const Mat2<R> Ua = block_matrix<R>(ga.kind, -theta[(int64_t)b * stride + ga.param]);
-  const Mat2<R> Ub = block_matrix<R>(gb.kind, -theta[(int64_t)b * stride + gb.param]);
-  const int q = ga.q0;
-  const uint64_t np = 1ull << (n - 1);
-  Acc<R> acca, accb;
-  for (uint64_t p = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; p < np; p += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t i0 = insert0(p, q), i1 = i0 | (1ull << q);
-    Cx<R> p0 = IO::ld(s + i0), p1 = IO::ld(s + i1);
-    Cx<R> l0 = IO::ld(l + i0), l1 = IO::ld(l + i1);
-    acc_generator<R>(accb, gb.kind, p0, p1, l0, l1);
-    apply_any<R>(gb.kind, Ub, p0, p1);
-    apply_any<R>(gb.kind, Ub, l0, l1);
-    acc_generator<R>(acca, ga.kind, p0, p1, l0, l1);
-    apply_any<R>(ga.kind, Ua, p0, p1);
-    apply_any<R>(ga.kind, Ua, l0, l1);
-    IO::st(s + i0, p0);
-    IO::st(s + i1, p1);
-    IO::st(l + i0, l0);
-    IO::st(l + i1, l1);
+struct BwdSums {
+  typename Bwd<R>::Z* z;
+  void* y;
+  int bad;  // this thread saw a non-finite sum
+};
+template <typename R>
+__host__ __device__ inline size_t bwd_sum_bytes(int T, int nop) {
+  return sizeof(typename Bwd<R>::Z) * 4 * T + (sizeof(R) == 4 ? (size_t)8 * (T / 32) * nop : (size_t)8 * T * nop);
+}
+
+template <typename R>
+__device__ __forceinline__ void bwd_zero_sums(BwdSums<R>& S, int nop) {
+  const int T = blockDim.x, words = (int)(bwd_sum_bytes<R>(T, nop) / 8);
+  for (int i = threadIdx.x; i < words; i += T) reinterpret_cast<unsigned long long*>(S.z)[i] = 0ull;
+}
+
+// kq: the fixed point of complex64 sums (k_prep adds each operator's own part)
+template <typename R>
+__device__ __forceinline__ void bwd_rounds(const TilePass& P, typename CT<R>::V2* sp, typename CT<R>::V2* sl,
+                                           const PassRec<R>* rec, BwdSums<R>& S, int kq) {
+  constexpr int RB = 3, NA = 8;
+  const int tid = threadIdx.x, T = blockDim.x;
+  const bool active = tid < (1 << (P.kt - RB));
+#pragma unroll 1
+  for (int r = 0; r < P.nround; ++r) {
+    const TileRound& rd = P.rd[r];
+    const int base = active ? tp_round_base<R, RB>(rd) : 0;
+    int bas[RB];
+#pragma unroll
+    for (int x = 0; x < RB; ++x) bas[x] = rd.bas[x];
+    Cx<R> p[NA], l[NA];
+#pragma unroll
+    for (int j = 0; j < NA; ++j) {
+      const int at = tp_round_at<RB>(base, bas, j);
+      p[j] = AmpIO<R>::ld(sm_at(sp, at));
+      l[j] = AmpIO<R>::ld(sm_at(sl, at));
+    }
+    if (!active) {  // lanes past a small tile take part in the warp sums only
+#pragma unroll
+      for (int j = 0; j < NA; ++j) p[j] = l[j] = cmake<R>((R)0, (R)0);
+    }
+    if (r == 0 && P.has_diag) {
+      Acc<R> w[NA], z[RB];
+#pragma unroll
+      for (int j = 0; j < NA; ++j) {
+        w[j].add(l[j].re, p[j].im);
+        w[j].sub(l[j].im, p[j].re);
+      }
+#pragma unroll
+      for (int x = 0; x < RB; ++x) {
+#pragma unroll
+        for (int j = 0; j < (NA >> (x + 1)); ++j) {  // bit x: w[2j] - w[2j+1], then the sum for the next bits
+          z[x].merge(w[2 * j]);
+          z[x].merge_neg(w[2 * j + 1]);
+          w[j] = w[2 * j];
+          w[j].merge(w[2 * j + 1]);
+        }
+      }
+      w[0].into(S.z[tid]);
+#pragma unroll
+      for (int x = 0; x < RB; ++x) z[x].into(S.z[(1 + x) * T + tid]);
+      S.bad |= !w[0].finite();
+    }
+    if (r == 0 && (P.has_diag || P.nop)) {
+      const auto A = rec->tab[tid & 31], Bw = rec->tab[32 + (tid >> 5)];
+      const Cx<R> d = cmul(cmake<R>(A.x, A.y), cmake<R>(Bw.x, Bw.y));
+#pragma unroll
+      for (int j = 0; j < NA; ++j) {
+        const auto J = rec->tab[48 + j];
+        const Cx<R> f = cmul(d, cmake<R>(J.x, J.y));
+        p[j] = cmul(p[j], f);
+        l[j] = cmul(l[j], f);
+      }
+    }
+#pragma unroll 1
+    for (int k = rd.op0; k < rd.op1; ++k) {
+      const OpRec<R> o = rec->op[k];
+      Acc<R> acc;
+      switch (P.op[k].bit) {
+        case 0:
+          if (o.mode != OM_H) grad_bit<0>(acc, o.mode, p, l);
+          op_bit<0, RB, R>(o, p);
+          op_bit<0, RB, R>(o, l);
+          break;
+        case 1:
+          if (o.mode != OM_H) grad_bit<1>(acc, o.mode, p, l);
+          op_bit<1, RB, R>(o, p);
+          op_bit<1, RB, R>(o, l);
+          break;
+        default:
+          if (o.mode != OM_H) grad_bit<2>(acc, o.mode, p, l);
+          op_bit<2, RB, R>(o, p);
+          op_bit<2, RB, R>(o, l);
+          break;
+      }
+      S.bad |= !acc.finite();
+      if constexpr (sizeof(R) == 4) {
+        const long long v = warp_sum(acc.fixed(kq + o.eq));
+        long long* y = reinterpret_cast<long long*>(S.y) + (tid >> 5) * P.nop + k;
+        if ((tid & 31) == 0) *y += v;
+      } else {
+        reinterpret_cast<double*>(S.y)[k * T + tid] += acc.value();
+      }
+    }
+    if (active) {
+#pragma unroll
+      for (int j = 0; j < NA; ++j) {
+        const int at = tp_round_at<RB>(base, bas, j);
+        AmpIO<R>::st(sm_at(sp, at), p[j]);
+        AmpIO<R>::st(sm_at(sl, at), l[j]);
+      }
+    }
+    __syncthreads();
   }
-  acca.flush();
-  accb.flush();
-  const double ta = block_reduce(acca.value());
-  const double tb = block_reduce(accb.value());
-  if (threadIdx.x == 0) {
-    part_a[(int64_t)b * gridDim.x + blockIdx.x] = ta;
-    part_b[(int64_t)b * gridDim.x + blockIdx.x] = tb;
+}
+
+// acc[2 slot + word] of one batch element; a non-finite sum sets the flag.
+__device__ __forceinline__ void bwd_add(unsigned long long* acc, int slot, double v, int k) {
+  const double x = scale2(v, k), hi = rint(x);
+  if (!isfinite(x)) return;
+  atomicAdd(acc + 2 * slot, (unsigned long long)(long long)hi);
+  atomicAdd(acc + 2 * slot + 1, (unsigned long long)__double2ll_rn((x - hi) * 4503599627370496.0));
+}
+template <typename R>
+__device__ __forceinline__ void bwd_flush(const TilePass& P, const PassRec<R>* rec, BwdSums<R>& S, int kq,
+                                          unsigned long long* __restrict__ acc, int* __restrict__ flag) {
+  const int tid = threadIdx.x, T = blockDim.x, lane = tid & 31, wp = tid >> 5, nw = T >> 5;
+  if (S.bad) *flag = 1;
+  __syncthreads();
+  if constexpr (sizeof(R) == 4) {
+    const long long* y = reinterpret_cast<const long long*>(S.y);
+    for (int k = tid; k < P.nop; k += T) {
+      long long v = 0;
+      for (int w = 0; w < nw; ++w) v += y[w * P.nop + k];
+      if (v) atomicAdd(acc + 2 * k, (unsigned long long)v);
+    }
+  } else {
+    const double* y = reinterpret_cast<const double*>(S.y);
+    for (int k = wp; k < P.nop; k += nw) {
+      double v = 0.0;
+      for (int i = lane; i < T; i += 32) v += y[k * T + i];
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (lane == 0) bwd_add(acc, k, v, kq + rec->op[k].eq);
+    }
+  }
+  if (!P.has_diag) return;
+  int i = 0, x = 0;
+  for (int p = 0; p < P.kt; ++p) {
+    const bool reg = x < 3 && P.rd[0].r[x] == p;
+    const int slot = reg ? 1 + x : 0, bit = reg ? -1 : i;
+    if (reg) ++x;
+    else ++i;
+    if (P.dp[p] < 0 || (p % nw) != wp) continue;
+    if constexpr (sizeof(R) == 4) {
+      long long v = 0;
+      for (int t = lane; t < T; t += 32) {
+        Acc<float> a;
+        a.s = S.z[slot * T + t].x;
+        a.c = S.z[slot * T + t].y;
+        const long long f = a.fixed(kq);
+        v += (bit >= 0 && ((t >> bit) & 1)) ? -f : f;
+      }
+      v = warp_sum(v);
+      if (lane == 0 && v) atomicAdd(acc + 2 * (TP_MAXOP + p), (unsigned long long)v);
+    } else {
+      double v = 0.0;
+      for (int t = lane; t < T; t += 32) {
+        const double f = S.z[slot * T + t];
+        v += (bit >= 0 && ((t >> bit) & 1)) ? -f : f;
+      }
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (lane == 0) bwd_add(acc, TP_MAXOP + p, v, kq);
+    }
+  }
+}
+
+// One pass over the batch: tiles blockIdx.x + gridDim.x i of state blockIdx.y.
+template <typename R>
+__global__ void __launch_bounds__(Bwd<R>::T, 2) k_bwd_tile(typename CT<R>::V2* __restrict__ psi,
+                                                           typename CT<R>::V2* __restrict__ lam, int n, int ntiles,
+                                                           const __grid_constant__ TilePass P,
+                                                           const PassRec<R>* __restrict__ recs, int kq,
+                                                           unsigned long long* __restrict__ acc, int* __restrict__ flag) {
+  using V2 = typename CT<R>::V2;
+  using V = typename Vec<R>::T;
+  constexpr int NV = 1 << Bwd<R>::LV;
+  extern __shared__ __align__(16) unsigned char dynsm[];
+  V2* sp = reinterpret_cast<V2*>(dynsm);
+  V2* sl = sp + (1 << P.kt);
+  PassRec<R>* rec = reinterpret_cast<PassRec<R>*>(sl + (1 << P.kt));
+  BwdSums<R> S{reinterpret_cast<typename Bwd<R>::Z*>(rec + 1), nullptr, 0};
+  S.y = S.z + 4 * blockDim.x;
+  const int tid = threadIdx.x, T = blockDim.x;
+  const bool al = ((reinterpret_cast<uintptr_t>(psi) | reinterpret_cast<uintptr_t>(lam)) & 15) == 0;
+  {
+    const uint4* src = reinterpret_cast<const uint4*>(recs + blockIdx.y);
+    for (int i = tid; i < (int)(sizeof(PassRec<R>) / 16); i += T) reinterpret_cast<uint4*>(rec)[i] = src[i];
+  }
+  bwd_zero_sums<R>(S, P.nop);
+  TileShare<R, Bwd<R>::LV> sh;
+  sh.init(P, T);
+  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const uint64_t base = tp_tile_base(P, tile);
+    V2* gp = psi + ((uint64_t)blockIdx.y << n) + base;
+    V2* gl = lam + ((uint64_t)blockIdx.y << n) + base;
+    const int cst = tp_cst(P, base);
+    V vp[NV], vl[NV];
+#pragma unroll
+    for (int u = 0; u < NV; ++u) vp[u] = Vec<R>::ld(gp + sh.g(u), al);
+#pragma unroll
+    for (int u = 0; u < NV; ++u) vl[u] = Vec<R>::ld(gl + sh.g(u), al);
+#pragma unroll
+    for (int u = 0; u < NV; ++u) {
+      const int s = sh.s(u) ^ cst;
+      Vec<R>::to_sm(sp, s, s ^ sh.s1, vp[u]);
+      Vec<R>::to_sm(sl, s, s ^ sh.s1, vl[u]);
+    }
+    __syncthreads();
+    bwd_rounds<R>(P, sp, sl, rec, S, kq);
+#pragma unroll
+    for (int u = 0; u < NV; ++u) {
+      const int a = sh.a(u), a1 = a ^ tp_at<R>(1);
+      Vec<R>::st(gp + sh.g(u), Vec<R>::from_sm(sp, a, a1), al);
+      Vec<R>::st(gl + sh.g(u), Vec<R>::from_sm(sl, a, a1), al);
+    }
+    __syncthreads();
+  }
+  bwd_flush<R>(P, rec, S, kq, acc + (size_t)blockIdx.y * BWD_SLOTS * 2, flag + blockIdx.y);
+}
+
+// The whole backward sweep of states that fit one tile, one block a state.
+template <typename R>
+__global__ void __launch_bounds__(Bwd<R>::T, 2) k_bwd_whole(const typename CT<R>::V2* __restrict__ psi,
+                                                            const typename CT<R>::V2* __restrict__ lam, int n,
+                                                            const TilePass* __restrict__ passes, int npass,
+                                                            const PassRec<R>* __restrict__ recs, int kq,
+                                                            unsigned long long* __restrict__ acc, int* __restrict__ flag,
+                                                            int B) {
+  using V2 = typename CT<R>::V2;
+  using V = typename Vec<R>::T;
+  constexpr int NV = 1 << Bwd<R>::LV, VE = Bwd<R>::VE;
+  extern __shared__ __align__(16) unsigned char dynsm[];
+  __shared__ TilePass P;
+  const int tid = threadIdx.x, T = blockDim.x, kt = passes[0].kt, b = blockIdx.x;
+  V2* sp = reinterpret_cast<V2*>(dynsm);
+  V2* sl = sp + (1 << kt);
+  PassRec<R>* rec = reinterpret_cast<PassRec<R>*>(sl + (1 << kt));
+  BwdSums<R> S{reinterpret_cast<typename Bwd<R>::Z*>(rec + 1), nullptr, 0};
+  S.y = S.z + 4 * T;
+  const V2 zero = CT<R>::make((R)0, (R)0);
+  for (int e = tid; e < (1 << kt); e += T) {
+    *sm_at(sp, tp_at<R>(e)) = e < (1 << n) ? psi[((uint64_t)b << n) + e] : zero;
+    *sm_at(sl, tp_at<R>(e)) = e < (1 << n) ? lam[((uint64_t)b << n) + e] : zero;
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int k = npass - 1; k >= 0; --k) {
+    for (int i = tid; i < (int)sizeof(TilePass) / 4; i += T)
+      reinterpret_cast<uint32_t*>(&P)[i] = reinterpret_cast<const uint32_t*>(passes + k)[i];
+    const uint4* src = reinterpret_cast<const uint4*>(recs + (size_t)k * B + b);
+    for (int i = tid; i < (int)(sizeof(PassRec<R>) / 16); i += T) reinterpret_cast<uint4*>(rec)[i] = src[i];
+    __syncthreads();
+    bwd_zero_sums<R>(S, P.nop);
+    if (P.has_perm) {
+      TileShare<R, Bwd<R>::LV> sh;
+      sh.init(P, T);
+      V vp[NV], vl[NV];
+#pragma unroll
+      for (int u = 0; u < NV; ++u)
+        if ((tid + T * u) * VE < (1 << kt)) {
+          const int a = sh.a(u), a1 = a ^ tp_at<R>(1);
+          vp[u] = Vec<R>::from_sm(sp, a, a1);
+          vl[u] = Vec<R>::from_sm(sl, a, a1);
+        }
+      __syncthreads();
+#pragma unroll
+      for (int u = 0; u < NV; ++u)
+        if ((tid + T * u) * VE < (1 << kt)) {
+          const int s = sh.s(u);
+          Vec<R>::to_sm(sp, s, s ^ sh.s1, vp[u]);
+          Vec<R>::to_sm(sl, s, s ^ sh.s1, vl[u]);
+        }
+    }
+    __syncthreads();
+    bwd_rounds<R>(P, sp, sl, rec, S, kq);
+    bwd_flush<R>(P, rec, S, kq, acc + ((size_t)k * B + b) * BWD_SLOTS * 2, flag + b);
+    __syncthreads();
+  }
+}
+
+// The sums of pass blockIdx.x, element blockIdx.y, into the gradient.
+template <typename R>
+__global__ void __launch_bounds__(64) k_bwd_finish(const TilePass* __restrict__ passes, const PassRec<R>* __restrict__ recs,
+                                                   const unsigned long long* __restrict__ acc,
+                                                   const int* __restrict__ flag, int B, int kq, double* __restrict__ grad,
+                                                   int64_t stride) {
+  const TilePass& P = passes[blockIdx.x];
+  const int64_t pb = (int64_t)blockIdx.x * B + blockIdx.y;
+  for (int slot = threadIdx.x; slot < BWD_SLOTS; slot += blockDim.x) {
+    const bool op = slot < TP_MAXOP;
+    if (op ? slot >= P.nop : P.dp[slot - TP_MAXOP] < 0) continue;
+    const int par = op ? P.op[slot].pa : P.dp[slot - TP_MAXOP];
+    if (par < 0) continue;  // H
+    const OpRec<R>* o = op ? &recs[pb].op[slot] : nullptr;
+    const unsigned long long* a = acc + (pb * BWD_SLOTS + slot) * 2;
+    double v = (double)(long long)a[0] + (double)(long long)a[1] * 2.220446049250313e-16;
+    v = scale2(v, -(kq + (op ? o->eq : 0)));
+    if (op) v *= o->f;
+    if (flag[blockIdx.y]) v = __longlong_as_double(0x7ff8000000000000ll);
+    grad[(int64_t)blockIdx.y * stride + par] = v;
   }
 }
 
@@ -726,15 +948,15 @@ struct TermsDev {
 template <typename R>
 __global__ void __launch_bounds__(ADJ_T) k_apply_h(const typename CT<R>::V2* __restrict__ psi,
                                                    typename CT<R>::V2* __restrict__ lam, int n,
-                                                   const TermsDev* __restrict__ T) {
+                                                   const __grid_constant__ TermsDev T) {
   const int b = blockIdx.y;
   const typename CT<R>::V2* s = psi + ((uint64_t)b << n);
   typename CT<R>::V2* l = lam + ((uint64_t)b << n);
   const uint64_t N = 1ull << n;
   for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j < N; j += (uint64_t)gridDim.x * blockDim.x) {
     R ar = 0, ai = 0;
-    for (int k = 0; k < T->nt; ++k) {
-      const uint64_t x = T->x[k], z = T->z[k];
+    for (int k = 0; k < T.nt; ++k) {
+      const uint64_t x = T.x[k], z = T.z[k];
       const auto v = s[j ^ x];
       R vr = v.x, vi = v.y;
       if (__popcll((j ^ x) & z) & 1) {
@@ -746,7 +968,7 @@ __global__ void __launch_bounds__(ADJ_T) k_apply_h(const typename CT<R>::V2* __r
       if (ny == 1) { wr = -vi; wi = vr; }
       else if (ny == 2) { wr = -vr; wi = -vi; }
       else if (ny == 3) { wr = vi; wi = -vr; }
-      const R c = (R)T->c[k];
+      const R c = (R)T.c[k];
       ar = fma(c, wr, ar);
       ai = fma(c, wi, ai);
     }
@@ -775,38 +997,6 @@ __global__ void __launch_bounds__(ADJ_T) k_energy(const typename CT<R>::V2* __re
 }
 
 // ------------------------------------------------------------ host side --
-enum AdjOpKind { AOP_GATE = 0, AOP_ROT2 = 1, AOP_RING = 2 };
-struct AdjOp {
-  int kind;
-  GateDev a, b;
-};
-
-static GateDev gdev(const qc_gate& g) { return GateDev{g.kind, g.q0, g.q1, g.param}; }
-
-// Compile the gate list into passes (see the file comment).
-static std::vector<AdjOp> compile_ops(const qc_gate* gates, int ng, int n) {
-  std::vector<AdjOp> ops;
-  int i = 0;
-  while (i < ng) {
-    bool ring = (i + n <= ng) && n >= 2;
-    for (int k = 0; ring && k < n; ++k)
-      ring = gates[i + k].kind == QC_G_CNOT && gates[i + k].q0 == k && gates[i + k].q1 == (k + 1) % n;
-    if (ring) {
-      ops.push_back(AdjOp{AOP_RING, GateDev{QC_G_CNOT, 0, 1, 0}, GateDev{QC_G_CNOT, 0, 1, 0}});
-      i += n;
-      continue;
-    }
-    if (i + 1 < ng && gates[i].kind <= QC_G_RZ && gates[i + 1].kind <= QC_G_RZ && gates[i].q0 == gates[i + 1].q0) {
-      ops.push_back(AdjOp{AOP_ROT2, gdev(gates[i]), gdev(gates[i + 1])});
-      i += 2;
-      continue;
-    }
-    ops.push_back(AdjOp{AOP_GATE, gdev(gates[i]), gdev(gates[i])});
-    ++i;
-  }
-  return ops;
-}
-
 static qc_status check_circuit(int n, qc_dtype dt, int B, const qc_gate* gates, int n_gates, int64_t stride,
                                int n_params) {
   if (n < 2 || n > 30) {
@@ -848,20 +1038,12 @@ template <typename R>
 static unsigned gx_for(int n, int B) {
   const uint64_t pairs = 1ull << (n - 1);
   uint64_t gx = (pairs + ADJ_T - 1) / ADJ_T;
-  const int res = std::min(resident_blocks((const void*)k_bwd_rot2<R>, ADJ_T, 0),
-                           resident_blocks((const void*)k_bwd_gate<R>, ADJ_T, 0));
+  const int res = std::min(resident_blocks((const void*)k_apply_h<R>, ADJ_T, 0),
+                           resident_blocks((const void*)k_energy<R>, ADJ_T, 0));
   const uint64_t cap = std::max<uint64_t>(1, (uint64_t)sm_count() * res / (uint64_t)B);
   gx = std::min<uint64_t>(gx, std::min<uint64_t>(cap, ADJ_GX_MAX));
   return (unsigned)std::max<uint64_t>(gx, 1);
 }
-
-// Buffers rotate among the caller's psi and lam and one workspace.
-template <typename R>
-struct Bufs {
-  typename CT<R>::V2* psi;
-  typename CT<R>::V2* lam;
-  typename CT<R>::V2* spare;
-};
 
 // Passes of a forward sweep on the device, with room for the operators of as
 // many batch elements at a time as fit PREP_BYTES.
@@ -884,7 +1066,6 @@ static cudaError_t fwd_plan(FwdPlan<R>& F, const qc_gate* gates, int ng, int n, 
   F.chunk = (int)std::max<size_t>(1, std::min<size_t>(B, PREP_BYTES / per));
   cudaError_t e = cudaMallocAsync((void**)&F.dpass, (F.passes.size() * sizeof(TilePass) + 15) / 16 * 16, st);
   if (e == cudaSuccess) e = cudaMallocAsync((void**)&F.recs, per * F.chunk, st);
-  if (e != cudaSuccess && F.dpass) cudaFreeAsync(F.dpass, st);
   return e;
 }
 template <typename R>
@@ -933,21 +1114,89 @@ static int forward_passes(const FwdPlan<R>& F, int n, int B, const double* theta
   return nk;
 }
 
-static bool has_ring(const std::vector<AdjOp>& ops) {
-  for (const AdjOp& o : ops)
-    if (o.kind == AOP_RING) return true;
-  return false;
-}
-
 template <typename R>
 static qc_status forward_impl(int n, int B, const qc_gate* gates, int n_gates, const double* theta,
                               int64_t stride, void* psi, cudaStream_t st) {
   FwdPlan<R> F;
   const cudaError_t e = fwd_plan(F, gates, n_gates, n, B, st);
-  if (e != cudaSuccess) return cuda_fail(e, "forward workspace");
+  if (e != cudaSuccess) {
+    fwd_plan_free(F, st);
+    return cuda_fail(e, "forward workspace");
+  }
   const int nk = forward_passes<R>(F, n, B, theta, stride, reinterpret_cast<typename CT<R>::V2*>(psi), st);
   fwd_plan_free(F, st);
   return check_launch("circuit forward", nk);
+}
+
+// The backward sweep on the device: passes, and the operators and sums of as
+// many batch elements at a time as fit PREP_BYTES.
+template <typename R>
+struct BwdPlan {
+  std::vector<TilePass> passes;
+  TilePass* dpass = nullptr;
+  PassRec<R>* recs = nullptr;
+  unsigned long long* acc = nullptr;  // sums, then a flag per element
+  int chunk = 0;
+  size_t acc_bytes(int nb) const { return passes.size() * nb * BWD_SLOTS * 16 + sizeof(int) * (size_t)nb; }
+};
+template <typename R>
+static cudaError_t bwd_plan(BwdPlan<R>& W, const qc_gate* gates, int ng, int n, int B, cudaStream_t st) {
+  W.passes = build_passes<R>(gates, ng, n, TileCfg{Bwd<R>::KT, Bwd<R>::C0, 3, false, true});
+  if (W.passes.empty()) return cudaSuccess;
+  const size_t np = W.passes.size();
+  W.chunk = (int)std::max<size_t>(1, std::min<size_t>(B, PREP_BYTES / (np * (sizeof(PassRec<R>) + BWD_SLOTS * 16))));
+  cudaError_t e = cudaMallocAsync((void**)&W.dpass, (np * sizeof(TilePass) + 15) / 16 * 16, st);
+  if (e == cudaSuccess) e = cudaMallocAsync((void**)&W.recs, np * W.chunk * sizeof(PassRec<R>), st);
+  if (e == cudaSuccess) e = cudaMallocAsync((void**)&W.acc, W.acc_bytes(W.chunk), st);
+  return e;
+}
+template <typename R>
+static void bwd_plan_free(BwdPlan<R>& W, cudaStream_t st) {
+  if (W.dpass) cudaFreeAsync(W.dpass, st);
+  if (W.recs) cudaFreeAsync(W.recs, st);
+  if (W.acc) cudaFreeAsync(W.acc, st);
+}
+
+// Walks the circuit back from psi and lambda; kq: fixed point of the sums.
+template <typename R>
+static int backward_passes(const BwdPlan<R>& W, int n, int B, const double* theta, int64_t stride, int kq,
+                           typename CT<R>::V2* psi, typename CT<R>::V2* lam, double* grad, cudaStream_t st) {
+  if (W.passes.empty()) return 0;
+  const int np = (int)W.passes.size();
+  int nk = put_bytes(W.dpass, W.passes.data(), np * sizeof(TilePass), st), maxop = 0;
+  for (const TilePass& P : W.passes) maxop = std::max<int>(maxop, P.nop);
+  const int kt = W.passes[0].kt, T = std::max(32, 1 << (kt - 3));
+  const size_t tiles2 = 2 * (sizeof(typename CT<R>::V2) << kt) + sizeof(PassRec<R>);
+  allow_smem(k_bwd_tile<R>, tiles2 + bwd_sum_bytes<R>(T, maxop));
+  allow_smem(k_bwd_whole<R>, tiles2 + bwd_sum_bytes<R>(T, maxop));
+  for (int b0 = 0; b0 < B; b0 += W.chunk) {
+    const int nb = std::min(W.chunk, B - b0);
+    const double* th = theta + (int64_t)b0 * stride;
+    typename CT<R>::V2 *p = psi + ((uint64_t)b0 << n), *l = lam + ((uint64_t)b0 << n);
+    cudaMemsetAsync(W.acc, 0, W.acc_bytes(nb), st);
+    int* flag = reinterpret_cast<int*>(W.acc + (size_t)np * nb * BWD_SLOTS * 2);
+    k_prep<R><<<dim3(np, nb), 128, 0, st>>>(W.dpass, W.recs, nb, th, stride, -1);
+    ++nk;
+    if (n <= kt) {
+      k_bwd_whole<R><<<nb, T, tiles2 + bwd_sum_bytes<R>(T, maxop), st>>>(p, l, n, W.dpass, np, W.recs, kq, W.acc, flag,
+                                                                        nb);
+      ++nk;
+    } else {
+      // a block takes up to eight tiles of a state (its sums then cost
+      // little), as long as six waves of blocks remain
+      const int64_t tiles = 1ll << (n - kt), all = tiles * nb;
+      const int64_t per = std::max<int64_t>(1, std::min<int64_t>({8, tiles, all / (12ll * sm_count())}));
+      const dim3 grid((unsigned)((tiles + per - 1) / per), nb);
+      for (int k = np - 1; k >= 0; --k, ++nk)
+        k_bwd_tile<R><<<grid, T, tiles2 + bwd_sum_bytes<R>(T, W.passes[k].nop), st>>>(
+            p, l, n, (int)tiles, W.passes[k], W.recs + (size_t)k * nb, kq, W.acc + (size_t)k * nb * BWD_SLOTS * 2,
+            flag);
+    }
+    k_bwd_finish<R><<<dim3(np, nb), 64, 0, st>>>(W.dpass, W.recs, W.acc, flag, nb, kq, grad + (int64_t)b0 * stride,
+                                                 stride);
+    ++nk;
+  }
+  return nk;
 }
 
 template <typename R>
@@ -955,76 +1204,46 @@ static qc_status adjoint_impl(int n, int B, const qc_gate* gates, int n_gates, c
                               int64_t stride, const qc_pauli_term* H, int n_terms, void* psi, void* lam,
                               double* energy, double* grad, cudaStream_t st) {
   using V2 = typename CT<R>::V2;
-  const std::vector<AdjOp> ops = compile_ops(gates, n_gates, n);
-  const size_t bytes = ((size_t)B << n) * sizeof(V2);
   const unsigned gx = gx_for<R>(n, B);
   const dim3 grid(gx, B);
-  // workspace: Hamiltonian terms, two partial arrays, one state buffer
-  TermsDev* dT = nullptr;
+  V2 *p = reinterpret_cast<V2*>(psi), *l = reinterpret_cast<V2*>(lam);
   double* part = nullptr;
-  V2* ws = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&dT, sizeof(TermsDev), st);
-  if (e == cudaSuccess) e = cudaMallocAsync((void**)&part, sizeof(double) * 2 * (size_t)gx * B, st);
-  if (e == cudaSuccess && has_ring(ops)) e = cudaMallocAsync((void**)&ws, bytes, st);
   FwdPlan<R> F;
+  BwdPlan<R> W;
+  cudaError_t e = cudaMallocAsync((void**)&part, sizeof(double) * (size_t)gx * B, st);
   if (e == cudaSuccess) e = fwd_plan(F, gates, n_gates, n, B, st);
-  TermsDev* hT = nullptr;
-  if (e == cudaSuccess) e = cudaMallocHost((void**)&hT, sizeof(TermsDev));
-  if (e != cudaSuccess) {
-    if (dT) cudaFreeAsync(dT, st);
-    if (part) cudaFreeAsync(part, st);
-    if (ws) cudaFreeAsync(ws, st);
-    fwd_plan_free(F, st);
-    return cuda_fail(e, "adjoint workspace");
-  }
-  double* part_b = part + (size_t)gx * B;
-  hT->nt = n_terms;
-  for (int k = 0; k < n_terms; ++k) {
-    hT->x[k] = H[k].xmask;
-    hT->z[k] = H[k].zmask;
-    hT->c[k] = H[k].coeff;
-  }
-  e = cudaMemcpyAsync(dT, hT, sizeof(TermsDev), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(grad, 0, sizeof(double) * (size_t)B * stride, st);
+  if (e == cudaSuccess) e = bwd_plan(W, gates, n_gates, n, B, st);
   qc_status s = QC_OK;
-  if (e != cudaSuccess) s = cuda_fail(e, "adjoint setup");
-  if (!s) {
-    Bufs<R> bf{reinterpret_cast<V2*>(psi), reinterpret_cast<V2*>(lam), ws};
-    int nk = forward_passes<R>(F, n, B, theta, stride, bf.psi, st);
-    k_apply_h<R><<<grid, ADJ_T, 0, st>>>(bf.psi, bf.lam, n, dT);
-    k_energy<R><<<grid, ADJ_T, 0, st>>>(bf.psi, bf.lam, n, part);
-    k_final_batch<<<B, ADJ_T, 0, st>>>(part, gx, energy, 1, 0);
-    nk += 3;
-    for (int i = (int)ops.size() - 1; i >= 0; --i) {
-      const AdjOp& op = ops[i];
-      if (op.kind == AOP_RING) {
-        k_ring<R><<<grid, ADJ_T, 0, st>>>(bf.psi, bf.spare, n, 1);
-        std::swap(bf.psi, bf.spare);
-        k_ring<R><<<grid, ADJ_T, 0, st>>>(bf.lam, bf.spare, n, 1);
-        std::swap(bf.lam, bf.spare);
-        nk += 2;
-      } else if (op.kind == AOP_ROT2) {
-        k_bwd_rot2<R><<<grid, ADJ_T, 0, st>>>(bf.psi, bf.lam, n, op.a, op.b, theta, stride, part, part_b);
-        k_final_batch<<<B, ADJ_T, 0, st>>>(part_b, gx, grad, stride, op.b.param);
-        k_final_batch<<<B, ADJ_T, 0, st>>>(part, gx, grad, stride, op.a.param);
-        nk += 3;
-      } else {
-        k_bwd_gate<R><<<grid, ADJ_T, 0, st>>>(bf.psi, bf.lam, n, op.a, theta, stride, part);
-        ++nk;
-        if (op.a.kind <= QC_G_RZ) {
-          k_final_batch<<<B, ADJ_T, 0, st>>>(part, gx, grad, stride, op.a.param);
-          ++nk;
-        }
-      }
+  if (e == cudaSuccess) {
+    TermsDev T;
+    double bound = 0.0;  // ||H|| <= sum |c_k|
+    T.nt = n_terms;
+    for (int k = 0; k < n_terms; ++k) {
+      T.x[k] = H[k].xmask;
+      T.z[k] = H[k].zmask;
+      T.c[k] = H[k].coeff;
+      bound += std::fabs(H[k].coeff) / 64.0;
     }
-    s = check_launch("adjoint", nk);
+    // sums stay below 2^55 units: bound * 64 < 2^(ilogb + 7)
+    int kq = 55 - (bound > 0.0 ? std::ilogb(bound) + 7 : 0);
+    if (sizeof(R) == 4) kq = std::min(160, std::max(-160, kq));  // past this H is 0 or infinite in complex64
+    e = cudaMemsetAsync(grad, 0, sizeof(double) * (size_t)B * stride, st);
+    if (e != cudaSuccess) s = cuda_fail(e, "adjoint setup");
+    if (!s) {
+      int nk = forward_passes<R>(F, n, B, theta, stride, p, st);
+      k_apply_h<R><<<grid, ADJ_T, 0, st>>>(p, l, n, T);
+      k_energy<R><<<grid, ADJ_T, 0, st>>>(p, l, n, part);
+      k_final_batch<<<B, ADJ_T, 0, st>>>(part, gx, energy, 1, 0);
+      nk += 3 + backward_passes<R>(W, n, B, theta, stride, kq, p, l, grad, st);
+      s = check_launch("adjoint", nk);
+    }
+  } else {
+    s = cuda_fail(e, "adjoint workspace");
   }
-  e = cudaStreamSynchronize(st);  // the pinned term list is freed below
-  cudaFreeHost(hT);
-  cudaFreeAsync(dT, st);
-  cudaFreeAsync(part, st);
-  if (ws) cudaFreeAsync(ws, st);
+  e = cudaStreamSynchronize(st);
+  if (part) cudaFreeAsync(part, st);
   fwd_plan_free(F, st);
+  bwd_plan_free(W, st);
   if (!s && e != cudaSuccess) s = cuda_fail(e, "adjoint");
   return s;
 }
