@@ -109,10 +109,14 @@ template <> struct Acc<float> {
     z = make_float2(t.s, t.c);
   }
   __device__ bool finite() const { return isfinite(s); }
-  // (s + c) 2^k rounded to an integer (k may exceed a float's range of exponents)
-  __device__ long long fixed(int k) const {
-    const float f0 = __int_as_float((127 + k / 2) << 23), f1 = __int_as_float((127 + k - k / 2) << 23);
-    return __float2ll_rn(s * f0 * f1) + __float2ll_rn(c * f0 * f1);
+  // (s + c) 2^k as hi 2^26 + lo, to a unit (k may exceed a float's range of
+  // exponents; no 64-bit conversion, which would run on the FP64 pipe)
+  __device__ int2 fixed(int k) const {
+    const int e = k - 26;
+    const float f0 = __int_as_float((127 + e / 2) << 23), f1 = __int_as_float((127 + e - e / 2) << 23);
+    const float x = s * f0 * f1;
+    const int hi = __float2int_rn(x);
+    return make_int2(hi, __float2int_rn(((x - (float)hi) + c * f0 * f1) * 67108864.f));
   }
 };
 
@@ -590,34 +594,46 @@ template <> struct Bwd<double> {
 };
 constexpr int BWD_SLOTS = TP_MAXOP + TP_MAXK + 3;  // sums of a pass: operators, then tile positions of D
 
-// Im <l|P|p> over the pairs of register bit BIT for a rotation's generator.
-template <int BIT, typename R>
-__device__ __forceinline__ void grad_bit(Acc<R>& acc, int mode, const Cx<R>* p, const Cx<R>* l) {
+// An operator's derivative term Im <l|P|p>, P its generator, over the pairs of
+// register bit BIT; then the operator on both states.
+template <int MODE, int BIT, typename R>
+__device__ __forceinline__ void bwd_mode(const R t, const R u, Acc<R>& acc, Cx<R>* p, Cx<R>* l) {
   // Im(conj(a) b) = a.re b.im - a.im b.re
 #pragma unroll
   for (int m = 0; m < 4; ++m) {
     const int j0 = ((m >> BIT) << (BIT + 1)) | (m & ((1 << BIT) - 1)), j1 = j0 | (1 << BIT);
-    if (mode == OM_RZ) {  // Z: conj(l0) p0 - conj(l1) p1
+    if (MODE == OM_RZ) {  // Z: conj(l0) p0 - conj(l1) p1
       acc.add(l[j0].re, p[j0].im); acc.sub(l[j0].im, p[j0].re);
       acc.sub(l[j1].re, p[j1].im); acc.add(l[j1].im, p[j1].re);
-    } else if (mode == OM_RX0 || mode == OM_RX1) {  // X: conj(l0) p1 + conj(l1) p0
+    } else if (MODE == OM_RX0 || MODE == OM_RX1) {  // X: conj(l0) p1 + conj(l1) p0
       acc.add(l[j0].re, p[j1].im); acc.sub(l[j0].im, p[j1].re);
       acc.add(l[j1].re, p[j0].im); acc.sub(l[j1].im, p[j0].re);
-    } else {  // Y: conj(l0)(-i p1) + conj(l1)(i p0); Im(conj(a)(-i b)) = -Re(conj(a) b)
+    } else if (MODE != OM_H) {  // Y: conj(l0)(-i p1) + conj(l1)(i p0); Im(conj(a)(-i b)) = -Re(conj(a) b)
       acc.sub(l[j0].re, p[j1].re); acc.sub(l[j0].im, p[j1].im);
       acc.add(l[j1].re, p[j0].re); acc.add(l[j1].im, p[j0].im);
     }
+  }
+  op_mode<MODE, BIT, 3>(t, u, p);
+  op_mode<MODE, BIT, 3>(t, u, l);
+}
+template <int BIT, typename R>
+__device__ __forceinline__ void bwd_bit(const OpRec<R>& o, Acc<R>& acc, Cx<R>* p, Cx<R>* l) {
+  switch (o.mode) {
+    case OM_RY0: bwd_mode<OM_RY0, BIT>(o.t, o.u, acc, p, l); break;
+    case OM_RY1: bwd_mode<OM_RY1, BIT>(o.t, o.u, acc, p, l); break;
+    case OM_RX0: bwd_mode<OM_RX0, BIT>(o.t, o.u, acc, p, l); break;
+    case OM_RX1: bwd_mode<OM_RX1, BIT>(o.t, o.u, acc, p, l); break;
+    case OM_RZ: bwd_mode<OM_RZ, BIT>(o.t, o.u, acc, p, l); break;
+    default: bwd_mode<OM_H, BIT>(o.t, o.u, acc, p, l); break;
   }
 }
 
 // value * 2^k, k up to twice an exponent's range
 __device__ __forceinline__ double scale2(double v, int k) { return ldexp(ldexp(v, k / 2), k - k / 2); }
 
-// Sum of a 64-bit integer over the warp (in every lane); |sum| < 2^57.
-__device__ __forceinline__ long long warp_sum(long long v) {
-  const unsigned lo = __reduce_add_sync(0xffffffffu, (unsigned)(v & 0x3ffffff));
-  const int hi = __reduce_add_sync(0xffffffffu, (int)(v >> 26));
-  return ((long long)hi << 26) + (long long)lo;
+// Sum of fixed-point values over the warp (in every lane); |sum| < 2^56.
+__device__ __forceinline__ long long warp_sum(int2 v) {
+  return ((long long)__reduce_add_sync(0xffffffffu, v.x) << 26) + __reduce_add_sync(0xffffffffu, v.y);
 }
 
 // A block's sums: shared memory behind the two tiles.
@@ -703,21 +719,9 @@ __device__ __forceinline__ void bwd_rounds(const TilePass& P, typename CT<R>::V2
       const OpRec<R> o = rec->op[k];
       Acc<R> acc;
       switch (P.op[k].bit) {
-        case 0:
-          if (o.mode != OM_H) grad_bit<0>(acc, o.mode, p, l);
-          op_bit<0, RB, R>(o, p);
-          op_bit<0, RB, R>(o, l);
-          break;
-        case 1:
-          if (o.mode != OM_H) grad_bit<1>(acc, o.mode, p, l);
-          op_bit<1, RB, R>(o, p);
-          op_bit<1, RB, R>(o, l);
-          break;
-        default:
-          if (o.mode != OM_H) grad_bit<2>(acc, o.mode, p, l);
-          op_bit<2, RB, R>(o, p);
-          op_bit<2, RB, R>(o, l);
-          break;
+        case 0: bwd_bit<0>(o, acc, p, l); break;
+        case 1: bwd_bit<1>(o, acc, p, l); break;
+        default: bwd_bit<2>(o, acc, p, l); break;
       }
       S.bad |= !acc.finite();
       if constexpr (sizeof(R) == 4) {
@@ -783,10 +787,10 @@ __device__ __forceinline__ void bwd_flush(const TilePass& P, const PassRec<R>* r
         Acc<float> a;
         a.s = S.z[slot * T + t].x;
         a.c = S.z[slot * T + t].y;
-        const long long f = a.fixed(kq);
-        v += (bit >= 0 && ((t >> bit) & 1)) ? -f : f;
+        const int2 f = a.fixed(kq);
+        const long long w = warp_sum((bit >= 0 && ((t >> bit) & 1)) ? make_int2(-f.x, -f.y) : f);
+        v += w;
       }
-      v = warp_sum(v);
       if (lane == 0 && v) atomicAdd(acc + 2 * (TP_MAXOP + p), (unsigned long long)v);
     } else {
       double v = 0.0;
