@@ -1063,7 +1063,7 @@ struct FwdPlan {
 
 template <typename R>
 static cudaError_t fwd_plan(FwdPlan<R>& F, const qc_gate* gates, int ng, int n, int B, cudaStream_t st) {
-  const TileCfg cfg = sizeof(R) == 4 ? TileCfg{13, 4, 4, true, false} : TileCfg{12, 3, 3, false, false};
+  const PassCfg cfg = sizeof(R) == 4 ? PassCfg{13, 4, 4, true, false} : PassCfg{12, 3, 3, false, false};
   F.passes = build_passes<R>(gates, ng, n, cfg);
   if (F.passes.empty()) return cudaSuccess;
   const size_t per = F.passes.size() * F.nrec * sizeof(typename Fwd<R>::Ops);
@@ -1145,7 +1145,7 @@ struct BwdPlan {
 };
 template <typename R>
 static cudaError_t bwd_plan(BwdPlan<R>& W, const qc_gate* gates, int ng, int n, int B, cudaStream_t st) {
-  W.passes = build_passes<R>(gates, ng, n, TileCfg{Bwd<R>::KT, Bwd<R>::C0, 3, false, true});
+  W.passes = build_passes<R>(gates, ng, n, PassCfg{Bwd<R>::KT, Bwd<R>::C0, 3, false, true});
   if (W.passes.empty()) return cudaSuccess;
   const size_t np = W.passes.size();
   W.chunk = (int)std::max<size_t>(1, std::min<size_t>(B, PREP_BYTES / (np * (sizeof(PassRec<R>) + BWD_SLOTS * 16))));

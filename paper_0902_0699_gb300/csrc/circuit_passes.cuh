@@ -152,13 +152,13 @@ __device__ __forceinline__ int tp_round_at(int base, const int* bas, int j) {
 // register bits of a round; merge: two neighbouring rotations on a qubit
 // become one operator and nothing goes to D; reverse: the rounds run the
 // operators last to first (the backward sweep).
-struct TileCfg {
+struct PassCfg {
   int kmax, c0, rb;
   bool merge, reverse;
 };
 
 template <typename R>
-inline std::vector<TilePass> build_passes(const qc_gate* gates, int ng, int n, const TileCfg& cfg) {
+inline std::vector<TilePass> build_passes(const qc_gate* gates, int ng, int n, const PassCfg& cfg) {
   struct Item {
     bool cx;
     int q, c, ka, kb, pa, pb;

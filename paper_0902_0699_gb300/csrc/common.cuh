@@ -329,6 +329,7 @@ qc_status launch_layer(qc_state* s, const double* U, uint64_t mask);
 int hadamard_layer_min_qubits(qc_dtype dt);
 qc_status launch_hadamard_layer(qc_state* s, uint64_t mask);
 qc_status launch_qft(qc_state* s);
+qc_status launch_qft_range(qc_state* s, int lo, int w);
 qc_status launch_grover_step(qc_state* s, const uint64_t* marked, int m);
 qc_status launch_grover_run(qc_state* s, const uint64_t* marked, int m, int iters);
 qc_status launch_grover_partial(qc_state* s, const uint64_t* marked, int m, double* out_host);

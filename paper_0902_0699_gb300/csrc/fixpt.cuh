@@ -1,0 +1,45 @@
+// binary64 <-> 64-bit fixed point with a common exponent per tile (wht.cu and
+// the register QFT of tile.cu): sums are exact integer additions and no FP64
+// instruction is issued.
+#pragma once
+
+namespace qc {
+
+// binary64 -> fixed point round(x 2^(1075 - G)) for a tile's G,
+// rounding half away from zero (symmetric, so unbiased; exact
+// values need no rounding at all).  x = m 2^(ex - 1075), so the value is
+// m 2^(ex - G).
+__device__ __forceinline__ long long d2fix(double x, int G) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(x);
+  const int ex = (int)((b >> 52) & 0x7FFu);
+  if (ex == 0) return 0;  // zero or subnormal (below 2^-1022): dropped
+  const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+  const int sh = ex - G;
+  unsigned long long v;
+  if (sh >= 0) {
+    v = m << sh;  // sh <= 9 - |B|: no overflow
+  } else {
+    const int r = -sh;
+    v = r > 54 ? 0ull : ((m >> (r - 1)) + 1ull) >> 1;
+  }
+  return (b >> 63) ? -(long long)v : (long long)v;
+}
+
+// fixed point v 2^-F -> binary64, rounded half away from zero (results
+// below 2^-1022 flush to zero)
+__device__ __forceinline__ double fix2d(long long v, int F) {
+  if (v == 0) return 0.0;
+  const unsigned long long sgn = v < 0 ? (1ull << 63) : 0ull;
+  const unsigned long long a = v < 0 ? (unsigned long long)(-v) : (unsigned long long)v;
+  const int lz = __clzll((long long)a);
+  unsigned long long keep = (((a << lz) >> 10) + 1ull) >> 1;  // 53 bits, rounded
+  int e = 63 - lz - F + 1023;
+  if (keep >> 53) {
+    keep >>= 1;
+    ++e;
+  }
+  if (e <= 0) return __longlong_as_double((long long)sgn);
+  return __longlong_as_double((long long)(sgn | ((unsigned long long)e << 52) | (keep & 0xFFFFFFFFFFFFFull)));
+}
+
+}  // namespace qc

@@ -81,16 +81,16 @@ __global__ void k_shor_fill(typename CT<R>::V2* __restrict__ s, uint64_t n1count
 }
 
 // ------------------------------------------------- ProjA, Eq. projreg2 ---
-// Probability of bits [lo, lo+w) == value (FP64 partials per block).
+// Probability of bits [lo, lo+w) == value (FP64 partials per block): only the
+// matching amplitudes are read.
 template <typename R>
-__global__ void __launch_bounds__(256) k_proj_prob(const typename CT<R>::V2* __restrict__ s, uint64_t N, int lo,
-                                                   uint64_t wmask, uint64_t value, double* __restrict__ part) {
+__global__ void __launch_bounds__(256) k_proj_prob(const typename CT<R>::V2* __restrict__ s, uint64_t count, int lo,
+                                                   int w, uint64_t value, double* __restrict__ part) {
   __shared__ double sh[32];
   double a = 0.0;
-  const uint64_t G = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += G) {
-    if (((i >> lo) & wmask) != value) continue;
-    const auto v = s[i];
+  const uint64_t G = (uint64_t)gridDim.x * blockDim.x, low = (1ull << lo) - 1ull;
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += G) {
+    const auto v = s[(i & low) | (value << lo) | ((i >> lo) << (lo + w))];
     a = fma((double)v.x, (double)v.x, a);
     a = fma((double)v.y, (double)v.y, a);
   }
@@ -99,24 +99,23 @@ __global__ void __launch_bounds__(256) k_proj_prob(const typename CT<R>::V2* __r
   __syncthreads();
   if (threadIdx.x == 0) {
     double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += sh[w];
+    for (int w2 = 0; w2 < (int)(blockDim.x >> 5); ++w2) t += sh[w2];
     part[blockIdx.x] = t;
   }
 }
 
-// Zero the amplitudes outside the outcome, scale the rest by f.
+// Zero the amplitudes outside the outcome (without reading them), scale the
+// rest by f.
 template <typename R>
-__global__ void k_proj_apply(typename CT<R>::V2* __restrict__ s, uint64_t N, int lo, uint64_t wmask, uint64_t value,
-                             R f) {
+__global__ void __launch_bounds__(256) k_proj_apply(typename CT<R>::V2* __restrict__ s, uint64_t N, int lo,
+                                                    uint64_t wmask, uint64_t value, R f) {
   const uint64_t G = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += G) {
-    auto v = s[i];
+    auto v = CT<R>::make((R)0, (R)0);
     if (((i >> lo) & wmask) == value) {
+      v = s[i];
       v.x *= f;
       v.y *= f;
-    } else {
-      v.x = 0;
-      v.y = 0;
     }
     s[i] = v;
   }
@@ -207,13 +206,14 @@ QC_API qc_status qc_project(qc_state* s, int lo, int width, uint64_t value, doub
   const uint64_t N = 1ull << s->n;
   const uint64_t wmask = (width >= 64) ? ~0ull : ((1ull << width) - 1ull);
   double* part = s->scratch + QC_SCR_PARTIALS;
-  const unsigned nb = std::min<unsigned>(grid_for(N, 256 * 4, 8), QC_PARTIALS);
+  const uint64_t count = N >> width;
+  const unsigned nb = std::min<unsigned>(grid_for(count, 256 * 4, 8), QC_PARTIALS);
   if (s->dt == QC_C128)
-    k_proj_prob<double><<<nb, 256, 0, s->stream>>>(reinterpret_cast<const double2*>(s->data), N, lo, wmask, value,
-                                                   part);
+    k_proj_prob<double><<<nb, 256, 0, s->stream>>>(reinterpret_cast<const double2*>(s->data), count, lo, width,
+                                                   value, part);
   else
-    k_proj_prob<float><<<nb, 256, 0, s->stream>>>(reinterpret_cast<const float2*>(s->data), N, lo, wmask, value,
-                                                  part);
+    k_proj_prob<float><<<nb, 256, 0, s->stream>>>(reinterpret_cast<const float2*>(s->data), count, lo, width,
+                                                  value, part);
   st = check_launch("project (probability)");
   if (st) return st;
   std::vector<double> h(nb);
@@ -238,10 +238,8 @@ QC_API qc_status qc_project(qc_state* s, int lo, int width, uint64_t value, doub
   return check_launch("project (apply)");
 }
 
-// Appendix A's circuit on the register of qubits [lo, lo+width): for the
-// register's qubits from the most significant down, a Hadamard, then
-// CPHASEK with each lower register qubit; then the pair swaps that restore
-// the register's bit order.  Built from the gate kernels.
+// Appendix A's circuit on the register of qubits [lo, lo+width), as tile
+// passes (tile.cu).
 QC_API qc_status qc_qft_range(qc_state* s, int lo, int width) {
   clear_error();
   qc_status st = check_state(s);
@@ -250,26 +248,5 @@ QC_API qc_status qc_qft_range(qc_state* s, int lo, int width) {
     set_error("bad register [%d, %d) for n = %d", lo, lo + width, s->n);
     return QC_EINVAL;
   }
-  const double h = 1.0 / sqrt(2.0);
-  const double H[8] = {h, 0, h, 0, h, 0, -h, 0};
-  for (int i = width - 1; i >= 0 && !st; --i) {
-    st = launch_1q(s, lo + i, H);
-    for (int j = i - 1; j >= 0 && !st; --j) {
-      const int k = i - j + 1;
-      double U[8] = {1, 0, 0, 0, 0, 0, 0, 0};
-      if (k == 1) {
-        U[6] = -1.0;
-      } else if (k == 2) {
-        U[7] = 1.0;
-      } else {
-        double sn, cs;
-        sincospi(2.0 / ldexp(1.0, k), &sn, &cs);
-        U[6] = cs;
-        U[7] = sn;
-      }
-      st = launch_ctrl(s, lo + i, lo + j, U);
-    }
-  }
-  for (int i = 0; i < width / 2 && !st; ++i) st = launch_swap(s, lo + i, lo + width - 1 - i);
-  return st;
+  return launch_qft_range(s, lo, width);
 }

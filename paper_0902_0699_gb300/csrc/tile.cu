@@ -29,11 +29,13 @@
 // (ff.cuh) on the FP32 pipe: the FP64 pipe of GB300 (0.5 Top/s) would
 // otherwise bound every pass many times over the memory time.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <vector>
 
 #include "common.cuh"
 #include "ff.cuh"
+#include "fixpt.cuh"
 
 namespace qc {
 
@@ -153,8 +155,10 @@ template <> struct TA<double> {
 template <typename R> struct TileProg {
   int nops;
   int lo, k, c;     // group [lo, lo+k), c low contiguous bits (c <= lo)
-  int n;
-  int twiddle;      // apply the QFT cross phase with the bits below lo
+  int n;            // bits of the QFT's root tables (the transformed register's width)
+  int base;         // the register's lowest qubit: the QFT's phases use the index bits from here up
+  int rev;          // store the group bits in reversed order (a register of one group)
+  int twiddle;      // apply the QFT cross phase with the register bits below lo
   int qft;          // the program contains QFT levels (build the ladder table)
   int nl;           // global root table split: low table has 2^nl entries
   int scale_p;      // unnormalised butterflies: multiply by 2^{-scale_p/2} at the end
@@ -248,36 +252,50 @@ __device__ __forceinline__ typename TA<R>::E ladder_at(const typename TA<R>::E* 
   return (y & 1) ? TA<R>::mul(m, LAD[(1 << kl) - 1]) : m;
 }
 
-// Shared tables of a pass: the ladders (QFT programs) and the twiddle
-// remainder tables TWA, TWB (QFT programs with a twiddle).
-template <typename R>
-__device__ __forceinline__ void tile_tables(const TileProg<R>& P, typename TA<R>::E* LAD, typename TA<R>::E* TWA,
-                                            typename TA<R>::E* TWB, int kl) {
-  using A = TA<R>;
-  const int k = P.k, hi = P.lo + P.k - 1;
-  if (!P.qft) return;
-  // ladder tables, one per level: LAD[2^j - 1 + x] = e^{2 pi i x / 2^{j+1}}
-  for (int a = threadIdx.x; a < (1 << kl) - 1; a += blockDim.x) {
-    const int j = 31 - __clz(a + 1);
-    LAD[a] = A::root((uint64_t)(a + 1 - (1 << j)), j + 1);
+// A ladder table entry in global memory (16 bytes for double-float).
+template <typename R> struct LadIO;
+template <> struct LadIO<float> {
+  __device__ static Cx<float> ld(const float2* p) { return cmake<float>(p->x, p->y); }
+  __device__ static void st(float2* p, Cx<float> z) { *p = make_float2(z.re, z.im); }
+};
+template <> struct LadIO<double> {
+  __device__ static ffc ld(const double2* p) {
+    const float4 v = *reinterpret_cast<const float4*>(p);
+    return ffc_make(ff_make(v.x, v.y), ff_make(v.z, v.w));
   }
-  if (k > kl && threadIdx.x == 0) LAD[(1 << kl) - 1] = A::root(1, k);  // e^{2 pi i / 2^k}
+  __device__ static void st(double2* p, ffc z) {
+    *reinterpret_cast<float4*>(p) = make_float4(z.re.hi, z.re.lo, z.im.hi, z.im.lo);
+  }
+};
+
+// Shared tables of a pass: the ladders (QFT programs, copied from the
+// transform's table: one FP64 sincospi per entry and block costs more than
+// the pass itself on states of up to 2^20 amplitudes) and the twiddle
+// remainder tables TWA, TWB (QFT programs with a twiddle whose contiguous
+// bits belong to the register).
+template <typename R>
+__device__ __forceinline__ void tile_tables(const TileProg<R>& P, const typename CT<R>::V2* __restrict__ lad,
+                                            typename TA<R>::E* LAD, typename TA<R>::E* TWA, typename TA<R>::E* TWB) {
+  using A = TA<R>;
+  const int hi = P.lo + P.k - 1 - P.base;
+  if (!P.qft) return;
+  for (int a = threadIdx.x; a < lad_entries<R>(P.k); a += blockDim.x) LAD[a] = LadIO<R>::ld(lad + a);
   // twiddle remainder: Omega_{hi+1}^x = TWA[x & 127] * TWB[x >> 7], x < 2^{c+k}
-  if (P.twiddle)
+  if (P.twiddle && P.base < P.c)
     for (int i = threadIdx.x; i < TS_TWA + TS_TWB; i += blockDim.x) {
       if (i < TS_TWA) TWA[i] = A::root((uint64_t)i, hi + 1);
       else TWB[i - TS_TWA] = A::root((uint64_t)(i - TS_TWA) << 7, hi + 1);
     }
 }
 
-// V[f] = 2^{-p/2} Omega_{hi+1}^{Ltile f} for tile T (Ltile = the tile's bits
-// between c and lo).
+// V[f] = 2^{-p/2} Omega_{hi+1}^{Ltile f} for tile T (Ltile = the tile's
+// register bits between c and lo; hi counted within the register).
 template <typename R>
 __device__ __forceinline__ void tile_twiddle_v(const TileProg<R>& P, uint64_t T, typename TA<R>::E* V,
                                                const typename CT<R>::V2* __restrict__ tlo,
                                                const typename CT<R>::V2* __restrict__ thi, typename TA<R>::S sc) {
-  const int lo = P.lo, k = P.k, c = P.c, hi = lo + k - 1;
-  const uint64_t Lt = (T & ((1ull << (lo - c)) - 1ull)) << c;
+  const int lo = P.lo, k = P.k, c = P.c, hi = lo + k - 1 - P.base;
+  const uint64_t Lt = ((T & ((1ull << (lo - c)) - 1ull)) << c) >> P.base;
   for (int f = threadIdx.x; f < (1 << k); f += blockDim.x) {
     const uint64_t r = (Lt * (uint64_t)f) & ((2ull << hi) - 1ull);
     V[f] = TA<R>::scale_by(omega<R>(tlo, thi, r << (P.n - hi - 1), P.nl), sc);
@@ -406,29 +424,32 @@ __device__ __forceinline__ void tile_store(typename CT<R>::V2* __restrict__ s, u
   using E = typename A::E;
   using V2 = typename CT<R>::V2;
   const int lo = P.lo, k = P.k, c = P.c;
-  const int NE = 1 << (k + c);
+  const int NE = 1 << (k + c), cm = (1 << c) - 1;
+  const bool own = P.base < c;  // contiguous bits of the register's
+  // the staged element that goes to place e
+  auto from = [&](int e) { return P.rev ? (int)((__brev((unsigned)(e >> c)) >> (32 - k)) << c) | (e & cm) : e; };
+  auto twiddled = [&](int e, E z) {
+    const int f = (int)(__brev((unsigned)(e >> c)) >> (32 - k));
+    E w = V[f];
+    if (own) {
+      const int x = ((e & cm) >> P.base) * f;  // < 2^{c+k}
+      w = A::mul(w, A::mul(TWA[x & 127], TWB[x >> 7]));
+    }
+    return A::mul(w, z);
+  };
   if (sizeof(R) == 8) {
     for (int e = threadIdx.x; e < NE; e += blockDim.x) {
-      E z = sm[e];
-      if (P.twiddle) {
-        const int f = (int)(__brev((unsigned)(e >> c)) >> (32 - k));
-        const int x = (e & ((1 << c) - 1)) * f;  // < 2^{c+k}
-        z = A::mul(A::mul(V[f], A::mul(TWA[x & 127], TWB[x >> 7])), z);
-      } else if (P.scale_p) {
-        z = A::scale_by(z, sc);
-      }
+      E z = sm[from(e)];
+      if (P.twiddle) z = twiddled(e, z);
+      else if (P.scale_p) z = A::scale_by(z, sc);
       s[tile_global(e, T, lo, k, c)] = A::to(z);
     }
   } else {
     for (int e = 2 * threadIdx.x; e < NE; e += 2 * blockDim.x) {
-      E z0 = sm[e], z1 = sm[e + 1];
+      E z0 = sm[from(e)], z1 = sm[from(e + 1)];
       if (P.twiddle) {
-        // e and e+1 share the group bits (c >= 1 whenever lo > 0)
-        const int f = (int)(__brev((unsigned)(e >> c)) >> (32 - k));
-        const int x0 = (e & ((1 << c) - 1)) * f, x1 = x0 + f;
-        const E v = V[f];
-        z0 = A::mul(A::mul(v, A::mul(TWA[x0 & 127], TWB[x0 >> 7])), z0);
-        z1 = A::mul(A::mul(v, A::mul(TWA[x1 & 127], TWB[x1 >> 7])), z1);
+        z0 = twiddled(e, z0);
+        z1 = twiddled(e + 1, z1);
       } else if (P.scale_p) {
         z0 = A::scale_by(z0, sc);
         z1 = A::scale_by(z1, sc);
@@ -443,7 +464,8 @@ __device__ __forceinline__ void tile_store(typename CT<R>::V2* __restrict__ s, u
 template <typename R>
 __global__ void __launch_bounds__(512, 2) k_tile(typename CT<R>::V2* __restrict__ s, uint64_t ntiles,
                                                  const TileProg<R> P, const typename CT<R>::V2* __restrict__ tlo,
-                                                 const typename CT<R>::V2* __restrict__ thi) {
+                                                 const typename CT<R>::V2* __restrict__ thi,
+                                                 const typename CT<R>::V2* __restrict__ lad) {
   using A = TA<R>;
   using E = typename A::E;
   using V2 = typename CT<R>::V2;
@@ -457,7 +479,7 @@ __global__ void __launch_bounds__(512, 2) k_tile(typename CT<R>::V2* __restrict_
   E* TWA = LAD + (P.qft ? lad_entries<R>(k) : 0);
   E* TWB = TWA + TS_TWA;
   const typename A::S sc = A::scale_const(P.scale_p);
-  tile_tables<R>(P, LAD, TWA, TWB, kl);
+  tile_tables<R>(P, lad, LAD, TWA, TWB);
   for (uint64_t T = blockIdx.x; T < ntiles; T += gridDim.x) {
     if (P.twiddle) tile_twiddle_v<R>(P, T, V, tlo, thi, sc);
     // load: 16-byte vectors; for complex64 two neighbouring elements (c >= 1
@@ -600,7 +622,8 @@ __device__ __forceinline__ double2 ffc_pack(ffc z) {
 template <int K>
 __global__ void __launch_bounds__(512, 2) k_qft_c128_k(double2* __restrict__ s, uint64_t ntiles, const TileProg<double> P,
                                                        const double2* __restrict__ tlo,
-                                                       const double2* __restrict__ thi, int ld_ff, int st_ff) {
+                                                       const double2* __restrict__ thi,
+                                                       const double2* __restrict__ lad, int ld_ff, int st_ff) {
   using A = TA<double>;
   constexpr int C = 12 - K, NE = 1 << 12, PER = NE / 512;
   static_assert(C <= 9, "512-element strides stay inside the group bits");
@@ -611,11 +634,7 @@ __global__ void __launch_bounds__(512, 2) k_qft_c128_k(double2* __restrict__ s, 
   const bool tw = P.twiddle != 0;
   ffc* LAD = sm + NE;
   constexpr int kl = lad_levels<double>(K);
-  for (int a = threadIdx.x; a < (1 << kl) - 1; a += blockDim.x) {
-    const int j = 31 - __clz(a + 1);
-    LAD[a] = A::root((uint64_t)(a + 1 - (1 << j)), j + 1);
-  }
-  if (K > kl && threadIdx.x == 0) LAD[(1 << kl) - 1] = A::root(1, K);
+  for (int a = threadIdx.x; a < lad_entries<double>(K); a += blockDim.x) LAD[a] = LadIO<double>::ld(lad + a);
   const typename A::S sc = A::scale_const(K);
   const int tid = threadIdx.x;
   const int st = tsw(tid);
@@ -1052,12 +1071,21 @@ __global__ void __launch_bounds__(512, 1) k_qft_db_c64(float2* __restrict__ s, u
 }
 
 // Tables of Omega^a (a < 2^nl) and Omega^{a 2^nl} (a < 2^{n-nl}),
-// Omega = e^{2 pi i / 2^n}, from sincospi in double precision.
+// Omega = e^{2 pi i / 2^n}, from sincospi in double precision, and the first
+// nlad entries of the ladder table: level j's e^{2 pi i x / 2^{j+1}} at
+// 2^j - 1 + x (complex128: e^{2 pi i / 2^12} at 2047).
 template <typename R>
-__global__ void k_roots(typename CT<R>::V2* tlo, typename CT<R>::V2* thi, int n, int nl) {
+__global__ void k_roots(typename CT<R>::V2* tlo, typename CT<R>::V2* thi, int n, int nl, typename CT<R>::V2* lad,
+                        int nlad) {
   const uint64_t nlo = 1ull << nl, nhi = 1ull << (n - nl);
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nlo + nhi;
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nlo + nhi + (uint64_t)nlad;
        i += (uint64_t)gridDim.x * blockDim.x) {
+    if (i >= nlo + nhi) {
+      const int a = (int)(i - nlo - nhi), j = 31 - __clz(a + 1);
+      const bool extra = sizeof(R) == 8 && a == 2047;
+      LadIO<R>::st(lad + a, extra ? TA<R>::root(1, 12) : TA<R>::root((uint64_t)(a + 1 - (1 << j)), j + 1));
+      continue;
+    }
     const bool low = i < nlo;
     const uint64_t a = low ? i : (i - nlo);
     // angle / pi = 2 a 2^{shift} / 2^n, reduced mod 2 exactly in integers
@@ -1123,22 +1151,21 @@ static size_t tile_smem(int k, int c, bool twiddle, bool qft) {
 }
 
 template <typename R>
-static qc_status run_tile(qc_state* s, TileProg<R>& P, const typename CT<R>::V2* tlo,
-                          const typename CT<R>::V2* thi) {
+static qc_status run_tile(qc_state* s, TileProg<R>& P, const typename CT<R>::V2* tlo = nullptr,
+                          const typename CT<R>::V2* thi = nullptr, const typename CT<R>::V2* lad = nullptr) {
   using V2 = typename CT<R>::V2;
   if (P.nops == 0 && !P.twiddle) return QC_OK;
-  P.n = s->n;
   const int tb = P.k + P.c;
   const uint64_t ntiles = 1ull << (s->n - tb);
   const size_t smem = tile_smem<R>(P.k, P.c, P.twiddle != 0, P.qft != 0);
-  constexpr int threads = 512;
+  const int threads = std::max(64, std::min(512, (1 << tb) >> 2));  // four amplitudes a thread
   static bool attr_set = false;
   if (!attr_set) {
     cudaFuncSetAttribute(k_tile<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     attr_set = true;
   }
   const unsigned grid = resident_grid(k_tile<R>, threads, (int64_t)ntiles, 1, smem);
-  k_tile<R><<<grid, threads, smem, s->stream>>>(reinterpret_cast<V2*>(s->data), ntiles, P, tlo, thi);
+  k_tile<R><<<grid, threads, smem, s->stream>>>(reinterpret_cast<V2*>(s->data), ntiles, P, tlo, thi, lad);
   return check_launch("tile pass");
 }
 
@@ -1151,9 +1178,8 @@ static bool qft_c128_compiled(const TileProg<double>& P) {
 // ld_ff / st_ff: the pass reads / leaves the double-float form (compiled
 // passes only; the transform's first pass reads IEEE doubles, and the bit
 // reversal after its last pass converts back).
-static qc_status run_qft_c128(qc_state* s, TileProg<double>& P, const double2* tlo, const double2* thi, bool ld_ff,
-                              bool st_ff) {
-  P.n = s->n;
+static qc_status run_qft_c128(qc_state* s, TileProg<double>& P, const double2* tlo, const double2* thi,
+                              const double2* lad, bool ld_ff, bool st_ff) {
   if (qft_c128_compiled(P)) {
     const uint64_t ntiles = 1ull << (s->n - 12);
     const size_t smem = sizeof(ffc) * (((size_t)1 << 12) + (size_t)lad_entries<double>(P.k));
@@ -1167,7 +1193,7 @@ static qc_status run_qft_c128(qc_state* s, TileProg<double>& P, const double2* t
       a = true;                                                                                     \
     }                                                                                               \
     const unsigned g = resident_grid(k_qft_c128_k<KK>, 512, (int64_t)ntiles, 1, smem);             \
-    k_qft_c128_k<KK><<<g, 512, smem, s->stream>>>(d, ntiles, P, tlo, thi, ld_ff, st_ff);            \
+    k_qft_c128_k<KK><<<g, 512, smem, s->stream>>>(d, ntiles, P, tlo, thi, lad, ld_ff, st_ff);       \
     return check_launch("qft pass");                                                                \
   }
       QC_QFT_C128(3) QC_QFT_C128(4) QC_QFT_C128(5) QC_QFT_C128(6) QC_QFT_C128(7) QC_QFT_C128(8)
@@ -1177,7 +1203,7 @@ static qc_status run_qft_c128(qc_state* s, TileProg<double>& P, const double2* t
     }
   }
   if (ld_ff || st_ff) return QC_EINVAL;
-  return run_tile<double>(s, P, tlo, thi);
+  return run_tile<double>(s, P, tlo, thi, lad);
 }
 
 // complex64 QFT pass through the double-buffered kernel: two tile buffers
@@ -1188,7 +1214,6 @@ static size_t qft_db_smem(int k, int c, bool twiddle) {
 }
 
 static qc_status run_qft_db_c64(qc_state* s, TileProg<float>& P, const float2* tlo, const float2* thi) {
-  P.n = s->n;
   const uint64_t ntiles = 1ull << (s->n - (P.k + P.c));
   const size_t smem = qft_db_smem(P.k, P.c, P.twiddle != 0);
   static bool attr_set = false;
@@ -1240,6 +1265,8 @@ static void prog_init(TileProg<R>& P, const Group& g, int n) {
   P.k = g.k;
   P.c = tile_c<R>(g);
   P.n = n;
+  P.base = 0;
+  P.rev = 0;
   P.twiddle = 0;
   P.qft = 0;
   P.nl = 0;
@@ -1275,7 +1302,7 @@ static qc_status layer_impl(qc_state* s, const double* U, uint64_t mask) {
       }
       ++P.nops;
     }
-    qc_status st = run_tile<R>(s, P, nullptr, nullptr);
+    qc_status st = run_tile<R>(s, P);
     if (st) return st;
   }
   return QC_OK;
@@ -1414,22 +1441,40 @@ static qc_status bitrev_impl(qc_state* s, bool from_ff = false) {
   return check_launch("bitrev");
 }
 
+__global__ void k_roots_fix(longlong2* tlo, longlong2* thi, int n, int nl, longlong2* lad, int nlad);
+
+// Root and ladder tables of a transform over n bits, in one allocation (tlo);
+// fixed: in 64-bit fixed point (complex128 register passes).
+template <typename R>
+struct QftTables {
+  typename CT<R>::V2 *tlo, *thi, *lad;
+};
+template <typename R>
+static qc_status qft_tables(qc_state* s, int n, int nl, int nlad, QftTables<R>* t, bool fixed = false) {
+  const size_t tot = ((size_t)1 << nl) + ((size_t)1 << (n - nl)) + (size_t)nlad;
+  cudaError_t e = cudaMallocAsync((void**)&t->tlo, tot * sizeof(typename CT<R>::V2), s->stream);
+  if (e != cudaSuccess) return cuda_fail(e, "qft tables");
+  t->thi = t->tlo + ((size_t)1 << nl);
+  t->lad = t->thi + ((size_t)1 << (n - nl));
+  const unsigned grid = grid_for((int64_t)tot, 64, 8);
+  if (fixed && sizeof(R) == 8)  // complex128 register passes
+    k_roots_fix<<<grid, 64, 0, s->stream>>>(reinterpret_cast<longlong2*>(t->tlo), reinterpret_cast<longlong2*>(t->thi), n,
+                                            nl, reinterpret_cast<longlong2*>(t->lad), nlad);
+  else
+    k_roots<R><<<grid, 64, 0, s->stream>>>(t->tlo, t->thi, n, nl, t->lad, nlad);
+  return check_launch("qft roots");
+}
+
 template <typename R>
 static qc_status qft_impl(qc_state* s) {
   using V2 = typename CT<R>::V2;
   const int n = s->n;
   const int nl = (n + 1) / 2;
-  const size_t tbytes = (((size_t)1 << nl) + ((size_t)1 << (n - nl))) * sizeof(V2);
-  V2* tab = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&tab, tbytes, s->stream);
-  if (e != cudaSuccess) return cuda_fail(e, "qft tables");
-  V2* tlo = tab;
-  V2* thi = tab + ((size_t)1 << nl);
-  {
-    const uint64_t tot = (1ull << nl) + (1ull << (n - nl));
-    k_roots<R><<<grid_for(tot, 256, 4), 256, 0, s->stream>>>(tlo, thi, n, nl);
-  }
-  qc_status st = check_launch("qft roots");
+  const int nlad = sizeof(R) == 8 ? 1 << std::min(n, 11) : 0;  // complex64 passes build theirs from the roots
+  QftTables<R> tab;
+  qc_status st = qft_tables(s, n, nl, nlad, &tab);
+  if (st) return st;
+  V2 *tlo = tab.tlo, *thi = tab.thi;
   // complex64: groups of at most 9 above the lowest 13 (64 KiB tiles)
   std::vector<Group> groups = sizeof(R) == 4 ? plan_groups_k(n, 13, 9) : plan_groups<R>(n);
   std::vector<TileProg<R>> progs(groups.size());
@@ -1453,17 +1498,286 @@ static qc_status qft_impl(qc_state* s) {
   for (int gi = (int)groups.size() - 1; gi >= 0 && !st; --gi) {
     if constexpr (sizeof(R) == 4) st = run_qft_db_c64(s, progs[gi], tlo, thi);
     else
-      st = run_qft_c128(s, progs[gi], tlo, thi, all_compiled && gi + 1 < (int)groups.size(), all_compiled);
+      st = run_qft_c128(s, progs[gi], tlo, thi, tab.lad, all_compiled && gi + 1 < (int)groups.size(), all_compiled);
   }
   // the bit reversal converts the complex128 passes' double-float form back
   if (!st) st = bitrev_impl<R>(s, sizeof(R) == 8 && all_compiled);
-  cudaFreeAsync(tab, s->stream);
+  cudaFreeAsync(tab.tlo, s->stream);
   return st;
 }
 
 qc_status launch_qft(qc_state* s) {
   s->sum_valid = false;
   return s->dt == QC_C128 ? qft_impl<double>(s) : qft_impl<float>(s);
+}
+
+// ---------------------------------------------------- register QFT -------
+// Reversal of the bits [lo, lo + w) of every index, in place: amplitude rows
+// of 2^lo swap (runs of 2^lo amplitudes stream).
+template <typename V2>
+__global__ void __launch_bounds__(256) k_reg_rev(V2* __restrict__ s, uint64_t N, int lo, int w) {
+  const uint64_t mask = (1ull << w) - 1ull;
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < N; i += (uint64_t)gridDim.x * blockDim.x) {
+    const uint64_t r = (i >> lo) & mask, q = __brevll(r) >> (64 - w);
+    if (q <= r) continue;
+    const uint64_t j = i ^ ((r ^ q) << lo);
+    const V2 a = s[i], b = s[j];
+    s[i] = b;
+    s[j] = a;
+  }
+}
+
+// complex128 register passes in 64-bit fixed point.  The tile's largest
+// exponent sets the binary point; sums are exact, a radix-4 step's two
+// 1/sqrt 2 are one halving (a shift, or the factor 1/2 that the high word of a
+// product by a root scaled by 2^63 brings), and the result is rounded once to
+// binary64.  Against double-float (k_tile) a sum costs two integer additions
+// instead of about 20 FP32 operations and a value keeps 54 bits or more of
+// the tile's largest instead of 47: an 11-qubit register of a 17-qubit state
+// has a relative error of 4e-16 where double-float passes have 1.2e-14 and
+// one pass per gate had 5.8e-15.  Double-float passes take 0.8 of the time
+// (two 9-qubit passes of a 26-qubit state 2.37 ms against 2.96 ms) but would
+// lose accuracy against the gates.
+struct RqftProg {
+  int lo, k, c;      // group [lo, lo+k), c contiguous low bits
+  int base, w, nl;   // the register's lowest qubit and width, split of its root table
+  int twiddle, rev;
+  long long rsqrt2;  // floor(2^62.5)
+};
+
+__device__ __forceinline__ longlong2 fx_mul(longlong2 a, longlong2 r) {
+  return make_longlong2(__mul64hi(a.x, r.x) - __mul64hi(a.y, r.y), __mul64hi(a.x, r.y) + __mul64hi(a.y, r.x));
+}
+__device__ __forceinline__ longlong2 fx_add(longlong2 a, longlong2 b) { return make_longlong2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ longlong2 fx_sub(longlong2 a, longlong2 b) { return make_longlong2(a.x - b.x, a.y - b.y); }
+__device__ __forceinline__ longlong2 fx_half(longlong2 a) { return make_longlong2((a.x + 1) >> 1, (a.y + 1) >> 1); }
+
+// The tables of k_roots scaled by 2^63 (1 itself saturates, 2^-63 low).
+__global__ void k_roots_fix(longlong2* tlo, longlong2* thi, int n, int nl, longlong2* lad, int nlad) {
+  const uint64_t nlo = 1ull << nl, nhi = 1ull << (n - nl);
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nlo + nhi + (uint64_t)nlad;
+       i += (uint64_t)gridDim.x * blockDim.x) {
+    double x;
+    longlong2* out;
+    if (i < nlo + nhi) {
+      const bool low = i < nlo;
+      const uint64_t a = low ? i : (i - nlo);
+      x = ldexp((double)((a << ((low ? 0 : nl) + 1)) & ((2ull << n) - 1ull)), -n);
+      out = low ? tlo + a : thi + a;
+    } else {
+      const int a = (int)(i - nlo - nhi), j = 31 - __clz(a + 1);
+      x = ldexp((double)(a + 1 - (1 << j)), -j);
+      out = lad + a;
+    }
+    double sn, cs;
+    sincospi(x, &sn, &cs);
+    *out = make_longlong2(__double2ll_rn(cs * 9223372036854775808.0), __double2ll_rn(sn * 9223372036854775808.0));
+  }
+}
+
+// Omega_w^r / 2 at scale 2^63 (the product's factor)
+__device__ __forceinline__ longlong2 fx_omega(const longlong2* __restrict__ tlo, const longlong2* __restrict__ thi,
+                                              uint64_t r, int nl) {
+  return fx_mul(tlo[r & ((1ull << nl) - 1ull)], thi[r >> nl]);
+}
+
+__global__ void __launch_bounds__(512, 2) k_rqft_c128(double2* __restrict__ s, uint64_t ntiles,
+                                                      const __grid_constant__ RqftProg P,
+                                                      const longlong2* __restrict__ tlo,
+                                                      const longlong2* __restrict__ thi,
+                                                      const longlong2* __restrict__ lad) {
+  constexpr int PER = 8;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  __shared__ int wmax[16];
+  const int k = P.k, c = P.c, lo = P.lo, NE = 1 << (k + c), T = blockDim.x, tid = threadIdx.x, cm = (1 << c) - 1;
+  const int hi = lo + k - 1 - P.base, sh = P.w - hi - 1, ns = (k + 1) / 2;
+  const uint64_t hm = (2ull << hi) - 1ull;
+  const bool own = P.base < c;  // contiguous bits of the register's: no common twiddle table of a tile
+  longlong2* sm = reinterpret_cast<longlong2*>(smraw);
+  longlong2* LAD = sm + NE;
+  longlong2* V = LAD + (1 << k) - 1;
+  for (int a = tid; a < (1 << k) - 1; a += T) LAD[a] = lad[a];
+  for (uint64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    double2 v[PER];
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+      const int e = tid + T * u;
+      v[u] = e < NE ? s[tile_global(e, tile, lo, k, c)] : make_double2(0.0, 0.0);
+    }
+    int em = 0;
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+      em = max(em, (int)((__double_as_longlong(v[u].x) >> 52) & 0x7FF));
+      em = max(em, (int)((__double_as_longlong(v[u].y) >> 52) & 0x7FF));
+    }
+    em = __reduce_max_sync(0xffffffffu, em);
+    if ((tid & 31) == 0) wmax[tid >> 5] = em;
+    __syncthreads();
+    for (int q = 0; q < (T >> 5); ++q) em = max(em, wmax[q]);
+    // |x| < 2^(em - 1022) times 2^(1075 - G) is below 2^(61 - ns).  A step's
+    // values grow by at most 2 and its sums of four by 4: below 2^63.
+    const int G = em - 8 + ns;
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+      const int e = tid + T * u;
+      if (e < NE) sm[tsw(e)] = make_longlong2(d2fix(v[u].x, G), d2fix(v[u].y, G));
+    }
+    const uint64_t Lt = (tile & ((1ull << (lo - c)) - 1ull)) << c;  // the tile's index bits below the group
+    if (P.twiddle && !own)
+      for (int f = tid; f < (1 << k); f += T) V[f] = fx_omega(tlo, thi, (((Lt >> P.base) * (uint64_t)f) & hm) << sh, P.nl);
+    __syncthreads();
+    int jh = k - 1;
+    for (; jh >= 1; jh -= 2) {  // levels jh, jh - 1 as in k_tile
+      const int jl = jh - 1, bl = c + jl;
+      for (int p = tid; p < (NE >> 2); p += T) {
+        const int e00 = ((p >> bl) << (bl + 2)) | (p & ((1 << bl) - 1));
+        const int b = tsw(e00), o01 = tsw(1 << bl), o10 = tsw(2 << bl), o11 = tsw(3 << bl);
+        const longlong2 a00 = sm[b], a01 = sm[b ^ o01], a10 = sm[b ^ o10], a11 = sm[b ^ o11];
+        const longlong2 s0 = fx_add(a00, a10), d0 = fx_sub(a00, a10), s1 = fx_add(a01, a11), d1 = fx_sub(a01, a11);
+        const longlong2 id1 = make_longlong2(-d1.y, d1.x);
+        longlong2 u0 = fx_sub(s0, s1), t1 = fx_add(d0, id1), u1 = fx_sub(d0, id1);
+        const int x = (e00 >> c) & ((1 << jl) - 1);
+        if (x) {
+          const longlong2* L = LAD + (1 << jh) - 1;
+          const int x3 = 3 * x, m = (1 << jh) - 1;
+          u0 = fx_mul(u0, L[2 * x]);
+          t1 = fx_mul(t1, L[x]);
+          u1 = fx_mul(u1, L[x3 & m]);
+          if (x3 >> jh) u1 = make_longlong2(-u1.x, -u1.y);
+        } else {
+          u0 = fx_half(u0);
+          t1 = fx_half(t1);
+          u1 = fx_half(u1);
+        }
+        sm[b] = fx_half(fx_add(s0, s1));
+        sm[b ^ o01] = u0;
+        sm[b ^ o10] = t1;
+        sm[b ^ o11] = u1;
+      }
+      __syncthreads();
+    }
+    if (jh == 0) {
+      for (int p = tid; p < (NE >> 1); p += T) {
+        const int b = tsw(((p >> c) << (c + 1)) | (p & cm)), o = tsw(1 << c);
+        const longlong2 a0 = sm[b], a1 = sm[b ^ o];
+        sm[b] = fx_add(a0, a1);
+        sm[b ^ o] = fx_sub(a0, a1);
+      }
+      __syncthreads();
+    }
+    // odd k: the last level's 1/sqrt 2 (the high word of 2^62.5 v is v / sqrt 2 / 2)
+    const int F = 1075 - G - (k & 1) - (P.twiddle ? 2 : 0);
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+      const int e = tid + T * u;
+      if (e < NE) {
+        const int f = (int)(__brev((unsigned)(e >> c)) >> (32 - k));
+        longlong2 z = sm[tsw(P.rev ? (f << c) | (e & cm) : e)];
+        if (k & 1) z = make_longlong2(__mul64hi(z.x, P.rsqrt2), __mul64hi(z.y, P.rsqrt2));
+        if (P.twiddle) {
+          const longlong2 W =
+              own ? fx_omega(tlo, thi, ((((Lt | (uint64_t)(e & cm)) >> P.base) * (uint64_t)f) & hm) << sh, P.nl) : V[f];
+          z = fx_mul(z, W);
+        }
+        // a tile with an infinity or a NaN comes out as NaN
+        const double nan = __longlong_as_double(0x7ff8000000000000ll);
+        s[tile_global(e, tile, lo, k, c)] =
+            em == 0x7FF ? make_double2(nan, nan) : make_double2(fix2d(z.x, F), fix2d(z.y, F));
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// Appendix A's circuit on the register [lo, lo + w) as tile passes: the
+// register's qubits in groups from the top, each pass one read and write of
+// the state; the phases between groups as in qft_impl, over the register's
+// bits.  A register of up to eleven qubits is a single pass (rows of 32 bytes
+// or longer: c contiguous bits below it) that also stores the reversed order;
+// larger ones take groups of up to nine with longer rows and one reversal
+// pass.  Gate by gate this is w Hadamard, w (w - 1) / 2 phase and w / 2 swap
+// passes: 195 us (71 launches) for 11 qubits of 17.
+struct RangePlan {
+  std::vector<Group> groups;
+  int kmax = 0;
+};
+static RangePlan plan_range(int lo, int w) {
+  RangePlan R;
+  if (w <= 11) {
+    R.groups.push_back({lo, w});
+  } else if (lo == 0) {
+    R.groups = plan_groups_k(w, 11, 9);
+  } else {
+    const int ng = (w + 8) / 9;
+    for (int i = 0, at = lo, left = w; i < ng; ++i) {
+      const int k = (left + (ng - i) - 1) / (ng - i);  // balanced
+      R.groups.push_back({at, k});
+      at += k;
+      left -= k;
+    }
+  }
+  for (const Group& g : R.groups) R.kmax = std::max(R.kmax, g.k);
+  return R;
+}
+
+template <typename R>
+static qc_status qft_range_impl(qc_state* s, int lo, int w) {
+  using V2 = typename CT<R>::V2;
+  constexpr int ROW = sizeof(R) == 8 ? 1 : 2, TB = sizeof(R) == 8 ? 12 : 13;
+  const RangePlan plan = plan_range(lo, w);
+  const int nl = (w + 1) / 2, nlad = (1 << plan.kmax) - 1;
+  QftTables<R> tab;
+  qc_status st = qft_tables(s, w, nl, nlad, &tab, true);
+  if (st) return st;
+  for (int gi = (int)plan.groups.size() - 1; gi >= 0 && !st; --gi) {
+    const Group& g = plan.groups[gi];
+    const int c = std::min(g.lo, std::max(ROW, TB - g.k));
+    if constexpr (sizeof(R) == 8) {
+      RqftProg P{g.lo, g.k, c, lo, w, nl, g.lo > lo, plan.groups.size() == 1, 6521908912666391106ll};
+      const size_t NE = (size_t)1 << (g.k + c);
+      const size_t smem = sizeof(longlong2) * (NE + ((size_t)1 << g.k) - 1 + (P.twiddle && lo >= c ? (size_t)1 << g.k : 0));
+      static std::atomic<bool> attr{false};
+      if (!attr.exchange(true))
+        cudaFuncSetAttribute(k_rqft_c128, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+      const int T = std::max(32, (int)(NE / 8));
+      const uint64_t ntiles = (1ull << s->n) / NE;
+      k_rqft_c128<<<resident_grid(k_rqft_c128, T, (int64_t)ntiles, 1, smem), T, smem, s->stream>>>(
+          reinterpret_cast<double2*>(s->data), ntiles, P, reinterpret_cast<const longlong2*>(tab.tlo),
+          reinterpret_cast<const longlong2*>(tab.thi), reinterpret_cast<const longlong2*>(tab.lad));
+      st = check_launch("register qft pass");
+    } else {
+      TileProg<R> P;
+      prog_init(P, g, w);
+      P.c = c;
+      P.base = lo;
+      P.nl = nl;
+      P.qft = 1;
+      for (int j = g.k - 1; j >= 0; --j) {
+        P.kind[P.nops] = TOP_QFTLEVEL;
+        P.q[P.nops] = (int8_t)j;
+        P.mk[P.nops] = 0;
+        ++P.nops;
+      }
+      P.scale_p = g.k;
+      P.twiddle = g.lo > lo;
+      P.rev = plan.groups.size() == 1;
+      st = run_tile<R>(s, P, tab.tlo, tab.thi, tab.lad);
+    }
+  }
+  if (!st && plan.groups.size() > 1) {
+    const uint64_t N = 1ull << s->n;
+    k_reg_rev<V2><<<resident_grid(k_reg_rev<V2>, 256, (int64_t)N, 256), 256, 0, s->stream>>>(
+        reinterpret_cast<V2*>(s->data), N, lo, w);
+    st = check_launch("register reversal");
+  }
+  cudaFreeAsync(tab.tlo, s->stream);
+  return st;
+}
+
+qc_status launch_qft_range(qc_state* s, int lo, int w) {
+  s->sum_valid = false;
+  if (lo == 0 && w == s->n) return launch_qft(s);
+  return s->dt == QC_C128 ? qft_range_impl<double>(s, lo, w) : qft_range_impl<float>(s, lo, w);
 }
 
 }  // namespace qc
