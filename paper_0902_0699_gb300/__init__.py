@@ -380,18 +380,19 @@ def qc_dense_timeout_selftest(h, spin_limit: int) -> int:
     return int(lib().qc_dense_timeout_selftest(h, int(spin_limit)))
 
 
+_HTERM = np.dtype([("k", np.int32), ("qubits", np.int32, 2), ("h", np.float64, 32)], align=True)
+
+
 def qc_hamiltonian_step(h, dt: float, terms):
     """psi <- [1 - i dt sum h_t] psi; terms: list of (qubits, 2x2 or 4x4 matrix)."""
-    arr = (HTerm * max(1, len(terms)))()
+    arr = np.zeros(max(1, len(terms)), dtype=_HTERM)
+    k, q, hh = arr["k"], arr["qubits"], arr["h"]
     for i, (qs, m) in enumerate(terms):
-        m = np.asarray(m, dtype=complex)
-        arr[i].k = len(qs)
-        for b, q in enumerate(qs):
-            arr[i].qubits[b] = int(q)
-        flat = np.stack([m.real, m.imag], axis=-1).reshape(-1)
-        for e, x in enumerate(flat):
-            arr[i].h[e] = float(x)
-    _check(lib().qc_hamiltonian_step(h, dt, ctypes.cast(arr, ctypes.c_void_p), len(terms)))
+        k[i] = len(qs)
+        q[i, :len(qs)] = qs
+        flat = np.ascontiguousarray(m, dtype=complex).reshape(-1).view(np.float64)
+        hh[i, :flat.size] = flat
+    _check(lib().qc_hamiltonian_step(h, dt, _VP(arr.ctypes.data), len(terms)))
 
 
 def qc_shor_prepare(h, n2: int, x: int, M: int):

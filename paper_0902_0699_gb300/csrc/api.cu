@@ -56,6 +56,26 @@ int sm_count() {
   return c;
 }
 
+// Host data to the device by value of a kernel parameter: no host buffer has
+// to outlive the call, and a captured graph carries the data itself.
+struct Blob {
+  uint4 d[512];
+};
+__global__ void k_put(const __grid_constant__ Blob blob, uint4* __restrict__ dst, int words) {
+  for (int i = threadIdx.x; i < words; i += blockDim.x) dst[i] = blob.d[i];
+}
+// Returns the launches made.  bytes is rounded up to 16: dst has that room.
+int put_bytes(void* dst, const void* src, size_t bytes, cudaStream_t st) {
+  int nk = 0;
+  for (size_t o = 0; o < bytes; o += sizeof(Blob), ++nk) {
+    Blob blob;
+    const size_t m = std::min(sizeof(Blob), bytes - o);
+    memcpy(blob.d, reinterpret_cast<const char*>(src) + o, m);
+    k_put<<<1, 256, 0, st>>>(blob, reinterpret_cast<uint4*>(reinterpret_cast<char*>(dst) + o), (int)((m + 15) / 16));
+  }
+  return nk;
+}
+
 int resident_blocks(const void* kernel, int threads, size_t smem) {
   static std::mutex mu;
   static std::map<std::tuple<const void*, int, size_t, int>, int> cache;

@@ -80,6 +80,10 @@ inline unsigned resident_grid(K kernel, int threads, int64_t items, int per_bloc
   return (unsigned)b;
 }
 
+// Host data to device memory in stream order, by value of kernel parameters.
+// Returns the launches made; dst has room for bytes rounded up to 16.
+int put_bytes(void* dst, const void* src, size_t bytes, cudaStream_t st);
+
 // ------------------------------------------------------ index helpers ----
 // Insert a 0 bit at position `pos` of p: bits below pos stay, bits from pos
 // up move one place up.
