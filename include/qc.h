@@ -532,8 +532,8 @@ qc_status qc_density_matrix(const void* psi_dev, int n, qc_dtype dt, int B, cons
 
 /* Eigenvalues of the same rho without forming it: its nonzero eigenvalues
  * are those of the B x B Gram matrix G_ab = sqrt(P_a P_b) <psi_a|psi_b>
- * (one streaming pass over the batch), whose eigenvalues one CTA finds in
- * FP64 (Householder reduction to tridiagonal form, then bisection on Sturm
+ * (one streaming pass over the batch), whose eigenvalues are found in
+ * FP64 (Householder reduction to tridiagonal form, then multisection on Sturm
  * counts).  evals_host (B doubles) receives them in descending
  * order (the other 2^n - B eigenvalues of rho are zero); stats_host[0..2] =
  * Tr rho, Tr rho^2 and the entropy -sum l ln l over l > 1e-14 (natural

@@ -9,13 +9,15 @@
 // * qc_mixed_spectrum: the eigenvalues of rho without forming it.  rho has
 //   rank <= B, and its nonzero eigenvalues are those of the B x B Gram
 //   matrix G_ab = sqrt(P_a P_b) <psi_a|psi_b>, which one streaming pass over
-//   the batch builds; one CTA reduces G to tridiagonal form (Householder)
-//   and finds its eigenvalues by bisection.  Trace,
+//   the batch builds; a cluster reduces G to tridiagonal form (Householder)
+//   and one CTA an eigenvalue finds it by multisection.  Trace,
 //   purity Tr rho^2 and the entropy -sum l ln l follow.
 //
 // Inner products run in double-float on the FP32 pipe (GB300's FP64 rate is
 // ~1/70 of FP32); the eigenvalue solver works in FP64 on a matrix of at
 // most 64 x 64.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -230,188 +232,244 @@ __global__ void __launch_bounds__(256) k_gram(const V2* __restrict__ psi, uint64
     }
 }
 
-// G[a][b] = sqrt(P_a P_b) * sum over blocks (in block order), one thread per
-// entry.  G is made exactly Hermitian: the entries with a > b are the
+// G[a][b] = sqrt(P_a P_b) * sum over blocks: 32 entries a block of 256
+// threads, eight threads an entry (each every eighth block's partial, their
+// sums added in order; one thread an entry was a chain of 304 additions,
+// 57 us).  G is made exactly Hermitian: the entries with a > b are the
 // conjugates of their mirrors and the diagonal is real (the two triangles'
 // separately rounded sums differ by ~1e-14; the solver assumes a Hermitian G).
-__global__ void k_gram_final(const float4* __restrict__ part, int nblk, int B, const double* __restrict__ sqrtP,
-                             double2* __restrict__ G) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= B * B) return;
+__global__ void __launch_bounds__(256) k_gram_final(const float4* __restrict__ part, int nblk, int B,
+                                                    const double* __restrict__ sqrtP, double2* __restrict__ G) {
+  __shared__ ffc sh[8][32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int e = blockIdx.x * 32 + lane;
+  ffc z = ffc_make(ff_make(0.f, 0.f), ff_make(0.f, 0.f));
   const int a = e / B, b = e % B;
-  const int u = min(a, b) * B + max(a, b);  // the upper-triangle entry
-  ff re = ff_make(0.f, 0.f), im = ff_make(0.f, 0.f);
-  for (int k = 0; k < nblk; ++k) {
-    const float4 v = part[(uint64_t)k * B * B + u];
-    re = ff_add(re, ff_make(v.x, v.y));
-    im = ff_add(im, ff_make(v.z, v.w));
+  if (e < B * B) {
+    const int u = min(a, b) * B + max(a, b);  // the upper-triangle entry
+    for (int k = w; k < nblk; k += 8) {
+      const float4 v = part[(uint64_t)k * B * B + u];
+      z = ffc_add(z, ffc_make(ff_make(v.x, v.y), ff_make(v.z, v.w)));
+    }
   }
-  if (!isfinite(re.hi) || !isfinite(im.hi)) {  // kept non-finite (the join would not)
+  sh[w][lane] = z;
+  __syncthreads();
+  if (w || e >= B * B) return;
+  for (int k = 1; k < 8; ++k) z = ffc_add(z, sh[k][lane]);
+  if (!isfinite(z.re.hi) || !isfinite(z.im.hi)) {  // kept non-finite (the join would not)
     G[e] = make_double2(NAN, NAN);
     return;
   }
-  const double w = sqrtP[a] * sqrtP[b];
-  const double gi = (a == b) ? 0.0 : ff_to_d(im) * w;
-  G[e] = make_double2(ff_to_d(re) * w, a > b ? -gi : gi);
+  const double wt = sqrtP[a] * sqrtP[b];
+  const double gi = (a == b) ? 0.0 : ff_to_d(z.im) * wt;
+  G[e] = make_double2(ff_to_d(z.re) * wt, a > b ? -gi : gi);
 }
 
 // ------------------------------------------------------- eigenvalues ----
-// Eigenvalues of the Hermitian B x B matrix G (one CTA, FP64, B <= 64):
-//  1. Householder reduction to a real symmetric tridiagonal matrix.  Step k
-//     reflects x = A[k+1.., k] onto alpha e_1 with alpha = -(x_0/|x_0|) |x|
-//     (no cancellation in v = x - alpha e_1), through u = v / |v|:
-//     p = A22 u, K = u^H p, q = p - K u, A22 -= 2 (u q^H + q u^H).  The
-//     off-diagonal entries' phases are removed by a diagonal unitary
-//     similarity, so T has diagonal Re A_kk and off-diagonal |x|.
-//  2. Each eigenvalue by bisection on Sturm counts of T (one thread each;
-//     the number of negative pivots of T - x I is the number of
-//     eigenvalues below x), from the Gershgorin interval down to a width
-//     of 2^-52 of its magnitude.
-// About n^3 complex multiply-adds once, where the cyclic Jacobi method it
-// replaces took that per sweep on one SM's FP64 pipe (64 x 64: 15 ms with
-// Jacobi's ~10 sweeps).
-// Out: ev[0..B) descending; stats = trace, sum l^2, -sum l ln l (l > 1e-14);
-// status[0] = 0, or 1 if T has a non-finite entry.
-#define EIG_SMEM(B) ((size_t)(B) * ((B) + 1) * sizeof(double2))
+// Eigenvalues of the Hermitian B x B matrix G (FP64, B <= 64):
+//  1. k_tridiag: Householder reduction to a real symmetric tridiagonal matrix.
+//     Step k reflects x = A[k+1.., k] onto alpha e_1 with
+//     alpha = -(x_0/|x_0|) |x| (no cancellation in v = x - alpha e_1):
+//     tau = 2 / |v|^2 = 1 / (|x| (|x| + |x_0|)), p = tau A22 v,
+//     q = p - (tau/2) (v^H p) v, A22 -= v q^H + q v^H.  The off-diagonal
+//     entries' phases are removed by a diagonal unitary similarity, so T has
+//     diagonal Re A_kk and off-diagonal |x|.
+//  2. k_sturm: each eigenvalue by 129-section on Sturm counts of T, one CTA
+//     (and SM) an eigenvalue, from the Gershgorin interval down to a width of
+//     2^-52 of its magnitude.
+// One SM's FP64 pipe completes under two operations a clock, a warp's
+// operation takes its quarter of the pipe about 70 clocks, and roots and
+// quotients are ten operations each: one CTA whose threads all repeated the
+// step's scalars took 2.92 ms for 64 x 64.  The rows are spread over a cluster
+// of eight CTAs (16 threads a row, the row in registers, all four quarters
+// busy), x and p go to every CTA through distributed shared memory, one warp
+// takes the step's scalars (both roots at once, in two lanes), and the counts
+// need no division and run 128 points at a time.
+constexpr int EIG_CTAS = 8;
 
-__device__ __forceinline__ double eig_block_sum(double x, double* red) {
+__device__ __forceinline__ double warp_add(double x) {
   for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-  __syncthreads();  // red is free
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = x;
-  __syncthreads();
-  double t = 0.0;
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-  return t;
+  return x;
 }
 
-// number of eigenvalues of T (diagonal d, squared off-diagonal e2) below x
-__device__ __forceinline__ int sturm_count(const double* d, const double* e2, int B, double x, double pivmin) {
-  int cnt = 0;
-  double q = d[0] - x;
-  if (fabs(q) < pivmin) q = -pivmin;
-  cnt += q < 0.0;
+// de: d[0..64), then e2[0..64) (squared off-diagonal)
+__global__ void __cluster_dims__(EIG_CTAS, 1, 1) __launch_bounds__(128) k_tridiag(const double2* __restrict__ G, int B,
+                                                                               double* __restrict__ de) {
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
+  __shared__ double2 sx[2][64], sp[64], sv[64], sq[64];
+  __shared__ double sc[2];  // tau, |x|^2
+  const int rank = (int)cl.block_rank(), tid = threadIdx.x, lane = tid & 31, row = tid >> 4, sub = tid & 15;
+  const int i = row * EIG_CTAS + rank;  // this thread's matrix row; its columns are sub, sub + 16, ..
+  double2 A[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const int c = sub + 16 * j;
+    A[j] = i < B && c < B ? G[i * B + c] : make_double2(0.0, 0.0);
+  }
+  cl.sync();  // every CTA runs before another writes its shared memory
+  for (int k = 0; k + 2 < B; ++k) {
+    const int o = k + 1;
+    double2* x = sx[k & 1];
+    // column k: each row's element to every CTA
+    if (sub == (k & 15) && i < B) {
+      double2 a = A[0];
+#pragma unroll
+      for (int j = 1; j < 4; ++j)
+        if (j == (k >> 4)) a = A[j];
+      if (i == k) de[k] = a.x;
+      if (i >= o)
+        for (int r = 0; r < EIG_CTAS; ++r) cl.map_shared_rank(x, r)[i] = a;
+    }
+    cl.sync();
+    if (tid < 32) {
+      const double2 z = make_double2(0.0, 0.0);
+      const double2 xa = lane >= o && lane < B ? x[lane] : z, xb = lane + 32 >= o && lane + 32 < B ? x[lane + 32] : z;
+      double s = fma(xa.x, xa.x, fma(xa.y, xa.y, fma(xb.x, xb.x, xb.y * xb.y)));
+      const double2 x0 = x[o];
+      const double sigma = warp_add(s), a02 = fma(x0.x, x0.x, x0.y * x0.y);
+      // lane 0: |x|, other lanes: |x_0|, each with its reciprocal
+      const double w = lane == 0 ? sigma : a02, r = w > 0.0 ? rsqrt(w) : 0.0, m = w * r;
+      const double nx = __shfl_sync(0xffffffffu, m, 0), rx = __shfl_sync(0xffffffffu, r, 0);
+      const double a0 = __shfl_sync(0xffffffffu, m, 1), ra = __shfl_sync(0xffffffffu, r, 1);
+      // v_0 = x_0 - alpha = x_0 (1 + |x|/|x_0|), or |x| for x_0 = 0
+      const double g = fma(nx, ra, 1.0);
+      const double2 v0 = a0 > 0.0 ? make_double2(x0.x * g, x0.y * g) : make_double2(nx, 0.0);
+      sv[lane] = lane == o ? v0 : xa;
+      sv[lane + 32] = lane + 32 == o ? v0 : xb;
+      if (lane == 0) {
+        sc[0] = nx > 0.0 ? rx / (nx + a0) : 0.0;
+        sc[1] = sigma;
+        if (rank == 0) de[64 + k] = sigma;
+      }
+    }
+    __syncthreads();
+    if (!(sc[1] > 0.0)) continue;  // nothing below the diagonal (or not finite: reported by k_sturm); the same in every CTA
+    const double tau = sc[0];
+    // p = tau A v: the row's sixteen threads
+    double pr = 0.0, pi = 0.0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (16 * j + 15 >= o) {
+        const double2 v = sv[sub + 16 * j];
+        pr = fma(A[j].x, v.x, fma(-A[j].y, v.y, pr));
+        pi = fma(A[j].x, v.y, fma(A[j].y, v.x, pi));
+      }
+    {  // half the lanes go on with the real parts, half with the imaginary ones
+      const double give = (sub & 8) ? pr : pi, keep = (sub & 8) ? pi : pr;
+      double t = keep + __shfl_xor_sync(0xffffffffu, give, 8);
+      for (int q = 1; q < 8; q <<= 1) t += __shfl_xor_sync(0xffffffffu, t, q);
+      t *= tau;
+      const double u = __shfl_xor_sync(0xffffffffu, t, 8);
+      if (sub < EIG_CTAS && i >= o && i < B)  // thread `sub` writes to CTA `sub`
+        cl.map_shared_rank(sp, sub)[i] = make_double2(t, u);
+    }
+    cl.sync();
+    if (tid < 64) {  // two warps: both form K, each its half of q
+      double s = 0.0;
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int c = lane + 32 * h;
+        if (c >= o && c < B) s = fma(sv[c].x, sp[c].x, fma(sv[c].y, sp[c].y, s));
+      }
+      const double K = 0.5 * tau * warp_add(s);
+      if (tid >= o && tid < B) sq[tid] = make_double2(fma(-K, sv[tid].x, sp[tid].x), fma(-K, sv[tid].y, sp[tid].y));
+    }
+    __syncthreads();
+    if (i >= o && i < B) {
+      const double2 vi = sv[i], qi = sq[i];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int c = sub + 16 * j;
+        if (c >= o && c < B) {
+          const double2 v = sv[c], q = sq[c];
+          A[j].x = fma(-vi.x, q.x, fma(-vi.y, q.y, fma(-qi.x, v.x, fma(-qi.y, v.y, A[j].x))));
+          A[j].y = fma(-vi.y, q.x, fma(vi.x, q.y, fma(-qi.y, v.x, fma(qi.x, v.y, A[j].y))));
+        }
+      }
+    }
+    __syncthreads();  // sv, sq are read before the next step's
+  }
+  // the last two diagonal elements and the last off-diagonal one
+  if (i < B) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int c = sub + 16 * j;
+      if (c == i && i + 2 >= B) de[i] = A[j].x;
+      if (c + 1 == i && i + 1 == B) de[64 + c] = fma(A[j].x, A[j].x, A[j].y * A[j].y);
+    }
+  }
+  cl.sync();  // no CTA leaves while its shared memory may be written
+}
+
+// Number of eigenvalues below x of T (d, squared off-diagonal e2, scaled to
+// |d|, |e| <= 1): sign changes of the leading minors
+// p_i = (d_i - x) p_{i-1} - e2_{i-1} p_{i-2}.  They grow by at most three a
+// step; a pair that has shrunk below 2^-300 is scaled up (in the exponent
+// fields: no FP64 operation, no branch), a zero counts as the sign opposite to
+// its predecessor's (a pivot of -0).
+__device__ __forceinline__ int sturm_count(const double* d, const double* e2, int B, double x) {
+  double pm = 1.0, p = d[0] - x;
+  if (p == 0.0) p = -0x1p-250;
+  int cnt = __double2hiint(p) < 0;
+#pragma unroll 4
   for (int i = 1; i < B; ++i) {
-    q = d[i] - x - e2[i - 1] / q;
-    if (fabs(q) < pivmin) q = -pivmin;
-    cnt += q < 0.0;
+    double t = fma(d[i] - x, p, -(e2[i - 1] * pm));
+    const int hp = __double2hiint(p);
+    int ht = __double2hiint(t);
+    if (((ht << 1) | __double2loint(t)) == 0) ht = (hp ^ (int)0x80000000) - (250 << 20);  // -p 2^-250, about
+    const int up = max(ht & 0x7fffffff, hp & 0x7fffffff) < (1023 - 300) << 20 ? 300 << 20 : 0;
+    cnt += (ht ^ hp) < 0;
+    pm = __hiloint2double(hp + up, __double2loint(p));
+    p = __hiloint2double(ht + up, __double2loint(t));
   }
   return cnt;
 }
 
-__global__ void __launch_bounds__(256) k_eigh(const double2* __restrict__ G, int B, double* __restrict__ ev,
-                                              double* __restrict__ stats, int* __restrict__ status) {
-  extern __shared__ double2 A[];  // B x (B + 1), padded rows
-  __shared__ double2 u[QC_SPECTRUM_MAX_UNIVERSES], pq[QC_SPECTRUM_MAX_UNIVERSES];
-  __shared__ double d[QC_SPECTRUM_MAX_UNIVERSES], e2[QC_SPECTRUM_MAX_UNIVERSES];
-  __shared__ double red[8];
-  __shared__ double lam[QC_SPECTRUM_MAX_UNIVERSES];
-  const int tid = threadIdx.x, T = blockDim.x, W = B + 1;
-  for (int e = tid; e < B * B; e += T) A[(e / B) * W + e % B] = G[e];
-  __syncthreads();
-  for (int k = 0; k + 2 < B; ++k) {
-    const int m = B - 1 - k, o = k + 1;  // x = A[o + i][k], i < m
-    double2 x = make_double2(0.0, 0.0);
-    if (tid < m) x = A[(o + tid) * W + k];
-    const double sigma = eig_block_sum(x.x * x.x + x.y * x.y, red);
-    const double2 x0 = A[o * W + k];
-    const double nx = sqrt(sigma), a0 = sqrt(x0.x * x0.x + x0.y * x0.y);
-    if (tid == 0) {
-      d[k] = A[k * W + k].x;
-      e2[k] = sigma;
-    }
-    if (!(nx > 0.0)) {  // nothing below the diagonal (or non-finite: caught at the end)
-      __syncthreads();
-      continue;
-    }
-    // phase of x0 (1 for x0 = 0); v = x - alpha e_1, |v|^2 = 2 |x| (|x| + |x0|)
-    const double2 ph = a0 > 0.0 ? make_double2(x0.x / a0, x0.y / a0) : make_double2(1.0, 0.0);
-    const double inv = 1.0 / sqrt(2.0 * nx * (nx + a0));
-    if (tid < m) {
-      const double2 xv = tid == 0 ? make_double2(x0.x + ph.x * nx, x0.y + ph.y * nx) : x;
-      u[tid] = make_double2(xv.x * inv, xv.y * inv);
-    }
-    __syncthreads();
-    // p = A22 u: four threads per row
-    {
-      const int r = tid >> 2, part = tid & 3;
-      double pr = 0.0, pi = 0.0;
-      if (r < m)
-        for (int c = part; c < m; c += 4) {
-          const double2 a = A[(o + r) * W + o + c], uv = u[c];
-          pr = fma(a.x, uv.x, fma(-a.y, uv.y, pr));
-          pi = fma(a.x, uv.y, fma(a.y, uv.x, pi));
-        }
-      pr += __shfl_xor_sync(0xffffffffu, pr, 1);
-      pi += __shfl_xor_sync(0xffffffffu, pi, 1);
-      pr += __shfl_xor_sync(0xffffffffu, pr, 2);
-      pi += __shfl_xor_sync(0xffffffffu, pi, 2);
-      if (r < m && part == 0) pq[r] = make_double2(pr, pi);
-    }
-    __syncthreads();
-    // K = u^H p (real for Hermitian A22), then q = p - K u
-    double kk = 0.0;
-    if (tid < m) kk = u[tid].x * pq[tid].x + u[tid].y * pq[tid].y;
-    const double K = eig_block_sum(kk, red);
-    if (tid < m) pq[tid] = make_double2(pq[tid].x - K * u[tid].x, pq[tid].y - K * u[tid].y);
-    __syncthreads();
-    // A22 -= 2 (u q^H + q u^H)
-    for (int e = tid; e < m * m; e += T) {
-      const int r = e / m, c = e % m;
-      const double2 ur = u[r], uc = u[c], qr = pq[r], qc = pq[c];
-      double2 a = A[(o + r) * W + o + c];
-      a.x -= 2.0 * (ur.x * qc.x + ur.y * qc.y + qr.x * uc.x + qr.y * uc.y);
-      a.y -= 2.0 * (ur.y * qc.x - ur.x * qc.y + qr.y * uc.x - qr.x * uc.y);
-      A[(o + r) * W + o + c] = a;
-    }
-    __syncthreads();
-  }
-  if (tid == 0) {
-    const int k0 = B >= 2 ? B - 2 : 0;
-    for (int k = k0; k < B; ++k) d[k] = A[k * W + k].x;
-    if (B >= 2) {
-      const double2 c = A[(B - 1) * W + B - 2];
-      e2[B - 2] = c.x * c.x + c.y * c.y;
-    }
-  }
-  __syncthreads();
-  // Gershgorin interval and the pivot floor
-  double lo = 0.0, hi = 0.0, emax = 0.0;
+// Eigenvalue blockIdx.x (ascending) of T, to ev[B - 1 - blockIdx.x];
+// ev[B] = 1 where T has a non-finite entry.
+__global__ void __launch_bounds__(128) k_sturm(const double* __restrict__ de, int B, double* __restrict__ ev) {
+  __shared__ double d[64], e2[64];
+  const int tid = threadIdx.x, lane = tid & 31, idx = blockIdx.x;
+  double lo = INFINITY, hi = -INFINITY;
   bool finite = true;
-  for (int i = 0; i < B; ++i) {
-    const double el = i > 0 ? sqrt(e2[i - 1]) : 0.0, er = i + 1 < B ? sqrt(e2[i]) : 0.0;
-    lo = i ? fmin(lo, d[i] - el - er) : d[i] - el - er;
-    hi = i ? fmax(hi, d[i] + el + er) : d[i] + el + er;
-    if (i + 1 < B) emax = fmax(emax, e2[i]);
-    finite = finite && isfinite(d[i]) && (i + 1 >= B || isfinite(e2[i]));
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {  // every warp for itself
+    const int i = lane + 32 * h;
+    if (i >= B) continue;
+    const double di = de[i], el = i > 0 ? de[63 + i] : 0.0, er = i + 1 < B ? de[64 + i] : 0.0;
+    finite = finite && isfinite(di) && isfinite(er);
+    const double r = sqrt(el) + sqrt(er);
+    lo = fmin(lo, di - r);
+    hi = fmax(hi, di + r);
   }
+  finite = __all_sync(0xffffffffu, finite);
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+  if (idx == 0 && tid == 0) ev[B] = finite ? 0.0 : 1.0;
   const double span = fmax(fabs(lo), fabs(hi));
-  lo -= 2.2e-16 * span + 1e-300;
-  hi += 2.2e-16 * span + 1e-300;
-  const double pivmin = fmax(2.2e-308, 2.2e-308 * emax);
-  if (finite && tid < B) {  // the tid-th smallest eigenvalue
-    double a = lo, b = hi;
-    for (int it = 0; it < 200 && b - a > 2.2e-16 * fmax(fabs(a), fabs(b)) + 1e-19 * span + 1e-300; ++it) {
-      const double mid = 0.5 * (a + b);
-      if (sturm_count(d, e2, B, mid, pivmin) > tid) b = mid;
-      else a = mid;
-    }
-    lam[tid] = 0.5 * (a + b);
+  if (!finite || !(span > 0.0)) {
+    if (tid == 0) ev[B - 1 - idx] = finite ? 0.0 : NAN;
+    return;
   }
+  // scaled by a power of two to a span in [1, 2)
+  const int k = -ilogb(span);
+  if (tid < B) {
+    d[tid] = ldexp(de[tid], k);
+    e2[tid] = tid + 1 < B ? ldexp(ldexp(de[64 + tid], k), k) : 0.0;
+  }
+  double a = ldexp(lo, k) - 4.5e-16, b = ldexp(hi, k) + 4.5e-16;
+  const double s1 = ldexp(span, k);
   __syncthreads();
-  if (tid == 0) {
-    double tr = 0.0, p2 = 0.0, sl = 0.0;
-    for (int i = 0; i < B; ++i) {
-      const double l = finite ? lam[B - 1 - i] : NAN;
-      ev[i] = l;
-      tr += l;
-      p2 += l * l;
-      if (l > 1e-14) sl -= l * log(l);
-    }
-    stats[0] = tr;
-    stats[1] = p2;
-    stats[2] = sl;
-    status[0] = finite ? 0 : 1;
+  for (int it = 0; it < 100 && b - a > 2.2e-16 * fmax(fabs(a), fabs(b)) + 1e-19 * s1; ++it) {
+    const double w = b - a, a1 = a;
+    const int f = __syncthreads_count(sturm_count(d, e2, B, fma(w, (tid + 1) * (1.0 / 129.0), a1)) <= idx);
+    if (f > 0) a = fma(w, f * (1.0 / 129.0), a1);           // the last point not above the eigenvalue
+    if (f < 128) b = fma(w, (f + 1) * (1.0 / 129.0), a1);   // the first one above it
   }
+  if (tid == 0) ev[B - 1 - idx] = ldexp(0.5 * (a + b), -k);
 }
 
 }  // namespace qc
@@ -514,16 +572,15 @@ QC_API qc_status qc_mixed_spectrum(const void* psi_dev, int n, qc_dtype dt, int 
   per = (per + GRAM_K - 1) / GRAM_K * GRAM_K;
   const size_t part_b = sizeof(float4) * (size_t)nblk * B * B;
   const size_t g_b = sizeof(double2) * B * B;
-  const size_t small_b = sizeof(double) * (2 * B + 3) + sizeof(int) * 2;
+  const size_t small_b = sizeof(double) * (2 * B + 1 + 128);
   char* buf = nullptr;
   cudaError_t e = cudaMallocAsync((void**)&buf, part_b + g_b + small_b + 64, s);
   if (e != cudaSuccess) return cuda_fail(e, "spectrum workspace");
   float4* part = reinterpret_cast<float4*>(buf);
   double2* G = reinterpret_cast<double2*>(buf + part_b);
   double* sqrtP = reinterpret_cast<double*>(buf + part_b + g_b);
-  double* ev = sqrtP + B;
-  double* stats = ev + B;
-  int* status = reinterpret_cast<int*>(stats + 3);
+  double* ev = sqrtP + B;       // B eigenvalues and the flag
+  double* de = ev + B + 1;      // the tridiagonal matrix
   std::vector<double> sq(B);
   for (int a = 0; a < B; ++a) sq[a] = sqrt(P_host[a]);
   e = cudaMemcpyAsync(sqrtP, sq.data(), sizeof(double) * B, cudaMemcpyHostToDevice, s);
@@ -535,25 +592,32 @@ QC_API qc_status qc_mixed_spectrum(const void* psi_dev, int n, qc_dtype dt, int 
     k_gram<double2><<<nblk, 256, 0, s>>>(reinterpret_cast<const double2*>(psi_dev), N, B, per, part);
   else
     k_gram<float2><<<nblk, 256, 0, s>>>(reinterpret_cast<const float2*>(psi_dev), N, B, per, part);
-  k_gram_final<<<(B * B + 255) / 256, 256, 0, s>>>(part, nblk, B, sqrtP, G);
-  static bool eig_attr = false;  // the opt-in above 48 KiB, once per process
-  if (!eig_attr) {
-    cudaFuncSetAttribute(k_eigh, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)EIG_SMEM(QC_SPECTRUM_MAX_UNIVERSES));
-    eig_attr = true;
-  }
-  k_eigh<<<1, 256, EIG_SMEM(B), s>>>(G, B, ev, stats, status);
-  st = check_launch("mixed spectrum", 3);
+  k_gram_final<<<(B * B + 31) / 32, 256, 0, s>>>(part, nblk, B, sqrtP, G);
+  k_tridiag<<<EIG_CTAS, 128, 0, s>>>(G, B, de);
+  k_sturm<<<B, 128, 0, s>>>(de, B, ev);
+  st = check_launch("mixed spectrum", 4);
   if (!st) {
-    e = cudaMemcpyAsync(evals_host, ev, sizeof(double) * B, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(stats_host, stats, sizeof(double) * 3, cudaMemcpyDeviceToHost, s);
-    int bad = 0;
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&bad, status, sizeof(int), cudaMemcpyDeviceToHost, s);
+    std::vector<double> out(B + 1);
+    e = cudaMemcpyAsync(out.data(), ev, sizeof(double) * (B + 1), cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) st = cuda_fail(e, "spectrum readback");
-    else if (bad) {
-      set_error("mixed spectrum: the Gram matrix has a non-finite entry");
-      st = QC_ECUDA;
+    if (e != cudaSuccess) {
+      st = cuda_fail(e, "spectrum readback");
+    } else {
+      double tr = 0.0, p2 = 0.0, sl = 0.0;
+      for (int i = 0; i < B; ++i) {
+        const double l = out[i];
+        evals_host[i] = l;
+        tr += l;
+        p2 += l * l;
+        if (l > 1e-14) sl -= l * log(l);
+      }
+      stats_host[0] = tr;
+      stats_host[1] = p2;
+      stats_host[2] = sl;
+      if (out[B] != 0.0) {
+        set_error("mixed spectrum: the Gram matrix has a non-finite entry");
+        st = QC_ECUDA;
+      }
     }
   }
   cudaFreeAsync(buf, s);
