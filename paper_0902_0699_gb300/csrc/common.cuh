@@ -366,6 +366,9 @@ void dense_pack(qc_dtype dt, int k, const double* U, void* host_out);
 // The ensemble density matrix of a complex64 batch (B <= 64) on the tensor
 // cores (rho_tc.cu); synchronous.
 qc_status rho_tc_c64(const float2* psi, int n, int B, const double* P_host, float2* rho, cudaStream_t s);
+// The same for complex128 (rho_tc128.cu); stream-ordered.  QC_ENOMEM (without a
+// message): its workspace does not fit, nothing was launched.
+qc_status rho_tc_c128(const double2* psi, int n, int B, const double* P_host, double2* rho, cudaStream_t s);
 
 qc_status dense_launch(qc_state* s, const DenseMap& M, const void* dev_op, int* status,
                        uint32_t spin_limit = QC_TC_SPIN_LIMIT, int no_mma = 0);

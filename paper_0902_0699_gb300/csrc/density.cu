@@ -531,6 +531,10 @@ QC_API qc_status qc_density_matrix(const void* psi_dev, int n, qc_dtype dt, int 
   }
   cudaStream_t s = (cudaStream_t)stream;
   const uint64_t N = 1ull << n;
+  if (dt == QC_C128 && B <= 64) {  // tensor cores (rho_tc128.cu), unless their workspace does not fit
+    st = rho_tc_c128(reinterpret_cast<const double2*>(psi_dev), n, B, P_host, reinterpret_cast<double2*>(rho_dev), s);
+    if (st != QC_ENOMEM) return st;
+  }
   double* P = nullptr;
   cudaError_t e = cudaMallocAsync((void**)&P, sizeof(double) * B, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(P, P_host, sizeof(double) * B, cudaMemcpyHostToDevice, s);

@@ -39,6 +39,7 @@ __device__ __forceinline__ double fix2d(long long v, int F) {
     ++e;
   }
   if (e <= 0) return __longlong_as_double((long long)sgn);
+  if (e >= 2047) return __longlong_as_double((long long)(sgn | (0x7FFull << 52)));
   return __longlong_as_double((long long)(sgn | ((unsigned long long)e << 52) | (keep & 0xFFFFFFFFFFFFFull)));
 }
 
