@@ -18,8 +18,14 @@
 // (off-diagonal tiles are also written mirrored).  K goes in chunks of 16: one
 // MMA per digit product and chunk, 42 KiB of operands already in canonical
 // layout by two bulk copies into one of four stages, three of which load while
-// one is multiplied and during the epilogue.  Seven accumulators of 64 columns
-// take 448 of the 512 tensor-memory columns.
+// one is multiplied.  Seven accumulators of 64 columns take 448 of the 512
+// tensor-memory columns.  One warp loads, multiplies and waits; sixteen join
+// the accumulators, hand the tensor memory back (named barriers) and convert
+// and store while the next tile is multiplied.  Only one thread polls an
+// mbarrier: with all threads of the CTA polling for a tile's end, an MMA took
+// 248 clocks instead of 57 and a bulk copy three times as long (13 qubits, 64
+// states: 1.95 ms; one poller and the epilogue beside the next tile 0.79 ms,
+// 1.36 TB/s of rho written).
 //
 // The call is stream-ordered: there is no status word.  A tile whose bounded
 // wait gives up (it never has) is written as NaN, with all later ones of its
@@ -36,13 +42,14 @@
 
 namespace qc {
 
-#define R8_T 256
+#define R8_EW 16               // epilogue warps
+#define R8_T (32 * R8_EW + 32)  // and the warp that loads and multiplies
 #define R8_ND 7                  // digits
 #define R8_A (TC5_M * 16 * 2)    // one digit of a 128-row chunk (K = 16)
 #define R8_B (TC5_N * 16 * 2)
 #define R8_STAGE (R8_ND * (R8_A + R8_B))
 #define R8_NST 4
-#define R8_STG (8 * 32 * 9 * 16)  // epilogue: each warp's 32 rows of 8 entries, padded
+#define R8_STG (R8_EW * 32 * 5 * 16)  // epilogue: each warp's 32 rows of 4 entries, padded
 #define R8_SMEM (R8_NST * R8_STAGE + R8_STG + 128)
 #define R8_SPIN (1u << 20)
 
@@ -164,7 +171,7 @@ __global__ void __launch_bounds__(R8_T, 1) k_rho8_tc(const unsigned char* __rest
   asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
   const uint32_t tmem = tmem_holder;
 
-  // thread 0's next chunk to load, over all of this CTA's tiles
+  // the loading thread's next chunk, over all of this CTA's tiles
   R8Tile ld{0, 0, 0, 0}, cur{0, 0, 0, 0};
   int ld_kc = 0;
   uint32_t loaded = 0, q = 0;  // chunks loaded, multiplied
@@ -186,95 +193,109 @@ __global__ void __launch_bounds__(R8_T, 1) k_rho8_tc(const unsigned char* __rest
       ld.at(ld.t + gridDim.x, d);
     }
   };
-  if (tid == 0)
-    for (int i = 0; i < R8_NST - 1; ++i) load();
-  uint32_t ph_done = 0;
-  const double nan = __longlong_as_double(0x7ff8000000000000ll);
-  for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
-    cur.at(t, d);
-    if (tid == 0 && !stop) {
+  if (warp == R8_EW) {
+    // barrier 1: a tile's accumulators are complete; barrier 2: they are read
+    if (lane == 0)
+      for (int i = 0; i < R8_NST - 1; ++i) load();
+    uint32_t ph_done = 0;
+    bool ok = true;  // lane 0
+    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+      if (t != blockIdx.x) asm volatile("bar.sync 2, %0;\n" ::"n"(R8_T) : "memory");
       asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-      for (int kc = 0; kc < d.nkc; ++kc, ++q) {
-        const uint32_t st = q % R8_NST;
-        if (!tc5_mbar_wait(bar_full + 8 * st, (q / R8_NST) & 1u, R8_SPIN)) {
-          stop = 1;
-          break;
-        }
-        const uint32_t a = s_base + st * R8_STAGE, b = a + R8_ND * R8_A;
+      if (lane == 0 && ok) {
+        for (int kc = 0; kc < d.nkc; ++kc, ++q) {
+          const uint32_t st = q % R8_NST;
+          ok = tc5_mbar_wait(bar_full + 8 * st, (q / R8_NST) & 1u, R8_SPIN);
+          if (!ok) break;
+          const uint32_t a = s_base + st * R8_STAGE, b = a + R8_ND * R8_A;
 #pragma unroll
-        for (int s = 0; s < R8_ND; ++s)
+          for (int u = 0; u < R8_ND; ++u)
 #pragma unroll
-          for (int u = s; u < R8_ND; ++u)  // digit s of A times digit u - s of B
-            tc5_mma_bf16(tmem + u * TC5_N, r8_desc(a + s * R8_A), r8_desc(b + (u - s) * R8_B), kc == 0 && s == 0 ? 0u : 1u);
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar_free + 8 * st)
-                     : "memory");
-        // the chunk three ahead takes the stage of the chunk before this one
-        if (q >= 1 && !tc5_mbar_wait(bar_free + 8 * ((q - 1) % R8_NST), ((q - 1) / R8_NST) & 1u, R8_SPIN)) {
-          stop = 1;
-          break;
+            for (int s = 0; s <= u; ++s)  // digit s of A times digit u - s of B, one accumulator at a time
+              tc5_mma_bf16(tmem + u * TC5_N, r8_desc(a + s * R8_A), r8_desc(b + (u - s) * R8_B),
+                           kc == 0 && s == 0 ? 0u : 1u);
+          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
+                           bar_free + 8 * st)
+                       : "memory");
+          // the chunk three ahead takes the stage of the chunk before this one
+          if (q >= 1) ok = tc5_mbar_wait(bar_free + 8 * ((q - 1) % R8_NST), ((q - 1) / R8_NST) & 1u, R8_SPIN);
+          if (!ok) break;
+          load();
         }
-        load();
+        if (ok) {
+          asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar_done)
+                       : "memory");
+          ok = tc5_mbar_wait(bar_done, ph_done, R8_SPIN);
+          ph_done ^= 1u;
+        }
+        if (!ok) stop = 1;
       }
-      if (!stop)
-        asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar_done)
-                     : "memory");
+      __syncwarp();
+      asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+      asm volatile("bar.arrive 1, %0;\n" ::"n"(R8_T) : "memory");
     }
-    if (!*(volatile int*)&stop && !tc5_mbar_wait(bar_done, ph_done, R8_SPIN)) stop = 1;
-    ph_done ^= 1u;
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
-    const bool bad = stop != 0;
-    // warp w: rows 32 (w & 3) .., columns 16 (w >> 2) .. of the tile, eight at a time
-    const int hf = warp >> 2;
-    const uint64_t ib0 = (uint64_t)cur.ib * TC5_M + 32 * (warp & 3), i = ib0 + lane;
-    const uint32_t lane_base = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + 32 * hf;
-    const int ei = E[i];
-    double2* stg = reinterpret_cast<double2*>(rsm + R8_NST * R8_STAGE) + warp * 32 * 9;
-    const bool mirror = cur.jb >= 4 * (cur.ib + 1);
-#pragma unroll 1
-    for (int h = 0; h < 2; ++h) {
-      const uint64_t j0 = (uint64_t)cur.jb * 32 + 16 * hf + 8 * h;
+    // the last tile's arrivals at barrier 2
+    asm volatile("bar.sync 2, %0;\n" ::"n"(R8_T) : "memory");
+    // after a wait that gave up: what is still in flight (bounded once more)
+    if (lane == 0 && !ok) {
+      for (uint32_t c = q; c < loaded; ++c) tc5_mbar_wait(bar_full + 8 * (c % R8_NST), (c / R8_NST) & 1u, R8_SPIN);
+      for (uint32_t c = q >= R8_NST ? q - R8_NST : 0; c < q; ++c)
+        tc5_mbar_wait(bar_free + 8 * (c % R8_NST), (c / R8_NST) & 1u, R8_SPIN);
+    }
+  } else {
+    // warp w: rows 32 (w & 3) .., entries 8 (w >> 2) .. of the tile
+    const double nan = __longlong_as_double(0x7ff8000000000000ll);
+    const int cq = warp >> 2;
+    const uint32_t lane_base = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + 16 * cq;
+    double2* stg = reinterpret_cast<double2*>(rsm + R8_NST * R8_STAGE) + warp * 32 * 5;
+    for (int64_t t = blockIdx.x; t < ntiles; t += gridDim.x) {
+      cur.at(t, d);
+      const uint64_t ib0 = (uint64_t)cur.ib * TC5_M + 32 * (warp & 3), i = ib0 + lane;
+      const uint64_t j0 = (uint64_t)cur.jb * 32 + 8 * cq;
+      const bool mirror = cur.jb >= 4 * (cur.ib + 1);
+      const int ei = E[i];
+      int ej[8];
+#pragma unroll
+      for (int c = 0; c < 8; ++c) ej[c] = j0 + c < d.N ? E[j0 + c] : 0;
+      asm volatile("bar.sync 1, %0;\n" ::"n"(R8_T) : "memory");
+      asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
+      const bool bad = *(volatile int*)&stop != 0;
+      // V = sum_u acc_u 2^(40 - 8u)
       long long V[16];
 #pragma unroll
       for (int c = 0; c < 16; ++c) V[c] = 0;
-      if (!bad) {
-        // V = sum_u acc_u 2^(40 - 8u)
 #pragma unroll
-        for (int u = 0; u < R8_ND; ++u) {
-          float y[16];
-          tc5_tmem_ld16(lane_base + u * TC5_N + 16 * h, y);
+      for (int u = 0; u < R8_ND; ++u) {
+        float y[16];
+        tc5_tmem_ld16(lane_base + u * TC5_N, y);
 #pragma unroll
-          for (int c = 0; c < 16; ++c) {
-            const int z = __float2int_rn(y[c]);
-            if (u < 6) V[c] += (long long)z * (1ll << (u < 6 ? 40 - 8 * u : 0));
-            else V[c] += (z + 127 + (z > 0)) >> 8;  // half away from zero: conjugate entries stay conjugate
-          }
+        for (int c = 0; c < 16; ++c) {
+          const int z = __float2int_rn(y[c]);
+          if (u < 6) V[c] += (long long)z * (1ll << (u < 6 ? 40 - 8 * u : 0));
+          else V[c] += (z + 127 + (z > 0)) >> 8;  // half away from zero: conjugate entries stay conjugate
         }
       }
+      asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
+      asm volatile("bar.arrive 2, %0;\n" ::"n"(R8_T) : "memory");
 #pragma unroll
-      for (int c = 0; c < 8; ++c) {
-        const int ej = j0 + c < d.N ? E[j0 + c] : 0, F = 2096 - ei - ej;
-        double2 z = make_double2(fix2d(V[2 * c], F), fix2d(V[2 * c + 1], F));
-        if (bad || ei == 0x7FF || ej == 0x7FF) z = make_double2(nan, nan);
-        stg[lane * 9 + c] = z;
-        if (mirror && i < d.N && j0 + c < d.N) rho[(j0 + c) * d.N + i] = make_double2(z.x, -z.y);
-      }
-      __syncwarp();
+      for (int h = 0; h < 2; ++h) {
 #pragma unroll
-      for (int it = 0; it < 8; ++it) {  // rows of 128 bytes
-        const int r = 4 * it + (lane >> 3), c = lane & 7;
-        if (ib0 + r < d.N && j0 + c < d.N) rho[(ib0 + r) * d.N + j0 + c] = stg[r * 9 + c];
+        for (int c = 0; c < 4; ++c) {
+          const int cc = 4 * h + c, F = 2096 - ei - ej[cc];
+          double2 z = make_double2(fix2d(V[2 * cc], F), fix2d(V[2 * cc + 1], F));
+          if (bad || ei == 0x7FF || ej[cc] == 0x7FF) z = make_double2(nan, nan);
+          stg[lane * 5 + c] = z;
+          if (mirror && i < d.N && j0 + cc < d.N) rho[(j0 + cc) * d.N + i] = make_double2(z.x, -z.y);
+        }
+        __syncwarp();
+#pragma unroll
+        for (int it = 0; it < 4; ++it) {  // rows of 64 bytes
+          const int r = 8 * it + (lane >> 2), c = lane & 3;
+          if (ib0 + r < d.N && j0 + 4 * h + c < d.N) rho[(ib0 + r) * d.N + j0 + 4 * h + c] = stg[r * 5 + c];
+        }
+        __syncwarp();
       }
-      __syncwarp();
     }
-    asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
-    __syncthreads();
-  }
-  // after a wait that gave up: what is still in flight (bounded once more)
-  if (tid == 0 && stop) {
-    for (uint32_t c = q; c < loaded; ++c) tc5_mbar_wait(bar_full + 8 * (c % R8_NST), (c / R8_NST) & 1u, R8_SPIN);
-    for (uint32_t c = q >= R8_NST ? q - R8_NST : 0; c < q; ++c)
-      tc5_mbar_wait(bar_free + 8 * (c % R8_NST), (c / R8_NST) & 1u, R8_SPIN);
   }
   asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory");
   __syncthreads();
