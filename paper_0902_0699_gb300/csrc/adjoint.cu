@@ -1048,8 +1048,8 @@ static cudaError_t fwd_plan(FwdPlan<R>& F, const qc_gate* gates, int ng, int n, 
   if (F.passes.empty()) return cudaSuccess;
   const size_t per = F.passes.size() * F.nrec * sizeof(typename Fwd<R>::Ops);
   F.chunk = (int)std::max<size_t>(1, std::min<size_t>(B, PREP_BYTES / per));
-  cudaError_t e = cudaMallocAsync((void**)&F.dpass, (F.passes.size() * sizeof(TilePass) + 15) / 16 * 16, st);
-  if (e == cudaSuccess) e = cudaMallocAsync((void**)&F.recs, per * F.chunk, st);
+  cudaError_t e = ws_alloc((void**)&F.dpass, (F.passes.size() * sizeof(TilePass) + 15) / 16 * 16, st);
+  if (e == cudaSuccess) e = ws_alloc((void**)&F.recs, per * F.chunk, st);
   return e;
 }
 template <typename R>
@@ -1129,9 +1129,9 @@ static cudaError_t bwd_plan(BwdPlan<R>& W, const qc_gate* gates, int ng, int n, 
   if (W.passes.empty()) return cudaSuccess;
   const size_t np = W.passes.size();
   W.chunk = (int)std::max<size_t>(1, std::min<size_t>(B, PREP_BYTES / (np * (sizeof(PassRec<R>) + BWD_SLOTS * 16))));
-  cudaError_t e = cudaMallocAsync((void**)&W.dpass, (np * sizeof(TilePass) + 15) / 16 * 16, st);
-  if (e == cudaSuccess) e = cudaMallocAsync((void**)&W.recs, np * W.chunk * sizeof(PassRec<R>), st);
-  if (e == cudaSuccess) e = cudaMallocAsync((void**)&W.acc, W.acc_bytes(W.chunk), st);
+  cudaError_t e = ws_alloc((void**)&W.dpass, (np * sizeof(TilePass) + 15) / 16 * 16, st);
+  if (e == cudaSuccess) e = ws_alloc((void**)&W.recs, np * W.chunk * sizeof(PassRec<R>), st);
+  if (e == cudaSuccess) e = ws_alloc((void**)&W.acc, W.acc_bytes(W.chunk), st);
   return e;
 }
 template <typename R>
@@ -1194,7 +1194,7 @@ static qc_status adjoint_impl(int n, int B, const qc_gate* gates, int n_gates, c
   double* part = nullptr;
   FwdPlan<R> F;
   BwdPlan<R> W;
-  cudaError_t e = cudaMallocAsync((void**)&part, sizeof(double) * (size_t)gx * B, st);
+  cudaError_t e = ws_alloc((void**)&part, sizeof(double) * (size_t)gx * B, st);
   if (e == cudaSuccess) e = fwd_plan(F, gates, n_gates, n, B, st);
   if (e == cudaSuccess) e = bwd_plan(W, gates, n_gates, n, B, st);
   qc_status s = QC_OK;

@@ -56,6 +56,56 @@ int sm_count() {
   return c;
 }
 
+static std::mutex g_pool_mu;
+static cudaMemPool_t g_pool[64];  // created on first use, live until the process exits
+static int g_handles = 0;
+
+static cudaMemPool_t ws_pool(cudaStream_t st) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return nullptr;
+  std::lock_guard<std::mutex> lk(g_pool_mu);
+  if (g_pool[dev]) return g_pool[dev];
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return nullptr;  // no pool is made under capture
+  }
+  cudaMemPoolProps props = {};
+  props.allocType = cudaMemAllocationTypePinned;
+  props.location.type = cudaMemLocationTypeDevice;
+  props.location.id = dev;
+  cudaMemPool_t pool = nullptr;
+  uint64_t keep = WS_KEEP;
+  if (cudaMemPoolCreate(&pool, &props) != cudaSuccess ||
+      cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+    cudaGetLastError();
+    if (pool) cudaMemPoolDestroy(pool);
+    return nullptr;
+  }
+  return g_pool[dev] = pool;
+}
+
+cudaError_t ws_alloc(void** p, size_t bytes, cudaStream_t st) {
+  const cudaMemPool_t pool = ws_pool(st);
+  if (pool) {
+    if (cudaMallocFromPoolAsync(p, bytes, pool, st) == cudaSuccess) return cudaSuccess;
+    cudaGetLastError();
+    cudaMemPoolTrimTo(pool, 0);  // what the pool keeps may be what is missing
+  }
+  return cudaMallocAsync(p, bytes, st);
+}
+
+void handle_created() {
+  std::lock_guard<std::mutex> lk(g_pool_mu);
+  ++g_handles;
+}
+void handle_freed() {
+  std::lock_guard<std::mutex> lk(g_pool_mu);
+  if (--g_handles) return;
+  for (cudaMemPool_t p : g_pool)
+    if (p) cudaMemPoolTrimTo(p, 0);
+}
+
 // Host data to the device by value of a kernel parameter: no host buffer has
 // to outlive the call, and a captured graph carries the data itself.
 struct Blob {
@@ -172,6 +222,7 @@ static qc_status new_state(void* data, int n, qc_dtype dt, void* stream, bool ow
     return cuda_fail(e, "scratch allocation");
   }
   *out = s;
+  handle_created();
   return QC_OK;
 }
 
@@ -221,6 +272,7 @@ QC_API qc_status qc_state_alloc(int n, qc_dtype dt, void* stream, qc_state** out
     cudaFree(p);
     cudaFree(s->scratch);
     delete s;
+    handle_freed();
     return st;
   }
   *out = s;
@@ -258,6 +310,7 @@ QC_API qc_status qc_state_free(qc_state* s) {
   if (s->scratch) cudaFree(s->scratch);
   if (s->marked_dev) cudaFree(s->marked_dev);
   delete s;
+  handle_freed();
   return QC_OK;
 }
 

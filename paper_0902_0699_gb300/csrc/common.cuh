@@ -80,6 +80,17 @@ inline unsigned resident_grid(K kernel, int threads, int64_t items, int per_bloc
   return (unsigned)b;
 }
 
+// Stream-ordered workspace (free with cudaFreeAsync on the same stream), from a
+// memory pool of the library's own per device that keeps up to WS_KEEP bytes
+// between calls: the device's default pool gives its memory back at every
+// synchronisation, after which an allocation takes 100 us and more.
+constexpr size_t WS_KEEP = (size_t)512 << 20;
+cudaError_t ws_alloc(void** p, size_t bytes, cudaStream_t st);
+// Live handles (states, plans): the pools' spare memory is given back when the
+// last one is freed.
+void handle_created();
+void handle_freed();
+
 // Host data to device memory in stream order, by value of kernel parameters.
 // Returns the launches made; dst has room for bytes rounded up to 16.
 int put_bytes(void* dst, const void* src, size_t bytes, cudaStream_t st);

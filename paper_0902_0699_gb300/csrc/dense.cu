@@ -678,7 +678,7 @@ static qc_status apply_dense_impl(qc_state* s, int k, const int* qubits, const d
   std::vector<unsigned char> host(ob);
   dense_pack(s->dt, k, U, host.data());
   void* dbuf = nullptr;
-  cudaError_t e = cudaMallocAsync(&dbuf, ob + 16, s->stream);
+  cudaError_t e = ws_alloc(&dbuf, ob + 16, s->stream);
   if (e != cudaSuccess) return cuda_fail(e, "dense operator buffer");
   int* status = reinterpret_cast<int*>(reinterpret_cast<char*>(dbuf) + ob);
   e = cudaMemcpyAsync(dbuf, host.data(), ob, cudaMemcpyHostToDevice, s->stream);

@@ -536,7 +536,7 @@ QC_API qc_status qc_density_matrix(const void* psi_dev, int n, qc_dtype dt, int 
     if (st != QC_ENOMEM) return st;
   }
   double* P = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&P, sizeof(double) * B, s);
+  cudaError_t e = ws_alloc((void**)&P, sizeof(double) * B, s);
   if (e == cudaSuccess) e = cudaMemcpyAsync(P, P_host, sizeof(double) * B, cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) {
     if (P) cudaFreeAsync(P, s);
@@ -578,7 +578,7 @@ QC_API qc_status qc_mixed_spectrum(const void* psi_dev, int n, qc_dtype dt, int 
   const size_t g_b = sizeof(double2) * B * B;
   const size_t small_b = sizeof(double) * (2 * B + 1 + 128);
   char* buf = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&buf, part_b + g_b + small_b + 64, s);
+  cudaError_t e = ws_alloc((void**)&buf, part_b + g_b + small_b + 64, s);
   if (e != cudaSuccess) return cuda_fail(e, "spectrum workspace");
   float4* part = reinterpret_cast<float4*>(buf);
   double2* G = reinterpret_cast<double2*>(buf + part_b);

@@ -303,7 +303,7 @@ static qc_status run_hstep(qc_state* s, const std::vector<HTermHost>& terms) {
                bf = sizeof(HFlip) * flips.size(), bd = sizeof(HDiag) * diags.size(), bi = (4 * (size_t)npass + 15) / 16 * 16,
                bt = (sizeof(float4) << HS_KT) * npass;
   char* w = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&w, state + bt + bp + bf + bd + bi, s->stream);
+  cudaError_t e = ws_alloc((void**)&w, state + bt + bp + bf + bd + bi, s->stream);
   if (e != cudaSuccess) return cuda_fail(e, "Hamiltonian step workspace");
   V* acc = reinterpret_cast<V*>(w);
   float4* tab = reinterpret_cast<float4*>(w + state);

@@ -267,7 +267,7 @@ qc_status rho_tc_c64(const float2* psi, int n, int B, const double* P_host, floa
   const size_t bytesE = (size_t)(d.nib * TC5_M + 16);
   const size_t total = bytesA + bytesB + ((bytesE + 255) / 256) * 256 + 256 + sizeof(float) * B + 16;
   char* buf = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&buf, total, s);
+  cudaError_t e = ws_alloc((void**)&buf, total, s);
   if (e != cudaSuccess) return cuda_fail(e, "density matrix workspace");
   uint16_t* Aop = reinterpret_cast<uint16_t*>(buf);
   uint16_t* Bop = reinterpret_cast<uint16_t*>(buf + bytesA);

@@ -314,7 +314,7 @@ qc_status rho_tc_c128(const double2* psi, int n, int B, const double* P_host, do
   const size_t bytesA = (size_t)d.nib * d.nkc * R8_ND * R8_A, bytesB = (size_t)d.njb * d.nkc * R8_ND * R8_B,
                bytesE = (size_t)d.nib * TC5_M * sizeof(int16_t);
   unsigned char* buf = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&buf, bytesA + bytesB + bytesE + sizeof(double) * 64, s);
+  cudaError_t e = ws_alloc((void**)&buf, bytesA + bytesB + bytesE + sizeof(double) * 64, s);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return QC_ENOMEM;

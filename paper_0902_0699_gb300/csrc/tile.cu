@@ -1452,7 +1452,7 @@ struct QftTables {
 template <typename R>
 static qc_status qft_tables(qc_state* s, int n, int nl, int nlad, QftTables<R>* t, bool fixed = false) {
   const size_t tot = ((size_t)1 << nl) + ((size_t)1 << (n - nl)) + (size_t)nlad;
-  cudaError_t e = cudaMallocAsync((void**)&t->tlo, tot * sizeof(typename CT<R>::V2), s->stream);
+  cudaError_t e = ws_alloc((void**)&t->tlo, tot * sizeof(typename CT<R>::V2), s->stream);
   if (e != cudaSuccess) return cuda_fail(e, "qft tables");
   t->thi = t->tlo + ((size_t)1 << nl);
   t->lad = t->thi + ((size_t)1 << (n - nl));
