@@ -28,6 +28,9 @@
  *    return QC_EINVAL and leave the state unchanged.  A CUDA launch or
  *    runtime failure returns QC_ECUDA.  qc_last_error() returns a message
  *    describing the last failure on the calling host thread.
+ *  - Temporary device buffers come from a memory pool of the library's own
+ *    per device, which keeps up to 512 MiB between calls and gives them back
+ *    when the last state handle is freed.
  *  - Device code never traps: a bounded wait that gives up reports
  *    QC_ETIMEOUT through a status word the host reads.
  */
@@ -334,8 +337,8 @@ qc_status qc_renormalize(qc_state* s, double* norm_out_host);
  * rescans the one block of 2048 amplitudes that holds its target, and the
  * temporary device buffer is 8 * (2^n / 2048 + 2) bytes (plus 8 bytes per
  * 4096 blocks for n >= 24, whose block sums are scanned in chunks); with
- * more shots the full W is written as well, 8 * 2^n bytes more (QC_ENOMEM
- * if it does not fit).  Both give the outcomes above.  Synchronises the stream
+ * more shots the sums of 32 weights are kept as well, 8 * (2^n / 32) bytes
+ * more (QC_ENOMEM if they do not fit), and a shot rescans 32.  Both give the outcomes above.  Synchronises the stream
  * once (to read the total back). */
 qc_status qc_sample(const qc_state* s, uint64_t seed, int64_t shots, uint64_t* out_dev);
 
@@ -358,7 +361,7 @@ qc_status qc_probs_sample(const qc_state* s, double* probs_dev, uint64_t seed, i
  * for its own pool (a cudaMalloc here would fail or force it to give memory
  * back), and code on a latency-critical path that cannot take the
  * device-wide synchronisation that cudaMalloc / cudaFree imply.  qc_sample
- * allocates its 8 * 2^n-byte CDF per call and needs a qc_state handle, whose
+ * allocates its buffers per call and needs a qc_state handle, whose
  * creation allocates scratch too; this variant takes the raw state pointer
  * and calls no cudaMalloc, cudaFree or other allocating routine.
  *

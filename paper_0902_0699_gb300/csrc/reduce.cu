@@ -460,7 +460,8 @@ qc_status reduce_expect(const qc_state* s, uint64_t x, uint64_t z, double* out_h
 // Only the per-block weight sums (one per SMP_BLOCK amplitudes) are scanned
 // over the whole state.  With few shots, each shot finds its block by
 // bisection over the block offsets and rescans that block's weights; with
-// many shots the full CDF is written once and bisected per shot.
+// many shots the same pass also leaves the sums of 32 weights, and a shot
+// rescans 32.
 #define SMP_PER 8
 #define SMP_T 256
 #define SMP_BLOCK (SMP_PER * SMP_T)
@@ -555,57 +556,73 @@ __device__ __forceinline__ void block_wsum_out(uint64_t t, bool bad, uint64_t* _
   }
 }
 
-// Per-block weight sums (coalesced: the saturating sum does not depend on
-// which thread adds which weight); status bits for unusable probabilities.
-template <typename R>
-__global__ void __launch_bounds__(SMP_T) k_wsum(const typename CT<R>::V2* __restrict__ s, uint64_t N,
-                                                uint64_t* __restrict__ bsum, uint64_t* __restrict__ status) {
-  const uint64_t base = (uint64_t)blockIdx.x * SMP_BLOCK;
-  bool bad = false;
-  uint64_t t = 0;
+// Sums of the weights of 32 neighbouring amplitudes: of each of a lane's
+// SMP_PER values (value k: amplitude 256 k + thread of the block) over the
+// warp, each step halving the values a lane goes on with (nine exchanges
+// instead of five per value).  Lane 4 k holds value k's sum afterwards.
+#define SMP_SUB 32
+#define SMP_NSUB (SMP_BLOCK / SMP_SUB)
+__device__ __forceinline__ uint64_t warp_sub_sums(uint64_t* v) {
+  const int lane = threadIdx.x & 31;
 #pragma unroll
-  for (int k = 0; k < SMP_PER; ++k) {
-    const uint64_t i = base + (uint64_t)k * SMP_T + threadIdx.x;
-    if (i < N) t = sat_add(t, weight_of<R>(s[i], &bad));
-  }
-  block_wsum_out(t, bad, bsum, status);
-}
-
-// The same block sums, and the probabilities p_i written out, from one read
-// of the state (the Born probability is computed once and used for both).
-template <typename R>
-__global__ void __launch_bounds__(SMP_T) k_probs_wsum(const typename CT<R>::V2* __restrict__ s, uint64_t N,
-                                                      double* __restrict__ p, uint64_t* __restrict__ bsum,
-                                                      uint64_t* __restrict__ status) {
-  const uint64_t base = (uint64_t)blockIdx.x * SMP_BLOCK;
-  bool bad = false;
-  uint64_t t = 0;
+  for (int d = 16; d >= 4; d >>= 1) {
+    const int half = d / 4;  // 4, 2, 1 values kept
 #pragma unroll
-  for (int k = 0; k < SMP_PER; ++k) {
-    const uint64_t i = base + (uint64_t)k * SMP_T + threadIdx.x;
-    if (i < N) {
-      const double pi = prob_of<R>(s[i]);
-      p[i] = pi;
-      t = sat_add(t, weight_of_p(pi, &bad));
+    for (int j = 0; j < half; ++j) {
+      const uint64_t give = (lane & d) ? v[j] : v[j + half], keep = (lane & d) ? v[j + half] : v[j];
+      v[j] = sat_add(keep, __shfl_xor_sync(0xffffffffu, give, d));
     }
   }
+  uint64_t t = v[0];
+  t = sat_add(t, __shfl_xor_sync(0xffffffffu, t, 2));
+  return sat_add(t, __shfl_xor_sync(0xffffffffu, t, 1));
+}
+
+// Per-block weight sums (coalesced: the saturating sum does not depend on
+// which thread adds which weight); status bits for unusable probabilities.
+// PROBS: the probabilities p_i are written too, from the same read of the
+// state.  SUB: so are the sums of 32 amplitudes (SMP_NSUB a block).
+template <typename R, bool PROBS, bool SUB>
+__global__ void __launch_bounds__(SMP_T) k_wsum(const typename CT<R>::V2* __restrict__ s, uint64_t N,
+                                                double* __restrict__ p, uint64_t* __restrict__ bsum,
+                                                uint64_t* __restrict__ sub, uint64_t* __restrict__ status) {
+  const uint64_t base = (uint64_t)blockIdx.x * SMP_BLOCK;
+  bool bad = false;
+  uint64_t t = 0, w[SMP_PER];
+#pragma unroll
+  for (int k = 0; k < SMP_PER; ++k) {
+    const uint64_t i = base + (uint64_t)k * SMP_T + threadIdx.x;
+    w[k] = 0;
+    if (i < N) {
+      const double pi = prob_of<R>(s[i]);
+      if (PROBS) p[i] = pi;
+      w[k] = weight_of_p(pi, &bad);
+    }
+    if (!SUB) t = sat_add(t, w[k]);
+  }
+  if (SUB) {
+    const int lane = threadIdx.x & 31;
+    t = warp_sub_sums(w);
+    if (lane & 3) t = 0;
+    else sub[(uint64_t)blockIdx.x * SMP_NSUB + (lane >> 2) * (SMP_T / 32) + (threadIdx.x >> 5)] = t;
+  }
   block_wsum_out(t, bad, bsum, status);
 }
 
-static void launch_wsum(qc_dtype dt, const void* psi, uint64_t N, uint64_t* bsum, uint64_t* status,
-                        cudaStream_t st, double* probs = nullptr) {
+template <typename R>
+static void launch_wsum_r(const void* psi, uint64_t N, uint64_t* bsum, uint64_t* status, cudaStream_t st, double* probs,
+                          uint64_t* sub) {
   const unsigned nb = (unsigned)((N + SMP_BLOCK - 1) / SMP_BLOCK);
-  if (probs) {
-    if (dt == QC_C128)
-      k_probs_wsum<double><<<nb, SMP_T, 0, st>>>(reinterpret_cast<const double2*>(psi), N, probs, bsum, status);
-    else
-      k_probs_wsum<float><<<nb, SMP_T, 0, st>>>(reinterpret_cast<const float2*>(psi), N, probs, bsum, status);
-    return;
-  }
-  if (dt == QC_C128)
-    k_wsum<double><<<nb, SMP_T, 0, st>>>(reinterpret_cast<const double2*>(psi), N, bsum, status);
-  else
-    k_wsum<float><<<nb, SMP_T, 0, st>>>(reinterpret_cast<const float2*>(psi), N, bsum, status);
+  const auto* d = reinterpret_cast<const typename CT<R>::V2*>(psi);
+  if (probs && sub) k_wsum<R, true, true><<<nb, SMP_T, 0, st>>>(d, N, probs, bsum, sub, status);
+  else if (probs) k_wsum<R, true, false><<<nb, SMP_T, 0, st>>>(d, N, probs, bsum, sub, status);
+  else if (sub) k_wsum<R, false, true><<<nb, SMP_T, 0, st>>>(d, N, probs, bsum, sub, status);
+  else k_wsum<R, false, false><<<nb, SMP_T, 0, st>>>(d, N, probs, bsum, sub, status);
+}
+static void launch_wsum(qc_dtype dt, const void* psi, uint64_t N, uint64_t* bsum, uint64_t* status,
+                        cudaStream_t st, double* probs = nullptr, uint64_t* sub = nullptr) {
+  if (dt == QC_C128) launch_wsum_r<double>(psi, N, bsum, status, st, probs, sub);
+  else launch_wsum_r<float>(psi, N, bsum, status, st, probs, sub);
 }
 
 // Exclusive scan of the block sums in place (one block); tail[0] receives
@@ -708,7 +725,7 @@ __device__ __forceinline__ uint64_t shot_target(int64_t sh, uint64_t seed, uint6
   return __umul64hi(r, total);
 }
 
-// Many shots: bisection of the full CDF.
+// The full CDF bisected, a thread a shot (qc_sample_noalloc).
 __global__ void k_sample(const uint64_t* __restrict__ cdf, uint64_t N, uint64_t seed, int64_t shots,
                          uint64_t* __restrict__ out) {
   const uint64_t total = cdf[N - 1];
@@ -722,6 +739,57 @@ __global__ void k_sample(const uint64_t* __restrict__ cdf, uint64_t N, uint64_t 
       else lo = mid + 1;
     }
     out[sh] = lo;
+  }
+}
+
+// Many shots, a warp a shot: 32-ary search of the block offsets for the last
+// block whose offset is <= target, the block's SMP_NSUB sums of 32 weights,
+// then the 32 weights themselves.  No CDF of 8 bytes an amplitude is written
+// and kept (26 qubits complex64, 100000 shots: 424 us and a 512 MiB buffer).
+template <typename R>
+__global__ void __launch_bounds__(256) k_sample_warp(const typename CT<R>::V2* __restrict__ s, uint64_t N,
+                                                     const uint64_t* __restrict__ boff, uint64_t nb,
+                                                     const uint64_t* __restrict__ sub, const uint64_t* __restrict__ tail,
+                                                     uint64_t seed, int64_t shots, uint64_t* __restrict__ out) {
+  const int lane = threadIdx.x & 31;
+  const uint64_t total = tail[0];
+  for (int64_t sh = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; sh < shots;
+       sh += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    const uint64_t target = shot_target(sh, seed, total);
+    uint64_t lo = 0, cnt = nb;  // the block is in [lo, lo + cnt), boff[lo] <= target
+    while (cnt > 1) {
+      const uint64_t step = (cnt + 31) / 32, at = lo + lane * step;
+      const bool le = at < lo + cnt && boff[at] <= target;
+      const int k = 31 - __clz(__ballot_sync(0xffffffffu, le));  // lane 0 always holds
+      const uint64_t end = lo + cnt;
+      lo += k * step;
+      cnt = min(step, end - lo);
+    }
+    static_assert(SMP_NSUB == 64, "two sums a lane");
+    const ulonglong2 v = reinterpret_cast<const ulonglong2*>(sub + lo * SMP_NSUB)[lane];
+    uint64_t run = v.x + v.y;  // inclusive over lanes
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint64_t y = __shfl_up_sync(0xffffffffu, run, o);
+      if (lane >= o) run += y;
+    }
+    const uint64_t rest = target - boff[lo];
+    const int f = __ffs(__ballot_sync(0xffffffffu, run > rest)) - 1;  // the lane whose pair holds it
+    uint64_t before = __shfl_sync(0xffffffffu, run - v.x - v.y, f);
+    const uint64_t first = __shfl_sync(0xffffffffu, v.x, f);
+    int sb = 2 * f;
+    if (rest >= before + first) {
+      before += first;
+      ++sb;
+    }
+    const uint64_t i = lo * SMP_BLOCK + (uint64_t)sb * SMP_SUB + lane;
+    bool bad = false;
+    run = i < N ? weight_of<R>(s[i], &bad) : 0ull;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint64_t y = __shfl_up_sync(0xffffffffu, run, o);
+      if (lane >= o) run += y;
+    }
+    const unsigned m = __ballot_sync(0xffffffffu, before + run > rest);
+    if (m && lane == __ffs(m) - 1) out[sh] = i;
   }
 }
 
@@ -761,13 +829,14 @@ qc_status launch_sample(const qc_state* s, uint64_t seed, int64_t shots, uint64_
   const uint64_t N = 1ull << s->n;
   const uint64_t nb = (N + SMP_BLOCK - 1) / SMP_BLOCK;
   const bool local = (uint64_t)shots <= nb;
-  // [cdf (many shots only)] [block offsets nb] [total] [status] [chunk sums]
-  const uint64_t words = (local ? 0 : N) + nb + 2 + scan_words(nb);
+  // [sums of 32 weights (many shots only)] [block offsets nb] [total] [status] [chunk sums]
+  const uint64_t nsub = local ? 0 : nb * SMP_NSUB;
+  const uint64_t words = nsub + nb + 2 + scan_words(nb);
   uint64_t* buf = nullptr;
-  cudaError_t e = cudaMallocAsync((void**)&buf, words * sizeof(uint64_t), s->stream);
+  cudaError_t e = ws_alloc((void**)&buf, words * sizeof(uint64_t), s->stream);
   if (e != cudaSuccess) return cuda_fail(e, "sampler buffer");
-  uint64_t* cdf = buf;
-  uint64_t* bsum = buf + (local ? 0 : N);
+  uint64_t* sub = local ? nullptr : buf;
+  uint64_t* bsum = buf + nsub;
   uint64_t* tail = bsum + nb;
   uint64_t* status = tail + 1;
   uint64_t* csum = status + 1;
@@ -776,7 +845,7 @@ qc_status launch_sample(const qc_state* s, uint64_t seed, int64_t shots, uint64_
     cudaFreeAsync(buf, s->stream);
     return cuda_fail(e, "sampler status reset");
   }
-  launch_wsum(s->dt, s->data, N, bsum, status, s->stream, probs);
+  launch_wsum(s->dt, s->data, N, bsum, status, s->stream, probs, sub);
   scan_block_sums(bsum, nb, csum, tail, status, s->stream);
   qc_status st = check_launch("sample weights", nb <= SCAN_CHUNK ? 2 : 4);
   uint64_t h[2] = {0, 0};
@@ -801,13 +870,14 @@ qc_status launch_sample(const qc_state* s, uint64_t seed, int64_t shots, uint64_
                                                           tail, seed, shots, out);
       st = check_launch("sample", 1);
     } else {
+      const unsigned g = (unsigned)std::min<int64_t>((shots + 7) / 8, (int64_t)sm_count() * 8);
       if (s->dt == QC_C128)
-        k_wcdf<double><<<(unsigned)nb, SMP_T, 0, s->stream>>>(reinterpret_cast<const double2*>(s->data), N, bsum, cdf);
+        k_sample_warp<double><<<g, 256, 0, s->stream>>>(reinterpret_cast<const double2*>(s->data), N, bsum, nb, sub,
+                                                        tail, seed, shots, out);
       else
-        k_wcdf<float><<<(unsigned)nb, SMP_T, 0, s->stream>>>(reinterpret_cast<const float2*>(s->data), N, bsum, cdf);
-      const unsigned g = (unsigned)std::min<int64_t>((shots + 255) / 256, (int64_t)sm_count() * 8);
-      k_sample<<<g, 256, 0, s->stream>>>(cdf, N, seed, shots, out);
-      st = check_launch("sample", 2);
+        k_sample_warp<float><<<g, 256, 0, s->stream>>>(reinterpret_cast<const float2*>(s->data), N, bsum, nb, sub,
+                                                       tail, seed, shots, out);
+      st = check_launch("sample", 1);
     }
   }
   cudaFreeAsync(buf, s->stream);
