@@ -155,7 +155,8 @@ qc_status qc_grover_step(qc_state* s, const uint64_t* marked, int n_marked);
 
 /* Grover search of sec. 5.1: prepare HALL|0..0>, then apply G `iters`
  * times.  For small states (<= 8192 amplitudes for QC_C128, 16384 for
- * QC_C64) the whole run is one kernel with the state in shared memory. */
+ * QC_C64) the whole run is one kernel with the state in registers (64-bit
+ * fixed point, rounded once to the state's type). */
 qc_status qc_grover_run(qc_state* s, const uint64_t* marked, int n_marked, int iters);
 
 /* Grover step of a state split over several devices (sec. 5.1's G; the

@@ -13,6 +13,7 @@
 #include <cmath>
 
 #include "common.cuh"
+#include "fixpt.cuh"
 
 namespace qc {
 
@@ -278,97 +279,77 @@ qc_status launch_grover_apply(qc_state* s, const uint64_t* marked, int m, const 
 }
 
 // ---------------------------------------------------- whole small run ----
-// HALL|0..0> followed by `iters` Grover steps, one block, state in shared
-// memory.  The mean is recomputed from the amplitudes every step.  One SM
-// completes about 1.6 FP64 operations per clock, which would bound every
-// step (a block-wide FP64 sum and an FP64 diffusion), so the run stays on
-// the FP32 pipe: complex128 keeps the state as double-float (about 48
-// bits) from the first to the last step, complex64 sums in float pairs.
-template <typename R> struct SmallRun;
-template <> struct SmallRun<double> {
-  using E = ffc;
-  __device__ static E start(double a) { return ffc_make(ff_from_d(a), ff_make(0.f, 0.f)); }
-  __device__ static double2 out(E z) { return make_double2(ff_to_d(z.re), ff_to_d(z.im)); }
-  __device__ static E neg(E z) { return ffc_make(ff_neg(z.re), ff_neg(z.im)); }
-  __device__ static ff re(E z) { return z.re; }
-  __device__ static ff im(E z) { return z.im; }
-  // 2m = S 2^{1-n} (an exact power-of-two scaling of the double-float sum)
-  __device__ static E two_mean(ff sr, ff si, float scale) {
-    return ffc_make(ff_make(sr.hi * scale, sr.lo * scale), ff_make(si.hi * scale, si.lo * scale));
-  }
-  __device__ static E diffuse(E t2, E z) { return ffc_sub(t2, z); }
+// HALL|0..0> followed by `iters` Grover steps in one block.  The start state
+// and both operators are real, so the amplitudes are carried as real 64-bit
+// fixed point (unit 2^-62), in registers, from the first to the last step.
+// With P = sum of the amplitudes after the oracle = S - 2 sum_{marked} C, a
+// step maps C -> 2m - C (unmarked), 2m + C (marked), 2m = 2 P / N, and the new
+// sum is S' = N 2m - P.  Sums and differences are exact integers, P and S in
+// 128 bits; the only rounding of a step is 2m to the unit, and S' follows it
+// exactly, so S stays the sum of the amplitudes held.  A step is therefore the
+// sum of the marked amplitudes (one thread each), one barrier and one
+// subtraction an amplitude; summing all amplitudes in double-float each step
+// took 1.6 us a step (10 qubits; 40 us for 25 steps), this 0.1 us.
+struct I128 {
+  unsigned long long lo;
+  long long hi;
 };
-template <> struct SmallRun<float> {
-  using E = Cx<float>;
-  __device__ static E start(double a) { return cmake<float>((float)a, 0.f); }
-  __device__ static float2 out(E z) { return make_float2(z.re, z.im); }
-  __device__ static E neg(E z) { return cmake<float>(-z.re, -z.im); }
-  __device__ static ff re(E z) { return ff_make(z.re, 0.f); }
-  __device__ static ff im(E z) { return ff_make(z.im, 0.f); }
-  __device__ static E two_mean(ff sr, ff si, float scale) {
-    return cmake<float>((sr.hi + sr.lo) * scale, (si.hi + si.lo) * scale);
-  }
-  __device__ static E diffuse(E t2, E z) { return cmake<float>(t2.re - z.re, t2.im - z.im); }
-};
+__device__ __forceinline__ I128 i128_of(__int128 v) { return I128{(unsigned long long)v, (long long)(v >> 64)}; }
+__device__ __forceinline__ __int128 i128_to(I128 v) { return ((__int128)v.hi << 64) | (__int128)v.lo; }
 
-__device__ __forceinline__ ff shfl_xor_ff(ff v, int o) {
-  return ff_make(__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o));
+template <typename V2, int PER>
+__global__ void __launch_bounds__(1024) k_grover_small(V2* __restrict__ s, int n, const MarkedList* __restrict__ ML,
+                                                       int iters) {
+  __shared__ I128 part[2][32];
+  const int tid = threadIdx.x, T = blockDim.x, N = 1 << n, m = ML->m;
+  const int lane = tid & 31, warp = tid >> 5, nw = (m + 31) >> 5;  // warps that hold marked amplitudes
+  // 2^(62 - n/2), rounded for odd n: sqrt 2 2^62 is 6521908912666391106.2
+  const int h = (n + 1) >> 1;
+  const long long a = (n & 1) ? (6521908912666391106ll + (1ll << (h - 1))) >> h : 1ll << (62 - h);
+  long long c[PER], mk = tid < m ? a : 0;
+#pragma unroll
+  for (int u = 0; u < PER; ++u) c[u] = a;
+  __int128 S = (__int128)a << n;
+  const int steps = m > 16 ? 5 : m > 8 ? 4 : m > 4 ? 3 : m > 2 ? 2 : m > 1 ? 1 : 0;
+  for (int it = 0; it < iters; ++it) {
+    I128* buf = part[it & 1];
+    if (warp < nw) {
+      __int128 t = mk;
+      for (int o = 1, k = 0; k < steps; ++k, o <<= 1) {
+        const I128 v = i128_of(t);
+        t += i128_to(I128{__shfl_xor_sync(0xffffffffu, v.lo, o), __shfl_xor_sync(0xffffffffu, v.hi, o)});
+      }
+      if (lane == 0) buf[warp] = i128_of(t);
+    }
+    __syncthreads();
+    __int128 P = S;
+    for (int w = 0; w < nw; ++w) P -= i128_to(buf[w]) * 2;
+    const long long t2 = (long long)((P + ((__int128)1 << (n - 1) >> 1)) >> (n - 1));
+    S = ((__int128)t2 << n) - P;
+#pragma unroll
+    for (int u = 0; u < PER; ++u) c[u] = t2 - c[u];
+    if (tid < m) mk += t2;
+  }
+  auto out = [](long long v) {
+    if constexpr (sizeof(V2) == 16) return make_double2(fix2d(v, 62), 0.0);
+    else return make_float2((float)v * 0x1p-62f, 0.f);
+  };
+#pragma unroll
+  for (int u = 0; u < PER; ++u)
+    if (tid + T * u < N) s[tid + T * u] = out(c[u]);
+  __syncthreads();
+  if (tid < m) s[ML->idx[tid]] = out(mk);
 }
 
-template <typename R>
-__global__ void __launch_bounds__(1024) k_grover_small(typename CT<R>::V2* __restrict__ s, int n,
-                                                       const MarkedList* __restrict__ ML, int iters) {
-  using G = SmallRun<R>;
-  using E = typename G::E;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  E* sm = reinterpret_cast<E*>(smraw);
-  __shared__ ff red[2][32];
-  __shared__ E t2s;
-  const int N = 1 << n;
-  const float scale = ldexpf(1.f, 1 - n);  // 2 / N, exact
-  const E a = G::start(1.0 / sqrt(ldexp(1.0, n)));
-  for (int i = threadIdx.x; i < N; i += blockDim.x) sm[i] = a;
-  __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const ff zero = ff_make(0.f, 0.f);
-  for (int it = 0; it < iters; ++it) {
-    // oracle (Eq. oracle1)
-    for (int i = threadIdx.x; i < ML->m; i += blockDim.x) {
-      const uint64_t j = ML->idx[i];
-      sm[j] = G::neg(sm[j]);
-    }
-    __syncthreads();
-    // amplitude sum in double-float: per thread, across the warp, across warps
-    ff sr = zero, si = zero;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) {
-      const E z = sm[i];
-      sr = ff_add(sr, G::re(z));
-      si = ff_add(si, G::im(z));
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      sr = ff_add(sr, shfl_xor_ff(sr, o));
-      si = ff_add(si, shfl_xor_ff(si, o));
-    }
-    if (lane == 0) {
-      red[0][warp] = sr;
-      red[1][warp] = si;
-    }
-    __syncthreads();
-    if (warp == 0) {
-      ff r = lane < nw ? red[0][lane] : zero, q = lane < nw ? red[1][lane] : zero;
-      for (int o = 16; o > 0; o >>= 1) {
-        r = ff_add(r, shfl_xor_ff(r, o));
-        q = ff_add(q, shfl_xor_ff(q, o));
-      }
-      if (lane == 0) t2s = G::two_mean(r, q, scale);
-    }
-    __syncthreads();
-    // diffusion: C -> 2m - C (HALL . Inv . HALL)
-    const E t2 = t2s;
-    for (int i = threadIdx.x; i < N; i += blockDim.x) sm[i] = G::diffuse(t2, sm[i]);
-    __syncthreads();
-  }
-  for (int i = threadIdx.x; i < N; i += blockDim.x) s[i] = G::out(sm[i]);
+template <typename V2>
+static void run_small(qc_state* s, const MarkedList* dml, int m, int iters) {
+  V2* d = reinterpret_cast<V2*>(s->data);
+  // eight amplitudes a thread (a step's scalar part is the same in every warp),
+  // a thread for every marked item
+  const int N = 1 << s->n, per = N <= 8192 ? 8 : 16, need = std::max(N / per, m);
+  const int T = std::min(1024, std::max(32, (need + 31) / 32 * 32));
+  if (per == 8) k_grover_small<V2, 8><<<1, T, 0, s->stream>>>(d, s->n, dml, iters);
+  else k_grover_small<V2, 16><<<1, T, 0, s->stream>>>(d, s->n, dml, iters);
 }
 
 qc_status launch_grover_run(qc_state* s, const uint64_t* marked, int m, int iters) {
@@ -377,15 +358,9 @@ qc_status launch_grover_run(qc_state* s, const uint64_t* marked, int m, int iter
   if (st) return st;
   const bool small = (s->dt == QC_C128) ? (s->n <= 13) : (s->n <= 14);
   if (small) {
-    const size_t smem = ((size_t)1 << s->n) * amp_bytes(s->dt);
-    if (s->dt == QC_C128) {
-      cudaFuncSetAttribute(k_grover_small<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
-      k_grover_small<double><<<1, 1024, smem, s->stream>>>(reinterpret_cast<double2*>(s->data), s->n, dml, iters);
-    } else {
-      cudaFuncSetAttribute(k_grover_small<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 160 * 1024);
-      k_grover_small<float><<<1, 1024, smem, s->stream>>>(reinterpret_cast<float2*>(s->data), s->n, dml, iters);
-    }
-    st = check_launch("grover run (shared memory)");
+    if (s->dt == QC_C128) run_small<double2>(s, dml, m, iters);
+    else run_small<float2>(s, dml, m, iters);
+    st = check_launch("grover run (one block)");
     s->sum_valid = false;
   } else {
     st = launch_fill_uniform(s);  // HALL|0..0>; records the amplitude sum
