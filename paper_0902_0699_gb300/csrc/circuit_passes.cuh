@@ -155,10 +155,11 @@ __device__ __forceinline__ int tp_round_at(int base, const int* bas, int j) {
 struct PassCfg {
   int kmax, c0, rb;
   bool merge, reverse;
+  bool grow = true;  // operators behind a left-out gate may still bring new tile bits
 };
 
 template <typename R>
-inline std::vector<TilePass> build_passes(const qc_gate* gates, int ng, int n, const PassCfg& cfg) {
+inline std::vector<TilePass> build_passes_as(const qc_gate* gates, int ng, int n, const PassCfg& cfg) {
   struct Item {
     bool cx;
     int q, c, ka, kb, pa, pb;
@@ -178,16 +179,19 @@ inline std::vector<TilePass> build_passes(const qc_gate* gates, int ng, int n, c
   }
   const int kt = std::min(n, cfg.kmax);
   std::vector<TilePass> out;
+  out.reserve(64);
   std::vector<char> done(items.size(), 0);
+  std::vector<Item> S, keep;
+  std::vector<std::pair<int, int>> cx;  // (control, target) in order
   size_t first = 0;
   while (first < items.size()) {
     uint64_t tile = (1ull << std::min(n, cfg.c0)) - 1, skip = 0, inp = 0;
     bool closed = false;  // no more operators
-    std::vector<Item> S;
-    std::vector<std::pair<int, int>> cx;  // (control, target) in order
+    S.clear();
+    cx.clear();
     auto fits = [&](int q) {
       if ((tile >> q) & 1) return true;
-      if (__builtin_popcountll(tile) >= kt) return false;
+      if (__builtin_popcountll(tile) >= kt || (skip && !cfg.grow)) return false;
       tile |= 1ull << q;
       return true;
     };
@@ -219,7 +223,7 @@ inline std::vector<TilePass> build_passes(const qc_gate* gates, int ng, int n, c
         bool ok = !closed && !((skip | inp) & b) && S.size() < (size_t)TP_MAXOP && fits(it.q);
         if (ok) {
           S.push_back(it);
-          if (rounds_of(S) > TP_MAXRD) {
+          if (S.size() > (size_t)TP_MAXRD && rounds_of(S) > TP_MAXRD) {
             S.pop_back();
             ok = false;
           }
@@ -227,7 +231,7 @@ inline std::vector<TilePass> build_passes(const qc_gate* gates, int ng, int n, c
         if (ok) done[i] = 1;
         else skip |= b, closed = cfg.merge;
       }
-      if (__builtin_popcountll(tile) >= kt && (tile & ~skip) == 0) break;
+      if ((__builtin_popcountll(tile) >= kt || (skip && !cfg.grow)) && (tile & ~skip) == 0) break;
     }
     while (first < items.size() && done[first]) ++first;
     for (int q = 0; q < n && __builtin_popcountll(tile) < kt; ++q) tile |= 1ull << q;
@@ -238,8 +242,7 @@ inline std::vector<TilePass> build_passes(const qc_gate* gates, int ng, int n, c
     int where[64];
     for (int q = 0; q < n; ++q) {
       if ((tile >> q) & 1) {
-        int p = 0;
-        for (int x = 0; x < q; ++x) p += (int)((tile >> x) & 1);
+        const int p = __builtin_popcountll(tile & ((1ull << q) - 1));
         where[q] = p;
         P.pos[p] = (int8_t)q;
       } else {
@@ -251,7 +254,7 @@ inline std::vector<TilePass> build_passes(const qc_gate* gates, int ng, int n, c
     for (int p = 0; p < TP_MAXK + 3; ++p) P.dp[p] = -1;
     if (!cfg.merge) {
       uint64_t later = 0;
-      std::vector<Item> keep;
+      keep.clear();
       for (size_t k = S.size(); k-- > 0;) {
         const uint64_t b = 1ull << S[k].q;
         if (S[k].ka == QC_G_RZ && !(later & b)) {
@@ -299,7 +302,7 @@ inline std::vector<TilePass> build_passes(const qc_gate* gates, int ng, int n, c
     };
     auto tile_part = [&](uint64_t v) {
       int r = 0;
-      for (int p = 0; p < kt; ++p) r |= (int)((v >> P.pos[p]) & 1ull) << p;
+      for (v &= tile; v; v &= v - 1) r |= 1 << where[__builtin_ctzll(v)];
       return r;
     };
     P.has_perm = !cx.empty();
@@ -314,6 +317,25 @@ inline std::vector<TilePass> build_passes(const qc_gate* gates, int ng, int n, c
     out.push_back(P);
   }
   return out;
+}
+
+// The shortest list over both ways to grow a tile and rows of 2^c0 or half as
+// many amplitudes.  A tile that takes in a later layer's qubits can leave the
+// passes after it out of step with the layers: 20 qubits, ten layers of
+// rotations and a ring on 2^11-amplitude tiles are 41 passes grown greedily
+// and 20 on 64-byte rows.
+template <typename R>
+inline std::vector<TilePass> build_passes(const qc_gate* gates, int ng, int n, const PassCfg& cfg) {
+  std::vector<TilePass> best;
+  for (int k = 0; k < 4; ++k) {
+    PassCfg c = cfg;
+    c.c0 -= k >> 1;
+    c.grow = !(k & 1);
+    std::vector<TilePass> p = build_passes_as<R>(gates, ng, n, c);
+    if (k == 0 || p.size() < best.size()) best.swap(p);
+    if (n <= cfg.kmax) break;  // one tile holds every qubit
+  }
+  return best;
 }
 
 }  // namespace qc
