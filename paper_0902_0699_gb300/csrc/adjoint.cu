@@ -922,61 +922,79 @@ __global__ void __launch_bounds__(64) k_bwd_finish(const TilePass* __restrict__ 
 }
 
 // lam = H psi = sum_k c_k P_k psi, P_k = i^{|x&z|} X^x Z^z:
-// (P psi)[j] = i^{|x&z|} (-1)^{|(j^x)&z|} psi[j^x].
+// (P psi)[j] = i^{|x&z|} (-1)^{|(j^x)&z|} psi[j^x],
+// and Re <psi|lam> per batch element (block partials).  The factor of i and
+// (-1)^{|x&z|} are folded into the coefficient on the host; what is left of a
+// term is a load, the parity of j & z if z is not zero, and two multiply-adds.
+// A thread takes four amplitudes a term, and a block a contiguous chunk, so
+// that partners across the low index bits come from its L1.  64 states of 20
+// qubits, 21 terms: 3.55 ms with one amplitude a thread and a pass of its own
+// for the energy.
+template <typename R>
 struct TermsDev {
   int nt;
-  uint64_t x[64], z[64];
-  double c[64];
+  uint32_t x[64], z[64];
+  R c[64];
+  uint8_t imag[64];  // the coefficient is i c
 };
+constexpr int AH_UNR = 4, AH_CHUNK = 4096;
 
 template <typename R>
 __global__ void __launch_bounds__(ADJ_T) k_apply_h(const typename CT<R>::V2* __restrict__ psi,
                                                    typename CT<R>::V2* __restrict__ lam, int n,
-                                                   const __grid_constant__ TermsDev T) {
+                                                   const __grid_constant__ TermsDev<R> T, double* __restrict__ part) {
+  using V2 = typename CT<R>::V2;
   const int b = blockIdx.y;
-  const typename CT<R>::V2* s = psi + ((uint64_t)b << n);
-  typename CT<R>::V2* l = lam + ((uint64_t)b << n);
-  const uint64_t N = 1ull << n;
-  for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j < N; j += (uint64_t)gridDim.x * blockDim.x) {
-    R ar = 0, ai = 0;
-    for (int k = 0; k < T.nt; ++k) {
-      const uint64_t x = T.x[k], z = T.z[k];
-      const auto v = s[j ^ x];
-      R vr = v.x, vi = v.y;
-      if (__popcll((j ^ x) & z) & 1) {
-        vr = -vr;
-        vi = -vi;
+  const V2* s = psi + ((uint64_t)b << n);
+  V2* l = lam + ((uint64_t)b << n);
+  const uint32_t N = 1u << n;
+  double e = 0.0;
+  for (uint64_t c0 = (uint64_t)blockIdx.x * AH_CHUNK; c0 < N; c0 += (uint64_t)gridDim.x * AH_CHUNK) {
+    Acc<R> acc;
+    for (uint32_t j0 = (uint32_t)c0 + threadIdx.x; j0 < (uint32_t)min((uint64_t)N, c0 + AH_CHUNK); j0 += AH_UNR * ADJ_T) {
+      R ar[AH_UNR], ai[AH_UNR];
+#pragma unroll
+      for (int u = 0; u < AH_UNR; ++u) ar[u] = ai[u] = 0;
+      for (int k = 0; k < T.nt; ++k) {
+        const uint32_t x = T.x[k], z = T.z[k];
+        const R c = T.c[k];
+        const bool imag = T.imag[k];
+        V2 v[AH_UNR];
+#pragma unroll
+        for (int u = 0; u < AH_UNR; ++u) {
+          const uint32_t j = j0 + u * ADJ_T;
+          if (j < N) v[u] = s[j ^ x];
+        }
+#pragma unroll
+        for (int u = 0; u < AH_UNR; ++u) {
+          const uint32_t j = j0 + u * ADJ_T;
+          if (j < N) {
+            const R cj = z && (__popc(j & z) & 1) ? -c : c;
+            if (imag) {
+              ar[u] = fma(-cj, v[u].y, ar[u]);
+              ai[u] = fma(cj, v[u].x, ai[u]);
+            } else {
+              ar[u] = fma(cj, v[u].x, ar[u]);
+              ai[u] = fma(cj, v[u].y, ai[u]);
+            }
+          }
+        }
       }
-      const int ny = __popcll(x & z) & 3;
-      R wr = vr, wi = vi;  // times i^ny
-      if (ny == 1) { wr = -vi; wi = vr; }
-      else if (ny == 2) { wr = -vr; wi = -vi; }
-      else if (ny == 3) { wr = vi; wi = -vr; }
-      const R c = (R)T.c[k];
-      ar = fma(c, wr, ar);
-      ai = fma(c, wi, ai);
+#pragma unroll
+      for (int u = 0; u < AH_UNR; ++u) {
+        const uint32_t j = j0 + u * ADJ_T;
+        if (j < N) {
+          const V2 v = s[j];
+          l[j] = CT<R>::make(ar[u], ai[u]);
+          acc.add(v.x, ar[u]);
+          acc.add(v.y, ai[u]);
+        }
+      }
     }
-    l[j] = CT<R>::make(ar, ai);
+    acc.flush();
+    e += acc.value();
   }
-}
-
-// Re <psi|lam> per batch element (block partials).
-template <typename R>
-__global__ void __launch_bounds__(ADJ_T) k_energy(const typename CT<R>::V2* __restrict__ psi,
-                                                  const typename CT<R>::V2* __restrict__ lam, int n,
-                                                  double* __restrict__ part) {
-  const int b = blockIdx.y;
-  const typename CT<R>::V2* s = psi + ((uint64_t)b << n);
-  const typename CT<R>::V2* l = lam + ((uint64_t)b << n);
-  const uint64_t N = 1ull << n;
-  Acc<R> acc;
-  for (uint64_t j = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; j < N; j += (uint64_t)gridDim.x * blockDim.x) {
-    const auto v = s[j], w = l[j];
-    acc.add(v.x, w.x);
-    acc.add(v.y, w.y);
-  }
-  acc.flush();
-  const double t = block_reduce(acc.value());
+  const double t = block_reduce(e);
   if (threadIdx.x == 0) part[(int64_t)b * gridDim.x + blockIdx.x] = t;
 }
 
@@ -1017,16 +1035,13 @@ static qc_status check_circuit(int n, qc_dtype dt, int B, const qc_gate* gates, 
   return QC_OK;
 }
 
-// Blocks per batch element: all blocks of the (gx, B) grid resident at once.
+// Blocks per batch element of the H psi pass.
 template <typename R>
 static unsigned gx_for(int n, int B) {
-  const uint64_t pairs = 1ull << (n - 1);
-  uint64_t gx = (pairs + ADJ_T - 1) / ADJ_T;
-  const int res = std::min(resident_blocks((const void*)k_apply_h<R>, ADJ_T, 0),
-                           resident_blocks((const void*)k_energy<R>, ADJ_T, 0));
-  const uint64_t cap = std::max<uint64_t>(1, (uint64_t)sm_count() * res / (uint64_t)B);
-  gx = std::min<uint64_t>(gx, std::min<uint64_t>(cap, ADJ_GX_MAX));
-  return (unsigned)std::max<uint64_t>(gx, 1);
+  const uint64_t chunks = std::max<uint64_t>(1, (1ull << n) / AH_CHUNK);
+  const uint64_t cap = std::max<uint64_t>(
+      1, 4ull * sm_count() * resident_blocks((const void*)k_apply_h<R>, ADJ_T, 0) / (uint64_t)B);
+  return (unsigned)std::min<uint64_t>({chunks, cap, ADJ_GX_MAX});
 }
 
 // Passes of a forward sweep on the device, with room for the operators of as
@@ -1196,16 +1211,18 @@ static qc_status adjoint_impl(int n, int B, const qc_gate* gates, int n_gates, c
   BwdPlan<R> W;
   cudaError_t e = ws_alloc((void**)&part, sizeof(double) * (size_t)gx * B, st);
   if (e == cudaSuccess) e = fwd_plan(F, gates, n_gates, n, B, st);
-  if (e == cudaSuccess) e = bwd_plan(W, gates, n_gates, n, B, st);
   qc_status s = QC_OK;
   if (e == cudaSuccess) {
-    TermsDev T;
+    TermsDev<R> T;
     double bound = 0.0;  // ||H|| <= sum |c_k|
     T.nt = n_terms;
     for (int k = 0; k < n_terms; ++k) {
-      T.x[k] = H[k].xmask;
-      T.z[k] = H[k].zmask;
-      T.c[k] = H[k].coeff;
+      const uint64_t x = H[k].xmask, z = H[k].zmask;
+      const int ny = __builtin_popcountll(x & z);  // i^ny (-1)^ny = (-i)^ny
+      T.x[k] = (uint32_t)x;
+      T.z[k] = (uint32_t)z;
+      T.imag[k] = ny & 1;
+      T.c[k] = (R)(((ny & 3) == 1 || (ny & 3) == 2) ? -H[k].coeff : H[k].coeff);
       bound += std::fabs(H[k].coeff) / 64.0;
     }
     // sums stay below 2^55 units: bound * 64 < 2^(ilogb + 7)
@@ -1215,11 +1232,15 @@ static qc_status adjoint_impl(int n, int B, const qc_gate* gates, int n_gates, c
     if (e != cudaSuccess) s = cuda_fail(e, "adjoint setup");
     if (!s) {
       int nk = forward_passes<R>(F, n, B, theta, stride, p, st);
-      k_apply_h<R><<<grid, ADJ_T, 0, st>>>(p, l, n, T);
-      k_energy<R><<<grid, ADJ_T, 0, st>>>(p, l, n, part);
+      k_apply_h<R><<<grid, ADJ_T, 0, st>>>(p, l, n, T, part);
       k_final_batch<<<B, ADJ_T, 0, st>>>(part, gx, energy, 1, 0);
-      nk += 3 + backward_passes<R>(W, n, B, theta, stride, kq, p, l, grad, st);
-      s = check_launch("adjoint", nk);
+      nk += 2;
+      // the backward passes are planned while the forward ones run
+      e = bwd_plan(W, gates, n_gates, n, B, st);
+      if (e != cudaSuccess) s = cuda_fail(e, "adjoint workspace");
+      else nk += backward_passes<R>(W, n, B, theta, stride, kq, p, l, grad, st);
+      const qc_status sl = check_launch("adjoint", nk);
+      if (!s) s = sl;
     }
   } else {
     s = cuda_fail(e, "adjoint workspace");
