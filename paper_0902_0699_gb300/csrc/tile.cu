@@ -848,7 +848,7 @@ __device__ __forceinline__ void qft_levels_c64_ct(float2* sm, const float2* LAD)
 // Consecutive threads hold consecutive low bits (2^C >= 16 amplitudes, at
 // least 128 contiguous bytes per warp and element).
 template <int K, int QR>
-__device__ __forceinline__ void qft_last_block_store_c64(const float2* sm, const float2* LAD, const float2* W,
+__device__ __forceinline__ void qft_last_block_store_c64(const float2* sm, const float2* LAD, const float2* __restrict__ W,
                                                          const float2* V, float2* __restrict__ s, uint64_t T,
                                                          int lo) {
   constexpr int NR = 1 << QR, NE = 1 << 13, C = 13 - K, BL = C;
@@ -885,20 +885,24 @@ __device__ __forceinline__ void qft_last_block_store_c64(const float2* sm, const
 }
 
 template <int K>
-__global__ void __launch_bounds__(512, 1) k_qft_db_c64_k(float2* __restrict__ s, uint64_t ntiles, const TileProg<float> P,
-                                                         const float2* __restrict__ tlo,
-                                                         const float2* __restrict__ thi) {
+__global__ void __launch_bounds__(512, 2) k_qft_c64_k(float2* __restrict__ s, uint64_t ntiles, const TileProg<float> P,
+                                                      const float2* __restrict__ tlo,
+                                                      const float2* __restrict__ thi,
+                                                      const float2* __restrict__ W,
+                                                      const float2* __restrict__ lad) {
   using A = TA<float>;
   constexpr int C = 13 - K, NE = 1 << 13;
   static_assert(C <= 10, "1024-element copy strides stay inside the group bits");
   extern __shared__ __align__(16) unsigned char smraw[];
   const int lo = P.lo, hi = lo + K - 1;
   const bool tw = P.twiddle != 0;
-  float2* buf0 = reinterpret_cast<float2*>(smraw);
-  float2* buf1 = buf0 + NE;
-  float2* W = buf1 + NE;
-  float2* V = W + (tw ? NE : 0);
-  float2* LAD = V + (tw ? (1 << K) : 0);
+  float2* cur = reinterpret_cast<float2*>(smraw);
+  float2* V = cur + NE;
+  // the ladders in shared memory; the lowest group's 64 KiB stay in global
+  // memory (read through L1), so that two blocks fit an SM
+  constexpr bool LSM = K <= 9;
+  float2* Ls = V + (tw ? (1 << K) : 0);
+  const float2* LAD = LSM ? Ls : lad;
   const float sc = (float)exp2(-0.5 * K);
   const int e0 = 2 * threadIdx.x;
   const int se0 = qsw(e0);
@@ -906,35 +910,18 @@ __global__ void __launch_bounds__(512, 1) k_qft_db_c64_k(float2* __restrict__ s,
   // this thread's copy / store elements e0 + 1024 u share the group bits'
   // low part; their reversed group bits are f0 | brev(u) at the top
   const int f0 = (int)(__brev((unsigned)(e0 >> C)) >> (32 - K));
-  auto issue = [&](uint64_t T, float2* dst) {
+  auto issue = [&](uint64_t T) {
     const uint64_t g = tile_global((uint64_t)e0, T, lo, K, C);
 #pragma unroll
     for (int u = 0; u < NE / 1024; ++u) {
-      const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst + (se0 ^ qsw(1024 * u)));
+      const uint32_t d = (uint32_t)__cvta_generic_to_shared(cur + (se0 ^ qsw(1024 * u)));
       asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(s + g + u * gstep) : "memory");
     }
   };
-  uint64_t T = blockIdx.x;
-  if (T < ntiles) issue(T, buf0);
-  asm volatile("cp.async.commit_group;\n" ::: "memory");
-  // the pass's tables from the global root tables (powers of Omega_n), in
-  // FP32: e^{2 pi i x / 2^{j+1}} = Omega_n^{x 2^{n-j-1}}
-  for (int a = threadIdx.x; a < (1 << K) - 1; a += blockDim.x) {
-    const int j = 31 - __clz(a + 1);
-    const A::E z = omega<float>(tlo, thi, (uint64_t)(a + 1 - (1 << j)) << (P.n - j - 1), P.nl);
-    LAD[a] = make_float2(z.re, z.im);
-  }
-  if (tw)
-    for (int e = threadIdx.x; e < NE; e += blockDim.x) {
-      const int f = (int)(__brev((unsigned)(e >> C)) >> (32 - K));
-      const uint64_t x = (uint64_t)((e & ((1 << C) - 1)) * f);  // < 2^13 <= 2^{hi+1}
-      const A::E z = omega<float>(tlo, thi, x << (P.n - hi - 1), P.nl);
-      W[e] = make_float2(z.re, z.im);
-    }
-  for (int it = 0; T < ntiles; T += gridDim.x, ++it) {
-    float2* cur = (it & 1) ? buf1 : buf0;
-    float2* nxt = (it & 1) ? buf0 : buf1;
-    if (T + gridDim.x < ntiles) issue(T + gridDim.x, nxt);
+  if (LSM)
+    for (int a = threadIdx.x; a < (1 << K) - 1; a += blockDim.x) Ls[a] = lad[a];
+  for (uint64_t T = blockIdx.x; T < ntiles; T += gridDim.x) {
+    issue(T);
     asm volatile("cp.async.commit_group;\n" ::: "memory");
     if (tw) {
       const uint64_t Lt = (T & ((1ull << (lo - C)) - 1ull)) << C;
@@ -944,7 +931,7 @@ __global__ void __launch_bounds__(512, 1) k_qft_db_c64_k(float2* __restrict__ s,
         V[f] = make_float2(z.re, z.im);
       }
     }
-    asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
     __syncthreads();
     if constexpr (C >= 4) {
       if (tw) {
@@ -977,7 +964,6 @@ __global__ void __launch_bounds__(512, 1) k_qft_db_c64_k(float2* __restrict__ s,
     }
     __syncthreads();
   }
-  asm volatile("cp.async.wait_all;\n" ::: "memory");
 }
 
 // P holds the pass: group [lo, lo+k), c contiguous bits, twiddle = lo > 0,
@@ -1213,7 +1199,8 @@ static size_t qft_db_smem(int k, int c, bool twiddle) {
   return sizeof(float2) * (2 * NE + (twiddle ? NE + ((size_t)1 << k) : 0) + ((size_t)1 << k) - 1);
 }
 
-static qc_status run_qft_db_c64(qc_state* s, TileProg<float>& P, const float2* tlo, const float2* thi) {
+static qc_status run_qft_db_c64(qc_state* s, TileProg<float>& P, const float2* tlo, const float2* thi,
+                                const float2* W, const float2* lad) {
   const uint64_t ntiles = 1ull << (s->n - (P.k + P.c));
   const size_t smem = qft_db_smem(P.k, P.c, P.twiddle != 0);
   static bool attr_set = false;
@@ -1229,11 +1216,12 @@ static qc_status run_qft_db_c64(qc_state* s, TileProg<float>& P, const float2* t
   case KK: {                                                                                       \
     static bool a = false;                                                                         \
     if (!a) {                                                                                      \
-      cudaFuncSetAttribute(k_qft_db_c64_k<KK>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024); \
+      cudaFuncSetAttribute(k_qft_c64_k<KK>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024); \
       a = true;                                                                                    \
     }                                                                                              \
-    const unsigned g = resident_grid(k_qft_db_c64_k<KK>, 512, (int64_t)ntiles, 1, smem);          \
-    k_qft_db_c64_k<KK><<<g, 512, smem, s->stream>>>(d, ntiles, P, tlo, thi);                       \
+    const size_t sm1 = sizeof(float2) * ((1 << 13) + (P.twiddle ? 1 << KK : 0) + (KK <= 9 ? (1 << KK) - 1 : 0)); \
+    const unsigned g = resident_grid(k_qft_c64_k<KK>, 512, (int64_t)ntiles, 1, sm1);               \
+    k_qft_c64_k<KK><<<g, 512, sm1, s->stream>>>(d, ntiles, P, tlo, thi, W, lad);                   \
     return check_launch("qft pass");                                                               \
   }
       QC_QFT_DB(3) QC_QFT_DB(4) QC_QFT_DB(5) QC_QFT_DB(6) QC_QFT_DB(7) QC_QFT_DB(8) QC_QFT_DB(9) QC_QFT_DB(13)
@@ -1450,12 +1438,13 @@ struct QftTables {
   typename CT<R>::V2 *tlo, *thi, *lad;
 };
 template <typename R>
-static qc_status qft_tables(qc_state* s, int n, int nl, int nlad, QftTables<R>* t, bool fixed = false) {
+static qc_status qft_tables(qc_state* s, int n, int nl, int nlad, QftTables<R>* t, bool fixed = false,
+                            size_t room = 0) {
   const size_t tot = ((size_t)1 << nl) + ((size_t)1 << (n - nl)) + (size_t)nlad;
-  cudaError_t e = ws_alloc((void**)&t->tlo, tot * sizeof(typename CT<R>::V2), s->stream);
+  cudaError_t e = ws_alloc((void**)&t->tlo, (tot + 2 + room) * sizeof(typename CT<R>::V2), s->stream);
   if (e != cudaSuccess) return cuda_fail(e, "qft tables");
   t->thi = t->tlo + ((size_t)1 << nl);
-  t->lad = t->thi + ((size_t)1 << (n - nl));
+  t->lad = t->thi + (((size_t)1 << (n - nl)) + 1) / 2 * 2;  // 16-byte aligned
   const unsigned grid = grid_for((int64_t)tot, 64, 8);
   if (fixed && sizeof(R) == 8)  // complex128 register passes
     k_roots_fix<<<grid, 64, 0, s->stream>>>(reinterpret_cast<longlong2*>(t->tlo), reinterpret_cast<longlong2*>(t->thi), n,
@@ -1465,18 +1454,44 @@ static qc_status qft_tables(qc_state* s, int n, int nl, int nlad, QftTables<R>* 
   return check_launch("qft roots");
 }
 
+// W[e] = Omega_{hi+1}^{l f} of the complex64 pass blockIdx.y on group
+// [lo, lo + k): l = tile element e's c = 13 - k low bits, f its group bits
+// reversed.  Every tile of a pass uses the same 64 KiB, read through L1.
+struct QftGroups {
+  int np;
+  int lo[8], k[8];
+};
+__global__ void __launch_bounds__(256) k_qft_w(const float2* __restrict__ tlo, const float2* __restrict__ thi, int n,
+                                               int nl, const QftGroups G, float2* __restrict__ W) {
+  const int lo = G.lo[blockIdx.y], k = G.k[blockIdx.y], c = 13 - k;
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  const int f = (int)(__brev((unsigned)(e >> c)) >> (32 - k));
+  const uint64_t x = (uint64_t)((e & ((1 << c) - 1)) * f);
+  const TA<float>::E z = omega<float>(tlo, thi, x << (n - lo - k), nl);
+  W[((size_t)blockIdx.y << 13) + e] = make_float2(z.re, z.im);
+}
+
 template <typename R>
 static qc_status qft_impl(qc_state* s) {
   using V2 = typename CT<R>::V2;
   const int n = s->n;
   const int nl = (n + 1) / 2;
-  const int nlad = sizeof(R) == 8 ? 1 << std::min(n, 11) : 0;  // complex64 passes build theirs from the roots
-  QftTables<R> tab;
-  qc_status st = qft_tables(s, n, nl, nlad, &tab);
-  if (st) return st;
-  V2 *tlo = tab.tlo, *thi = tab.thi;
   // complex64: groups of at most 9 above the lowest 13 (64 KiB tiles)
   std::vector<Group> groups = sizeof(R) == 4 ? plan_groups_k(n, 13, 9) : plan_groups<R>(n);
+  const int nw = sizeof(R) == 4 ? (int)groups.size() - 1 : 0;  // W tables
+  const int nlad = sizeof(R) == 8 ? 1 << std::min(n, 11) : n >= 13 ? (1 << 13) - 1 : 0;
+  QftTables<R> tab;
+  qc_status st = qft_tables(s, n, nl, nlad, &tab, false, (size_t)nw << 13);
+  if (st) return st;
+  V2 *tlo = tab.tlo, *thi = tab.thi;
+  if constexpr (sizeof(R) == 4) {
+    if (nw) {
+      QftGroups G{nw, {}, {}};
+      for (int i = 0; i < nw; ++i) G.lo[i] = groups[i + 1].lo, G.k[i] = groups[i + 1].k;
+      k_qft_w<<<dim3(32, nw), 256, 0, s->stream>>>(tlo, thi, n, nl, G, tab.lad + (1 << 13));
+      st = check_launch("qft twiddle tables");
+    }
+  }
   std::vector<TileProg<R>> progs(groups.size());
   bool all_compiled = true;  // complex128: double-float form between the passes
   for (int gi = (int)groups.size() - 1; gi >= 0; --gi) {
@@ -1496,7 +1511,8 @@ static qc_status qft_impl(qc_state* s) {
     if constexpr (sizeof(R) == 8) all_compiled = all_compiled && qft_c128_compiled(P);
   }
   for (int gi = (int)groups.size() - 1; gi >= 0 && !st; --gi) {
-    if constexpr (sizeof(R) == 4) st = run_qft_db_c64(s, progs[gi], tlo, thi);
+    if constexpr (sizeof(R) == 4)
+      st = run_qft_db_c64(s, progs[gi], tlo, thi, gi ? tab.lad + ((size_t)gi << 13) : nullptr, tab.lad);
     else
       st = run_qft_c128(s, progs[gi], tlo, thi, tab.lad, all_compiled && gi + 1 < (int)groups.size(), all_compiled);
   }
