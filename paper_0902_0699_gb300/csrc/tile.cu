@@ -687,9 +687,15 @@ __global__ void __launch_bounds__(512, 2) k_qft_c128_k(double2* __restrict__ s, 
 }
 
 // ------------------------------------------------- complex64 QFT passes --
-// One CTA per SM with two 64 KiB tile buffers: the next tile's loads
-// (cp.async, 16 bytes each) are in flight while the current tile is
-// transformed and written back.  The group's levels run in register blocks
+// Bound by memory latency and shared-memory round trips.  On a 2^13-amplitude
+// tile (k_qft_c64_k) two CTAs share an SM, each with one 64 KiB tile: while
+// one waits at its barriers or for its loads, the other computes.  What is the
+// same for every tile (the twiddles W, the ladders) is built once per
+// transform and read through L1, which is what makes room for the second tile.
+// 29 qubits, an 8-level pass above the lowest group: 2.16 ms with one CTA of
+// two buffers, 1.48 with two CTAs, the first levels straight from the state and
+// the last straight to it (0.86 of the copy bandwidth); the QFT 8.16 -> 6.76.
+// The group's levels run in register blocks
 // of up to four levels (one shared-memory round trip each).  Within a block
 // on group qubits jlo .. jlo+QR-1, level j = jlo + lv multiplies the
 // difference of the pair with local low bits m by
@@ -781,6 +787,27 @@ __device__ __forceinline__ void qft_levels_c64(float2* sm, int NE, int c, int k,
 // positions, the swizzled offsets of a block's elements and a thread's
 // copy and store offsets are constants, so the index arithmetic is one XOR
 // per element.  qsw is linear over XOR, qsw(x ^ y) = qsw(x) ^ qsw(y).
+template <int QR, int JLO>
+__device__ __forceinline__ void qft_butterflies_c64(float2* a, const float2* LAD, int xlow) {
+  constexpr int NR = 1 << QR;
+#pragma unroll
+  for (int lv = QR - 1; lv >= 0; --lv) {
+    const int j = JLO + lv;
+    const float2 u = JLO ? LAD[(1 << j) - 1 + xlow] : make_float2(1.f, 0.f);  // L_j(xlow), 1 for the lowest block
+#pragma unroll
+    for (int i = 0; i < NR; ++i) {
+      if ((i >> lv) & 1) continue;
+      const int i1 = i | (1 << lv);
+      const float2 x0 = a[i], x1 = a[i1];
+      a[i] = make_float2(x0.x + x1.x, x0.y + x1.y);
+      const int m = i & ((1 << lv) - 1);  // the factor e^{2 pi i m / 2^{lv+1}} L_j(xlow)
+      const float2 d = make_float2(x0.x - x1.x, x0.y - x1.y);
+      if (JLO) a[i1] = c2mul(d, m ? c2mul(qroot(lv, m), u) : u);
+      else a[i1] = m ? c2mul(d, qroot(lv, m)) : d;
+    }
+  }
+}
+
 template <int QR, int BL, int JLO>
 __device__ __forceinline__ void qft_block_c64_ct(float2* sm, const float2* LAD) {
   constexpr int NR = 1 << QR, NE = 1 << 13;
@@ -793,21 +820,29 @@ __device__ __forceinline__ void qft_block_c64_ct(float2* sm, const float2* LAD) 
     float2 a[NR];
 #pragma unroll
     for (int i = 0; i < NR; ++i) a[i] = sm[sb ^ qsw(i << BL)];
-    const int xlow = (base >> C) & ((1 << JLO) - 1);
+    qft_butterflies_c64<QR, JLO>(a, LAD, (base >> C) & ((1 << JLO) - 1));
 #pragma unroll
-    for (int lv = QR - 1; lv >= 0; --lv) {
-      const int j = JLO + lv;
-      const float2 u = LAD[(1 << j) - 1 + xlow];  // L_j(xlow)
+    for (int i = 0; i < NR; ++i) sm[sb ^ qsw(i << BL)] = a[i];
+  }
+}
+
+// The first block (the group's top QR levels, tile bits 13 - QR ..) straight
+// from the state: a warp's elements are rows of 2^C consecutive amplitudes,
+// and a thread's 2^QR loads are in flight together.  A round trip through
+// shared memory and its barrier fewer.
+template <int K, int QR>
+__device__ __forceinline__ void qft_first_block_load_c64(float2* sm, const float2* LAD, const float2* __restrict__ s,
+                                                         uint64_t T, int lo) {
+  constexpr int NR = 1 << QR, NE = 1 << 13, C = 13 - K, BL = 13 - QR, JLO = K - QR;
 #pragma unroll
-      for (int i = 0; i < NR; ++i) {
-        if ((i >> lv) & 1) continue;
-        const int i1 = i | (1 << lv);
-        const float2 x0 = a[i], x1 = a[i1];
-        a[i] = make_float2(x0.x + x1.x, x0.y + x1.y);
-        const int m = i & ((1 << lv) - 1);  // the factor e^{2 pi i m / 2^{lv+1}} L_j(xlow)
-        a[i1] = c2mul(make_float2(x0.x - x1.x, x0.y - x1.y), m ? c2mul(qroot(lv, m), u) : u);
-      }
-    }
+  for (int r = 0; r < (NE >> QR) / 512; ++r) {
+    const int base = threadIdx.x + 512 * r;
+    const uint64_t g = tile_global((uint64_t)base, T, lo, K, C), step = (uint64_t)(1 << JLO) << lo;
+    float2 a[NR];
+#pragma unroll
+    for (int i = 0; i < NR; ++i) a[i] = s[g + i * step];
+    qft_butterflies_c64<QR, JLO>(a, LAD, (base >> C) & ((1 << JLO) - 1));
+    const int sb = qsw(base);
 #pragma unroll
     for (int i = 0; i < NR; ++i) sm[sb ^ qsw(i << BL)] = a[i];
   }
@@ -860,20 +895,7 @@ __device__ __forceinline__ void qft_last_block_store_c64(const float2* sm, const
     float2 a[NR];
 #pragma unroll
     for (int i = 0; i < NR; ++i) a[i] = sm[sb ^ qsw(i << BL)];
-    // jlo = 0: every level's ladder phase is a constant root (xlow = 0)
-#pragma unroll
-    for (int lv = QR - 1; lv >= 0; --lv) {
-#pragma unroll
-      for (int i = 0; i < NR; ++i) {
-        if ((i >> lv) & 1) continue;
-        const int i1 = i | (1 << lv);
-        const float2 x0 = a[i], x1 = a[i1];
-        a[i] = make_float2(x0.x + x1.x, x0.y + x1.y);
-        const int m = i & ((1 << lv) - 1);
-        const float2 d = make_float2(x0.x - x1.x, x0.y - x1.y);
-        a[i1] = m ? c2mul(d, qroot(lv, m)) : d;
-      }
-    }
+    qft_butterflies_c64<QR, 0>(a, LAD, 0);  // every level's ladder phase is a constant root
     const uint64_t g = tile_global((uint64_t)base, T, lo, K, C);
     const int fb = (int)(__brev((unsigned)(base >> C)) >> (32 - K));
 #pragma unroll
@@ -910,19 +932,11 @@ __global__ void __launch_bounds__(512, 2) k_qft_c64_k(float2* __restrict__ s, ui
   // this thread's copy / store elements e0 + 1024 u share the group bits'
   // low part; their reversed group bits are f0 | brev(u) at the top
   const int f0 = (int)(__brev((unsigned)(e0 >> C)) >> (32 - K));
-  auto issue = [&](uint64_t T) {
-    const uint64_t g = tile_global((uint64_t)e0, T, lo, K, C);
-#pragma unroll
-    for (int u = 0; u < NE / 1024; ++u) {
-      const uint32_t d = (uint32_t)__cvta_generic_to_shared(cur + (se0 ^ qsw(1024 * u)));
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(s + g + u * gstep) : "memory");
-    }
-  };
   if (LSM)
     for (int a = threadIdx.x; a < (1 << K) - 1; a += blockDim.x) Ls[a] = lad[a];
+  __syncthreads();
+  constexpr int NB = qft_nblocks(K);
   for (uint64_t T = blockIdx.x; T < ntiles; T += gridDim.x) {
-    issue(T);
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
     if (tw) {
       const uint64_t Lt = (T & ((1ull << (lo - C)) - 1ull)) << C;
       for (int f = threadIdx.x; f < (1 << K); f += blockDim.x) {
@@ -931,19 +945,18 @@ __global__ void __launch_bounds__(512, 2) k_qft_c64_k(float2* __restrict__ s, ui
         V[f] = make_float2(z.re, z.im);
       }
     }
-    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    qft_first_block_load_c64<K, qft_block_size(K, 0)>(cur, LAD, s, T, lo);
     __syncthreads();
-    if constexpr (C >= 4) {
+    if constexpr (C >= 4 && NB >= 2) {
       if (tw) {
         // every pass above the lowest group: the last block goes straight to the state
-        constexpr int NB = qft_nblocks(K);
-        qft_levels_c64_ct<K, 0, NB - 1>(cur, LAD);
+        qft_levels_c64_ct<K, 1, NB - 1>(cur, LAD);
         qft_last_block_store_c64<K, qft_block_size(K, NB - 1)>(cur, LAD, W, V, s, T, lo);
         __syncthreads();
         continue;
       }
     }
-    qft_levels_c64_ct<K, 0, qft_nblocks(K)>(cur, LAD);
+    qft_levels_c64_ct<K, 1, NB>(cur, LAD);
     const uint64_t g = tile_global((uint64_t)e0, T, lo, K, C);
 #pragma unroll
     for (int u = 0; u < NE / 1024; ++u) {
@@ -966,6 +979,9 @@ __global__ void __launch_bounds__(512, 2) k_qft_c64_k(float2* __restrict__ s, ui
   }
 }
 
+// Registers below 13 qubits and groups of fewer than three levels: one CTA per
+// SM with two tile buffers, the next tile's copies (cp.async, 16 bytes each)
+// in flight while the current tile is transformed and written back.
 // P holds the pass: group [lo, lo+k), c contiguous bits, twiddle = lo > 0,
 // scale_p = k.  Shared memory: two tile buffers, then (twiddle passes) the
 // per-pass table W[e] = Omega_{hi+1}^{l f} (l = e's c low bits, f = its
