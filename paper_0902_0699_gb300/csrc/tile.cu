@@ -694,16 +694,15 @@ __global__ void __launch_bounds__(512, 2) k_qft_c128_k(double2* __restrict__ s, 
 // transform and read through L1, which is what makes room for the second tile.
 // 29 qubits, an 8-level pass above the lowest group: 2.16 ms with one CTA of
 // two buffers, 1.48 with two CTAs, the first levels straight from the state and
-// the last straight to it (0.86 of the copy bandwidth); the QFT 8.16 -> 6.76.
+// the last straight to it (0.91 of the copy bandwidth, 1.39 ms).
 // The group's levels run in register blocks
 // of up to four levels (one shared-memory round trip each).  Within a block
 // on group qubits jlo .. jlo+QR-1, level j = jlo + lv multiplies the
 // difference of the pair with local low bits m by
 //   L_j(x) = e^{2 pi i x / 2^{j+1}},  x = m 2^jlo + xlow,
-//   L_j(x) = e^{2 pi i m / 2^{lv+1}} L_j(xlow),
-// so a thread loads one ladder entry per level (its xlow is fixed) and
-// multiplies it by constant roots of unity.  The shared tile is swizzled in
-// 16-byte units (pairs of amplitudes stay together for the 16-byte copies):
+// read from the ladder table (one rounding; a constant root times L_j(xlow)
+// has two).  The lowest block's are constants.  The shared tile is swizzled in
+// 16-byte units:
 // strided register blocks then hit at most twice the minimum number of
 // shared-memory wavefronts instead of up to 16x.
 __device__ __forceinline__ int qsw(int e) { return e ^ (((e >> 4) & 7) << 1); }
@@ -735,55 +734,8 @@ __device__ __forceinline__ float2 qroot(int lv, int m) {
   }
 }
 
-template <int QR>
-__device__ __forceinline__ void qft_block_c64(float2* sm, int NE, int c, int jtop, const float2* LAD) {
-  constexpr int NR = 1 << QR;
-  const int jlo = jtop - QR + 1;
-  const int bl = c + jlo;
-  for (int p = threadIdx.x; p < (NE >> QR); p += blockDim.x) {
-    const int base = ((p >> bl) << (bl + QR)) | (p & ((1 << bl) - 1));
-    float2 a[NR];
-#pragma unroll
-    for (int i = 0; i < NR; ++i) a[i] = sm[qsw(base | (i << bl))];
-    const int xlow = (base >> c) & ((1 << jlo) - 1);
-#pragma unroll
-    for (int lv = QR - 1; lv >= 0; --lv) {
-      const int j = jlo + lv;
-      const float2 u = LAD[(1 << j) - 1 + xlow];  // L_j(xlow)
-#pragma unroll
-      for (int i = 0; i < NR; ++i) {
-        if ((i >> lv) & 1) continue;
-        const int i1 = i | (1 << lv);
-        const float2 x0 = a[i], x1 = a[i1];
-        a[i] = make_float2(x0.x + x1.x, x0.y + x1.y);
-        const int m = i & ((1 << lv) - 1);  // the factor e^{2 pi i m / 2^{lv+1}} L_j(xlow)
-        a[i1] = c2mul(make_float2(x0.x - x1.x, x0.y - x1.y), m ? c2mul(qroot(lv, m), u) : u);
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < NR; ++i) sm[qsw(base | (i << bl))] = a[i];
-  }
-}
-
-// Register blocks over levels k-1 .. 0: ceil(k/4) blocks, the larger first.
-__device__ __forceinline__ void qft_levels_c64(float2* sm, int NE, int c, int k, const float2* LAD) {
-  const int nb = (k + 3) >> 2;
-  int j = k - 1;
-  for (int b = 0; b < nb; ++b) {
-    const int qr = (j + 1 + (nb - b) - 1) / (nb - b);  // balanced, larger first
-    switch (qr) {
-      case 4: qft_block_c64<4>(sm, NE, c, j, LAD); break;
-      case 3: qft_block_c64<3>(sm, NE, c, j, LAD); break;
-      case 2: qft_block_c64<2>(sm, NE, c, j, LAD); break;
-      default: qft_block_c64<1>(sm, NE, c, j, LAD); break;
-    }
-    __syncthreads();
-    j -= qr;
-  }
-}
-
-// Compile-time forms for the passes of states of at least 13 qubits, where
-// every tile holds 2^13 amplitudes (k + c = 13): the register blocks' bit
+// States of at least 13 qubits (smaller ones: the general tile program).
+// Every tile holds 2^13 amplitudes (k + c = 13): the register blocks' bit
 // positions, the swizzled offsets of a block's elements and a thread's
 // copy and store offsets are constants, so the index arithmetic is one XOR
 // per element.  qsw is linear over XOR, qsw(x ^ y) = qsw(x) ^ qsw(y).
@@ -793,16 +745,15 @@ __device__ __forceinline__ void qft_butterflies_c64(float2* a, const float2* LAD
 #pragma unroll
   for (int lv = QR - 1; lv >= 0; --lv) {
     const int j = JLO + lv;
-    const float2 u = JLO ? LAD[(1 << j) - 1 + xlow] : make_float2(1.f, 0.f);  // L_j(xlow), 1 for the lowest block
 #pragma unroll
     for (int i = 0; i < NR; ++i) {
       if ((i >> lv) & 1) continue;
       const int i1 = i | (1 << lv);
       const float2 x0 = a[i], x1 = a[i1];
       a[i] = make_float2(x0.x + x1.x, x0.y + x1.y);
-      const int m = i & ((1 << lv) - 1);  // the factor e^{2 pi i m / 2^{lv+1}} L_j(xlow)
+      const int m = i & ((1 << lv) - 1);
       const float2 d = make_float2(x0.x - x1.x, x0.y - x1.y);
-      if (JLO) a[i1] = c2mul(d, m ? c2mul(qroot(lv, m), u) : u);
+      if (JLO) a[i1] = c2mul(d, LAD[(1 << j) - 1 + (m << JLO) + xlow]);  // L_j(m 2^jlo + xlow)
       else a[i1] = m ? c2mul(d, qroot(lv, m)) : d;
     }
   }
@@ -907,24 +858,16 @@ __device__ __forceinline__ void qft_last_block_store_c64(const float2* sm, const
 }
 
 template <int K>
-__global__ void __launch_bounds__(512, 2) k_qft_c64_k(float2* __restrict__ s, uint64_t ntiles, const TileProg<float> P,
-                                                      const float2* __restrict__ tlo,
-                                                      const float2* __restrict__ thi,
+__global__ void __launch_bounds__(512, 2) k_qft_c64_k(float2* __restrict__ s, uint64_t ntiles, int lo,
                                                       const float2* __restrict__ W,
                                                       const float2* __restrict__ lad) {
-  using A = TA<float>;
   constexpr int C = 13 - K, NE = 1 << 13;
   static_assert(C <= 10, "1024-element copy strides stay inside the group bits");
   extern __shared__ __align__(16) unsigned char smraw[];
-  const int lo = P.lo, hi = lo + K - 1;
-  const bool tw = P.twiddle != 0;
+  const int hi = lo + K - 1;
   float2* cur = reinterpret_cast<float2*>(smraw);
   float2* V = cur + NE;
-  // the ladders in shared memory; the lowest group's 64 KiB stay in global
-  // memory (read through L1), so that two blocks fit an SM
-  constexpr bool LSM = K <= 9;
-  float2* Ls = V + (tw ? (1 << K) : 0);
-  const float2* LAD = LSM ? Ls : lad;
+  float2* LAD = V + (1 << K);
   const float sc = (float)exp2(-0.5 * K);
   const int e0 = 2 * threadIdx.x;
   const int se0 = qsw(e0);
@@ -932,36 +875,31 @@ __global__ void __launch_bounds__(512, 2) k_qft_c64_k(float2* __restrict__ s, ui
   // this thread's copy / store elements e0 + 1024 u share the group bits'
   // low part; their reversed group bits are f0 | brev(u) at the top
   const int f0 = (int)(__brev((unsigned)(e0 >> C)) >> (32 - K));
-  if (LSM)
-    for (int a = threadIdx.x; a < (1 << K) - 1; a += blockDim.x) Ls[a] = lad[a];
+  for (int a = threadIdx.x; a < (1 << K) - 1; a += blockDim.x) LAD[a] = lad[a];
   __syncthreads();
   constexpr int NB = qft_nblocks(K);
   for (uint64_t T = blockIdx.x; T < ntiles; T += gridDim.x) {
-    if (tw) {
-      const uint64_t Lt = (T & ((1ull << (lo - C)) - 1ull)) << C;
-      for (int f = threadIdx.x; f < (1 << K); f += blockDim.x) {
-        const uint64_t r = (Lt * (uint64_t)f) & ((2ull << hi) - 1ull);
-        const A::E z = A::scale_by(omega<float>(tlo, thi, r << (P.n - hi - 1), P.nl), sc);
-        V[f] = make_float2(z.re, z.im);
-      }
+    // V[f] = Omega_{hi+1}^{Lt f} sc: the angle in two floats, the low one a
+    // small rotation (closer than a product of two rounded table entries)
+    const uint64_t Lt = (T & ((1ull << (lo - C)) - 1ull)) << C;
+    for (int f = threadIdx.x; f < (1 << K); f += blockDim.x) {
+      const uint64_t r = (Lt * (uint64_t)f) & ((2ull << hi) - 1ull);
+      const float ah = (float)r, al = (float)((int64_t)r - (int64_t)ah);
+      float vr, vi;
+      sincospif(ldexpf(ah, -hi), &vi, &vr);
+      const float d = ldexpf(al * 3.14159265358979f, -hi);
+      V[f] = make_float2(fmaf(-vi, d, vr) * sc, fmaf(vr, d, vi) * sc);
     }
     qft_first_block_load_c64<K, qft_block_size(K, 0)>(cur, LAD, s, T, lo);
     __syncthreads();
-    if constexpr (C >= 4 && NB >= 2) {
-      if (tw) {
-        // every pass above the lowest group: the last block goes straight to the state
-        qft_levels_c64_ct<K, 1, NB - 1>(cur, LAD);
-        qft_last_block_store_c64<K, qft_block_size(K, NB - 1)>(cur, LAD, W, V, s, T, lo);
-        __syncthreads();
-        continue;
-      }
-    }
-    qft_levels_c64_ct<K, 1, NB>(cur, LAD);
-    const uint64_t g = tile_global((uint64_t)e0, T, lo, K, C);
+    if constexpr (NB >= 2) {  // the last block goes straight to the state
+      qft_levels_c64_ct<K, 1, NB - 1>(cur, LAD);
+      qft_last_block_store_c64<K, qft_block_size(K, NB - 1)>(cur, LAD, W, V, s, T, lo);
+    } else {
+      const uint64_t g = tile_global((uint64_t)e0, T, lo, K, C);
 #pragma unroll
-    for (int u = 0; u < NE / 1024; ++u) {
-      float4 z = *reinterpret_cast<const float4*>(cur + (se0 ^ qsw(1024 * u)));
-      if (tw) {
+      for (int u = 0; u < NE / 1024; ++u) {
+        const float4 z = *reinterpret_cast<const float4*>(cur + (se0 ^ qsw(1024 * u)));
         // the group bits of e0 + 1024 u are (e0 >> C) + (1024 u >> C): reversed,
         // brev(u) lands below f0's bits
         const int f = f0 | (int)(__brev((unsigned)((1024 * u) >> C)) >> (32 - K));
@@ -969,107 +907,73 @@ __global__ void __launch_bounds__(512, 2) k_qft_c64_k(float2* __restrict__ s, ui
         const float4 w = *reinterpret_cast<const float4*>(W + e0 + 1024 * u);
         const float2 z0 = c2mul(c2mul(make_float2(z.x, z.y), make_float2(w.x, w.y)), v);
         const float2 z1 = c2mul(c2mul(make_float2(z.z, z.w), make_float2(w.z, w.w)), v);
-        z = make_float4(z0.x, z0.y, z1.x, z1.y);
-      } else {
-        z = make_float4(z.x * sc, z.y * sc, z.z * sc, z.w * sc);
+        *reinterpret_cast<float4*>(s + g + u * gstep) = make_float4(z0.x, z0.y, z1.x, z1.y);
       }
-      *reinterpret_cast<float4*>(s + g + u * gstep) = z;
     }
     __syncthreads();
   }
 }
 
-// Registers below 13 qubits and groups of fewer than three levels: one CTA per
-// SM with two tile buffers, the next tile's copies (cp.async, 16 bytes each)
-// in flight while the current tile is transformed and written back.
-// P holds the pass: group [lo, lo+k), c contiguous bits, twiddle = lo > 0,
-// scale_p = k.  Shared memory: two tile buffers, then (twiddle passes) the
-// per-pass table W[e] = Omega_{hi+1}^{l f} (l = e's c low bits, f = its
-// group bits reversed) and V[f] (per tile), then the ladder table.
-__global__ void __launch_bounds__(512, 1) k_qft_db_c64(float2* __restrict__ s, uint64_t ntiles, const TileProg<float> P,
-                                                       const float2* __restrict__ tlo, const float2* __restrict__ thi) {
-  using A = TA<float>;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  const int lo = P.lo, k = P.k, c = P.c, hi = lo + k - 1;
-  const int NE = 1 << (k + c);
-  float2* buf0 = reinterpret_cast<float2*>(smraw);
-  float2* buf1 = buf0 + NE;
-  float2* W = buf1 + NE;
-  float2* V = W + (P.twiddle ? NE : 0);
-  float2* LAD = V + (P.twiddle ? (1 << k) : 0);
-  const float sc = (float)exp2(-0.5 * P.scale_p);
-  // 16-byte copies of amplitude pairs (e, e+1); successive ones of a thread
-  // are 1024 tile elements apart
-  const bool step_ok = c <= 10;
-  const uint64_t gstep = step_ok ? ((uint64_t)(1024 >> c) << lo) : 0;
-  auto issue = [&](uint64_t T, float2* dst) {
-    const int e0 = 2 * threadIdx.x;
-    uint64_t g = tile_global((uint64_t)e0, T, lo, k, c);
-    for (int e = e0; e < NE; e += 1024) {
-      if (!step_ok) g = tile_global((uint64_t)e, T, lo, k, c);
-      const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst + qsw(e));
-      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(s + g) : "memory");
-      g += gstep;
-    }
-  };
-  uint64_t T = blockIdx.x;
-  if (T < ntiles) issue(T, buf0);
-  asm volatile("cp.async.commit_group;\n" ::: "memory");
-  // ladder table: LAD[2^j - 1 + x] = e^{2 pi i x / 2^{j+1}}, j < k
-  // (from the global root tables: e^{2 pi i x / 2^{j+1}} = Omega_n^{x 2^{n-j-1}})
-  for (int a = threadIdx.x; a < (1 << k) - 1; a += blockDim.x) {
-    const int j = 31 - __clz(a + 1);
-    const A::E z = omega<float>(tlo, thi, (uint64_t)(a + 1 - (1 << j)) << (P.n - j - 1), P.nl);
-    LAD[a] = make_float2(z.re, z.im);
-  }
-  if (P.twiddle)
-    for (int e = threadIdx.x; e < NE; e += blockDim.x) {
-      const int f = (int)(__brev((unsigned)(e >> c)) >> (32 - k));
-      const uint64_t x = (uint64_t)((e & ((1 << c) - 1)) * f);  // l f < 2^{c+k} <= 2^{hi+1}
-      const A::E z = omega<float>(tlo, thi, x << (P.n - hi - 1), P.nl);
-      W[e] = make_float2(z.re, z.im);
-    }
-  for (int it = 0; T < ntiles; T += gridDim.x, ++it) {
-    float2* cur = (it & 1) ? buf1 : buf0;
-    float2* nxt = (it & 1) ? buf0 : buf1;
-    // nxt was last read by the previous tile's store, which ended at that
-    // iteration's closing barrier
-    if (T + gridDim.x < ntiles) issue(T + gridDim.x, nxt);
-    asm volatile("cp.async.commit_group;\n" ::: "memory");
-    if (P.twiddle) {
-      // V[f] = 2^{-k/2} Omega_{hi+1}^{Ltile f}
-      const uint64_t Lt = (T & ((1ull << (lo - c)) - 1ull)) << c;
-      for (int f = threadIdx.x; f < (1 << k); f += blockDim.x) {
-        const uint64_t r = (Lt * (uint64_t)f) & ((2ull << hi) - 1ull);
-        const A::E z = A::scale_by(omega<float>(tlo, thi, r << (P.n - hi - 1), P.nl), sc);
-        V[f] = make_float2(z.re, z.im);
+// The lowest QFTR_B levels with the reversal of all n index bits (see the bit
+// reversal below for its tiles).  Index = (h, m, l), h and l of QFTR_B bits:
+// the transform of a row (the 2^QFTR_B values of l) gives, at position p,
+// frequency rev(p), whose place is (rev p, rev m, rev h).  The block for m
+// (m <= rev m) reads the tiles of m and rev m, one level on its loads' way
+// into shared memory and four on the way out, so that the levels cost no pass.
+// 29 qubits: a 13-level lowest group took 2.07 ms and the reversal 1.72;
+// an 8-level group and this kernel take 1.39 and 1.75 (0.73 of the copy
+// bandwidth: rows of 256 bytes), the whole QFT 6.76 -> 5.94 (8.16 with one CTA
+// an SM).  Six or eight blocks an SM run alike, ten are slower (1.87).
+constexpr int QFTR_B = 5;
+constexpr int QFTR_T = 128;
+__global__ void __launch_bounds__(QFTR_T, 8) k_qft_rev_c64(float2* __restrict__ s, int n, const float2* __restrict__ lad) {
+  constexpr int B = QFTR_B, W = 1 << B, WP = W + 1;
+  static_assert(B == 5 && QFTR_T == 128, "two warps a tile, sixteen amplitudes a thread");
+  __shared__ float2 A[2][W * WP];
+  const int lane = threadIdx.x & 31, w = (threadIdx.x >> 5) & 1, t = threadIdx.x >> 6;
+  const int nm = n - 2 * B;
+  const uint64_t M = 1ull << nm;
+  const float sc = (float)exp2(-0.5 * B);
+  // loads: l = 2j, 2j + 1 and 16 above them, of rows r0 + 8 u; a half-warp's
+  // two rows are neighbours, so that its stores to the padded tile hit every bank
+  const int j = lane & 7, r0 = (lane >> 3) | (w << 2);
+  const float2 c0 = lad[(1 << (B - 1)) - 1 + 2 * j], c1 = lad[(1 << (B - 1)) + 2 * j];
+  // stores: positions 16 w + i, i < 16, of row rev(lane)
+  const int rr = (int)(__brev((unsigned)lane) >> (32 - B));
+  for (uint64_t m = blockIdx.x; m < M; m += gridDim.x) {
+    const uint64_t mr = nm ? (__brevll((unsigned long long)m) >> (64 - nm)) : 0ull;
+    if (mr < m) continue;
+    const bool act = t == 0 || mr != m;
+    if (act) {
+      const float2* g = s + (((uint64_t)r0 << (n - B)) | ((t ? mr : m) << B) | (uint64_t)(2 * j));
+      float4 x[4], y[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        x[u] = *reinterpret_cast<const float4*>(g + ((uint64_t)(8 * u) << (n - B)));
+        y[u] = *reinterpret_cast<const float4*>(g + ((uint64_t)(8 * u) << (n - B)) + 16);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {  // the top level
+        float2* o = A[t] + (r0 + 8 * u) * WP + 2 * j;
+        o[0] = make_float2(x[u].x + y[u].x, x[u].y + y[u].y);
+        o[1] = make_float2(x[u].z + y[u].z, x[u].w + y[u].w);
+        o[16] = c2mul(make_float2(x[u].x - y[u].x, x[u].y - y[u].y), c0);
+        o[17] = c2mul(make_float2(x[u].z - y[u].z, x[u].w - y[u].w), c1);
       }
     }
-    asm volatile("cp.async.wait_group 1;\n" ::: "memory");  // this thread's copies of the current tile
-    __syncthreads();                                         // ... and everyone's; tables and V written
-    qft_levels_c64(cur, NE, c, k, LAD);
-    // store: pairs (e, e+1) share the group bits (c >= 1 whenever lo > 0)
-    const int e0 = 2 * threadIdx.x;
-    uint64_t g = tile_global((uint64_t)e0, T, lo, k, c);
-    for (int e = e0; e < NE; e += 1024) {
-      if (!step_ok) g = tile_global((uint64_t)e, T, lo, k, c);
-      float4 z = *reinterpret_cast<const float4*>(cur + qsw(e));
-      if (P.twiddle) {
-        const int f = (int)(__brev((unsigned)(e >> c)) >> (32 - k));
-        const float2 v = V[f];
-        const float4 w = *reinterpret_cast<const float4*>(W + e);
-        const float2 z0 = c2mul(c2mul(make_float2(z.x, z.y), make_float2(w.x, w.y)), v);
-        const float2 z1 = c2mul(c2mul(make_float2(z.z, z.w), make_float2(w.z, w.w)), v);
-        z = make_float4(z0.x, z0.y, z1.x, z1.y);
-      } else {
-        z = make_float4(z.x * sc, z.y * sc, z.z * sc, z.w * sc);
-      }
-      *reinterpret_cast<float4*>(s + g) = z;
-      g += gstep;
+    __syncthreads();
+    if (act) {
+      float2 a[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) a[i] = A[t][rr * WP + 16 * w + i];
+      qft_butterflies_c64<4, 0>(a, lad, 0);
+      float2* g = s + (((uint64_t)w << (n - B)) | ((t ? m : mr) << B) | (uint64_t)lane);
+#pragma unroll
+      for (int i = 0; i < 16; ++i)
+        g[(uint64_t)(__brev((unsigned)i) >> (32 - 4)) << (n - B + 1)] = make_float2(a[i].x * sc, a[i].y * sc);
     }
     __syncthreads();
   }
-  asm volatile("cp.async.wait_all;\n" ::: "memory");
 }
 
 // Tables of Omega^a (a < 2^nl) and Omega^{a 2^nl} (a < 2^{n-nl}),
@@ -1106,7 +1010,7 @@ __global__ void k_roots(typename CT<R>::V2* tlo, typename CT<R>::V2* thi, int n,
 // the tile holds 2^{k+c} amplitudes (64 KiB: 2^12 complex128 or 2^13
 // complex64 amplitudes, 128 KiB for complex64 layer groups of 10): 30
 // complex128 qubits in three QFT passes, 12 + 9 + 9, 32 complex64 qubits in
-// four, 13 + 7 + 6 + 6.
+// four, 5 + 9 + 9 + 9 (the lowest five with the bit reversal).
 template <typename R> struct TileCfg;
 template <> struct TileCfg<double> { static constexpr int C = 3, K = 9, BOT = 12; };
 // the ladder helper reaches one level past the table (levels 0..10)
@@ -1208,53 +1112,33 @@ static qc_status run_qft_c128(qc_state* s, TileProg<double>& P, const double2* t
   return run_tile<double>(s, P, tlo, thi, lad);
 }
 
-// complex64 QFT pass through the double-buffered kernel: two tile buffers
-// plus the pass's tables.
-static size_t qft_db_smem(int k, int c, bool twiddle) {
-  const size_t NE = (size_t)1 << (k + c);
-  return sizeof(float2) * (2 * NE + (twiddle ? NE + ((size_t)1 << k) : 0) + ((size_t)1 << k) - 1);
-}
-
-static qc_status run_qft_db_c64(qc_state* s, TileProg<float>& P, const float2* tlo, const float2* thi,
-                                const float2* W, const float2* lad) {
-  const uint64_t ntiles = 1ull << (s->n - (P.k + P.c));
-  const size_t smem = qft_db_smem(P.k, P.c, P.twiddle != 0);
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaFuncSetAttribute(k_qft_db_c64, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-    attr_set = true;
+// complex64 QFT pass on a group of three to ten qubits (2^13-amplitude tiles).
+static qc_status run_qft_c64(qc_state* s, const Group& g, const float2* W, const float2* lad) {
+  const int64_t ntiles = (int64_t)1 << (s->n - 13);
+  switch (g.k) {
+#define QC_QFT_C64(KK)                                                                                  \
+  case KK: {                                                                                            \
+    const size_t smem = sizeof(float2) * ((1 << 13) + 2 * (1 << KK));                                   \
+    static bool a = false;                                                                              \
+    if (!a) {                                                                                           \
+      cudaFuncSetAttribute(k_qft_c64_k<KK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);    \
+      a = true;                                                                                         \
+    }                                                                                                   \
+    const unsigned grid = resident_grid(k_qft_c64_k<KK>, 512, ntiles, 1, smem);                         \
+    k_qft_c64_k<KK><<<grid, 512, smem, s->stream>>>(reinterpret_cast<float2*>(s->data), (uint64_t)ntiles, g.lo, W, lad); \
+    return check_launch("qft pass");                                                                    \
   }
-  float2* d = reinterpret_cast<float2*>(s->data);
-  // 2^13-amplitude tiles (states of at least 13 qubits): the compile-time kernels
-  if (P.k + P.c == 13 && P.c == 13 - P.k && P.scale_p == P.k) {
-    switch (P.k) {
-#define QC_QFT_DB(KK)                                                                              \
-  case KK: {                                                                                       \
-    static bool a = false;                                                                         \
-    if (!a) {                                                                                      \
-      cudaFuncSetAttribute(k_qft_c64_k<KK>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024); \
-      a = true;                                                                                    \
-    }                                                                                              \
-    const size_t sm1 = sizeof(float2) * ((1 << 13) + (P.twiddle ? 1 << KK : 0) + (KK <= 9 ? (1 << KK) - 1 : 0)); \
-    const unsigned g = resident_grid(k_qft_c64_k<KK>, 512, (int64_t)ntiles, 1, sm1);               \
-    k_qft_c64_k<KK><<<g, 512, sm1, s->stream>>>(d, ntiles, P, tlo, thi, W, lad);                   \
-    return check_launch("qft pass");                                                               \
+    QC_QFT_C64(3) QC_QFT_C64(4) QC_QFT_C64(5) QC_QFT_C64(6) QC_QFT_C64(7) QC_QFT_C64(8) QC_QFT_C64(9) QC_QFT_C64(10)
+#undef QC_QFT_C64
+    default: return QC_EINVAL;
   }
-      QC_QFT_DB(3) QC_QFT_DB(4) QC_QFT_DB(5) QC_QFT_DB(6) QC_QFT_DB(7) QC_QFT_DB(8) QC_QFT_DB(9) QC_QFT_DB(13)
-#undef QC_QFT_DB
-      default: break;
-    }
-  }
-  const unsigned grid = resident_grid(k_qft_db_c64, 512, (int64_t)ntiles, 1, smem);
-  k_qft_db_c64<<<grid, 512, smem, s->stream>>>(d, ntiles, P, tlo, thi);
-  return check_launch("qft pass");
 }
 
 // Contiguous low bits of a group's tile: at least C (128-byte rows) and, for
 // small groups, enough to fill the tile to 2^TB amplitudes, so that a pass
 // has few large tiles with long rows rather than many small ones (each tile
 // costs a DRAM round trip before its compute).  TB: 64 KiB tiles (two CTAs
-// per SM; the complex64 QFT kernel holds two of them in one CTA).  The QFT
+// per SM).  The QFT
 // twiddle tables need c + k <= 14.
 template <typename R>
 static int tile_c(const Group& g) {
@@ -1335,17 +1219,17 @@ qc_status launch_hall(qc_state* s) {
 }
 
 // ------------------------------------------------------- bit reversal ----
-// In-place reversal of all n index bits.  Index = (h, m, l) with h, l of B
+// In-place reversal of all n index bits (complex128).  Index = (h, m, l) with h, l of B
 // bits: rev(h, m, l) = (rev l, rev m, rev h).  The block for middle value m
 // (with m <= rev m) exchanges the 2^B x 2^B tiles of m and rev m through
 // shared memory (rows of 2^B contiguous amplitudes, padded against bank
 // conflicts).  The pass is latency bound (load both tiles, synchronise,
-// store), so many small blocks beat few large ones: complex128 runs B = 4
+// store), so many small blocks beat few large ones: B = 4
 // with 128 threads (twelve blocks per SM; 0.76 of copy bandwidth on GB300
-// at 30 qubits, against 0.63 for B = 5 with 256 threads); complex64 keeps
-// B = 5 with 256 threads (rows of 256 bytes).
-template <typename V2, bool FF>
-__device__ __forceinline__ V2 bitrev_out(V2 v) {
+// at 30 qubits, against 0.63 for B = 5 with 256 threads).  complex128 states of
+// more than one group only: a single tile reverses on its store.
+template <bool FF>
+__device__ __forceinline__ double2 bitrev_out(double2 v) {
   if constexpr (FF) {
     const ffc z = ffc_unpack(v);
     return make_double2(ff_to_d_fast(z.re), ff_to_d_fast(z.im));
@@ -1354,17 +1238,15 @@ __device__ __forceinline__ V2 bitrev_out(V2 v) {
   }
 }
 
-// FF (complex128 only): the input holds double-float parts (the form the
+// FF: the input holds double-float parts (the form the
 // compiled QFT passes leave) and is converted to IEEE double on the way.
-template <typename R, int B, int T, bool FF = false>
-__global__ void __launch_bounds__(T) k_bitrev(typename CT<R>::V2* __restrict__ s, int n) {
-  using V2 = typename CT<R>::V2;
-  static_assert(!FF || sizeof(R) == 8, "double-float input is complex128");
-  constexpr int W = 1 << B, WP = W + 1, PER = W * W / T;
+constexpr int BITREV_B = 4, BITREV_T = 128;
+template <bool FF>
+__global__ void __launch_bounds__(BITREV_T) k_bitrev(double2* __restrict__ s, int n) {
+  using V2 = double2;
+  constexpr int B = BITREV_B, T = BITREV_T, W = 1 << B, WP = W + 1, PER = W * W / T;
   static_assert(PER * T == W * W, "whole tiles per block");
-  extern __shared__ __align__(16) unsigned char smraw[];
-  V2* A = reinterpret_cast<V2*>(smraw);
-  V2* Bt = A + W * WP;
+  __shared__ V2 A[W * WP], Bt[W * WP];
   const int nm = n - 2 * B;
   const uint64_t M = 1ull << nm;
   for (uint64_t m = blockIdx.x; m < M; m += gridDim.x) {
@@ -1394,54 +1276,26 @@ __global__ void __launch_bounds__(T) k_bitrev(typename CT<R>::V2* __restrict__ s
       const int rl = (int)(__brev((unsigned)l) >> (32 - B)), rh = (int)(__brev((unsigned)h) >> (32 - B));
       // element (h, m, l) of the output is the input at rev(h, m, l)
       if (mr != m) {
-        s[((uint64_t)h << (n - B)) | (m << B) | (uint64_t)l] = bitrev_out<V2, FF>(Bt[rl * WP + rh]);
-        s[((uint64_t)h << (n - B)) | (mr << B) | (uint64_t)l] = bitrev_out<V2, FF>(A[rl * WP + rh]);
+        s[((uint64_t)h << (n - B)) | (m << B) | (uint64_t)l] = bitrev_out<FF>(Bt[rl * WP + rh]);
+        s[((uint64_t)h << (n - B)) | (mr << B) | (uint64_t)l] = bitrev_out<FF>(A[rl * WP + rh]);
       } else {
-        s[((uint64_t)h << (n - B)) | (m << B) | (uint64_t)l] = bitrev_out<V2, FF>(A[rl * WP + rh]);
+        s[((uint64_t)h << (n - B)) | (m << B) | (uint64_t)l] = bitrev_out<FF>(A[rl * WP + rh]);
       }
     }
     __syncthreads();
   }
 }
 
-// Small states: the whole vector through shared memory, one block.
-template <typename R>
-__global__ void k_bitrev_small(typename CT<R>::V2* __restrict__ s, int n) {
-  using V2 = typename CT<R>::V2;
-  extern __shared__ __align__(16) unsigned char smraw[];
-  V2* A = reinterpret_cast<V2*>(smraw);
-  const int N = 1 << n;
-  for (int i = threadIdx.x; i < N; i += blockDim.x) A[i] = s[i];
-  __syncthreads();
-  for (int i = threadIdx.x; i < N; i += blockDim.x) {
-    const int r = n ? (int)(__brev((unsigned)i) >> (32 - n)) : 0;
-    s[i] = A[r];
+static qc_status bitrev_impl(qc_state* s, bool from_ff) {
+  double2* d = reinterpret_cast<double2*>(s->data);
+  const int64_t M = (int64_t)1 << (s->n - 2 * BITREV_B);
+  if (from_ff) {
+    const unsigned grid = resident_grid(k_bitrev<true>, BITREV_T, M, 1, 0);
+    k_bitrev<true><<<grid, BITREV_T, 0, s->stream>>>(d, s->n);
+  } else {
+    const unsigned grid = resident_grid(k_bitrev<false>, BITREV_T, M, 1, 0);
+    k_bitrev<false><<<grid, BITREV_T, 0, s->stream>>>(d, s->n);
   }
-}
-
-template <typename R>
-static qc_status bitrev_impl(qc_state* s, bool from_ff = false) {
-  using V2 = typename CT<R>::V2;
-  V2* d = reinterpret_cast<V2*>(s->data);
-  const int n = s->n;
-  constexpr int b = sizeof(R) == 8 ? 4 : 5, T = sizeof(R) == 8 ? 128 : 256;
-  if (n < 2 * b) {
-    if (from_ff) return QC_EINVAL;
-    k_bitrev_small<R><<<1, 256, sizeof(V2) << n, s->stream>>>(d, n);
-    return check_launch("bitrev small");
-  }
-  const size_t smem = 2 * (size_t)(1 << b) * ((1 << b) + 1) * sizeof(V2);
-  const uint64_t M = 1ull << (n - 2 * b);
-  if constexpr (sizeof(R) == 8) {
-    if (from_ff) {
-      const unsigned grid = resident_grid(k_bitrev<R, b, T, true>, T, (int64_t)M, 1, smem);
-      k_bitrev<R, b, T, true><<<grid, T, smem, s->stream>>>(d, n);
-      return check_launch("bitrev");
-    }
-  }
-  if (from_ff) return QC_EINVAL;
-  const unsigned grid = resident_grid(k_bitrev<R, b, T>, T, (int64_t)M, 1, smem);
-  k_bitrev<R, b, T><<<grid, T, smem, s->stream>>>(d, n);
   return check_launch("bitrev");
 }
 
@@ -1454,10 +1308,9 @@ struct QftTables {
   typename CT<R>::V2 *tlo, *thi, *lad;
 };
 template <typename R>
-static qc_status qft_tables(qc_state* s, int n, int nl, int nlad, QftTables<R>* t, bool fixed = false,
-                            size_t room = 0) {
+static qc_status qft_tables(qc_state* s, int n, int nl, int nlad, QftTables<R>* t, bool fixed = false) {
   const size_t tot = ((size_t)1 << nl) + ((size_t)1 << (n - nl)) + (size_t)nlad;
-  cudaError_t e = ws_alloc((void**)&t->tlo, (tot + 2 + room) * sizeof(typename CT<R>::V2), s->stream);
+  cudaError_t e = ws_alloc((void**)&t->tlo, (tot + 2) * sizeof(typename CT<R>::V2), s->stream);
   if (e != cudaSuccess) return cuda_fail(e, "qft tables");
   t->thi = t->tlo + ((size_t)1 << nl);
   t->lad = t->thi + (((size_t)1 << (n - nl)) + 1) / 2 * 2;  // 16-byte aligned
@@ -1473,18 +1326,67 @@ static qc_status qft_tables(qc_state* s, int n, int nl, int nlad, QftTables<R>* 
 // W[e] = Omega_{hi+1}^{l f} of the complex64 pass blockIdx.y on group
 // [lo, lo + k): l = tile element e's c = 13 - k low bits, f its group bits
 // reversed.  Every tile of a pass uses the same 64 KiB, read through L1.
+// Below the tables: the ladder, level j's e^{2 pi i x / 2^{j+1}} at 2^j - 1 + x
+// (blockIdx.y = np).
+constexpr int QFT_LAD = 1 << 10;
 struct QftGroups {
   int np;
   int lo[8], k[8];
 };
-__global__ void __launch_bounds__(256) k_qft_w(const float2* __restrict__ tlo, const float2* __restrict__ thi, int n,
-                                               int nl, const QftGroups G, float2* __restrict__ W) {
-  const int lo = G.lo[blockIdx.y], k = G.k[blockIdx.y], c = 13 - k;
+__global__ void __launch_bounds__(256) k_qft_w(const QftGroups G, float2* __restrict__ lad) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (blockIdx.y == G.np) {
+    if (e < QFT_LAD) {
+      const int j = 31 - __clz(e + 1);
+      const TA<float>::E z = TA<float>::root((uint64_t)(e + 1 - (1 << j)), j + 1);
+      lad[e] = make_float2(z.re, z.im);
+    }
+    return;
+  }
+  const int lo = G.lo[blockIdx.y], k = G.k[blockIdx.y], c = 13 - k;
   const int f = (int)(__brev((unsigned)(e >> c)) >> (32 - k));
-  const uint64_t x = (uint64_t)((e & ((1 << c) - 1)) * f);
-  const TA<float>::E z = omega<float>(tlo, thi, x << (n - lo - k), nl);
-  W[((size_t)blockIdx.y << 13) + e] = make_float2(z.re, z.im);
+  float zr, zi;  // an exact argument: one rounding
+  sincospif(ldexpf((float)((e & ((1 << c) - 1)) * f), 1 - lo - k), &zi, &zr);
+  lad[QFT_LAD + ((size_t)blockIdx.y << 13) + e] = make_float2(zr, zi);
+}
+
+// Groups of a complex64 transform of at least 13 qubits: the bit reversal's
+// kernel does the lowest QFTR_B levels, the others are balanced in groups of
+// at most nine (2^13-amplitude tiles with rows of 128 bytes or more), the
+// lowest of at least eight, so that its tiles are whole.  Ten levels (n = 15)
+// run as one group.
+static std::vector<Group> qft_groups_c64(int n) {
+  const int total = n - QFTR_B;
+  if (total <= 10) return {{QFTR_B, total}};
+  const int np = (total + 8) / 9, g0 = std::max(8, (total + np - 1) / np);
+  std::vector<Group> g{{QFTR_B, g0}};
+  for (int i = 1, lo = QFTR_B + g0; i < np; ++i) {
+    const int k = (n - lo + np - i - 1) / (np - i);
+    g.push_back({lo, k});
+    lo += k;
+  }
+  return g;
+}
+
+static qc_status qft_c64(qc_state* s) {
+  const std::vector<Group> groups = qft_groups_c64(s->n);
+  QftGroups G{(int)groups.size(), {}, {}};
+  for (int i = 0; i < G.np; ++i) G.lo[i] = groups[i].lo, G.k[i] = groups[i].k;
+  float2* lad = nullptr;  // the ladder, then the passes' W tables
+  cudaError_t e = ws_alloc((void**)&lad, sizeof(float2) * (QFT_LAD + ((size_t)G.np << 13)), s->stream);
+  if (e != cudaSuccess) return cuda_fail(e, "qft tables");
+  k_qft_w<<<dim3(32, G.np + 1), 256, 0, s->stream>>>(G, lad);
+  qc_status st = check_launch("qft tables");
+  for (int gi = G.np - 1; gi >= 0 && !st; --gi)
+    st = run_qft_c64(s, groups[gi], lad + QFT_LAD + ((size_t)gi << 13), lad);
+  if (!st) {
+    const uint64_t M = 1ull << (s->n - 2 * QFTR_B);
+    const unsigned grid = resident_grid(k_qft_rev_c64, QFTR_T, (int64_t)M, 1, 0);
+    k_qft_rev_c64<<<grid, QFTR_T, 0, s->stream>>>(reinterpret_cast<float2*>(s->data), s->n, lad);
+    st = check_launch("qft bit reversal");
+  }
+  cudaFreeAsync(lad, s->stream);
+  return st;
 }
 
 template <typename R>
@@ -1492,22 +1394,11 @@ static qc_status qft_impl(qc_state* s) {
   using V2 = typename CT<R>::V2;
   const int n = s->n;
   const int nl = (n + 1) / 2;
-  // complex64: groups of at most 9 above the lowest 13 (64 KiB tiles)
-  std::vector<Group> groups = sizeof(R) == 4 ? plan_groups_k(n, 13, 9) : plan_groups<R>(n);
-  const int nw = sizeof(R) == 4 ? (int)groups.size() - 1 : 0;  // W tables
-  const int nlad = sizeof(R) == 8 ? 1 << std::min(n, 11) : n >= 13 ? (1 << 13) - 1 : 0;
+  std::vector<Group> groups = plan_groups<R>(n);
   QftTables<R> tab;
-  qc_status st = qft_tables(s, n, nl, nlad, &tab, false, (size_t)nw << 13);
+  qc_status st = qft_tables(s, n, nl, 1 << std::min(n, sizeof(R) == 8 ? 11 : 12), &tab);
   if (st) return st;
   V2 *tlo = tab.tlo, *thi = tab.thi;
-  if constexpr (sizeof(R) == 4) {
-    if (nw) {
-      QftGroups G{nw, {}, {}};
-      for (int i = 0; i < nw; ++i) G.lo[i] = groups[i + 1].lo, G.k[i] = groups[i + 1].k;
-      k_qft_w<<<dim3(32, nw), 256, 0, s->stream>>>(tlo, thi, n, nl, G, tab.lad + (1 << 13));
-      st = check_launch("qft twiddle tables");
-    }
-  }
   std::vector<TileProg<R>> progs(groups.size());
   bool all_compiled = true;  // complex128: double-float form between the passes
   for (int gi = (int)groups.size() - 1; gi >= 0; --gi) {
@@ -1526,21 +1417,25 @@ static qc_status qft_impl(qc_state* s) {
     P.twiddle = g.lo > 0;
     if constexpr (sizeof(R) == 8) all_compiled = all_compiled && qft_c128_compiled(P);
   }
+  // one tile: it is stored in reversed order (every complex64 state that comes here)
+  if (groups.size() == 1 && !(sizeof(R) == 8 && all_compiled)) progs[0].rev = 1;
   for (int gi = (int)groups.size() - 1; gi >= 0 && !st; --gi) {
     if constexpr (sizeof(R) == 4)
-      st = run_qft_db_c64(s, progs[gi], tlo, thi, gi ? tab.lad + ((size_t)gi << 13) : nullptr, tab.lad);
+      st = run_tile<R>(s, progs[gi], tlo, thi, tab.lad);
     else
       st = run_qft_c128(s, progs[gi], tlo, thi, tab.lad, all_compiled && gi + 1 < (int)groups.size(), all_compiled);
   }
-  // the bit reversal converts the complex128 passes' double-float form back
-  if (!st) st = bitrev_impl<R>(s, sizeof(R) == 8 && all_compiled);
+  if constexpr (sizeof(R) == 8) {  // the bit reversal converts the double-float form back
+    if (!st && !progs[0].rev) st = bitrev_impl(s, all_compiled);
+  }
   cudaFreeAsync(tab.tlo, s->stream);
   return st;
 }
 
 qc_status launch_qft(qc_state* s) {
   s->sum_valid = false;
-  return s->dt == QC_C128 ? qft_impl<double>(s) : qft_impl<float>(s);
+  if (s->dt == QC_C128) return qft_impl<double>(s);
+  return s->n >= 13 ? qft_c64(s) : qft_impl<float>(s);
 }
 
 // ---------------------------------------------------- register QFT -------
