@@ -62,51 +62,71 @@ __device__ __forceinline__ Mat2<R> gate_matrix(int kind, double theta) {
 }
 
 // ----------------------------------------------------- accumulators ------
-template <typename R> struct Acc;
-template <> struct Acc<double> {
+// The energy's sum.  complex64: products exact as float pairs (two-product),
+// summed as a float pair with two-sum (relative error ~ terms * 2^-48),
+// converted to double every few terms.
+template <typename R> struct SumE;
+template <> struct SumE<double> {
   double a = 0.0;
   __device__ void add(double x, double y) { a = fma(x, y, a); }
-  __device__ void sub(double x, double y) { a = fma(-x, y, a); }
   __device__ void flush() {}
   __device__ double value() const { return a; }
-  __device__ void merge(const Acc& o) { a += o.a; }
-  __device__ void merge_neg(const Acc& o) { a -= o.a; }
-  __device__ void into(double& z) const { z += a; }
-  __device__ bool finite() const { return isfinite(a); }
 };
-// complex64: products exact as float pairs (two-product), summed as a float
-// pair with two-sum (relative error ~ terms * 2^-48), converted to double
-// once per thread -- no FP64 instruction in the loop.
-template <> struct Acc<float> {
+template <> struct SumE<float> {
   double a = 0.0;
   float s = 0.f, c = 0.f;
-  __device__ void put(float p, float e) {
+  __device__ void add(float x, float y) {
+    const float p = x * y, e = fmaf(x, y, -p);
     const float t = s + p;
     const float bp = t - s;
     c += ((s - (t - bp)) + (p - bp)) + e;
     s = t;
-  }
-  __device__ void add(float x, float y) {
-    const float p = x * y;
-    put(p, fmaf(x, y, -p));
-  }
-  __device__ void sub(float x, float y) {
-    const float p = -x * y;
-    put(p, fmaf(-x, y, -p));
   }
   __device__ void flush() {
     a += (double)s + (double)c;
     s = c = 0.f;
   }
   __device__ double value() const { return a; }
-  __device__ void merge(const Acc& o) { put(o.s, o.c); }
-  __device__ void merge_neg(const Acc& o) { put(-o.s, -o.c); }
-  __device__ void into(float2& z) const {
-    Acc t;
-    t.s = z.x;
-    t.c = z.y;
-    t.put(s, c);
-    z = make_float2(t.s, t.c);
+};
+
+// The derivatives' sums.
+template <typename R> struct Acc;
+template <> struct Acc<double> {
+  double a = 0.0;
+  __device__ void add(double x, double y) { a = fma(x, y, a); }
+  __device__ void sub(double x, double y) { a = fma(-x, y, a); }
+  __device__ void start(double) {}
+  __device__ void settle(double) {}
+  __device__ double value() const { return a; }
+  __device__ void merge(const Acc& o) { a += o.a; }
+  __device__ void merge_neg(const Acc& o) { a -= o.a; }
+  __device__ void into(double& z) const { z += a; }
+  __device__ bool finite() const { return isfinite(a); }
+};
+// complex64: a float pair, no FP64 instruction.  The high word starts at
+// C = 1.5 2^e with every partial sum below 2^{e-1}: it stays in one binade, so
+// that s' - s is the multiple of its unit that a product was rounded to,
+// exactly, and fma(x, y, -(s' - s)) what that left out.  Four instructions a
+// product; a two-product and a two-sum take ten (20 qubits, 64 states: the
+// backward passes 28.5 -> 24.9 ms; what is left waits: issue slots 0.53
+// busy, barriers, shared memory and the tile's loads in turn).
+// Error: 2^-24 units a term, a unit being 2^-16 of the largest product at most.
+template <> struct Acc<float> {
+  float s = 0.f, c = 0.f;
+  __device__ void start(float C) { s = C; }
+  __device__ void settle(float C) { s -= C; }
+  __device__ void add(float x, float y) {
+    const float t = fmaf(x, y, s);
+    c += fmaf(x, y, s - t);
+    s = t;
+  }
+  __device__ void sub(float x, float y) { add(-x, y); }
+  // sums with a common C, settled: the high words are multiples of one unit
+  __device__ void merge(const Acc& o) { s += o.s; c += o.c; }
+  __device__ void merge_neg(const Acc& o) { s -= o.s; c -= o.c; }
+  __device__ void into(float2& z) const {  // two-sum
+    const float t = z.x + s, bp = t - z.x;
+    z = make_float2(t, z.y + (((z.x - (t - bp)) + (s - bp)) + c));
   }
   __device__ bool finite() const { return isfinite(s); }
   // (s + c) 2^k as hi 2^26 + lo, to a unit (k may exceed a float's range of
@@ -114,9 +134,10 @@ template <> struct Acc<float> {
   __device__ int2 fixed(int k) const {
     const int e = k - 26;
     const float f0 = __int_as_float((127 + e / 2) << 23), f1 = __int_as_float((127 + e - e / 2) << 23);
-    const float x = s * f0 * f1;
+    const float t = s + c, b = t - s;  // two-sum: the low word below half a unit of the high one
+    const float x = t * f0 * f1, y = ((s - (t - b)) + (c - b)) * f0 * f1;
     const int hi = __float2int_rn(x);
-    return make_int2(hi, __float2int_rn(((x - (float)hi) + c * f0 * f1) * 67108864.f));
+    return make_int2(hi, __float2int_rn(((x - (float)hi) + y) * 67108864.f));
   }
 };
 
@@ -558,18 +579,18 @@ __global__ void k_final_batch(const double* __restrict__ part, int gx, double* _
 //    block is done (the sign is the thread's).
 //  - Those of S (RX, RY, inner RZ) are four products a pair.
 //
-// Sums: complex64 products exact as float pairs, a thread's pairs in float
+// Sums: complex64 products and a thread's sums in float
 // pairs (Acc), then 64-bit fixed point; complex128 in FP64 per thread, then
 // two 64-bit words of fixed point.  Every sum is bounded by ||psi|| ||lambda||
 // <= sum_k |c_k|, which sets the point (accumulated integers do not depend on
 // the order of the blocks).
 template <typename R> struct Bwd;
 template <> struct Bwd<float> {
-  static constexpr int KT = 12, C0 = 4, T = 512, LV = 2, VE = 2;
+  static constexpr int KT = 12, C0 = 4, T = 512, OCC = 2, LV = 2, VE = 2;
   using Z = float2;  // a thread's running sum
 };
 template <> struct Bwd<double> {
-  static constexpr int KT = 11, C0 = 3, T = 256, LV = 3, VE = 1;
+  static constexpr int KT = 11, C0 = 3, T = 256, OCC = 2, LV = 3, VE = 1;
   using Z = double;
 };
 constexpr int BWD_SLOTS = TP_MAXOP + TP_MAXK + 3;  // sums of a pass: operators, then tile positions of D
@@ -636,6 +657,26 @@ __device__ __forceinline__ void bwd_zero_sums(BwdSums<R>& S, int nop) {
   for (int i = threadIdx.x; i < words; i += T) reinterpret_cast<unsigned long long*>(S.z)[i] = 0ull;
 }
 
+// The C of complex64 sums of products of a thread's p and l, each component
+// taken once: they stay below |p| |l| < 2^ex.  (At the ends of the range the
+// sums lose the low word, not the high one.)
+constexpr float ACC_TOP = 0x1.8p126f;
+template <typename R>
+__device__ __forceinline__ R acc_point(const Cx<R>* p, const Cx<R>* l) {
+  if constexpr (sizeof(R) == 8) {
+    return 0.0;
+  } else {
+    float a = 0.f, b = 0.f;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      a = fmaxf(a, fmaxf(fabsf(p[j].re), fabsf(p[j].im)));
+      b = fmaxf(b, fmaxf(fabsf(l[j].re), fabsf(l[j].im)));
+    }
+    const int ex = (__float_as_int(a * b) >> 23) + 1 + 4 + 1;
+    return __int_as_float((min(ex, 253) << 23) | 0x400000);
+  }
+}
+
 // kq: the fixed point of complex64 sums (k_prep adds each operator's own part)
 template <typename R>
 __device__ __forceinline__ void bwd_rounds(const TilePass& P, typename CT<R>::V2* sp, typename CT<R>::V2* sl,
@@ -662,26 +703,31 @@ __device__ __forceinline__ void bwd_rounds(const TilePass& P, typename CT<R>::V2
       for (int j = 0; j < NA; ++j) p[j] = l[j] = cmake<R>((R)0, (R)0);
     }
     if (r == 0 && P.has_diag) {
-      Acc<R> w[NA], z[RB];
+      const R C = acc_point<R>(p, l);
+      Acc<R> z[RB], s[RB], w;  // s: the sum of the lower half of each bit's block
 #pragma unroll
       for (int j = 0; j < NA; ++j) {
-        w[j].add(l[j].re, p[j].im);
-        w[j].sub(l[j].im, p[j].re);
-      }
+        w = Acc<R>();
+        w.start(C);
+        w.add(l[j].re, p[j].im);
+        w.sub(l[j].im, p[j].re);
+        w.settle(C);
 #pragma unroll
-      for (int x = 0; x < RB; ++x) {
-#pragma unroll
-        for (int j = 0; j < (NA >> (x + 1)); ++j) {  // bit x: w[2j] - w[2j+1], then the sum for the next bits
-          z[x].merge(w[2 * j]);
-          z[x].merge_neg(w[2 * j + 1]);
-          w[j] = w[2 * j];
-          w[j].merge(w[2 * j + 1]);
+        for (int x = 0; x < RB; ++x) {  // bit x: lower half less upper half; their sum goes on to bit x + 1
+          if ((j >> x) & 1) {
+            z[x].merge(s[x]);
+            z[x].merge_neg(w);
+            w.merge(s[x]);
+          } else {
+            s[x] = w;
+            break;
+          }
         }
       }
-      w[0].into(S.z[tid]);
+      w.into(S.z[tid]);
 #pragma unroll
       for (int x = 0; x < RB; ++x) z[x].into(S.z[(1 + x) * T + tid]);
-      S.bad |= !w[0].finite();
+      S.bad |= !w.finite();
     }
     if (r == 0 && (P.has_diag || P.nop)) {
       const auto A = rec->tab[tid & 31], Bw = rec->tab[32 + (tid >> 5)];
@@ -694,17 +740,21 @@ __device__ __forceinline__ void bwd_rounds(const TilePass& P, typename CT<R>::V2
         l[j] = cmul(l[j], f);
       }
     }
+    R C = acc_point<R>(p, l);
 #pragma unroll 1
     for (int k = rd.op0; k < rd.op1; ++k) {
       const OpRec<R> o = rec->op[k];
       Acc<R> acc;
+      acc.start(C);
       switch (P.op[k].bit) {
         case 0: bwd_bit<0>(o, acc, p, l); break;
         case 1: bwd_bit<1>(o, acc, p, l); break;
         default: bwd_bit<2>(o, acc, p, l); break;
       }
+      acc.settle(C);
       S.bad |= !acc.finite();
       if constexpr (sizeof(R) == 4) {
+        C = fminf(2.f * C, ACC_TOP);  // an operator without its factor at most doubles a product
         const long long v = warp_sum(acc.fixed(kq + o.eq));
         long long* y = reinterpret_cast<long long*>(S.y) + (tid >> 5) * P.nop + k;
         if ((tid & 31) == 0) *y += v;
@@ -786,7 +836,7 @@ __device__ __forceinline__ void bwd_flush(const TilePass& P, const PassRec<R>* r
 
 // One pass over the batch: tiles blockIdx.x + gridDim.x i of state blockIdx.y.
 template <typename R>
-__global__ void __launch_bounds__(Bwd<R>::T, 2) k_bwd_tile(typename CT<R>::V2* __restrict__ psi,
+__global__ void __launch_bounds__(Bwd<R>::T, Bwd<R>::OCC) k_bwd_tile(typename CT<R>::V2* __restrict__ psi,
                                                            typename CT<R>::V2* __restrict__ lam, int n, int ntiles,
                                                            const __grid_constant__ TilePass P,
                                                            const PassRec<R>* __restrict__ recs, int kq,
@@ -840,7 +890,7 @@ __global__ void __launch_bounds__(Bwd<R>::T, 2) k_bwd_tile(typename CT<R>::V2* _
 
 // The whole backward sweep of states that fit one tile, one block a state.
 template <typename R>
-__global__ void __launch_bounds__(Bwd<R>::T, 2) k_bwd_whole(const typename CT<R>::V2* __restrict__ psi,
+__global__ void __launch_bounds__(Bwd<R>::T, Bwd<R>::OCC) k_bwd_whole(const typename CT<R>::V2* __restrict__ psi,
                                                             const typename CT<R>::V2* __restrict__ lam, int n,
                                                             const TilePass* __restrict__ passes, int npass,
                                                             const PassRec<R>* __restrict__ recs, int kq,
@@ -950,7 +1000,7 @@ __global__ void __launch_bounds__(ADJ_T) k_apply_h(const typename CT<R>::V2* __r
   const uint32_t N = 1u << n;
   double e = 0.0;
   for (uint64_t c0 = (uint64_t)blockIdx.x * AH_CHUNK; c0 < N; c0 += (uint64_t)gridDim.x * AH_CHUNK) {
-    Acc<R> acc;
+    SumE<R> acc;
     for (uint32_t j0 = (uint32_t)c0 + threadIdx.x; j0 < (uint32_t)min((uint64_t)N, c0 + AH_CHUNK); j0 += AH_UNR * ADJ_T) {
       R ar[AH_UNR], ai[AH_UNR];
 #pragma unroll
