@@ -634,6 +634,7 @@ __global__ void __launch_bounds__(512, 2) k_qft_c128_k(double2* __restrict__ s, 
   const bool tw = P.twiddle != 0;
   ffc* LAD = sm + NE;
   constexpr int kl = lad_levels<double>(K);
+#pragma unroll 1
   for (int a = threadIdx.x; a < lad_entries<double>(K); a += blockDim.x) LAD[a] = LadIO<double>::ld(lad + a);
   const typename A::S sc = A::scale_const(K);
   const int tid = threadIdx.x;
@@ -1246,7 +1247,9 @@ __global__ void __launch_bounds__(BITREV_T) k_bitrev(double2* __restrict__ s, in
   using V2 = double2;
   constexpr int B = BITREV_B, T = BITREV_T, W = 1 << B, WP = W + 1, PER = W * W / T;
   static_assert(PER * T == W * W, "whole tiles per block");
-  __shared__ V2 A[W * WP], Bt[W * WP];
+  extern __shared__ __align__(16) unsigned char smraw[];
+  V2* A = reinterpret_cast<V2*>(smraw);
+  V2* Bt = A + W * WP;
   const int nm = n - 2 * B;
   const uint64_t M = 1ull << nm;
   for (uint64_t m = blockIdx.x; m < M; m += gridDim.x) {
@@ -1289,12 +1292,13 @@ __global__ void __launch_bounds__(BITREV_T) k_bitrev(double2* __restrict__ s, in
 static qc_status bitrev_impl(qc_state* s, bool from_ff) {
   double2* d = reinterpret_cast<double2*>(s->data);
   const int64_t M = (int64_t)1 << (s->n - 2 * BITREV_B);
+  const size_t smem = 2 * sizeof(double2) * ((1 << BITREV_B) * ((1 << BITREV_B) + 1));
   if (from_ff) {
-    const unsigned grid = resident_grid(k_bitrev<true>, BITREV_T, M, 1, 0);
-    k_bitrev<true><<<grid, BITREV_T, 0, s->stream>>>(d, s->n);
+    const unsigned grid = resident_grid(k_bitrev<true>, BITREV_T, M, 1, smem);
+    k_bitrev<true><<<grid, BITREV_T, smem, s->stream>>>(d, s->n);
   } else {
-    const unsigned grid = resident_grid(k_bitrev<false>, BITREV_T, M, 1, 0);
-    k_bitrev<false><<<grid, BITREV_T, 0, s->stream>>>(d, s->n);
+    const unsigned grid = resident_grid(k_bitrev<false>, BITREV_T, M, 1, smem);
+    k_bitrev<false><<<grid, BITREV_T, smem, s->stream>>>(d, s->n);
   }
   return check_launch("bitrev");
 }
