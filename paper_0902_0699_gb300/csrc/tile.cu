@@ -23,7 +23,8 @@
 // the twiddle is V[f] * Omega^{l f}: V is built once per tile from global
 // root tables, Omega^{l f} (l f < 2^{c+k}) comes from a two-level table in
 // shared memory, the ladder phases from a direct table.  The final SWAPs
-// are one in-place blocked bit-reversal pass.
+// are one in-place blocked bit-reversal pass (complex64: with the lowest five
+// levels; a transform of one tile reverses on its store).
 //
 // complex64 tiles compute in FP32.  complex128 tiles compute in double-float
 // (ff.cuh) on the FP32 pipe: the FP64 pipe of GB300 (0.5 Top/s) would
@@ -922,9 +923,8 @@ __global__ void __launch_bounds__(512, 2) k_qft_c64_k(float2* __restrict__ s, ui
 // (m <= rev m) reads the tiles of m and rev m, one level on its loads' way
 // into shared memory and four on the way out, so that the levels cost no pass.
 // 29 qubits: a 13-level lowest group took 2.07 ms and the reversal 1.72;
-// an 8-level group and this kernel take 1.39 and 1.75 (0.73 of the copy
-// bandwidth: rows of 256 bytes), the whole QFT 6.76 -> 5.94 (8.16 with one CTA
-// an SM).  Six or eight blocks an SM run alike, ten are slower (1.87).
+// an 8-level group and this kernel take 1.39 each (0.91 of the copy
+// bandwidth), the whole QFT 6.76 -> 5.60 (8.16 with one CTA an SM).
 constexpr int QFTR_B = 5;
 constexpr int QFTR_T = 128;
 __global__ void __launch_bounds__(QFTR_T, 8) k_qft_rev_c64(float2* __restrict__ s, int n, const float2* __restrict__ lad) {
@@ -1226,8 +1226,8 @@ qc_status launch_hall(qc_state* s) {
 // shared memory (rows of 2^B contiguous amplitudes, padded against bank
 // conflicts).  The pass is latency bound (load both tiles, synchronise,
 // store), so many small blocks beat few large ones: B = 4
-// with 128 threads (twelve blocks per SM; 0.76 of copy bandwidth on GB300
-// at 30 qubits, against 0.63 for B = 5 with 256 threads).  complex128 states of
+// with 128 threads (twelve blocks per SM; 0.89 of copy bandwidth on GB300
+// at 30 qubits).  complex128 states of
 // more than one group only: a single tile reverses on its store.
 template <bool FF>
 __device__ __forceinline__ double2 bitrev_out(double2 v) {
@@ -1289,15 +1289,23 @@ __global__ void __launch_bounds__(BITREV_T) k_bitrev(double2* __restrict__ s, in
   }
 }
 
+// Blocks of a reversal over M middle values.  A block takes m = blockIdx +
+// i grid and skips m > rev m; with an even grid its m keep their low bit, so
+// that (rev m having it on top) the odd blocks skipped a quarter of theirs and
+// the even ones three quarters, which left half of the SMs idle half of the
+// time.  An odd grid: 30 complex128 qubits 6.81 -> 5.65 ms (0.89 of the copy
+// bandwidth), 29 complex64 1.74 -> 1.39 ms (0.91).
+static unsigned odd_grid(unsigned grid, int64_t M) { return grid < M ? (grid - 1) | 1 : grid; }
+
 static qc_status bitrev_impl(qc_state* s, bool from_ff) {
   double2* d = reinterpret_cast<double2*>(s->data);
   const int64_t M = (int64_t)1 << (s->n - 2 * BITREV_B);
   const size_t smem = 2 * sizeof(double2) * ((1 << BITREV_B) * ((1 << BITREV_B) + 1));
   if (from_ff) {
-    const unsigned grid = resident_grid(k_bitrev<true>, BITREV_T, M, 1, smem);
+    const unsigned grid = odd_grid(resident_grid(k_bitrev<true>, BITREV_T, M, 1, smem), M);
     k_bitrev<true><<<grid, BITREV_T, smem, s->stream>>>(d, s->n);
   } else {
-    const unsigned grid = resident_grid(k_bitrev<false>, BITREV_T, M, 1, smem);
+    const unsigned grid = odd_grid(resident_grid(k_bitrev<false>, BITREV_T, M, 1, smem), M);
     k_bitrev<false><<<grid, BITREV_T, smem, s->stream>>>(d, s->n);
   }
   return check_launch("bitrev");
@@ -1384,8 +1392,8 @@ static qc_status qft_c64(qc_state* s) {
   for (int gi = G.np - 1; gi >= 0 && !st; --gi)
     st = run_qft_c64(s, groups[gi], lad + QFT_LAD + ((size_t)gi << 13), lad);
   if (!st) {
-    const uint64_t M = 1ull << (s->n - 2 * QFTR_B);
-    const unsigned grid = resident_grid(k_qft_rev_c64, QFTR_T, (int64_t)M, 1, 0);
+    const int64_t M = (int64_t)1 << (s->n - 2 * QFTR_B);
+    const unsigned grid = odd_grid(resident_grid(k_qft_rev_c64, QFTR_T, M, 1, 0), M);
     k_qft_rev_c64<<<grid, QFTR_T, 0, s->stream>>>(reinterpret_cast<float2*>(s->data), s->n, lad);
     st = check_launch("qft bit reversal");
   }
