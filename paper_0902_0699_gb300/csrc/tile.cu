@@ -1452,7 +1452,8 @@ qc_status launch_qft(qc_state* s) {
 
 // ---------------------------------------------------- register QFT -------
 // Reversal of the bits [lo, lo + w) of every index, in place: amplitude rows
-// of 2^lo swap (runs of 2^lo amplitudes stream).
+// of 2^lo swap (runs of 2^lo amplitudes stream).  An odd grid, as above: 17
+// bits of a 26-qubit complex128 state 486 -> 423 us.
 template <typename V2>
 __global__ void __launch_bounds__(256) k_reg_rev(V2* __restrict__ s, uint64_t N, int lo, int w) {
   const uint64_t mask = (1ull << w) - 1ull;
@@ -1705,8 +1706,8 @@ static qc_status qft_range_impl(qc_state* s, int lo, int w) {
   }
   if (!st && plan.groups.size() > 1) {
     const uint64_t N = 1ull << s->n;
-    k_reg_rev<V2><<<resident_grid(k_reg_rev<V2>, 256, (int64_t)N, 256), 256, 0, s->stream>>>(
-        reinterpret_cast<V2*>(s->data), N, lo, w);
+    const unsigned grid = odd_grid(resident_grid(k_reg_rev<V2>, 256, (int64_t)N, 256), ((int64_t)N + 255) / 256);
+    k_reg_rev<V2><<<grid, 256, 0, s->stream>>>(reinterpret_cast<V2*>(s->data), N, lo, w);
     st = check_launch("register reversal");
   }
   cudaFreeAsync(tab.tlo, s->stream);
