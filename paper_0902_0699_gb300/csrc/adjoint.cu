@@ -358,11 +358,11 @@ __device__ __forceinline__ V2* sm_at(V2* sm, int byte) {
 // The register rounds of a pass on the tile in `sm`, each closed by a barrier.
 template <typename R> struct Fwd;
 template <> struct Fwd<float> {
-  static constexpr int RB = 4, VE = 2;
+  static constexpr int KT = 13, C0 = 4, RB = 4, VE = 2;
   using Ops = Mat2<float>;
 };
 template <> struct Fwd<double> {
-  static constexpr int RB = 3, VE = 1;
+  static constexpr int KT = 12, C0 = 3, RB = 3, VE = 1;
   using Ops = PassRec<double>;
 };
 
@@ -1108,7 +1108,7 @@ struct FwdPlan {
 
 template <typename R>
 static cudaError_t fwd_plan(FwdPlan<R>& F, const qc_gate* gates, int ng, int n, int B, cudaStream_t st) {
-  const PassCfg cfg = sizeof(R) == 4 ? PassCfg{13, 4, 4, true, false} : PassCfg{12, 3, 3, false, false};
+  const PassCfg cfg{Fwd<R>::KT, Fwd<R>::C0, Fwd<R>::RB, sizeof(R) == 4, false};
   F.passes = build_passes<R>(gates, ng, n, cfg);
   if (F.passes.empty()) return cudaSuccess;
   const size_t per = F.passes.size() * F.nrec * sizeof(typename Fwd<R>::Ops);
@@ -1123,11 +1123,6 @@ static void fwd_plan_free(FwdPlan<R>& F, cudaStream_t st) {
   if (F.recs) cudaFreeAsync(F.recs, st);
 }
 
-template <typename K>
-static void allow_smem(K kernel, size_t bytes) {
-  cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 // psi_b = U_G .. U_1 |0..0>; returns the launches made.
 template <typename R>
 static int forward_passes(const FwdPlan<R>& F, int n, int B, const double* theta, int64_t stride,
@@ -1139,9 +1134,10 @@ static int forward_passes(const FwdPlan<R>& F, int n, int B, const double* theta
   const int np = (int)F.passes.size();
   int nk = put_bytes(F.dpass, F.passes.data(), np * sizeof(TilePass), st);
   const int kt = F.passes[0].kt, T = std::max(32, 1 << (kt - Fwd<R>::RB));
-  const size_t smem = (sizeof(typename CT<R>::V2) << kt) + sizeof(typename Fwd<R>::Ops) * F.nrec;
-  allow_smem(k_fwd_tile<R>, smem);
-  allow_smem(k_fwd_whole<R>, smem);
+  const size_t ops = sizeof(typename Fwd<R>::Ops) * F.nrec, smem = (sizeof(typename CT<R>::V2) << kt) + ops;
+  constexpr size_t most = sizeof(typename CT<R>::V2) << Fwd<R>::KT;
+  allow_smem(k_fwd_tile<R>, most + ops);
+  allow_smem(k_fwd_whole<R>, most + ops);
   for (int b0 = 0; b0 < B; b0 += F.chunk) {
     const int nb = std::min(F.chunk, B - b0);
     const double* th = theta + (int64_t)b0 * stride;
@@ -1216,8 +1212,10 @@ static int backward_passes(const BwdPlan<R>& W, int n, int B, const double* thet
   for (const TilePass& P : W.passes) maxop = std::max<int>(maxop, P.nop);
   const int kt = W.passes[0].kt, T = std::max(32, 1 << (kt - 3));
   const size_t tiles2 = 2 * (sizeof(typename CT<R>::V2) << kt) + sizeof(PassRec<R>);
-  allow_smem(k_bwd_tile<R>, tiles2 + bwd_sum_bytes<R>(T, maxop));
-  allow_smem(k_bwd_whole<R>, tiles2 + bwd_sum_bytes<R>(T, maxop));
+  const size_t most = 2 * (sizeof(typename CT<R>::V2) << Bwd<R>::KT) + sizeof(PassRec<R>) +
+                      bwd_sum_bytes<R>(Bwd<R>::T, TP_MAXOP);
+  allow_smem(k_bwd_tile<R>, most);
+  allow_smem(k_bwd_whole<R>, most);
   for (int b0 = 0; b0 < B; b0 += W.chunk) {
     const int nb = std::min(W.chunk, B - b0);
     const double* th = theta + (int64_t)b0 * stride;

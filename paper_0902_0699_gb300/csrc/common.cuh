@@ -80,6 +80,16 @@ inline unsigned resident_grid(K kernel, int threads, int64_t items, int per_bloc
   return (unsigned)b;
 }
 
+// Lets `kernel` be launched with up to `bytes` of dynamic shared memory on the
+// current device.  The limit belongs to the function on the device, for every
+// host thread: callers pass the most the kernel ever needs, it is set once per
+// kernel and device and never lowered, and the call returns when it is set.
+cudaError_t allow_smem_bytes(const void* kernel, size_t bytes);
+template <typename K>
+inline cudaError_t allow_smem(K kernel, size_t bytes) {
+  return allow_smem_bytes((const void*)kernel, bytes);
+}
+
 // Stream-ordered workspace (free with cudaFreeAsync on the same stream), from a
 // memory pool of the library's own per device that keeps up to WS_KEEP bytes
 // between calls: the device's default pool gives its memory back at every

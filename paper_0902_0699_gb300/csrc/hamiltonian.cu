@@ -318,13 +318,16 @@ static qc_status run_hstep(qc_state* s, const std::vector<HTermHost>& terms) {
     k_hdiag<R><<<dim3(std::max(1, (1 << kt) / 128), npass), 128, 0, s->stream>>>(dp, dd, di, tab);
   }
   const size_t smem = sizeof(typename HT<R>::E) << kt;
-  cudaFuncSetAttribute(k_hstep<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  allow_smem(k_hstep<R>, sizeof(typename HT<R>::E) << HS_KT);
   const int T = std::max(32, (1 << kt) / HS_PER), ntiles = 1 << (n - kt);
   const unsigned grid = resident_grid(k_hstep<R>, T, ntiles, 1, smem);
-  for (int p = 0; p < npass; ++p, ++nk)
+  // a pass is launched only after the ones before it were: the last adds what they left in the workspace to psi
+  qc_status st = check_launch("Hamiltonian step setup", nk);
+  for (int p = 0; p < npass && !st; ++p) {
     k_hstep<R><<<grid, T, smem, s->stream>>>(reinterpret_cast<V*>(s->data), acc, ntiles, passes[p], df + ffirst[p],
                                              tab + ((size_t)p << HS_KT));
-  const qc_status st = check_launch("Hamiltonian step", nk);
+    st = check_launch("Hamiltonian step");
+  }
   cudaFreeAsync(w, s->stream);
   s->sum_valid = false;
   return st;

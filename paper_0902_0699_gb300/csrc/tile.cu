@@ -30,7 +30,6 @@
 // (ff.cuh) on the FP32 pipe: the FP64 pipe of GB300 (0.5 Top/s) would
 // otherwise bound every pass many times over the memory time.
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <vector>
 
@@ -1066,11 +1065,7 @@ static qc_status run_tile(qc_state* s, TileProg<R>& P, const typename CT<R>::V2*
   const uint64_t ntiles = 1ull << (s->n - tb);
   const size_t smem = tile_smem<R>(P.k, P.c, P.twiddle != 0, P.qft != 0);
   const int threads = std::max(64, std::min(512, (1 << tb) >> 2));  // four amplitudes a thread
-  static bool attr_set = false;
-  if (!attr_set) {
-    cudaFuncSetAttribute(k_tile<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-    attr_set = true;
-  }
+  allow_smem(k_tile<R>, 200 * 1024);
   const unsigned grid = resident_grid(k_tile<R>, threads, (int64_t)ntiles, 1, smem);
   k_tile<R><<<grid, threads, smem, s->stream>>>(reinterpret_cast<V2*>(s->data), ntiles, P, tlo, thi, lad);
   return check_launch("tile pass");
@@ -1094,11 +1089,7 @@ static qc_status run_qft_c128(qc_state* s, TileProg<double>& P, const double2* t
     switch (P.k) {
 #define QC_QFT_C128(KK)                                                                             \
   case KK: {                                                                                        \
-    static bool a = false;                                                                          \
-    if (!a) {                                                                                       \
-      cudaFuncSetAttribute(k_qft_c128_k<KK>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024); \
-      a = true;                                                                                     \
-    }                                                                                               \
+    allow_smem(k_qft_c128_k<KK>, 200 * 1024);                                                       \
     const unsigned g = resident_grid(k_qft_c128_k<KK>, 512, (int64_t)ntiles, 1, smem);             \
     k_qft_c128_k<KK><<<g, 512, smem, s->stream>>>(d, ntiles, P, tlo, thi, lad, ld_ff, st_ff);       \
     return check_launch("qft pass");                                                                \
@@ -1120,11 +1111,7 @@ static qc_status run_qft_c64(qc_state* s, const Group& g, const float2* W, const
 #define QC_QFT_C64(KK)                                                                                  \
   case KK: {                                                                                            \
     const size_t smem = sizeof(float2) * ((1 << 13) + 2 * (1 << KK));                                   \
-    static bool a = false;                                                                              \
-    if (!a) {                                                                                           \
-      cudaFuncSetAttribute(k_qft_c64_k<KK>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);    \
-      a = true;                                                                                         \
-    }                                                                                                   \
+    allow_smem(k_qft_c64_k<KK>, smem);                                                                  \
     const unsigned grid = resident_grid(k_qft_c64_k<KK>, 512, ntiles, 1, smem);                         \
     k_qft_c64_k<KK><<<grid, 512, smem, s->stream>>>(reinterpret_cast<float2*>(s->data), (uint64_t)ntiles, g.lo, W, lad); \
     return check_launch("qft pass");                                                                    \
@@ -1676,9 +1663,7 @@ static qc_status qft_range_impl(qc_state* s, int lo, int w) {
       RqftProg P{g.lo, g.k, c, lo, w, nl, g.lo > lo, plan.groups.size() == 1, 6521908912666391106ll};
       const size_t NE = (size_t)1 << (g.k + c);
       const size_t smem = sizeof(longlong2) * (NE + ((size_t)1 << g.k) - 1 + (P.twiddle && lo >= c ? (size_t)1 << g.k : 0));
-      static std::atomic<bool> attr{false};
-      if (!attr.exchange(true))
-        cudaFuncSetAttribute(k_rqft_c128, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+      allow_smem(k_rqft_c128, 200 * 1024);
       const int T = std::max(32, (int)(NE / 8));
       const uint64_t ntiles = (1ull << s->n) / NE;
       k_rqft_c128<<<resident_grid(k_rqft_c128, T, (int64_t)ntiles, 1, smem), T, smem, s->stream>>>(
