@@ -22,6 +22,7 @@
 
 #include "circuit_passes.cuh"
 #include "common.cuh"
+#include "fixpt.cuh"
 
 namespace qc {
 
@@ -776,10 +777,12 @@ __device__ __forceinline__ void bwd_rounds(const TilePass& P, typename CT<R>::V2
 
 // acc[2 slot + word] of one batch element; a non-finite sum sets the flag.
 __device__ __forceinline__ void bwd_add(unsigned long long* acc, int slot, double v, int k) {
-  const double x = scale2(v, k), hi = rint(x);
+  const double x = scale2(v, k);
   if (!isfinite(x)) return;
-  atomicAdd(acc + 2 * slot, (unsigned long long)(long long)hi);
-  atomicAdd(acc + 2 * slot + 1, (unsigned long long)__double2ll_rn((x - hi) * 4503599627370496.0));
+  long long hi, lo;
+  fx_split(x, hi, lo);
+  atomicAdd(acc + 2 * slot, (unsigned long long)hi);
+  atomicAdd(acc + 2 * slot + 1, (unsigned long long)lo);
 }
 template <typename R>
 __device__ __forceinline__ void bwd_flush(const TilePass& P, const PassRec<R>* rec, BwdSums<R>& S, int kq,
@@ -963,7 +966,7 @@ __global__ void __launch_bounds__(64) k_bwd_finish(const TilePass* __restrict__ 
     if (par < 0) continue;  // H
     const OpRec<R>* o = op ? &recs[pb].op[slot] : nullptr;
     const unsigned long long* a = acc + (pb * BWD_SLOTS + slot) * 2;
-    double v = (double)(long long)a[0] + (double)(long long)a[1] * 2.220446049250313e-16;
+    double v = fx_join((long long)a[0], (long long)a[1]);
     v = scale2(v, -(kq + (op ? o->eq : 0)));
     if (op) v *= o->f;
     if (flag[blockIdx.y]) v = __longlong_as_double(0x7ff8000000000000ll);

@@ -3,7 +3,29 @@
 // instruction is issued.
 #pragma once
 
+#include <math.h>
+
+#ifdef __CUDACC__
+#define FX_HD __host__ __device__ __forceinline__
+#else
+#define FX_HD inline
+#endif
+
 namespace qc {
+
+// One of many terms of a sum that is kept in two 64-bit integers:
+// x = hi + lo 2^-FX_LOW to half a unit of lo.  |lo| <= 2^(FX_LOW - 1), so the
+// low words of 2^27 terms add up without overflow, whatever their fractions
+// (2^52 for 2^-FX_LOW would leave room for 2^12 equal ones).
+constexpr int FX_LOW = 36;
+FX_HD void fx_split(double x, long long& hi, long long& lo) {
+  const double r = rint(x);
+  hi = (long long)r;
+  lo = (long long)rint((x - r) * (double)(1ll << FX_LOW));
+}
+FX_HD double fx_join(long long hi, long long lo) { return (double)hi + (double)lo * (1.0 / (double)(1ll << FX_LOW)); }
+
+#ifdef __CUDACC__
 
 // binary64 -> fixed point round(x 2^(1075 - G)) for a tile's G,
 // rounding half away from zero (symmetric, so unbiased; exact
@@ -42,5 +64,7 @@ __device__ __forceinline__ double fix2d(long long v, int F) {
   if (e >= 2047) return __longlong_as_double((long long)(sgn | (0x7FFull << 52)));
   return __longlong_as_double((long long)(sgn | ((unsigned long long)e << 52) | (keep & 0xFFFFFFFFFFFFFull)));
 }
+
+#endif  // __CUDACC__
 
 }  // namespace qc
