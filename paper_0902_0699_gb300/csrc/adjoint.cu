@@ -12,9 +12,10 @@
 // -- and U_j^dagger is applied to both.  No intermediate state is stored: psi
 // is uncomputed instead of checkpointed.
 //
-// Accumulation is FP64: complex128 with FMA in double; complex64 products
-// are formed exactly with the FP32 two-product and summed as float pairs
-// over short runs before they are added in double.
+// Accumulation: complex128 with FMA in double.  complex64: the energy's
+// products are exact float pairs (two-product), summed as float pairs over
+// short runs and then in double; a derivative's products are summed in float
+// pairs with a common high binade (Acc) and then in 64-bit fixed point.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -111,7 +112,9 @@ template <> struct Acc<double> {
 // product; a two-product and a two-sum take ten (20 qubits, 64 states: the
 // backward passes 28.5 -> 24.9 ms; what is left waits: issue slots 0.53
 // busy, barriers, shared memory and the tile's loads in turn).
-// Error: 2^-24 units a term, a unit being 2^-16 of the largest product at most.
+// Error: 2^-24 units a term, a unit being at most 2^-16 of the product of the
+// thread's largest |p| and |l| where C was set, and at most 2^-13 of it up to
+// ACC_SPAN operators later.
 template <> struct Acc<float> {
   float s = 0.f, c = 0.f;
   __device__ void start(float C) { s = C; }
@@ -662,6 +665,11 @@ __device__ __forceinline__ void bwd_zero_sums(BwdSums<R>& S, int nop) {
 // taken once: they stay below |p| |l| < 2^ex.  (At the ends of the range the
 // sums lose the low word, not the high one.)
 constexpr float ACC_TOP = 0x1.8p126f;
+// Operators of a round between two looks at the amplitudes: C doubles with
+// every operator, since one without its factor can double a product, but most
+// do not, and after some seventeen the high word would hold nothing of a
+// product.  Rounds of up to four operators (an ansatz's have three) look once.
+constexpr int ACC_SPAN = 4;
 template <typename R>
 __device__ __forceinline__ R acc_point(const Cx<R>* p, const Cx<R>* l) {
   if constexpr (sizeof(R) == 8) {
@@ -741,9 +749,10 @@ __device__ __forceinline__ void bwd_rounds(const TilePass& P, typename CT<R>::V2
         l[j] = cmul(l[j], f);
       }
     }
-    R C = acc_point<R>(p, l);
+    R C = 0;
 #pragma unroll 1
     for (int k = rd.op0; k < rd.op1; ++k) {
+      if ((k - rd.op0) % ACC_SPAN == 0) C = acc_point<R>(p, l);
       const OpRec<R> o = rec->op[k];
       Acc<R> acc;
       acc.start(C);
