@@ -341,7 +341,7 @@ FF_HD void ffacc_add(ffacc& A, ff a, ff b) {
 }
 // moves t into s (fast two-sum; |t| stays far below |s| between calls), so
 // that t's own roundings stay at 2^-24 of a few units of s.  Called after
-// every fourth term, the error of up to 64 terms stays below 2^-44 of
+// every fourth term, the error of up to 200 terms stays below 2^-44 of
 // sum |a_i b_i| (mostly the operands' own splitting error); without it the
 // low word's roundings grow with the square of the number of terms.
 FF_HD void ffacc_norm(ffacc& A) {

@@ -186,7 +186,9 @@ __global__ void __launch_bounds__(512, 2) k_hstep(typename HT<R>::V* __restrict_
             S[u].mac(re, im, f.c[((e >> sa) & 1) | ((e >> sb) & 1) << 1],
                      *reinterpret_cast<const E*>(sm + (a_of(h + u) ^ off)));
         }
-        if ((k & 1) && sizeof(R) == 8) {  // at most four products since the last
+        // at most four products since the last, and a complex diagonal's two
+        // before the first (a pass's up to 194 then stay within ff.cuh's bound)
+        if ((k & 1) && sizeof(R) == 8) {
 #pragma unroll
           for (int u = 0; u < 4; ++u) S[u].norm();
         }
