@@ -529,11 +529,14 @@ qc_status qc_wigner_d(int twoj, double alpha, double beta, double gamma, double*
  * tensor cores (a real GEMM of 128 x 32 tiles over K = 2B).  complex64: bf16
  * digit slices with exact leading sums, FP32-class accuracy; the call
  * synchronises the stream to read a status word (QC_ETIMEOUT if a device wait
- * gave up).  complex128: seven exact integer digits, rounded once to binary64;
- * stream-ordered (a tile whose device wait gave up is NaN).  B > 64 (or, for
- * complex128, no room for the operand workspace of about 11 * 2^n * B * 4
- * bytes) is stream-ordered on CUDA cores (complex128 inner products in
- * double-float). */
+ * gave up).  complex128: seven exact integer digits, rounded once to binary64,
+ * with an error of about 2^-52.3 sqrt(2 B) of the product of the two rows'
+ * largest magnitudes; entries whose terms are so much smaller that double-float
+ * products (2^-47.6 of sum_a P_a |C_a(n)| |C_a(n')|) are closer, and tiles whose
+ * device wait gave up, are taken on the CUDA cores; stream-ordered.  B > 64 (or,
+ * for complex128, no room for the operand workspace of 84 * 2^n * B bytes, B
+ * rounded up to a multiple of 8, and 26 * 2^n bytes, 2^n at least 128) is
+ * stream-ordered on CUDA cores (complex128 inner products in double-float). */
 qc_status qc_density_matrix(const void* psi_dev, int n, qc_dtype dt, int B, const double* P_host,
                             void* rho_dev, void* stream);
 

@@ -390,6 +390,10 @@ qc_status rho_tc_c64(const float2* psi, int n, int B, const double* P_host, floa
 // The same for complex128 (rho_tc128.cu); stream-ordered.  QC_ENOMEM (without a
 // message): its workspace does not fit, nothing was launched.
 qc_status rho_tc_c128(const double2* psi, int n, int B, const double* P_host, double2* rho, cudaStream_t s);
+// Then: its entries that double-float products give better, and the blocks a
+// CTA gave up (redo), on the CUDA cores (density.cu); returns the launches made.
+int launch_rho_fix(const double2* psi, int n, int B, const double* P, const int16_t* E, const ulonglong3* Big,
+                   const unsigned char* redo, double2* rho, cudaStream_t s);
 
 qc_status dense_launch(qc_state* s, const DenseMap& M, const void* dev_op, int* status,
                        uint32_t spin_limit = QC_TC_SPIN_LIMIT, int no_mma = 0);

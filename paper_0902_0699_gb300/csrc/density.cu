@@ -41,6 +41,7 @@ __device__ __forceinline__ ffc load_ffc(const float2* p, uint64_t i) {
 }
 template <typename V2> __device__ __forceinline__ V2 ffc_to_v2(const ffc& z);
 template <> __device__ __forceinline__ double2 ffc_to_v2<double2>(const ffc& z) {
+  if (!isfinite(z.re.hi) || !isfinite(z.im.hi)) return make_double2(NAN, NAN);  // the join would make it finite
   return make_double2(ff_to_d(z.re), ff_to_d(z.im));
 }
 template <> __device__ __forceinline__ float2 ffc_to_v2<float2>(const ffc& z) {
@@ -70,6 +71,52 @@ __device__ __forceinline__ void mac_conj_b(ffc& acc, const ffc& a, const ffc& b)
 // ------------------------------------------------------------- rho -------
 #define RHO_TILE 32
 #define RHO_KC 16
+
+// A thread's 2 x 2 entries of the 32 x 32 tile (rows r0 + 2 ty + i, columns
+// c0 + 2 tx + j) in double-float.  SIZES: also the sums of the terms' sizes
+// (|re| + |im| of each factor).
+template <bool SIZES>
+__device__ __forceinline__ void rho_tile_c128(const double2* __restrict__ psi, uint64_t N, int B,
+                                              const double* __restrict__ P, uint64_t r0, uint64_t c0,
+                                              ffc (*Ar)[RHO_TILE], ffc (*Ac)[RHO_TILE], ffc (*acc)[2],
+                                              float (*size)[2]) {
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  for (int i = 0; i < 2; ++i)
+    for (int j = 0; j < 2; ++j) {
+      acc[i][j] = ffc_make(ff_make(0.f, 0.f), ff_make(0.f, 0.f));
+      if (SIZES) size[i][j] = 0.f;
+    }
+  for (int a0 = 0; a0 < B; a0 += RHO_KC) {
+    const int kc = min(RHO_KC, B - a0);
+    for (int e = threadIdx.x; e < kc * RHO_TILE; e += blockDim.x) {
+      const int k = e / RHO_TILE, x = e % RHO_TILE;
+      const int a = a0 + k;
+      ffc vr = ffc_make(ff_make(0.f, 0.f), ff_make(0.f, 0.f)), vc = vr;
+      const ff w = ff_from_d(P[a]);
+      if (r0 + x < N) {
+        vr = load_ffc(psi, (uint64_t)a * N + r0 + x);
+        vr = ffc_make(ff_mul(vr.re, w), ff_mul(vr.im, w));
+      }
+      if (c0 + x < N) vc = load_ffc(psi, (uint64_t)a * N + c0 + x);
+      Ar[k][x] = vr;
+      Ac[k][x] = vc;
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int k = 0; k < kc; ++k) {
+      const ffc r[2] = {Ar[k][2 * ty], Ar[k][2 * ty + 1]}, c[2] = {Ac[k][2 * tx], Ac[k][2 * tx + 1]};
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          mac_conj_b(acc[i][j], r[i], c[j]);
+          if (SIZES)
+            size[i][j] = fmaf(fabsf(r[i].re.hi) + fabsf(r[i].im.hi), fabsf(c[j].re.hi) + fabsf(c[j].im.hi), size[i][j]);
+        }
+    }
+    __syncthreads();
+  }
+}
 
 // One CTA: a 32 x 32 tile of rho (rows r0.., columns c0..); each of the 256
 // threads owns 2 x 2 entries.  The weights P_a scale the row operands.
@@ -124,35 +171,7 @@ __global__ void __launch_bounds__(256) k_rho(const V2* __restrict__ psi, uint64_
     if (mirror) rho_mirror<V2>(Tm, rho, N, r0, c0);
   } else {
   ffc acc[2][2];
-  for (int i = 0; i < 2; ++i)
-    for (int j = 0; j < 2; ++j) acc[i][j] = ffc_make(ff_make(0.f, 0.f), ff_make(0.f, 0.f));
-  for (int a0 = 0; a0 < B; a0 += RHO_KC) {
-    for (int e = threadIdx.x; e < RHO_KC * RHO_TILE; e += blockDim.x) {
-      const int k = e / RHO_TILE, x = e % RHO_TILE;
-      const int a = a0 + k;
-      ffc vr = ffc_make(ff_make(0.f, 0.f), ff_make(0.f, 0.f)), vc = vr;
-      if (a < B) {
-        const ff w = ff_from_d(P[a]);
-        if (r0 + x < N) {
-          vr = load_ffc(psi, (uint64_t)a * N + r0 + x);
-          vr = ffc_make(ff_mul(vr.re, w), ff_mul(vr.im, w));
-        }
-        if (c0 + x < N) vc = load_ffc(psi, (uint64_t)a * N + c0 + x);
-      }
-      Ar[k][x] = vr;
-      Ac[k][x] = vc;
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int k = 0; k < RHO_KC; ++k) {
-      const ffc ra = Ar[k][2 * ty], rb = Ar[k][2 * ty + 1], ca = Ac[k][2 * tx], cb = Ac[k][2 * tx + 1];
-      mac_conj_b(acc[0][0], ra, ca);
-      mac_conj_b(acc[0][1], ra, cb);
-      mac_conj_b(acc[1][0], rb, ca);
-      mac_conj_b(acc[1][1], rb, cb);
-    }
-    __syncthreads();
-  }
+  rho_tile_c128<false>(psi, N, B, P, r0, c0, Ar, Ac, acc, nullptr);
   for (int i = 0; i < 2; ++i)
     for (int j = 0; j < 2; ++j) {
       const uint64_t r = r0 + 2 * ty + i, c = c0 + 2 * tx + j;
@@ -162,6 +181,176 @@ __global__ void __launch_bounds__(256) k_rho(const V2* __restrict__ psi, uint64_
     }
   if (mirror) rho_mirror<V2>(Tm, rho, N, r0, c0);
   }
+}
+
+// Entries of the digit products (rho_tc128.cu) that double-float products give
+// better, replaced by those; a CTA (or four, or sixteen, for few blocks) per
+// 128 x 128 block on or above the diagonal (the lower triangle gets the
+// conjugates).
+//
+// The digits' error is about 2^-52.3 sqrt(2 B) of the product of the rows'
+// scales 2^(E - 1023), that of the double-float products 2^-47.6 of the terms'
+// own sizes (both from sums of random rows against exact ones) and 2^-98 a
+// factor.  So an entry is replaced if its terms come to less than
+// sqrt(2 B) / 26 of the scales' product.  Which entries may be such:
+//  - Up to RHO_EXACT states: the terms' sizes are summed for every entry.
+//  - More states: a state that is at least a quarter (an eighth) of the scale in
+//    both rows has a term of 1/16 (1/64) of it or more, so K16 =
+//    ceil(16 sqrt(2 B) / 26) (K64 likewise) of those rule an entry out, and so
+//    does having no state in common, which makes it exactly zero.  Two rows of
+//    c1 and c2 such states share at least c1 + c2 - B: for some thirty states
+//    and more of an ordinary ensemble the block's smallest counts decide without
+//    a look at its pairs.
+// A 32 x 32 tile with few such entries takes them one by one (a thread an
+// entry, amplitudes from L2), one with more is formed whole as k_rho does.
+// 13 qubits, the call without and with it: ordinary batches of 64 states 829 ->
+// 837 us, of 2 states 410 -> 450 (no entry is replaced, bound by the sums);
+// states that are each large on amplitudes of their own and 1e-9 elsewhere: 64
+// 6.1 ms, 2 0.93 ms (k_rho alone 4.64 ms).
+// |x| to 2^-20, without an FP64 instruction (0 below FP32's range, infinite above)
+__device__ __forceinline__ float mag_f(double x) {
+  const int h = __double2hiint(x) & 0x7fffffff;
+  return h < (897 << 20) ? 0.f : h >= (1151 << 20) ? INFINITY : __int_as_float((h - (896 << 20)) << 3);
+}
+#define RHO_FEW 96
+#define RHO_EXACT 16
+#define RHO_MS (RHO_EXACT + 4)  // padded: 16-byte loads of 32 rows hit every bank
+__global__ void __launch_bounds__(256) k_rho_fix(const double2* __restrict__ psi, uint64_t N, int B,
+                                                 const double* __restrict__ P, const int16_t* __restrict__ E,
+                                                 const ulonglong3* __restrict__ Big, int K16, int K64, float lim,
+                                                 const unsigned char* __restrict__ redo, double2* __restrict__ rho) {
+  if (blockIdx.x < blockIdx.y) return;
+  __shared__ union {
+    ulonglong3 mask[2][128];
+    float size[2][128][RHO_MS];  // |re| + |im| of a row's amplitudes, of its scale
+  } M;
+  __shared__ float scale[2][128];  // of the rows; 0: none of its entries is replaced
+  __shared__ float wt[RHO_EXACT];
+  __shared__ int least[2], count[16];
+  __shared__ ffc Ar[RHO_KC][RHO_TILE], Ac[RHO_KC][RHO_TILE];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, tx = tid & 15, ty = tid >> 4;
+  const bool all = redo[blockIdx.y * gridDim.x + blockIdx.x] != 0, exact = B <= RHO_EXACT;
+  const int nh = (B + 3) / 4;
+  const uint64_t R0 = (uint64_t)blockIdx.y * 128, C0 = (uint64_t)blockIdx.x * 128;
+  const int side = tid >> 7, x = tid & 127;
+  const uint64_t row = (side ? C0 : R0) + x;
+  const int e = E[row] - 1023;
+  // a factor's 2^-98 forbids what lies lower, FP32's range what lies higher
+  const float sc = e >= -50 && e <= 60 ? __int_as_float((e + 127) << 23) : 0.f;
+  scale[side][x] = sc;
+  if (tid < 16) count[tid] = 0;
+  if (exact) {
+    if (tid < RHO_EXACT) wt[tid] = tid < B ? sqrtf((float)P[tid]) : 0.f;
+    __syncthreads();
+    const float inv = sc > 0.f ? 1.f / sc : 0.f;
+#pragma unroll
+    for (int h = 0; h < RHO_EXACT / 4; ++h) {
+      if (h >= nh) break;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        const int a = 4 * h + k;
+        double2 v = make_double2(0.0, 0.0);
+        if (a < B && row < N) v = psi[(uint64_t)a * N + row];
+        M.size[side][x][a] = (mag_f(v.x) + mag_f(v.y)) * (wt[a] * inv);
+      }
+    }
+    __syncthreads();
+  } else {
+    if (tid < 2) least[tid] = 64;
+    __syncthreads();
+    const ulonglong3 mine = Big[row];
+    M.mask[side][x] = mine;
+    const int cnt = __reduce_min_sync(0xffffffffu, mine.z ? __popcll(mine.y) : 64);
+    if (lane == 0) atomicMin(&least[side], cnt);
+    __syncthreads();
+    if (!all && least[0] + least[1] - B >= K64) return;
+  }
+  auto smaller = [&](float size, int r, int c) {
+    const float er = scale[0][r], ec = scale[1][c];
+    return fmaf(0x1p-48f, er + ec, size) < lim * er * ec;
+  };
+  auto put = [&](uint64_t r, uint64_t c, const ffc& z) {
+    // joined in FP64: such an entry may be below 2^-75, where ff_to_d keeps 24 bits
+    const double2 v = make_double2((double)z.re.hi + (double)z.re.lo, (double)z.im.hi + (double)z.im.lo);
+    rho[r * N + c] = r < c || !isfinite(v.x) ? v : make_double2(v.x, 0.0);
+    if (r < c) rho[c * N + r] = make_double2(v.x, -v.y);
+  };
+  for (int t = blockIdx.z; t < 16; t += gridDim.z) {
+    const int rl = 32 * (t >> 2), cl = 32 * (t & 3), c = cl + lane;
+    const uint64_t r0 = R0 + rl, c0 = C0 + cl;
+    if (r0 > c0 || c0 >= N) continue;
+    int hit = 0;  // of this thread's entries (rl + warp + 8 q, c); those past N have no state
+    if (!all) {
+      if (exact) {
+        float4 y[RHO_EXACT / 4];
+#pragma unroll
+        for (int h = 0; h < RHO_EXACT / 4; ++h)
+          if (h < nh) y[h] = *reinterpret_cast<const float4*>(&M.size[1][c][4 * h]);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int r = rl + warp + 8 * q;
+          float z = 0.f;
+#pragma unroll
+          for (int h = 0; h < RHO_EXACT / 4; ++h) {
+            if (h >= nh) break;
+            const float4 w = *reinterpret_cast<const float4*>(&M.size[0][r][4 * h]);
+            z = fmaf(w.x, y[h].x, fmaf(w.y, y[h].y, fmaf(w.z, y[h].z, fmaf(w.w, y[h].w, z))));
+          }
+          hit |= (z > 0.f && z < lim && R0 + r < C0 + c) << q;
+        }
+      } else {
+        const ulonglong3 b = M.mask[1][c];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int r = rl + warp + 8 * q;
+          const ulonglong3 a = M.mask[0][r];
+          hit |= ((a.z & b.z) && __popcll(a.x & b.x) < K16 && __popcll(a.y & b.y) < K64 && R0 + r < C0 + c) << q;
+        }
+      }
+      const int hits = __reduce_add_sync(0xffffffffu, __popc(hit));
+      if (lane == 0 && hits) atomicAdd(&count[t], hits);
+      __syncthreads();
+      if (count[t] == 0) continue;
+    }
+    if (!all && count[t] <= RHO_FEW) {
+      for (int q = 0; q < 4; ++q) {
+        if (!((hit >> q) & 1)) continue;
+        const int r = rl + warp + 8 * q;
+        ffc z = ffc_make(ff_make(0.f, 0.f), ff_make(0.f, 0.f));
+        float size = 0.f;
+        for (int a = 0; a < B; ++a) {
+          const ff w = ff_from_d(P[a]);
+          ffc u = load_ffc(psi, (uint64_t)a * N + R0 + r);
+          const ffc v = load_ffc(psi, (uint64_t)a * N + C0 + c);
+          u = ffc_make(ff_mul(u.re, w), ff_mul(u.im, w));
+          mac_conj_b(z, u, v);
+          size = fmaf(fabsf(u.re.hi) + fabsf(u.im.hi), fabsf(v.re.hi) + fabsf(v.im.hi), size);
+        }
+        if (smaller(size, r, c)) put(R0 + r, C0 + c, z);
+      }
+    } else {
+      ffc acc[2][2];
+      float size[2][2];
+      rho_tile_c128<true>(psi, N, B, P, r0, c0, Ar, Ac, acc, size);
+      for (int i = 0; i < 2; ++i)
+        for (int j = 0; j < 2; ++j) {
+          const int rr = 2 * ty + i, cc = 2 * tx + j;
+          const uint64_t r = r0 + rr, cg = c0 + cc;
+          if (r > cg || cg >= N) continue;
+          if (all || (r < cg && smaller(size[i][j], rl + rr, cl + cc))) put(r, cg, acc[i][j]);
+        }
+    }
+  }
+}
+int launch_rho_fix(const double2* psi, int n, int B, const double* P, const int16_t* E, const ulonglong3* Big,
+                   const unsigned char* redo, double2* rho, cudaStream_t s) {
+  const unsigned nb = (unsigned)(((1ull << n) + 127) / 128);
+  const double unit = std::sqrt(2.0 * B) / 26.0;
+  // sizes are sums of |re| + |im| of both factors: twice the terms' moduli at most
+  k_rho_fix<<<dim3(nb, nb, nb <= 16 ? 16 : nb <= 32 ? 4 : 1), 256, 0, s>>>(
+      psi, 1ull << n, B, P, E, Big, (int)std::ceil(16.0 * unit), (int)std::ceil(64.0 * unit), (float)(2.0 * unit), redo,
+      rho);
+  return 1;
 }
 
 // ------------------------------------------------------------ Gram -------

@@ -9,10 +9,16 @@
 // u = s + t <= 6, go to seven FP32 accumulators; a product is below 2^14, an
 // accumulator sums at most 7 x 128 of them, so every sum is an exact integer
 // below 2^24 and nothing is rounded until the seven are joined in 64-bit
-// integers and converted to binary64 once.  What is dropped (u > 6) is below
-// 2^-51 of the two rows' largest entries: the result is more accurate than the
-// double-float products of the CUDA cores (k_rho), whose rate bounds them at
-// about 13 FP32 operations a real product (13 qubits, 64 states: 4.64 ms).
+// integers and converted to binary64 once.
+//
+// What is dropped (u > 6) is a fraction of the product of the two rows' scales
+// (powers of two up to their largest magnitudes), about 2^-52.3 sqrt(2 B) of it.
+// The double-float products of the CUDA cores (k_rho; bound at about 13 FP32
+// operations a real product: 4.64 ms for 13 qubits and 64 states) are good to
+// about 2^-47.6 of the terms' own sizes.  Where many states are large in both
+// rows, as in an ensemble around a common state, the digits are the better
+// ones; where the rows are dominated by different states (universes near
+// different basis states), the others, and k_rho_fix (density.cu) replaces them.
 //
 // One CTA per SM works through 128 x 32 tiles on and above the block diagonal
 // (off-diagonal tiles are also written mirrored).  K goes in chunks of 16: one
@@ -28,7 +34,7 @@
 // 1.36 TB/s of rho written).
 //
 // The call is stream-ordered: there is no status word.  A tile whose bounded
-// wait gives up (it never has) is written as NaN, with all later ones of its
+// wait gives up (it never has) is left to k_rho_fix, with all later ones of its
 // CTA.
 #include <cuda_bf16.h>
 
@@ -67,10 +73,14 @@ __device__ __forceinline__ uint64_t r8_desc(uint32_t saddr) {
 
 // One block per 32 amplitude indices: their reals through shared memory, each
 // index's largest exponent, then 8 reals (one 16-byte core-matrix row per
-// digit) at a time: A's row, Bre's and Bim's.
+// digit) at a time: A's row, Bre's and Bim's.  Big: per row, the states of at
+// least a quarter of the row's scale, of at least an eighth, and the nonzero ones
+// (bit a for state a; all of them where the row is not finite, which makes its
+// entries NaN).  Clears redo.
 __global__ void __launch_bounds__(256) k_rho8_digits(const double2* __restrict__ psi, const double* __restrict__ sqrtP,
                                                      Rho8Dims d, unsigned char* __restrict__ Aop,
-                                                     unsigned char* __restrict__ Bop, int16_t* __restrict__ E) {
+                                                     unsigned char* __restrict__ Bop, int16_t* __restrict__ E,
+                                                     ulonglong3* __restrict__ Big, unsigned char* __restrict__ redo) {
   __shared__ double X[128][33];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, jb = blockIdx.x, ib = jb >> 2;
   const uint64_t i0 = (uint64_t)jb * 32;
@@ -81,6 +91,29 @@ __global__ void __launch_bounds__(256) k_rho8_digits(const double2* __restrict__
     X[a + d.B][lane] = sqrtP[a] * c.y;
   }
   __syncthreads();
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < d.nib * d.nib; i += gridDim.x * blockDim.x) redo[i] = 0;
+  for (int r = w; r < 32; r += 8) {
+    int e[2];  // exponents of this lane's states
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int a = lane + 32 * h;
+      e[h] = -1;  // no state, or a zero
+      if (a < d.B) {
+        const double x = fmax(fabs(X[a][r]), fabs(X[a + d.B][r]));
+        if (!isfinite(X[a][r]) || !isfinite(X[a + d.B][r])) e[h] = 0x7FF;
+        else if (x > 0.0) e[h] = (int)(__double_as_longlong(x) >> 52);
+      }
+    }
+    const int top = __reduce_max_sync(0xffffffffu, max(e[0], e[1]));
+    uint64_t m[3];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const int at = q == 2 ? 0 : max(0, top - 2 - q);
+      m[q] = __ballot_sync(0xffffffffu, e[0] >= at) | (uint64_t)__ballot_sync(0xffffffffu, e[1] >= at) << 32;
+      if (top == 0x7FF) m[q] = ~0ull;
+    }
+    if (lane == 0) Big[i0 + r] = make_ulonglong3(m[0], m[1], m[2]);
+  }
   const int K = 2 * d.B;
   for (int item = threadIdx.x; item < 512; item += 256) {
     const int r = item >> 4, kg = item & 15;
@@ -145,7 +178,7 @@ struct R8Tile {
 __global__ void __launch_bounds__(R8_T, 1) k_rho8_tc(const unsigned char* __restrict__ Aop,
                                                      const unsigned char* __restrict__ Bop,
                                                      const int16_t* __restrict__ E, Rho8Dims d, int64_t ntiles,
-                                                     double2* __restrict__ rho) {
+                                                     double2* __restrict__ rho, unsigned char* __restrict__ redo) {
   extern __shared__ __align__(1024) unsigned char rsm[];
   uint64_t* bars = reinterpret_cast<uint64_t*>(rsm + R8_NST * R8_STAGE + R8_STG);
   __shared__ uint32_t tmem_holder;
@@ -260,6 +293,7 @@ __global__ void __launch_bounds__(R8_T, 1) k_rho8_tc(const unsigned char* __rest
       asm volatile("bar.sync 1, %0;\n" ::"n"(R8_T) : "memory");
       asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory");
       const bool bad = *(volatile int*)&stop != 0;
+      if (bad && tid == 0) redo[cur.ib * d.nib + (cur.jb >> 2)] = 1;
       // V = sum_u acc_u 2^(40 - 8u)
       long long V[16];
 #pragma unroll
@@ -311,25 +345,30 @@ qc_status rho_tc_c128(const double2* psi, int n, int B, const double* P_host, do
   d.nkc = (2 * B + 15) / 16;
   d.nib = (int)((d.N + TC5_M - 1) / TC5_M);
   d.njb = (int)((d.N + 31) / 32);
-  const size_t bytesA = (size_t)d.nib * d.nkc * R8_ND * R8_A, bytesB = (size_t)d.njb * d.nkc * R8_ND * R8_B,
-               bytesE = (size_t)d.nib * TC5_M * sizeof(int16_t);
+  int64_t ntiles = 0;
+  for (int ib = 0; ib < d.nib; ++ib) ntiles += d.njb - 4 * ib;
+  const size_t rows = (size_t)d.nib * TC5_M, bytesA = (size_t)d.nib * d.nkc * R8_ND * R8_A,
+               bytesB = (size_t)d.njb * d.nkc * R8_ND * R8_B;
   unsigned char* buf = nullptr;
-  cudaError_t e = ws_alloc((void**)&buf, bytesA + bytesB + bytesE + sizeof(double) * 64, s);
+  cudaError_t e = ws_alloc((void**)&buf, bytesA + bytesB + rows * (sizeof(ulonglong3) + sizeof(int16_t)) +
+                                             sizeof(double) * 128 + (size_t)d.nib * d.nib, s);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return QC_ENOMEM;
   }
-  int16_t* E = reinterpret_cast<int16_t*>(buf + bytesA + bytesB);
-  double* sqrtP = reinterpret_cast<double*>(buf + bytesA + bytesB + bytesE);
-  double sp[64] = {};
-  for (int a = 0; a < B; ++a) sp[a] = std::sqrt(P_host[a]);
-  int nk = put_bytes(sqrtP, sp, sizeof sp, s);
-  k_rho8_digits<<<4 * d.nib, 256, 0, s>>>(psi, sqrtP, d, buf, buf + bytesA, E);
-  int64_t ntiles = 0;
-  for (int ib = 0; ib < d.nib; ++ib) ntiles += d.njb - 4 * ib;
-  cudaFuncSetAttribute(k_rho8_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, R8_SMEM);
-  k_rho8_tc<<<(unsigned)std::min<int64_t>(ntiles, sm_count()), R8_T, R8_SMEM, s>>>(buf, buf + bytesA, E, d, ntiles, rho);
-  const qc_status st = check_launch("density matrix (tensor cores)", nk + 2);
+  double* w = reinterpret_cast<double*>(buf + bytesA + bytesB);  // sqrt(P), then P
+  ulonglong3* Big = reinterpret_cast<ulonglong3*>(w + 128);
+  int16_t* E = reinterpret_cast<int16_t*>(Big + rows);
+  unsigned char* redo = reinterpret_cast<unsigned char*>(E + rows);
+  double host[128] = {};
+  for (int a = 0; a < B; ++a) host[a] = std::sqrt(P_host[a]), host[64 + a] = P_host[a];
+  int nk = put_bytes(w, host, sizeof host, s);
+  k_rho8_digits<<<4 * d.nib, 256, 0, s>>>(psi, w, d, buf, buf + bytesA, E, Big, redo);
+  allow_smem(k_rho8_tc, R8_SMEM);
+  k_rho8_tc<<<(unsigned)std::min<int64_t>(ntiles, sm_count()), R8_T, R8_SMEM, s>>>(buf, buf + bytesA, E, d, ntiles, rho,
+                                                                                  redo);
+  nk += 2 + launch_rho_fix(psi, n, B, w + 64, E, Big, redo, rho, s);
+  const qc_status st = check_launch("density matrix (tensor cores)", nk);
   cudaFreeAsync(buf, s);
   return st;
 }
