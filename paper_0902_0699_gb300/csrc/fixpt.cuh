@@ -30,12 +30,14 @@ FX_HD double fx_join(long long hi, long long lo) { return (double)hi + (double)l
 // binary64 -> fixed point round(x 2^(1075 - G)) for a tile's G,
 // rounding half away from zero (symmetric, so unbiased; exact
 // values need no rounding at all).  x = m 2^(ex - 1075), so the value is
-// m 2^(ex - G).
+// m 2^(ex - G).  Numbers below 2^-1022 are dropped, or kept with SUBNORMAL.
+template <bool SUBNORMAL = false>
 __device__ __forceinline__ long long d2fix(double x, int G) {
   const unsigned long long b = (unsigned long long)__double_as_longlong(x);
-  const int ex = (int)((b >> 52) & 0x7FFu);
-  if (ex == 0) return 0;  // zero or subnormal (below 2^-1022): dropped
-  const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+  int ex = (int)((b >> 52) & 0x7FFu);
+  if (!SUBNORMAL && ex == 0) return 0;
+  const unsigned long long m = (b & 0xFFFFFFFFFFFFFull) | (ex ? 1ull << 52 : 0ull);
+  if (SUBNORMAL) ex = max(ex, 1);
   const int sh = ex - G;
   unsigned long long v;
   if (sh >= 0) {
@@ -48,7 +50,8 @@ __device__ __forceinline__ long long d2fix(double x, int G) {
 }
 
 // fixed point v 2^-F -> binary64, rounded half away from zero (results
-// below 2^-1022 flush to zero)
+// below 2^-1022 flush to zero, or are kept with SUBNORMAL)
+template <bool SUBNORMAL = false>
 __device__ __forceinline__ double fix2d(long long v, int F) {
   if (v == 0) return 0.0;
   const unsigned long long sgn = v < 0 ? (1ull << 63) : 0ull;
@@ -59,6 +62,11 @@ __device__ __forceinline__ double fix2d(long long v, int F) {
   if (keep >> 53) {
     keep >>= 1;
     ++e;
+  }
+  if (SUBNORMAL && e <= 0) {  // a 2^-F in units of 2^-1074: below 2^52 of them
+    const int r = F - 1074;
+    const unsigned long long m = r > 63 ? 0ull : r > 0 ? ((a >> (r - 1)) + 1ull) >> 1 : a << -r;
+    return __longlong_as_double((long long)(sgn | m));
   }
   if (e <= 0) return __longlong_as_double((long long)sgn);
   if (e >= 2047) return __longlong_as_double((long long)(sgn | (0x7FFull << 52)));

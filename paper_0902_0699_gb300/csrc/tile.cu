@@ -1454,13 +1454,15 @@ __global__ void __launch_bounds__(256) k_reg_rev(V2* __restrict__ s, uint64_t N,
   }
 }
 
-// complex128 register passes in 64-bit fixed point.  The tile's largest
-// exponent sets the binary point; sums are exact, a radix-4 step's two
+// complex128 register passes in 64-bit fixed point.  A tile holds 2^c columns,
+// the transforms over the group's bits for each value of its contiguous low bits.
+// The largest exponent of a column sets its binary point, so that columns share
+// nothing: not a scale, nor an infinity or a NaN.  Sums are exact, a radix-4 step's two
 // 1/sqrt 2 are one halving (a shift, or the factor 1/2 that the high word of a
 // product by a root scaled by 2^63 brings), and the result is rounded once to
 // binary64.  Against double-float (k_tile) a sum costs two integer additions
 // instead of about 20 FP32 operations and a value keeps 54 bits or more of
-// the tile's largest instead of 47: an 11-qubit register of a 17-qubit state
+// the column's largest instead of 47: an 11-qubit register of a 17-qubit state
 // has a relative error of 4e-16 where double-float passes have 1.2e-14 and
 // one pass per gate had 5.8e-15.  Double-float passes take 0.8 of the time
 // (two 9-qubit passes of a 26-qubit state 2.37 ms against 2.96 ms) but would
@@ -1515,7 +1517,6 @@ __global__ void __launch_bounds__(512, 2) k_rqft_c128(double2* __restrict__ s, u
                                                       const longlong2* __restrict__ lad) {
   constexpr int PER = 8;
   extern __shared__ __align__(16) unsigned char smraw[];
-  __shared__ int wmax[16];
   const int k = P.k, c = P.c, lo = P.lo, NE = 1 << (k + c), T = blockDim.x, tid = threadIdx.x, cm = (1 << c) - 1;
   const int hi = lo + k - 1 - P.base, sh = P.w - hi - 1, ns = (k + 1) / 2;
   const uint64_t hm = (2ull << hi) - 1ull;
@@ -1523,7 +1524,13 @@ __global__ void __launch_bounds__(512, 2) k_rqft_c128(double2* __restrict__ s, u
   longlong2* sm = reinterpret_cast<longlong2*>(smraw);
   longlong2* LAD = sm + NE;
   longlong2* V = LAD + (1 << k) - 1;
+  // the columns' largest exponents, of this tile and of the next (cleared meanwhile)
+  int* const top0 = reinterpret_cast<int*>(V + (P.twiddle && !own ? 1 << k : 0));
+  int* top = top0;
+  const bool one = cm < T;  // a thread's elements are of one column (T is a power of two)
   for (int a = tid; a < (1 << k) - 1; a += T) LAD[a] = lad[a];
+  for (int i = tid; i < 2 << c; i += T) top0[i] = 0;
+  __syncthreads();
   for (uint64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     double2 v[PER];
 #pragma unroll
@@ -1531,24 +1538,29 @@ __global__ void __launch_bounds__(512, 2) k_rqft_c128(double2* __restrict__ s, u
       const int e = tid + T * u;
       v[u] = e < NE ? s[tile_global(e, tile, lo, k, c)] : make_double2(0.0, 0.0);
     }
-    int em = 0;
+    int em = 1;  // subnormal numbers count as 2^-1022
 #pragma unroll
     for (int u = 0; u < PER; ++u) {
-      em = max(em, (int)((__double_as_longlong(v[u].x) >> 52) & 0x7FF));
-      em = max(em, (int)((__double_as_longlong(v[u].y) >> 52) & 0x7FF));
+      const int ex = max((int)((__double_as_longlong(v[u].x) >> 52) & 0x7FF),
+                         (int)((__double_as_longlong(v[u].y) >> 52) & 0x7FF));
+      if (one) em = max(em, ex);
+      else if (tid + T * u < NE) atomicMax(&top[(tid + T * u) & cm], max(ex, 1));
     }
-    em = __reduce_max_sync(0xffffffffu, em);
-    if ((tid & 31) == 0) wmax[tid >> 5] = em;
+    if (one) {
+      for (int o = 16; o > cm; o >>= 1) em = max(em, __shfl_xor_sync(0xffffffffu, em, o));
+      if ((tid & 31) <= cm) atomicMax(&top[tid & cm], em);
+    }
     __syncthreads();
-    for (int q = 0; q < (T >> 5); ++q) em = max(em, wmax[q]);
     // |x| < 2^(em - 1022) times 2^(1075 - G) is below 2^(61 - ns).  A step's
     // values grow by at most 2 and its sums of four by 4: below 2^63.
-    const int G = em - 8 + ns;
+    const int G0 = ns - 8, mine = top[tid & cm];
 #pragma unroll
     for (int u = 0; u < PER; ++u) {
-      const int e = tid + T * u;
-      if (e < NE) sm[tsw(e)] = make_longlong2(d2fix(v[u].x, G), d2fix(v[u].y, G));
+      const int e = tid + T * u, G = (one ? mine : top[e & cm]) + G0;
+      if (e < NE) sm[tsw(e)] = make_longlong2(d2fix<true>(v[u].x, G), d2fix<true>(v[u].y, G));
     }
+    int* const next = top == top0 ? top0 + (1 << c) : top0;
+    for (int i = tid; i <= cm; i += T) next[i] = 0;
     const uint64_t Lt = (tile & ((1ull << (lo - c)) - 1ull)) << c;  // the tile's index bits below the group
     if (P.twiddle && !own)
       for (int f = tid; f < (1 << k); f += T) V[f] = fx_omega(tlo, thi, (((Lt >> P.base) * (uint64_t)f) & hm) << sh, P.nl);
@@ -1593,7 +1605,7 @@ __global__ void __launch_bounds__(512, 2) k_rqft_c128(double2* __restrict__ s, u
       __syncthreads();
     }
     // odd k: the last level's 1/sqrt 2 (the high word of 2^62.5 v is v / sqrt 2 / 2)
-    const int F = 1075 - G - (k & 1) - (P.twiddle ? 2 : 0);
+    const int F0 = 1075 - G0 - (k & 1) - (P.twiddle ? 2 : 0);
 #pragma unroll
     for (int u = 0; u < PER; ++u) {
       const int e = tid + T * u;
@@ -1606,12 +1618,14 @@ __global__ void __launch_bounds__(512, 2) k_rqft_c128(double2* __restrict__ s, u
               own ? fx_omega(tlo, thi, ((((Lt | (uint64_t)(e & cm)) >> P.base) * (uint64_t)f) & hm) << sh, P.nl) : V[f];
           z = fx_mul(z, W);
         }
-        // a tile with an infinity or a NaN comes out as NaN
+        // a column with an infinity or a NaN comes out as NaN
         const double nan = __longlong_as_double(0x7ff8000000000000ll);
+        const int t = one ? mine : top[e & cm], F = F0 - t;
         s[tile_global(e, tile, lo, k, c)] =
-            em == 0x7FF ? make_double2(nan, nan) : make_double2(fix2d(z.x, F), fix2d(z.y, F));
+            t == 0x7FF ? make_double2(nan, nan) : make_double2(fix2d<true>(z.x, F), fix2d<true>(z.y, F));
       }
     }
+    top = next;
     __syncthreads();
   }
 }
@@ -1662,7 +1676,8 @@ static qc_status qft_range_impl(qc_state* s, int lo, int w) {
     if constexpr (sizeof(R) == 8) {
       RqftProg P{g.lo, g.k, c, lo, w, nl, g.lo > lo, plan.groups.size() == 1, 6521908912666391106ll};
       const size_t NE = (size_t)1 << (g.k + c);
-      const size_t smem = sizeof(longlong2) * (NE + ((size_t)1 << g.k) - 1 + (P.twiddle && lo >= c ? (size_t)1 << g.k : 0));
+      const size_t smem = sizeof(longlong2) * (NE + ((size_t)1 << g.k) - 1 + (P.twiddle && lo >= c ? (size_t)1 << g.k : 0)) +
+                          2 * sizeof(int) * ((size_t)1 << c);
       allow_smem(k_rqft_c128, 200 * 1024);
       const int T = std::max(32, (int)(NE / 8));
       const uint64_t ntiles = (1ull << s->n) / NE;
