@@ -157,9 +157,9 @@ template <typename R> struct TileProg {
   int lo, k, c;     // group [lo, lo+k), c low contiguous bits (c <= lo)
   int n;            // bits of the QFT's root tables (the transformed register's width)
   int base;         // the register's lowest qubit: the QFT's phases use the index bits from here up
-  int rev;          // store the group bits in reversed order (a register of one group)
+  int rev;          // store the lowest `rev` group bits in reversed order (a register of one group)
   int twiddle;      // apply the QFT cross phase with the register bits below lo
-  int qft;          // the program contains QFT levels (build the ladder table)
+  int qft;          // QFT levels, on the lowest `qft` group bits (the ladder table has as many)
   int nl;           // global root table split: low table has 2^nl entries
   int scale_p;      // unnormalised butterflies: multiply by 2^{-scale_p/2} at the end
   int8_t kind[QC_TILE_MAXOPS];
@@ -279,7 +279,7 @@ __device__ __forceinline__ void tile_tables(const TileProg<R>& P, const typename
   using A = TA<R>;
   const int hi = P.lo + P.k - 1 - P.base;
   if (!P.qft) return;
-  for (int a = threadIdx.x; a < lad_entries<R>(P.k); a += blockDim.x) LAD[a] = LadIO<R>::ld(lad + a);
+  for (int a = threadIdx.x; a < lad_entries<R>(P.qft); a += blockDim.x) LAD[a] = LadIO<R>::ld(lad + a);
   // twiddle remainder: Omega_{hi+1}^x = TWA[x & 127] * TWB[x >> 7], x < 2^{c+k}
   if (P.twiddle && P.base < P.c)
     for (int i = threadIdx.x; i < TS_TWA + TS_TWB; i += blockDim.x) {
@@ -427,7 +427,10 @@ __device__ __forceinline__ void tile_store(typename CT<R>::V2* __restrict__ s, u
   const int NE = 1 << (k + c), cm = (1 << c) - 1;
   const bool own = P.base < c;  // contiguous bits of the register's
   // the staged element that goes to place e
-  auto from = [&](int e) { return P.rev ? (int)((__brev((unsigned)(e >> c)) >> (32 - k)) << c) | (e & cm) : e; };
+  const int keep = cm | ~0 << (c + P.rev);
+  auto from = [&](int e) {
+    return P.rev ? (int)((__brev((unsigned)(e >> c)) >> (32 - P.rev)) << c) | (e & keep) : e;
+  };
   auto twiddled = [&](int e, E z) {
     const int f = (int)(__brev((unsigned)(e >> c)) >> (32 - k));
     E w = V[f];
@@ -475,8 +478,8 @@ __global__ void __launch_bounds__(512, 2) k_tile(typename CT<R>::V2* __restrict_
   const int NE = 1 << (k + c);
   E* V = sm + NE;
   E* LAD = V + (P.twiddle ? (1 << k) : 0);
-  const int kl = lad_levels<R>(k);  // levels in the table
-  E* TWA = LAD + (P.qft ? lad_entries<R>(k) : 0);
+  const int kl = lad_levels<R>(P.qft);  // levels in the table
+  E* TWA = LAD + (P.qft ? lad_entries<R>(P.qft) : 0);
   E* TWB = TWA + TS_TWA;
   const typename A::S sc = A::scale_const(P.scale_p);
   tile_tables<R>(P, lad, LAD, TWA, TWB);
@@ -1050,10 +1053,10 @@ static std::vector<Group> plan_groups(int n) {
 }
 
 template <typename R>
-static size_t tile_smem(int k, int c, bool twiddle, bool qft) {
+static size_t tile_smem(int k, int c, bool twiddle, int qft) {
   using E = typename TA<R>::E;
   return sizeof(E) * (((size_t)1 << (k + c)) + (twiddle ? ((size_t)1 << k) : 0) +
-                      (qft ? (size_t)lad_entries<R>(k) : 0) + TS_TWA + TS_TWB);
+                      (qft ? (size_t)lad_entries<R>(qft) : 0) + TS_TWA + TS_TWB);
 }
 
 template <typename R>
@@ -1063,7 +1066,7 @@ static qc_status run_tile(qc_state* s, TileProg<R>& P, const typename CT<R>::V2*
   if (P.nops == 0 && !P.twiddle) return QC_OK;
   const int tb = P.k + P.c;
   const uint64_t ntiles = 1ull << (s->n - tb);
-  const size_t smem = tile_smem<R>(P.k, P.c, P.twiddle != 0, P.qft != 0);
+  const size_t smem = tile_smem<R>(P.k, P.c, P.twiddle != 0, P.qft);
   const int threads = std::max(64, std::min(512, (1 << tb) >> 2));  // four amplitudes a thread
   allow_smem(k_tile<R>, 200 * 1024);
   const unsigned grid = resident_grid(k_tile<R>, threads, (int64_t)ntiles, 1, smem);
@@ -1405,7 +1408,7 @@ static qc_status qft_impl(qc_state* s) {
     TileProg<R>& P = progs[gi];
     prog_init(P, g, n);
     P.nl = nl;
-    P.qft = 1;
+    P.qft = g.k;
     for (int j = g.k - 1; j >= 0; --j) {
       P.kind[P.nops] = TOP_QFTLEVEL;
       P.q[P.nops] = (int8_t)j;
@@ -1417,7 +1420,7 @@ static qc_status qft_impl(qc_state* s) {
     if constexpr (sizeof(R) == 8) all_compiled = all_compiled && qft_c128_compiled(P);
   }
   // one tile: it is stored in reversed order (every complex64 state that comes here)
-  if (groups.size() == 1 && !(sizeof(R) == 8 && all_compiled)) progs[0].rev = 1;
+  if (groups.size() == 1 && !(sizeof(R) == 8 && all_compiled)) progs[0].rev = n;
   for (int gi = (int)groups.size() - 1; gi >= 0 && !st; --gi) {
     if constexpr (sizeof(R) == 4)
       st = run_tile<R>(s, progs[gi], tlo, thi, tab.lad);
@@ -1468,7 +1471,7 @@ __global__ void __launch_bounds__(256) k_reg_rev(V2* __restrict__ s, uint64_t N,
 // (two 9-qubit passes of a 26-qubit state 2.37 ms against 2.96 ms) but would
 // lose accuracy against the gates.
 struct RqftProg {
-  int lo, k, c;      // group [lo, lo+k), c contiguous low bits
+  int lo, k, c, h;   // group [lo, lo+k), c contiguous low bits, h bits above the group
   int base, w, nl;   // the register's lowest qubit and width, split of its root table
   int twiddle, rev;
   long long rsqrt2;  // floor(2^62.5)
@@ -1510,6 +1513,8 @@ __device__ __forceinline__ longlong2 fx_omega(const longlong2* __restrict__ tlo,
   return fx_mul(tlo[r & ((1ull << nl) - 1ull)], thi[r >> nl]);
 }
 
+// ONE: a thread's elements are of one column (the eight differ in group bits only).
+template <bool ONE>
 __global__ void __launch_bounds__(512, 2) k_rqft_c128(double2* __restrict__ s, uint64_t ntiles,
                                                       const __grid_constant__ RqftProg P,
                                                       const longlong2* __restrict__ tlo,
@@ -1517,7 +1522,7 @@ __global__ void __launch_bounds__(512, 2) k_rqft_c128(double2* __restrict__ s, u
                                                       const longlong2* __restrict__ lad) {
   constexpr int PER = 8;
   extern __shared__ __align__(16) unsigned char smraw[];
-  const int k = P.k, c = P.c, lo = P.lo, NE = 1 << (k + c), T = blockDim.x, tid = threadIdx.x, cm = (1 << c) - 1;
+  const int k = P.k, c = P.c, lo = P.lo, NE = 1 << (k + c + P.h), T = blockDim.x, tid = threadIdx.x, cm = (1 << c) - 1;
   const int hi = lo + k - 1 - P.base, sh = P.w - hi - 1, ns = (k + 1) / 2;
   const uint64_t hm = (2ull << hi) - 1ull;
   const bool own = P.base < c;  // contiguous bits of the register's: no common twiddle table of a tile
@@ -1527,40 +1532,44 @@ __global__ void __launch_bounds__(512, 2) k_rqft_c128(double2* __restrict__ s, u
   // the columns' largest exponents, of this tile and of the next (cleared meanwhile)
   int* const top0 = reinterpret_cast<int*>(V + (P.twiddle && !own ? 1 << k : 0));
   int* top = top0;
-  const bool one = cm < T;  // a thread's elements are of one column (T is a power of two)
+  const int nc = 1 << (c + P.h), lb = min(5, c + k);
+  auto col = [&](int e) { return ONE ? e & cm : (e & cm) | (e >> (c + k)) << c; };
   for (int a = tid; a < (1 << k) - 1; a += T) LAD[a] = lad[a];
-  for (int i = tid; i < 2 << c; i += T) top0[i] = 0;
+  for (int i = tid; i < 2 * nc; i += T) top0[i] = 0;
   __syncthreads();
   for (uint64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
     double2 v[PER];
 #pragma unroll
     for (int u = 0; u < PER; ++u) {
       const int e = tid + T * u;
-      v[u] = e < NE ? s[tile_global(e, tile, lo, k, c)] : make_double2(0.0, 0.0);
+      v[u] = e < NE ? s[tile_global(e, tile, lo, k + P.h, c)] : make_double2(0.0, 0.0);
     }
-    int em = 1;  // subnormal numbers count as 2^-1022
+    // to the columns' maxima, the lanes of a column first (those that differ in
+    // lane bits [c, lb)); subnormal numbers count as 2^-1022
+    auto note = [&](int e, int ex) {
+      for (int o = (1 << lb) / 2; o > cm; o >>= 1) ex = max(ex, __shfl_xor_sync(0xffffffffu, ex, o));
+      if (((tid & ((1 << lb) - 1)) & ~cm) == 0 && e < NE) atomicMax(&top[col(e)], max(ex, 1));
+    };
+    int em = 0;
 #pragma unroll
     for (int u = 0; u < PER; ++u) {
       const int ex = max((int)((__double_as_longlong(v[u].x) >> 52) & 0x7FF),
                          (int)((__double_as_longlong(v[u].y) >> 52) & 0x7FF));
-      if (one) em = max(em, ex);
-      else if (tid + T * u < NE) atomicMax(&top[(tid + T * u) & cm], max(ex, 1));
+      if (ONE) em = max(em, ex);
+      else note(tid + T * u, ex);
     }
-    if (one) {
-      for (int o = 16; o > cm; o >>= 1) em = max(em, __shfl_xor_sync(0xffffffffu, em, o));
-      if ((tid & 31) <= cm) atomicMax(&top[tid & cm], em);
-    }
+    if (ONE) note(tid, em);
     __syncthreads();
     // |x| < 2^(em - 1022) times 2^(1075 - G) is below 2^(61 - ns).  A step's
     // values grow by at most 2 and its sums of four by 4: below 2^63.
-    const int G0 = ns - 8, mine = top[tid & cm];
+    const int G0 = ns - 8, mine = ONE ? top[tid & cm] : 0;
 #pragma unroll
     for (int u = 0; u < PER; ++u) {
-      const int e = tid + T * u, G = (one ? mine : top[e & cm]) + G0;
+      const int e = tid + T * u, G = (ONE || e >= NE ? mine : top[col(e)]) + G0;
       if (e < NE) sm[tsw(e)] = make_longlong2(d2fix<true>(v[u].x, G), d2fix<true>(v[u].y, G));
     }
-    int* const next = top == top0 ? top0 + (1 << c) : top0;
-    for (int i = tid; i <= cm; i += T) next[i] = 0;
+    int* const next = top == top0 ? top0 + nc : top0;
+    for (int i = tid; i < nc; i += T) next[i] = 0;
     const uint64_t Lt = (tile & ((1ull << (lo - c)) - 1ull)) << c;  // the tile's index bits below the group
     if (P.twiddle && !own)
       for (int f = tid; f < (1 << k); f += T) V[f] = fx_omega(tlo, thi, (((Lt >> P.base) * (uint64_t)f) & hm) << sh, P.nl);
@@ -1611,7 +1620,7 @@ __global__ void __launch_bounds__(512, 2) k_rqft_c128(double2* __restrict__ s, u
       const int e = tid + T * u;
       if (e < NE) {
         const int f = (int)(__brev((unsigned)(e >> c)) >> (32 - k));
-        longlong2 z = sm[tsw(P.rev ? (f << c) | (e & cm) : e)];
+        longlong2 z = sm[tsw(P.rev ? (f << c) | (e & (ONE ? cm : cm | ~0 << (c + k))) : e)];
         if (k & 1) z = make_longlong2(__mul64hi(z.x, P.rsqrt2), __mul64hi(z.y, P.rsqrt2));
         if (P.twiddle) {
           const longlong2 W =
@@ -1620,8 +1629,8 @@ __global__ void __launch_bounds__(512, 2) k_rqft_c128(double2* __restrict__ s, u
         }
         // a column with an infinity or a NaN comes out as NaN
         const double nan = __longlong_as_double(0x7ff8000000000000ll);
-        const int t = one ? mine : top[e & cm], F = F0 - t;
-        s[tile_global(e, tile, lo, k, c)] =
+        const int t = ONE ? mine : top[col(e)], F = F0 - t;
+        s[tile_global(e, tile, lo, k + P.h, c)] =
             t == 0x7FF ? make_double2(nan, nan) : make_double2(fix2d<true>(z.x, F), fix2d<true>(z.y, F));
       }
     }
@@ -1672,26 +1681,33 @@ static qc_status qft_range_impl(qc_state* s, int lo, int w) {
   if (st) return st;
   for (int gi = (int)plan.groups.size() - 1; gi >= 0 && !st; --gi) {
     const Group& g = plan.groups[gi];
-    const int c = std::min(g.lo, std::max(ROW, TB - g.k));
+    // near the bottom of the state there are few contiguous bits: bits above the
+    // group fill the tile, while 256 tiles (two per SM, about) are left.  26
+    // complex128 qubits, registers at qubit 0: tiles of 2^w amplitudes took 30 ms
+    // for w = 1 and 11.8 for w = 3, full ones 0.82 and 1.13
+    const int c = std::min(g.lo, std::max(ROW, TB - g.k)),
+              h = g.lo == lo && c == g.lo ? std::max(0, std::min(s->n - 8, TB) - g.k - c) : 0;
     if constexpr (sizeof(R) == 8) {
-      RqftProg P{g.lo, g.k, c, lo, w, nl, g.lo > lo, plan.groups.size() == 1, 6521908912666391106ll};
-      const size_t NE = (size_t)1 << (g.k + c);
+      RqftProg P{g.lo, g.k, c, h, lo, w, nl, g.lo > lo, plan.groups.size() == 1, 6521908912666391106ll};
+      const size_t NE = (size_t)1 << (g.k + c + h);
       const size_t smem = sizeof(longlong2) * (NE + ((size_t)1 << g.k) - 1 + (P.twiddle && lo >= c ? (size_t)1 << g.k : 0)) +
-                          2 * sizeof(int) * ((size_t)1 << c);
-      allow_smem(k_rqft_c128, 200 * 1024);
+                          2 * sizeof(int) * ((size_t)1 << (c + h));
       const int T = std::max(32, (int)(NE / 8));
       const uint64_t ntiles = (1ull << s->n) / NE;
-      k_rqft_c128<<<resident_grid(k_rqft_c128, T, (int64_t)ntiles, 1, smem), T, smem, s->stream>>>(
+      const auto kernel = h == 0 && (1 << c) <= T ? k_rqft_c128<true> : k_rqft_c128<false>;
+      allow_smem(kernel, 200 * 1024);
+      kernel<<<resident_grid(kernel, T, (int64_t)ntiles, 1, smem), T, smem, s->stream>>>(
           reinterpret_cast<double2*>(s->data), ntiles, P, reinterpret_cast<const longlong2*>(tab.tlo),
           reinterpret_cast<const longlong2*>(tab.thi), reinterpret_cast<const longlong2*>(tab.lad));
       st = check_launch("register qft pass");
     } else {
       TileProg<R> P;
       prog_init(P, g, w);
+      P.k = g.k + h;
       P.c = c;
       P.base = lo;
       P.nl = nl;
-      P.qft = 1;
+      P.qft = g.k;
       for (int j = g.k - 1; j >= 0; --j) {
         P.kind[P.nops] = TOP_QFTLEVEL;
         P.q[P.nops] = (int8_t)j;
@@ -1700,7 +1716,7 @@ static qc_status qft_range_impl(qc_state* s, int lo, int w) {
       }
       P.scale_p = g.k;
       P.twiddle = g.lo > lo;
-      P.rev = plan.groups.size() == 1;
+      P.rev = plan.groups.size() == 1 ? g.k : 0;
       st = run_tile<R>(s, P, tab.tlo, tab.thi, tab.lad);
     }
   }
@@ -1723,6 +1739,14 @@ qc_status launch_qft_range(qc_state* s, int lo, int w) {
   // gate by gate 9.3e-15; here 99 us and 8.6e-16): not for a register that
   // happens to be the state.
   if (lo == 0 && w == s->n && s->dt == QC_C64) return launch_qft(s);
+  // One qubit in complex64 is the Hadamard's own kernel (26 qubits: 175 us, and
+  // 210 through tiles; 20 qubits 5 us and 17).  In complex128 that kernel is
+  // faster too (335 us and 830), but its double-float drops what lies below
+  // 2^-100, which a column of a register here keeps.
+  if (w == 1 && s->dt == QC_C64) {
+    const double h = 1.0 / sqrt(2.0), H[8] = {h, 0, h, 0, h, 0, -h, 0};
+    return launch_1q(s, lo, H);
+  }
   return s->dt == QC_C128 ? qft_range_impl<double>(s, lo, w) : qft_range_impl<float>(s, lo, w);
 }
 
