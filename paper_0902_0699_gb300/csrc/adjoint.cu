@@ -406,7 +406,11 @@ __device__ __forceinline__ void fwd_rounds(const TilePass& P, typename CT<R>::V2
         }
       }
       if constexpr (sizeof(R) == 8) {
-        if (r == P.nround - 1 && (P.has_diag || P.nop)) {
+        if (r == P.nround - 1 && !P.has_diag && P.has_fac) {  // the factor alone
+          const R f = ops->tab[48].x;
+#pragma unroll
+          for (int j = 0; j < NA; ++j) v[j] = cmake<R>(v[j].re * f, v[j].im * f);
+        } else if (r == P.nround - 1 && P.has_diag) {
           const auto A = ops->tab[tid & 31], Bw = ops->tab[32 + (tid >> 5)];
           const Cx<R> d = cmul(cmake<R>(A.x, A.y), cmake<R>(Bw.x, Bw.y));
 #pragma unroll
@@ -1120,7 +1124,14 @@ struct FwdPlan {
 
 template <typename R>
 static cudaError_t fwd_plan(FwdPlan<R>& F, const qc_gate* gates, int ng, int n, int B, cudaStream_t st) {
-  const PassCfg cfg{Fwd<R>::KT, Fwd<R>::C0, Fwd<R>::RB, sizeof(R) == 4, false};
+  // complex128: an SM's FP64 pipe bounds a tile (2^12 amplitudes under two
+  // operators: 12 us), so that tiles shrink down to 2^10 until there are 256 of
+  // them.  60 x (RX, RY, CNOT) on three of 14 qubits: 888 us gate by gate, 855
+  // with tiles of 2^12, 514 of 2^10, 511 of 2^9 (whose lists get longer: over
+  // circuits of 5 to 20 qubits 1.01 times the time).
+  const int few = n - 8 + 31 - __builtin_clz((unsigned)B);
+  const int kt = sizeof(R) == 8 ? std::max(10, std::min<int>(Fwd<R>::KT, few)) : Fwd<R>::KT;
+  const PassCfg cfg{kt, Fwd<R>::C0, Fwd<R>::RB, sizeof(R) == 4, false};
   F.passes = build_passes<R>(gates, ng, n, cfg);
   if (F.passes.empty()) return cudaSuccess;
   const size_t per = F.passes.size() * F.nrec * sizeof(typename Fwd<R>::Ops);

@@ -44,7 +44,7 @@ struct TileRound {
 };
 struct TilePass {
   int16_t kt, nreal;  // tile bits; index bits among them (nreal < kt only for states smaller than a register block)
-  int16_t nfix, nround, nop, nfc, has_perm, has_diag;
+  int16_t nfix, nround, nop, nfc, has_perm, has_diag, has_fac, pad;
   int8_t pos[TP_MAXK + 3];   // index bit of tile position p, ascending
   int8_t fix[32];            // the other index bits, ascending
   // P: the source of tile element e is the XOR of col[p] over e's set bits and
@@ -250,7 +250,8 @@ inline std::vector<TilePass> build_passes_as(const qc_gate* gates, int ng, int n
         P.fix[P.nfix++] = (int8_t)q;
       }
     }
-    // D: RZ that nothing in S follows on its qubit
+    // D: RZ that nothing in S follows on its qubit.  Forward, one alone stays an
+    // operator: four multiplications an amplitude, D's phase takes eight
     for (int p = 0; p < TP_MAXK + 3; ++p) P.dp[p] = -1;
     if (!cfg.merge) {
       uint64_t later = 0;
@@ -266,8 +267,14 @@ inline std::vector<TilePass> build_passes_as(const qc_gate* gates, int ng, int n
         later |= b;
       }
       std::reverse(keep.begin(), keep.end());
-      S.swap(keep);
+      if (cfg.reverse || S.size() - keep.size() >= 2) {
+        S.swap(keep);
+      } else {
+        for (int p = 0; p < TP_MAXK + 3; ++p) P.dp[p] = -1;
+        P.has_diag = 0;
+      }
     }
+    for (const Item& it : S) P.has_fac |= it.ka != QC_G_RZ;  // operators applied without their factor
     if (cfg.reverse) std::reverse(S.begin(), S.end());
     // register rounds; spare register bits come from the top of the tile
     P.nop = (int16_t)S.size();
