@@ -339,7 +339,9 @@ qc_status qc_renormalize(qc_state* s, double* norm_out_host);
  * temporary device buffer is 8 * (2^n / 2048 + 2) bytes (plus 8 bytes per
  * 4096 blocks for n >= 24, whose block sums are scanned in chunks); with
  * more shots the sums of 32 weights are kept as well, 8 * (2^n / 32) bytes
- * more (QC_ENOMEM if they do not fit), and a shot rescans 32.  Both give the outcomes above.  Synchronises the stream
+ * more (QC_ENOMEM if they do not fit), and a shot rescans 32; from 2^14 shots
+ * and a 32nd of the amplitudes on, the full W is written instead if its
+ * 8 * 2^n bytes fit.  All give the outcomes above.  Synchronises the stream
  * once (to read the total back). */
 qc_status qc_sample(const qc_state* s, uint64_t seed, int64_t shots, uint64_t* out_dev);
 

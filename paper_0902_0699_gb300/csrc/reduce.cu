@@ -461,7 +461,8 @@ qc_status reduce_expect(const qc_state* s, uint64_t x, uint64_t z, double* out_h
 // over the whole state.  With few shots, each shot finds its block by
 // bisection over the block offsets and rescans that block's weights; with
 // many shots the same pass also leaves the sums of 32 weights, and a shot
-// rescans 32.
+// rescans 32; with very many for the state's size the full CDF is written and
+// bisected per shot.
 #define SMP_PER 8
 #define SMP_T 256
 #define SMP_BLOCK (SMP_PER * SMP_T)
@@ -725,7 +726,7 @@ __device__ __forceinline__ uint64_t shot_target(int64_t sh, uint64_t seed, uint6
   return __umul64hi(r, total);
 }
 
-// The full CDF bisected, a thread a shot (qc_sample_noalloc).
+// The full CDF bisected, a thread a shot.
 __global__ void k_sample(const uint64_t* __restrict__ cdf, uint64_t N, uint64_t seed, int64_t shots,
                          uint64_t* __restrict__ out) {
   const uint64_t total = cdf[N - 1];
@@ -829,13 +830,23 @@ qc_status launch_sample(const qc_state* s, uint64_t seed, int64_t shots, uint64_
   const uint64_t N = 1ull << s->n;
   const uint64_t nb = (N + SMP_BLOCK - 1) / SMP_BLOCK;
   const bool local = (uint64_t)shots <= nb;
-  // [sums of 32 weights (many shots only)] [block offsets nb] [total] [status] [chunk sums]
-  const uint64_t nsub = local ? 0 : nb * SMP_NSUB;
-  const uint64_t words = nsub + nb + 2 + scan_words(nb);
+  // The CDF costs 6 ps an amplitude to write and 0.05 ns a shot to bisect, a
+  // warp's search 0.3 ns a shot: the CDF from 32 amplitudes a shot down, and if it
+  // fits (10^6 shots of 18 complex128 qubits: 432 us by warps, 92 with it; of 26
+  // qubits 924 by warps).
+  bool full = !local && shots >= 1 << 14 && N / 32 <= (uint64_t)shots;
+  // [CDF, or sums of 32 weights (many shots only)] [block offsets nb] [total] [status] [chunk sums]
+  uint64_t nsub = 0;
   uint64_t* buf = nullptr;
-  cudaError_t e = ws_alloc((void**)&buf, words * sizeof(uint64_t), s->stream);
+  cudaError_t e = cudaErrorMemoryAllocation;
+  for (int retry = full ? 0 : 1; retry < 2 && e != cudaSuccess; ++retry) {
+    if (retry) full = false;
+    cudaGetLastError();
+    nsub = full ? N : local ? 0 : nb * SMP_NSUB;
+    e = ws_alloc((void**)&buf, (nsub + nb + 2 + scan_words(nb)) * sizeof(uint64_t), s->stream);
+  }
   if (e != cudaSuccess) return cuda_fail(e, "sampler buffer");
-  uint64_t* sub = local ? nullptr : buf;
+  uint64_t* sub = local || full ? nullptr : buf;
   uint64_t* bsum = buf + nsub;
   uint64_t* tail = bsum + nb;
   uint64_t* status = tail + 1;
@@ -869,6 +880,14 @@ qc_status launch_sample(const qc_state* s, uint64_t seed, int64_t shots, uint64_
         k_sample_local<float><<<g, SMP_T, 0, s->stream>>>(reinterpret_cast<const float2*>(s->data), N, bsum, nb,
                                                           tail, seed, shots, out);
       st = check_launch("sample", 1);
+    } else if (full) {
+      if (s->dt == QC_C128)
+        k_wcdf<double><<<(unsigned)nb, SMP_T, 0, s->stream>>>(reinterpret_cast<const double2*>(s->data), N, bsum, buf);
+      else
+        k_wcdf<float><<<(unsigned)nb, SMP_T, 0, s->stream>>>(reinterpret_cast<const float2*>(s->data), N, bsum, buf);
+      const unsigned g = (unsigned)std::min<int64_t>((shots + 255) / 256, (int64_t)sm_count() * 8);
+      k_sample<<<g, 256, 0, s->stream>>>(buf, N, seed, shots, out);
+      st = check_launch("sample", 2);
     } else {
       const unsigned g = (unsigned)std::min<int64_t>((shots + 7) / 8, (int64_t)sm_count() * 8);
       if (s->dt == QC_C128)
