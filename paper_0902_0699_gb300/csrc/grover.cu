@@ -323,7 +323,16 @@ __global__ void __launch_bounds__(1024) k_grover_small(V2* __restrict__ s, int n
     }
     __syncthreads();
     __int128 P = S;
-    for (int w = 0; w < nw; ++w) P -= i128_to(buf[w]) * 2;
+    if (nw <= 4) {
+      for (int w = 0; w < nw; ++w) P -= i128_to(buf[w]) * 2;
+    } else {  // many marked: a partial sum a lane (32 of them one by one: 2.6 us a step, 1.3 so)
+      __int128 t = lane < nw ? i128_to(buf[lane]) : 0;
+      for (int o = 16; o; o >>= 1) {
+        const I128 v = i128_of(t);
+        t += i128_to(I128{__shfl_xor_sync(0xffffffffu, v.lo, o), __shfl_xor_sync(0xffffffffu, v.hi, o)});
+      }
+      P -= t * 2;
+    }
     const long long t2 = (long long)((P + ((__int128)1 << (n - 1) >> 1)) >> (n - 1));
     S = ((__int128)t2 << n) - P;
 #pragma unroll
