@@ -29,8 +29,11 @@
  *    runtime failure returns QC_ECUDA.  qc_last_error() returns a message
  *    describing the last failure on the calling host thread.
  *  - Temporary device buffers come from a memory pool of the library's own
- *    per device, which keeps up to 512 MiB between calls and gives them back
- *    when the last state handle is freed.
+ *    per device, which keeps up to 512 MiB between calls.  It gives them back
+ *    when the last state handle is freed, and to any allocation of the process
+ *    that does not fit without them; a process that uses only the calls
+ *    without a handle (circuits, density matrices, spectra) and whose
+ *    allocations fit holds them until it exits or frees a state handle.
  *  - Device code never traps: a bounded wait that gives up reports
  *    QC_ETIMEOUT through a status word the host reads.
  */

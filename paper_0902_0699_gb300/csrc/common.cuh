@@ -96,8 +96,9 @@ inline cudaError_t allow_smem(K kernel, size_t bytes) {
 // synchronisation, after which an allocation takes 100 us and more.
 constexpr size_t WS_KEEP = (size_t)512 << 20;
 cudaError_t ws_alloc(void** p, size_t bytes, cudaStream_t st);
-// Live handles (states, plans): the pools' spare memory is given back when the
-// last one is freed.
+// Live state handles: the pools' spare memory is given back when the last one
+// is freed (an allocation that does not fit takes it before that; plans are not
+// counted, their next call allocates again).
 void handle_created();
 void handle_freed();
 
