@@ -1322,7 +1322,9 @@ static qc_status qft_tables(qc_state* s, int n, int nl, int nlad, QftTables<R>* 
                                             nl, reinterpret_cast<longlong2*>(t->lad), nlad);
   else
     k_roots<R><<<grid, 64, 0, s->stream>>>(t->tlo, t->thi, n, nl, t->lad, nlad);
-  return check_launch("qft roots");
+  const qc_status st = check_launch("qft roots");
+  if (st) cudaFreeAsync(t->tlo, s->stream);  // the callers go no further
+  return st;
 }
 
 // W[e] = Omega_{hi+1}^{l f} of the complex64 pass blockIdx.y on group
