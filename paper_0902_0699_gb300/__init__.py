@@ -380,7 +380,7 @@ def qc_dense_timeout_selftest(h, spin_limit: int) -> int:
     return int(lib().qc_dense_timeout_selftest(h, int(spin_limit)))
 
 
-_HTERM = np.dtype([("k", np.int32), ("qubits", np.int32, 2), ("h", np.float64, 32)], align=True)
+_HTERM = np.dtype(HTerm)
 
 
 def qc_hamiltonian_step(h, dt: float, terms):
@@ -389,8 +389,11 @@ def qc_hamiltonian_step(h, dt: float, terms):
     k, q, hh = arr["k"], arr["qubits"], arr["h"]
     for i, (qs, m) in enumerate(terms):
         k[i] = len(qs)
-        q[i, :len(qs)] = qs
+        for b, t in enumerate(qs):  # any iterable of integers; a third one is an IndexError
+            q[i, b] = int(t)
         flat = np.ascontiguousarray(m, dtype=complex).reshape(-1).view(np.float64)
+        if flat.size > 32:
+            raise IndexError("a term's matrix has at most 4 x 4 entries")
         hh[i, :flat.size] = flat
     _check(lib().qc_hamiltonian_step(h, dt, _VP(arr.ctypes.data), len(terms)))
 
