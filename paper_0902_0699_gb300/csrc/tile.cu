@@ -203,46 +203,6 @@ __device__ __forceinline__ typename TA<R>::E omega(const typename CT<R>::V2* __r
   return TA<R>::mul(TA<R>::from(a), TA<R>::from(b));
 }
 
-// QR consecutive QFT levels jtop, jtop-1, .., jtop-QR+1 in one shared-memory
-// round trip: each thread holds the 2^QR elements that differ in the block's
-// bits in registers.  Level j (local bit lv = j - jtop + QR - 1) pairs
-// elements across local bit lv; its ladder phase e^{2 pi i x / 2^{j+1}}
-// uses x = group bits below j = (local bits below lv, placed above the
-// block's lowest group qubit) | (the thread's group bits below the block).
-template <typename R, int QR>
-__device__ __forceinline__ void qft_levels_regs(typename TA<R>::E* sm, int NE, int c, int jtop,
-                                                const typename TA<R>::E* LAD) {
-  using A = TA<R>;
-  using E = typename A::E;
-  constexpr int NR = 1 << QR;
-  const int jlo = jtop - QR + 1;  // the block's lowest group qubit
-  const int bl = c + jlo;         // its index bit
-  for (int p = threadIdx.x; p < (NE >> QR); p += blockDim.x) {
-    const int base = ((p >> bl) << (bl + QR)) | (p & ((1 << bl) - 1));
-    E a[NR];
-#pragma unroll
-    for (int i = 0; i < NR; ++i) a[i] = sm[base | (i << bl)];
-    const int xlow = (base >> c) & ((1 << jlo) - 1);
-#pragma unroll
-    for (int lv = QR - 1; lv >= 0; --lv) {
-      const int j = jlo + lv;
-#pragma unroll
-      for (int i = 0; i < NR; ++i) {
-        if ((i >> lv) & 1) continue;
-        const int i1 = i | (1 << lv);
-        const E s0 = A::add(a[i], a[i1]);
-        E d = A::sub(a[i], a[i1]);
-        const int x = ((i & ((1 << lv) - 1)) << jlo) | xlow;
-        if (x) d = A::mul(LAD[(1 << j) - 1 + x], d);
-        a[i] = s0;
-        a[i1] = d;
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < NR; ++i) sm[base | (i << bl)] = a[i];
-  }
-}
-
 // L_j(y) = e^{2 pi i y / 2^{j+1}}, y < 2^j, from the ladder table (levels
 // below kl) or, for level kl, from level kl - 1 and the extra entry.
 template <typename R>
@@ -303,9 +263,8 @@ __device__ __forceinline__ void tile_twiddle_v(const TileProg<R>& P, uint64_t T,
 }
 
 // The program's operators on the staged tile sm (2^{k+c} elements), with a
-// barrier after each shared-memory round trip.  QREG: four descending QFT
-// levels at a time in registers.
-template <typename R, bool QREG>
+// barrier after each shared-memory round trip.
+template <typename R>
 __device__ __forceinline__ void tile_ops(typename TA<R>::E* sm, const TileProg<R>& P, const typename TA<R>::E* LAD,
                                          int kl) {
   using A = TA<R>;
@@ -315,16 +274,6 @@ __device__ __forceinline__ void tile_ops(typename TA<R>::E* sm, const TileProg<R
   for (int o = 0; o < P.nops; ++o) {
     const int b = c + P.q[o];
     const int kind = P.kind[o];
-    // four descending QFT levels in registers (complex64: the passes are
-    // bound by shared-memory traffic)
-    if (QREG && kind == TOP_QFTLEVEL && o + 3 < P.nops && P.kind[o + 1] == kind &&
-        P.kind[o + 2] == kind && P.kind[o + 3] == kind && P.q[o + 1] == P.q[o] - 1 &&
-        P.q[o + 2] == P.q[o] - 2 && P.q[o + 3] == P.q[o] - 3) {
-      qft_levels_regs<R, 4>(sm, NE, c, P.q[o], LAD);
-      __syncthreads();
-      o += 3;
-      continue;
-    }
     // two butterfly levels on neighbouring qubits: one shared-memory round
     // trip (radix 4).  QFT levels come in descending order j, j-1; plain
     // Hadamard butterflies commute, so any neighbouring pair qualifies.
@@ -524,7 +473,7 @@ __global__ void __launch_bounds__(512, 2) k_tile(typename CT<R>::V2* __restrict_
       }
     }
     __syncthreads();
-    tile_ops<R, false>(sm, P, LAD, kl);
+    tile_ops<R>(sm, P, LAD, kl);
     tile_store<R>(s, T, sm, P, V, TWA, TWB, sc);
     __syncthreads();
   }
