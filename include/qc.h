@@ -301,8 +301,11 @@ qc_status qc_project(qc_state* s, int lo, int width, uint64_t value, double* pro
 
 /* QFT of the register of qubits [lo, lo+width) (Appendix A's circuit
  * applied to register 1 of Shor's algorithm, sec. 5.2 step 5): Hadamard /
- * CPHASEK ladder and the swaps restoring the register's bit order, as gate
- * passes.  On the whole state (lo = 0, width = n) it equals qc_qft. */
+ * CPHASEK ladder and the swaps restoring the register's bit order, as passes
+ * over shared-memory tiles.  complex128 in 64-bit fixed point with an exponent
+ * for each transform (each value of the qubits outside the register; an
+ * infinity or a NaN stays in its transform).  On the whole state (lo = 0,
+ * width = n) it is qc_qft's transform. */
 qc_status qc_qft_range(qc_state* s, int lo, int width);
 
 /* ----------------------------------------------------------- reductions -- */
@@ -495,12 +498,15 @@ qc_status qc_circuit_forward(int n, qc_dtype dt, int B, const qc_gate* gates, in
  * entries of parameters the circuit does not use are set to 0).  Runs the
  * forward pass, then walks the gates backwards applying U^dagger to psi and
  * to lambda = H psi (no intermediate states are stored); for a rotation
- * gate j with Pauli generator P: dE/dtheta_j = Im <lambda_j|P|psi_j>, with
- * FP64 accumulation.  psi_dev and lam_dev are caller-owned workspace of
- * B * 2^n amplitudes each; their contents on return are unspecified.  Two
- * rotations in a row on one qubit run as one pass, and a CNOT ring
- * CNOT(0,1), .., CNOT(n-1,0) as one gather pass (using one more temporary
- * buffer of B * 2^n amplitudes).  H is a host array of Pauli terms with real
+ * gate j with Pauli generator P: dE/dtheta_j = Im <lambda_j|P|psi_j>.  The
+ * energy and complex128 derivatives are summed in FP64 (a block's sums in
+ * fixed point of 2^-54 sum |c_k| and finer); complex64 derivatives in float
+ * pairs, to about 2^-37 of a thread's largest |lambda| |psi| a term, and then in
+ * 64-bit fixed point.  psi_dev and lam_dev are caller-owned workspace of
+ * B * 2^n amplitudes each; their contents on return are unspecified.  Both
+ * sweeps apply the gates in passes over shared-memory tiles, a pass's CNOTs as
+ * one index map; temporary buffers hold the passes' operators and sums (about
+ * 64 MiB each at most).  H is a host array of Pauli terms with real
  * coefficients. */
 qc_status qc_adjoint_grad(int n, qc_dtype dt, int B, const qc_gate* gates, int n_gates,
                           const double* theta_dev, int64_t theta_stride, int n_params,

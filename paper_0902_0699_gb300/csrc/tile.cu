@@ -645,9 +645,9 @@ __global__ void __launch_bounds__(512, 2) k_qft_c128_k(double2* __restrict__ s, 
 // one waits at its barriers or for its loads, the other computes.  What is the
 // same for every tile (the twiddles W, the ladders) is built once per
 // transform and read through L1, which is what makes room for the second tile.
-// 29 qubits, an 8-level pass above the lowest group: 2.16 ms with one CTA of
-// two buffers, 1.48 with two CTAs, the first levels straight from the state and
-// the last straight to it (0.91 of the copy bandwidth, 1.39 ms).
+// 29 qubits, an 8-level pass above the lowest group: 2.16 ms with one CTA of two
+// buffers; 1.39 ms (0.91 of the copy bandwidth) with two CTAs, the first levels
+// straight from the state and the last straight to it.
 // The group's levels run in register blocks
 // of up to four levels (one shared-memory round trip each).  Within a block
 // on group qubits jlo .. jlo+QR-1, level j = jlo + lv multiplies the
@@ -968,8 +968,8 @@ template <> struct TileCfg<double> { static constexpr int C = 3, K = 9, BOT = 12
 // the ladder helper reaches one level past the table (levels 0..10)
 static_assert(TileCfg<double>::BOT <= 12 && TileCfg<double>::K <= 12, "complex128 groups of at most 12 qubits");
 // complex64 layers: 128 KiB tiles for groups of 10 (c = 4, one CTA per SM),
-// 64 KiB for smaller ones; the complex64 QFT plans groups of at most 9 above
-// the lowest 13 (64 KiB tiles, two buffers in one CTA)
+// 64 KiB for smaller ones; the complex64 QFT of 13 qubits and more has groups of
+// its own (qft_groups_c64)
 template <> struct TileCfg<float> { static constexpr int C = 4, K = 10, BOT = 13; };
 
 struct Group {
