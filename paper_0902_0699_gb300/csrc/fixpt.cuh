@@ -1,6 +1,7 @@
-// binary64 <-> 64-bit fixed point with a common exponent per tile (wht.cu and
-// the register QFT of tile.cu): sums are exact integer additions and no FP64
-// instruction is issued.
+// binary64 <-> 64-bit fixed point with a common exponent per tile (wht.cu), column
+// (the register QFT of tile.cu) or row (rho_tc128.cu): sums are exact integer
+// additions and no FP64 instruction is issued.  And a sum of FP64 terms in two
+// words of fixed point, which does not depend on their order (adjoint.cu).
 #pragma once
 
 #include <math.h>
