@@ -393,7 +393,14 @@ qc_status rho_tc_c64(const float2* psi, int n, int B, const double* P_host, floa
 qc_status rho_tc_c128(const double2* psi, int n, int B, const double* P_host, double2* rho, cudaStream_t s);
 // Then: its entries that double-float products give better, and the blocks a
 // CTA gave up (redo), on the CUDA cores (density.cu); returns the launches made.
-int launch_rho_fix(const double2* psi, int n, int B, const double* P, const int16_t* E, const ulonglong3* Big,
+// Big: per amplitude index, the states of at least the full scale 2^(E - 1023) of
+// its row (its largest magnitude is below twice that), a half, a quarter and an
+// eighth of it, and the nonzero ones; bit a for state a, all where the row is not
+// finite.
+struct RhoBig {
+  uint64_t full, half, quarter, eighth, any;
+};
+int launch_rho_fix(const double2* psi, int n, int B, const double* P, const int16_t* E, const RhoBig* Big,
                    const unsigned char* redo, double2* rho, cudaStream_t s);
 
 qc_status dense_launch(qc_state* s, const DenseMap& M, const void* dev_op, int* status,

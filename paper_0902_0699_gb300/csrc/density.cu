@@ -183,6 +183,14 @@ __global__ void __launch_bounds__(256) k_rho(const V2* __restrict__ psi, uint64_
   }
 }
 
+// |x| to 2^-20, without an FP64 instruction (0 below FP32's range, infinite above)
+__device__ __forceinline__ float mag_f(double x) {
+  const int h = __double2hiint(x) & 0x7fffffff;
+  return h < (897 << 20) ? 0.f : h >= (1151 << 20) ? INFINITY : __int_as_float((h - (896 << 20)) << 3);
+}
+#define RHO_FEW 96
+#define RHO_EXACT 16
+
 // Entries of the digit products (rho_tc128.cu) that double-float products give
 // better, replaced by those; a CTA (or four, or sixteen, for few blocks) per
 // 128 x 128 block on or above the diagonal (the lower triangle gets the
@@ -192,157 +200,187 @@ __global__ void __launch_bounds__(256) k_rho(const V2* __restrict__ psi, uint64_
 // scales 2^(E - 1023), that of the double-float products 2^-47.6 of the terms'
 // own sizes (both from sums of random rows against exact ones) and 2^-98 a
 // factor.  So an entry is replaced if its terms come to less than
-// sqrt(2 B) / 26 of the scales' product.  Which entries may be such:
-//  - Up to RHO_EXACT states: the terms' sizes are summed for every entry.
-//  - More states: a state that is at least a quarter (an eighth) of the scale in
-//    both rows has a term of 1/16 (1/64) of it or more, so K16 =
-//    ceil(16 sqrt(2 B) / 26) (K64 likewise) of those rule an entry out, and so
-//    does having no state in common, which makes it exactly zero.  Two rows of
-//    c1 and c2 such states share at least c1 + c2 - B: for some thirty states
-//    and more of an ordinary ensemble the block's smallest counts decide without
-//    a look at its pairs.
-// A 32 x 32 tile with few such entries takes them one by one (a thread an
-// entry, amplitudes from L2), one with more is formed whole as k_rho does.
-// 13 qubits, the call without and with it: ordinary batches of 64 states 829 ->
-// 837 us, of 2 states 410 -> 450 (no entry is replaced, bound by the sums);
-// states that are each large on amplitudes of their own and 1e-9 elsewhere: 64
-// 6.1 ms, 2 0.93 ms (k_rho alone 4.64 ms).
-// |x| to 2^-20, without an FP64 instruction (0 below FP32's range, infinite above)
-__device__ __forceinline__ float mag_f(double x) {
-  const int h = __double2hiint(x) & 0x7fffffff;
-  return h < (897 << 20) ? 0.f : h >= (1151 << 20) ? INFINITY : __int_as_float((h - (896 << 20)) << 3);
-}
-#define RHO_FEW 96
-#define RHO_EXACT 16
-#define RHO_MS (RHO_EXACT + 4)  // padded: 16-byte loads of 32 rows hit every bank
+// sqrt(2 B) / 26 of the scales' product, and of that by its terms' sizes, summed
+// in FP32.  More than RHO_EXACT states: the sums are formed only for 32 x 32 tiles
+// that may hold such an entry.  A state that is at least a quarter (an eighth) of
+// the scale in both rows has a term of 1/16 (1/64) of it or more, so K16 =
+// ceil(16 sqrt(2 B) / 26) (K64 likewise) of those rule an entry out; so does one
+// state of the full scale in one row and half of it in the other (sqrt(2 B) / 26
+// is below 1/2), and having no state in common, which makes the entry exactly
+// zero.  Two rows of c1 and c2 such states share at least c1 + c2 - B: for some
+// thirty states and more of an ordinary ensemble the block's smallest counts
+// decide without a look at its pairs.
+// A tile with few entries to replace takes them one by one (a warp an entry, two
+// states a lane), one with more is formed whole as k_rho does.
+// The call without and with it, 13 qubits: ordinary batches of 64 states 830 ->
+// 837 us, of 2 states 410 -> 445 (no entry is replaced, bound by the sums); 64
+// Grover runs that noise strikes at different steps 830 -> 905 us, of 14 qubits
+// 3.17 -> 3.36 ms (a few rows dominated by one run, 0.001% replaced); states
+// that are each large on amplitudes of their own and 1e-9 elsewhere 6.4 ms, two
+// of them 0.98 (every tile whole; k_rho alone 4.64 ms).
 __global__ void __launch_bounds__(256) k_rho_fix(const double2* __restrict__ psi, uint64_t N, int B,
                                                  const double* __restrict__ P, const int16_t* __restrict__ E,
-                                                 const ulonglong3* __restrict__ Big, int K16, int K64, float lim,
+                                                 const RhoBig* __restrict__ Big, int K16, int K64, float lim,
                                                  const unsigned char* __restrict__ redo, double2* __restrict__ rho) {
   if (blockIdx.x < blockIdx.y) return;
+  // |re| + |im| of sqrt(P_a) C_a, of the row's scale: all 128 + 128 rows (up to RHO_EXACT states) or a
+  // tile's 32 + 32; padded rows, whose 16-byte loads hit every bank
+  constexpr int W16 = RHO_EXACT + 4, W64 = 64 + 4;
   __shared__ union {
-    ulonglong3 mask[2][128];
-    float size[2][128][RHO_MS];  // |re| + |im| of a row's amplitudes, of its scale
-  } M;
+    float all[2][128][W16];
+    struct {
+      RhoBig mask[2][128];
+      union {
+        float size[2][32][W64];
+        ffc op[2][RHO_KC][RHO_TILE];
+      } t;
+    } m;
+    struct {
+      float all[2][128][W16];
+      ffc op[2][RHO_KC][RHO_TILE];
+    } x;
+  } S;
   __shared__ float scale[2][128];  // of the rows; 0: none of its entries is replaced
-  __shared__ float wt[RHO_EXACT];
-  __shared__ int least[2], count[16];
-  __shared__ ffc Ar[RHO_KC][RHO_TILE], Ac[RHO_KC][RHO_TILE];
+  __shared__ float wt[64];
+  __shared__ int least[2], listed;
+  __shared__ uint16_t list[RHO_FEW];  // entries of a tile: row << 5 | column
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, tx = tid & 15, ty = tid >> 4;
-  const bool all = redo[blockIdx.y * gridDim.x + blockIdx.x] != 0, exact = B <= RHO_EXACT;
+  const bool redo_all = redo[blockIdx.y * gridDim.x + blockIdx.x] != 0, exact = B <= RHO_EXACT;
   const int nh = (B + 3) / 4;
   const uint64_t R0 = (uint64_t)blockIdx.y * 128, C0 = (uint64_t)blockIdx.x * 128;
   const int side = tid >> 7, x = tid & 127;
   const uint64_t row = (side ? C0 : R0) + x;
   const int e = E[row] - 1023;
   // a factor's 2^-98 forbids what lies lower, FP32's range what lies higher
-  const float sc = e >= -50 && e <= 60 ? __int_as_float((e + 127) << 23) : 0.f;
-  scale[side][x] = sc;
-  if (tid < 16) count[tid] = 0;
-  if (exact) {
-    if (tid < RHO_EXACT) wt[tid] = tid < B ? sqrtf((float)P[tid]) : 0.f;
-    __syncthreads();
-    const float inv = sc > 0.f ? 1.f / sc : 0.f;
+  scale[side][x] = e >= -50 && e <= 60 ? __int_as_float((e + 127) << 23) : 0.f;
+  if (tid < 64) wt[tid] = tid < B ? sqrtf((float)P[tid]) : 0.f;
+  if (tid < 2) least[tid] = 64;
+  __syncthreads();
+  // the sizes of a row (index i of the block's, side s), states 4 h .. 4 h + 3
+  auto sizes = [&](int s, int i, int h, float* to) {
+    const float sc = scale[s][i], inv = sc > 0.f ? 1.f / sc : 0.f;
+    const uint64_t at = (s ? C0 : R0) + i;
 #pragma unroll
-    for (int h = 0; h < RHO_EXACT / 4; ++h) {
-      if (h >= nh) break;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int a = 4 * h + k;
-        double2 v = make_double2(0.0, 0.0);
-        if (a < B && row < N) v = psi[(uint64_t)a * N + row];
-        M.size[side][x][a] = (mag_f(v.x) + mag_f(v.y)) * (wt[a] * inv);
-      }
+    for (int k = 0; k < 4; ++k) {
+      const int a = 4 * h + k;
+      double2 v = make_double2(0.0, 0.0);
+      if (a < B && at < N) v = psi[(uint64_t)a * N + at];
+      to[k] = (mag_f(v.x) + mag_f(v.y)) * (wt[a] * inv);
     }
-    __syncthreads();
-  } else {
-    if (tid < 2) least[tid] = 64;
-    __syncthreads();
-    const ulonglong3 mine = Big[row];
-    M.mask[side][x] = mine;
-    const int cnt = __reduce_min_sync(0xffffffffu, mine.z ? __popcll(mine.y) : 64);
-    if (lane == 0) atomicMin(&least[side], cnt);
-    __syncthreads();
-    if (!all && least[0] + least[1] - B >= K64) return;
-  }
-  auto smaller = [&](float size, int r, int c) {
-    const float er = scale[0][r], ec = scale[1][c];
-    return fmaf(0x1p-48f, er + ec, size) < lim * er * ec;
   };
+  if (exact) {
+#pragma unroll
+    for (int h = 0; h < RHO_EXACT / 4; ++h)
+      if (h < nh) sizes(side, x, h, &S.all[side][x][4 * h]);
+  } else {
+    const RhoBig mine = Big[row];
+    S.m.mask[side][x] = mine;
+    const int cnt = __reduce_min_sync(0xffffffffu, mine.any ? __popcll(mine.eighth) : 64);
+    if (lane == 0) atomicMin(&least[side], cnt);
+  }
+  __syncthreads();
+  if (!exact && !redo_all && least[0] + least[1] - B >= K64) return;
+  ffc(*op)[RHO_KC][RHO_TILE] = exact ? S.x.op : S.m.t.op;
   auto put = [&](uint64_t r, uint64_t c, const ffc& z) {
     // joined in FP64: such an entry may be below 2^-75, where ff_to_d keeps 24 bits
     const double2 v = make_double2((double)z.re.hi + (double)z.re.lo, (double)z.im.hi + (double)z.im.lo);
     rho[r * N + c] = r < c || !isfinite(v.x) ? v : make_double2(v.x, 0.0);
     if (r < c) rho[c * N + r] = make_double2(v.x, -v.y);
   };
+  auto smaller = [&](float size, int r, int c) {  // size: of the scales' product
+    const float er = scale[0][r], ec = scale[1][c];
+    return fmaf(0x1p-48f, er + ec, size * er * ec) < lim * er * ec;
+  };
+  // of this thread's entries (rl + warp + 8 q, cl + lane) of a tile, those to replace: bit q
+  auto small = [&](int rl, int cl) {
+    float z[4] = {0.f, 0.f, 0.f, 0.f};
+    const float* pr = exact ? S.all[0][rl + warp] : S.m.t.size[0][warp];
+    const float* pc = exact ? S.all[1][cl + lane] : S.m.t.size[1][lane];
+    const int ld = exact ? W16 : W64;
+#pragma unroll 4
+    for (int h = 0; h < nh; ++h) {
+      const float4 y = *reinterpret_cast<const float4*>(pc + 4 * h);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const float4 w = *reinterpret_cast<const float4*>(pr + 8 * q * ld + 4 * h);
+        z[q] = fmaf(w.x, y.x, fmaf(w.y, y.y, fmaf(w.z, y.z, fmaf(w.w, y.w, z[q]))));
+      }
+    }
+    unsigned mine = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int r = rl + warp + 8 * q, c = cl + lane;
+      mine |= (unsigned)(z[q] > 0.f && R0 + r < C0 + c && smaller(z[q], r, c)) << q;
+    }
+    return mine;
+  };
+  if (exact && !redo_all) {  // most blocks have none: one barrier for all of a block's tiles
+    unsigned any = 0;
+    for (int t = blockIdx.z; t < 16; t += gridDim.z) any |= small(32 * (t >> 2), 32 * (t & 3));
+    if (!__syncthreads_or(any)) return;
+  }
   for (int t = blockIdx.z; t < 16; t += gridDim.z) {
-    const int rl = 32 * (t >> 2), cl = 32 * (t & 3), c = cl + lane;
+    const int rl = 32 * (t >> 2), cl = 32 * (t & 3);
     const uint64_t r0 = R0 + rl, c0 = C0 + cl;
     if (r0 > c0 || c0 >= N) continue;
-    int hit = 0;  // of this thread's entries (rl + warp + 8 q, c); those past N have no state
-    if (!all) {
-      if (exact) {
-        float4 y[RHO_EXACT / 4];
-#pragma unroll
-        for (int h = 0; h < RHO_EXACT / 4; ++h)
-          if (h < nh) y[h] = *reinterpret_cast<const float4*>(&M.size[1][c][4 * h]);
+    int n = 1024;  // entries to replace
+    if (!redo_all) {
+      if (!exact) {  // does the tile need its sizes?
+        bool hit = false;
+        const RhoBig b = S.m.mask[1][cl + lane];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          const int r = rl + warp + 8 * q;
-          float z = 0.f;
-#pragma unroll
-          for (int h = 0; h < RHO_EXACT / 4; ++h) {
-            if (h >= nh) break;
-            const float4 w = *reinterpret_cast<const float4*>(&M.size[0][r][4 * h]);
-            z = fmaf(w.x, y[h].x, fmaf(w.y, y[h].y, fmaf(w.z, y[h].z, fmaf(w.w, y[h].w, z))));
-          }
-          hit |= (z > 0.f && z < lim && R0 + r < C0 + c) << q;
+          const RhoBig a = S.m.mask[0][rl + warp + 8 * q];
+          hit |= (a.any & b.any) && !((a.full & b.half) | (a.half & b.full)) &&
+                 __popcll(a.quarter & b.quarter) < K16 && __popcll(a.eighth & b.eighth) < K64 &&
+                 r0 + warp + 8 * q < c0 + lane;
         }
-      } else {
-        const ulonglong3 b = M.mask[1][c];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int r = rl + warp + 8 * q;
-          const ulonglong3 a = M.mask[0][r];
-          hit |= ((a.z & b.z) && __popcll(a.x & b.x) < K16 && __popcll(a.y & b.y) < K64 && R0 + r < C0 + c) << q;
-        }
+        if (!__syncthreads_or(hit)) continue;
+        for (int i = tid; i < 64 * nh; i += blockDim.x)
+          sizes((i >> 5) & 1, ((i >> 5) & 1 ? cl : rl) + (i & 31), i >> 6, &S.m.t.size[(i >> 5) & 1][i & 31][4 * (i >> 6)]);
+        __syncthreads();
       }
-      const int hits = __reduce_add_sync(0xffffffffu, __popc(hit));
-      if (lane == 0 && hits) atomicAdd(&count[t], hits);
+      unsigned mine = small(rl, cl);
+      if (tid == 0) listed = 0;
+      if (!__syncthreads_or(mine)) continue;
+      for (; mine; mine &= mine - 1) {
+        const int at = atomicAdd(&listed, 1);
+        if (at < RHO_FEW) list[at] = (uint16_t)((warp + 8 * (__ffs(mine) - 1)) << 5 | lane);
+      }
       __syncthreads();
-      if (count[t] == 0) continue;
+      n = listed;
     }
-    if (!all && count[t] <= RHO_FEW) {
-      for (int q = 0; q < 4; ++q) {
-        if (!((hit >> q) & 1)) continue;
-        const int r = rl + warp + 8 * q;
+    if (n <= RHO_FEW) {
+      for (int i = warp; i < n; i += 8) {
+        const uint64_t r = r0 + (list[i] >> 5), c = c0 + (list[i] & 31);
         ffc z = ffc_make(ff_make(0.f, 0.f), ff_make(0.f, 0.f));
-        float size = 0.f;
-        for (int a = 0; a < B; ++a) {
+        for (int a = lane; a < B; a += 32) {
           const ff w = ff_from_d(P[a]);
-          ffc u = load_ffc(psi, (uint64_t)a * N + R0 + r);
-          const ffc v = load_ffc(psi, (uint64_t)a * N + C0 + c);
-          u = ffc_make(ff_mul(u.re, w), ff_mul(u.im, w));
-          mac_conj_b(z, u, v);
-          size = fmaf(fabsf(u.re.hi) + fabsf(u.im.hi), fabsf(v.re.hi) + fabsf(v.im.hi), size);
+          const ffc u = load_ffc(psi, (uint64_t)a * N + r);
+          mac_conj_b(z, ffc_make(ff_mul(u.re, w), ff_mul(u.im, w)), load_ffc(psi, (uint64_t)a * N + c));
         }
-        if (smaller(size, r, c)) put(R0 + r, C0 + c, z);
+        for (int o = 16; o; o >>= 1)
+          z = ffc_add(z, ffc_make(ff_make(__shfl_xor_sync(0xffffffffu, z.re.hi, o), __shfl_xor_sync(0xffffffffu, z.re.lo, o)),
+                                  ff_make(__shfl_xor_sync(0xffffffffu, z.im.hi, o), __shfl_xor_sync(0xffffffffu, z.im.lo, o))));
+        if (lane == 0) put(r, c, z);
       }
     } else {
       ffc acc[2][2];
       float size[2][2];
-      rho_tile_c128<true>(psi, N, B, P, r0, c0, Ar, Ac, acc, size);
+      rho_tile_c128<true>(psi, N, B, P, r0, c0, op[0], op[1], acc, size);
       for (int i = 0; i < 2; ++i)
         for (int j = 0; j < 2; ++j) {
           const int rr = 2 * ty + i, cc = 2 * tx + j;
-          const uint64_t r = r0 + rr, cg = c0 + cc;
-          if (r > cg || cg >= N) continue;
-          if (all || (r < cg && smaller(size[i][j], rl + rr, cl + cc))) put(r, cg, acc[i][j]);
+          const uint64_t r = r0 + rr, c = c0 + cc;
+          if (r > c || c >= N) continue;
+          const float er = scale[0][rl + rr], ec = scale[1][cl + cc];
+          if (redo_all || (r < c && fmaf(0x1p-48f, er + ec, size[i][j]) < lim * er * ec)) put(r, c, acc[i][j]);
         }
     }
+    __syncthreads();  // listed and list are read
   }
 }
-int launch_rho_fix(const double2* psi, int n, int B, const double* P, const int16_t* E, const ulonglong3* Big,
+int launch_rho_fix(const double2* psi, int n, int B, const double* P, const int16_t* E, const RhoBig* Big,
                    const unsigned char* redo, double2* rho, cudaStream_t s) {
   const unsigned nb = (unsigned)(((1ull << n) + 127) / 128);
   const double unit = std::sqrt(2.0 * B) / 26.0;

@@ -73,14 +73,12 @@ __device__ __forceinline__ uint64_t r8_desc(uint32_t saddr) {
 
 // One block per 32 amplitude indices: their reals through shared memory, each
 // index's largest exponent, then 8 reals (one 16-byte core-matrix row per
-// digit) at a time: A's row, Bre's and Bim's.  Big: per row, the states of at
-// least a quarter of the row's scale, of at least an eighth, and the nonzero ones
-// (bit a for state a; all of them where the row is not finite, which makes its
-// entries NaN).  Clears redo.
+// digit) at a time: A's row, Bre's and Bim's.  Also each row's sets of large
+// states for k_rho_fix; clears redo.
 __global__ void __launch_bounds__(256) k_rho8_digits(const double2* __restrict__ psi, const double* __restrict__ sqrtP,
                                                      Rho8Dims d, unsigned char* __restrict__ Aop,
                                                      unsigned char* __restrict__ Bop, int16_t* __restrict__ E,
-                                                     ulonglong3* __restrict__ Big, unsigned char* __restrict__ redo) {
+                                                     RhoBig* __restrict__ Big, unsigned char* __restrict__ redo) {
   __shared__ double X[128][33];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, jb = blockIdx.x, ib = jb >> 2;
   const uint64_t i0 = (uint64_t)jb * 32;
@@ -105,14 +103,14 @@ __global__ void __launch_bounds__(256) k_rho8_digits(const double2* __restrict__
       }
     }
     const int top = __reduce_max_sync(0xffffffffu, max(e[0], e[1]));
-    uint64_t m[3];
+    uint64_t m[5];
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
-      const int at = q == 2 ? 0 : max(0, top - 2 - q);
+    for (int q = 0; q < 5; ++q) {
+      const int at = q == 4 ? 0 : max(0, top - q);
       m[q] = __ballot_sync(0xffffffffu, e[0] >= at) | (uint64_t)__ballot_sync(0xffffffffu, e[1] >= at) << 32;
       if (top == 0x7FF) m[q] = ~0ull;
     }
-    if (lane == 0) Big[i0 + r] = make_ulonglong3(m[0], m[1], m[2]);
+    if (lane == 0) Big[i0 + r] = RhoBig{m[0], m[1], m[2], m[3], m[4]};
   }
   const int K = 2 * d.B;
   for (int item = threadIdx.x; item < 512; item += 256) {
@@ -350,14 +348,14 @@ qc_status rho_tc_c128(const double2* psi, int n, int B, const double* P_host, do
   const size_t rows = (size_t)d.nib * TC5_M, bytesA = (size_t)d.nib * d.nkc * R8_ND * R8_A,
                bytesB = (size_t)d.njb * d.nkc * R8_ND * R8_B;
   unsigned char* buf = nullptr;
-  cudaError_t e = ws_alloc((void**)&buf, bytesA + bytesB + rows * (sizeof(ulonglong3) + sizeof(int16_t)) +
+  cudaError_t e = ws_alloc((void**)&buf, bytesA + bytesB + rows * (sizeof(RhoBig) + sizeof(int16_t)) +
                                              sizeof(double) * 128 + (size_t)d.nib * d.nib, s);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return QC_ENOMEM;
   }
   double* w = reinterpret_cast<double*>(buf + bytesA + bytesB);  // sqrt(P), then P
-  ulonglong3* Big = reinterpret_cast<ulonglong3*>(w + 128);
+  RhoBig* Big = reinterpret_cast<RhoBig*>(w + 128);
   int16_t* E = reinterpret_cast<int16_t*>(Big + rows);
   unsigned char* redo = reinterpret_cast<unsigned char*>(E + rows);
   double host[128] = {};
