@@ -546,7 +546,7 @@ qc_status qc_wigner_d(int twoj, double alpha, double beta, double gamma, double*
  * products (2^-47.6 of sum_a P_a |C_a(n)| |C_a(n')|) are closer, and tiles whose
  * device wait gave up, are taken on the CUDA cores; stream-ordered.  B > 64 (or,
  * for complex128, no room for the operand workspace of 84 * 2^n * B bytes, B
- * rounded up to a multiple of 8, and 42 * 2^n bytes, 2^n at least 128) is
+ * rounded up to a multiple of 8, and 66 * 2^n bytes, 2^n at least 128) is
  * stream-ordered on CUDA cores (complex128 inner products in double-float). */
 qc_status qc_density_matrix(const void* psi_dev, int n, qc_dtype dt, int B, const double* P_host,
                             void* rho_dev, void* stream);

@@ -393,14 +393,28 @@ qc_status rho_tc_c64(const float2* psi, int n, int B, const double* P_host, floa
 qc_status rho_tc_c128(const double2* psi, int n, int B, const double* P_host, double2* rho, cudaStream_t s);
 // Then: its entries that double-float products give better, and the blocks a
 // CTA gave up (redo), on the CUDA cores (density.cu); returns the launches made.
-// Big: per amplitude index, the states of at least the full scale 2^(E - 1023) of
-// its row (its largest magnitude is below twice that), a half, a quarter and an
-// eighth of it, and the nonzero ones; bit a for state a, all where the row is not
-// finite.
+// rows: per amplitude index, with the row's scale 2^(E - 1023) (its largest
+// magnitude is below twice that), for up to RHO_EXACT states their sizes
+// |re| + |im| of it (RHO_EXACT floats), for more the sets of those of at least
+// the full scale, a half, a quarter and an eighth of it, and of the nonzero ones
+// (bit a for state a; all where the row is not finite).
+constexpr int RHO_EXACT = 16;
 struct RhoBig {
   uint64_t full, half, quarter, eighth, any;
 };
-int launch_rho_fix(const double2* psi, int n, int B, const double* P, const int16_t* E, const RhoBig* Big,
+constexpr size_t RHO_ROW = 64;  // bytes a row of either
+static_assert(sizeof(RhoBig) <= RHO_ROW && sizeof(float) * RHO_EXACT <= RHO_ROW, "a row's record");
+// |x| to 2^-20, without an FP64 instruction (0 below FP32's range, infinite above)
+__device__ __forceinline__ float mag_f(double x) {
+  const int h = __double2hiint(x) & 0x7fffffff;
+  return h < (897 << 20) ? 0.f : h >= (1151 << 20) ? INFINITY : __int_as_float((h - (896 << 20)) << 3);
+}
+// The scale of a row of exponent E, 0 if none of its entries is replaced: a
+// double-float factor's 2^-98 forbids what lies lower, FP32's range what lies higher.
+__device__ __forceinline__ float rho_scale(int E) {
+  return E >= 1023 - 50 && E <= 1023 + 60 ? __int_as_float((E - 1023 + 127) << 23) : 0.f;
+}
+int launch_rho_fix(const double2* psi, int n, int B, const double* P, const int16_t* E, const void* rows,
                    const unsigned char* redo, double2* rho, cudaStream_t s);
 
 qc_status dense_launch(qc_state* s, const DenseMap& M, const void* dev_op, int* status,

@@ -183,13 +183,7 @@ __global__ void __launch_bounds__(256) k_rho(const V2* __restrict__ psi, uint64_
   }
 }
 
-// |x| to 2^-20, without an FP64 instruction (0 below FP32's range, infinite above)
-__device__ __forceinline__ float mag_f(double x) {
-  const int h = __double2hiint(x) & 0x7fffffff;
-  return h < (897 << 20) ? 0.f : h >= (1151 << 20) ? INFINITY : __int_as_float((h - (896 << 20)) << 3);
-}
 #define RHO_FEW 96
-#define RHO_EXACT 16
 
 // Entries of the digit products (rho_tc128.cu) that double-float products give
 // better, replaced by those; a CTA (or four, or sixteen, for few blocks) per
@@ -220,9 +214,13 @@ __device__ __forceinline__ float mag_f(double x) {
 // of them 0.98 (every tile whole; k_rho alone 4.64 ms).
 __global__ void __launch_bounds__(256) k_rho_fix(const double2* __restrict__ psi, uint64_t N, int B,
                                                  const double* __restrict__ P, const int16_t* __restrict__ E,
-                                                 const RhoBig* __restrict__ Big, int K16, int K64, float lim,
+                                                 const void* __restrict__ rows, int K16, int K64, float lim,
                                                  const unsigned char* __restrict__ redo, double2* __restrict__ rho) {
-  if (blockIdx.x < blockIdx.y) return;
+  // the upper triangle's blocks column by column: column J's rows are 0 .. J
+  int J = (int)(0.5f * (sqrtf(8.f * (float)blockIdx.x + 1.f) - 1.f));
+  while ((J + 1) * (J + 2) / 2 <= (int)blockIdx.x) ++J;
+  while (J * (J + 1) / 2 > (int)blockIdx.x) --J;
+  const int I = (int)blockIdx.x - J * (J + 1) / 2;
   // |re| + |im| of sqrt(P_a) C_a, of the row's scale: all 128 + 128 rows (up to RHO_EXACT states) or a
   // tile's 32 + 32; padded rows, whose 16-byte loads hit every bank
   constexpr int W16 = RHO_EXACT + 4, W64 = 64 + 4;
@@ -245,18 +243,16 @@ __global__ void __launch_bounds__(256) k_rho_fix(const double2* __restrict__ psi
   __shared__ int least[2], listed;
   __shared__ uint16_t list[RHO_FEW];  // entries of a tile: row << 5 | column
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, tx = tid & 15, ty = tid >> 4;
-  const bool redo_all = redo[blockIdx.y * gridDim.x + blockIdx.x] != 0, exact = B <= RHO_EXACT;
+  const bool redo_all = redo[I * (int)((N + 127) / 128) + J] != 0, exact = B <= RHO_EXACT;
   const int nh = (B + 3) / 4;
-  const uint64_t R0 = (uint64_t)blockIdx.y * 128, C0 = (uint64_t)blockIdx.x * 128;
+  const uint64_t R0 = (uint64_t)I * 128, C0 = (uint64_t)J * 128;
   const int side = tid >> 7, x = tid & 127;
   const uint64_t row = (side ? C0 : R0) + x;
-  const int e = E[row] - 1023;
-  // a factor's 2^-98 forbids what lies lower, FP32's range what lies higher
-  scale[side][x] = e >= -50 && e <= 60 ? __int_as_float((e + 127) << 23) : 0.f;
+  scale[side][x] = rho_scale(E[row]);
   if (tid < 64) wt[tid] = tid < B ? sqrtf((float)P[tid]) : 0.f;
   if (tid < 2) least[tid] = 64;
   __syncthreads();
-  // the sizes of a row (index i of the block's, side s), states 4 h .. 4 h + 3
+  // the sizes of a row (index i of the block's, side s), states 4 h .. 4 h + 3, from the amplitudes
   auto sizes = [&](int s, int i, int h, float* to) {
     const float sc = scale[s][i], inv = sc > 0.f ? 1.f / sc : 0.f;
     const uint64_t at = (s ? C0 : R0) + i;
@@ -269,11 +265,12 @@ __global__ void __launch_bounds__(256) k_rho_fix(const double2* __restrict__ psi
     }
   };
   if (exact) {
+    const float4* mine = reinterpret_cast<const float4*>(rows) + row * (RHO_EXACT / 4);
 #pragma unroll
     for (int h = 0; h < RHO_EXACT / 4; ++h)
-      if (h < nh) sizes(side, x, h, &S.all[side][x][4 * h]);
+      if (h < nh) *reinterpret_cast<float4*>(&S.all[side][x][4 * h]) = mine[h];
   } else {
-    const RhoBig mine = Big[row];
+    const RhoBig mine = reinterpret_cast<const RhoBig*>(rows)[row];
     S.m.mask[side][x] = mine;
     const int cnt = __reduce_min_sync(0xffffffffu, mine.any ? __popcll(mine.eighth) : 64);
     if (lane == 0) atomicMin(&least[side], cnt);
@@ -316,10 +313,10 @@ __global__ void __launch_bounds__(256) k_rho_fix(const double2* __restrict__ psi
   };
   if (exact && !redo_all) {  // most blocks have none: one barrier for all of a block's tiles
     unsigned any = 0;
-    for (int t = blockIdx.z; t < 16; t += gridDim.z) any |= small(32 * (t >> 2), 32 * (t & 3));
+    for (int t = blockIdx.y; t < 16; t += gridDim.y) any |= small(32 * (t >> 2), 32 * (t & 3));
     if (!__syncthreads_or(any)) return;
   }
-  for (int t = blockIdx.z; t < 16; t += gridDim.z) {
+  for (int t = blockIdx.y; t < 16; t += gridDim.y) {
     const int rl = 32 * (t >> 2), cl = 32 * (t & 3);
     const uint64_t r0 = R0 + rl, c0 = C0 + cl;
     if (r0 > c0 || c0 >= N) continue;
@@ -380,13 +377,13 @@ __global__ void __launch_bounds__(256) k_rho_fix(const double2* __restrict__ psi
     __syncthreads();  // listed and list are read
   }
 }
-int launch_rho_fix(const double2* psi, int n, int B, const double* P, const int16_t* E, const RhoBig* Big,
+int launch_rho_fix(const double2* psi, int n, int B, const double* P, const int16_t* E, const void* rows,
                    const unsigned char* redo, double2* rho, cudaStream_t s) {
   const unsigned nb = (unsigned)(((1ull << n) + 127) / 128);
   const double unit = std::sqrt(2.0 * B) / 26.0;
   // sizes are sums of |re| + |im| of both factors: twice the terms' moduli at most
-  k_rho_fix<<<dim3(nb, nb, nb <= 16 ? 16 : nb <= 32 ? 4 : 1), 256, 0, s>>>(
-      psi, 1ull << n, B, P, E, Big, (int)std::ceil(16.0 * unit), (int)std::ceil(64.0 * unit), (float)(2.0 * unit), redo,
+  k_rho_fix<<<dim3(nb * (nb + 1) / 2, nb <= 8 ? 16 : nb <= 16 ? 4 : 1), 256, 0, s>>>(
+      psi, 1ull << n, B, P, E, rows, (int)std::ceil(16.0 * unit), (int)std::ceil(64.0 * unit), (float)(2.0 * unit), redo,
       rho);
   return 1;
 }

@@ -73,12 +73,12 @@ __device__ __forceinline__ uint64_t r8_desc(uint32_t saddr) {
 
 // One block per 32 amplitude indices: their reals through shared memory, each
 // index's largest exponent, then 8 reals (one 16-byte core-matrix row per
-// digit) at a time: A's row, Bre's and Bim's.  Also each row's sets of large
-// states for k_rho_fix; clears redo.
+// digit) at a time: A's row, Bre's and Bim's.  Also each row's record for
+// k_rho_fix; clears redo.
 __global__ void __launch_bounds__(256) k_rho8_digits(const double2* __restrict__ psi, const double* __restrict__ sqrtP,
                                                      Rho8Dims d, unsigned char* __restrict__ Aop,
                                                      unsigned char* __restrict__ Bop, int16_t* __restrict__ E,
-                                                     RhoBig* __restrict__ Big, unsigned char* __restrict__ redo) {
+                                                     unsigned char* __restrict__ rows, unsigned char* __restrict__ redo) {
   __shared__ double X[128][33];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, jb = blockIdx.x, ib = jb >> 2;
   const uint64_t i0 = (uint64_t)jb * 32;
@@ -103,6 +103,13 @@ __global__ void __launch_bounds__(256) k_rho8_digits(const double2* __restrict__
       }
     }
     const int top = __reduce_max_sync(0xffffffffu, max(e[0], e[1]));
+    if (d.B <= RHO_EXACT) {
+      const float sc = rho_scale(top), inv = sc > 0.f ? 1.f / sc : 0.f;
+      if (lane < RHO_EXACT)
+        reinterpret_cast<float*>(rows)[(i0 + r) * RHO_EXACT + lane] =
+            lane < d.B ? (mag_f(X[lane][r]) + mag_f(X[lane + d.B][r])) * inv : 0.f;
+      continue;
+    }
     uint64_t m[5];
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
@@ -110,7 +117,7 @@ __global__ void __launch_bounds__(256) k_rho8_digits(const double2* __restrict__
       m[q] = __ballot_sync(0xffffffffu, e[0] >= at) | (uint64_t)__ballot_sync(0xffffffffu, e[1] >= at) << 32;
       if (top == 0x7FF) m[q] = ~0ull;
     }
-    if (lane == 0) Big[i0 + r] = RhoBig{m[0], m[1], m[2], m[3], m[4]};
+    if (lane == 0) reinterpret_cast<RhoBig*>(rows)[i0 + r] = RhoBig{m[0], m[1], m[2], m[3], m[4]};
   }
   const int K = 2 * d.B;
   for (int item = threadIdx.x; item < 512; item += 256) {
@@ -345,27 +352,27 @@ qc_status rho_tc_c128(const double2* psi, int n, int B, const double* P_host, do
   d.njb = (int)((d.N + 31) / 32);
   int64_t ntiles = 0;
   for (int ib = 0; ib < d.nib; ++ib) ntiles += d.njb - 4 * ib;
-  const size_t rows = (size_t)d.nib * TC5_M, bytesA = (size_t)d.nib * d.nkc * R8_ND * R8_A,
+  const size_t nr = (size_t)d.nib * TC5_M, bytesA = (size_t)d.nib * d.nkc * R8_ND * R8_A,
                bytesB = (size_t)d.njb * d.nkc * R8_ND * R8_B;
   unsigned char* buf = nullptr;
-  cudaError_t e = ws_alloc((void**)&buf, bytesA + bytesB + rows * (sizeof(RhoBig) + sizeof(int16_t)) +
+  cudaError_t e = ws_alloc((void**)&buf, bytesA + bytesB + nr * (RHO_ROW + sizeof(int16_t)) +
                                              sizeof(double) * 128 + (size_t)d.nib * d.nib, s);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return QC_ENOMEM;
   }
   double* w = reinterpret_cast<double*>(buf + bytesA + bytesB);  // sqrt(P), then P
-  RhoBig* Big = reinterpret_cast<RhoBig*>(w + 128);
-  int16_t* E = reinterpret_cast<int16_t*>(Big + rows);
-  unsigned char* redo = reinterpret_cast<unsigned char*>(E + rows);
+  unsigned char* rows = reinterpret_cast<unsigned char*>(w + 128);
+  int16_t* E = reinterpret_cast<int16_t*>(rows + nr * RHO_ROW);
+  unsigned char* redo = reinterpret_cast<unsigned char*>(E + nr);
   double host[128] = {};
   for (int a = 0; a < B; ++a) host[a] = std::sqrt(P_host[a]), host[64 + a] = P_host[a];
   int nk = put_bytes(w, host, sizeof host, s);
-  k_rho8_digits<<<4 * d.nib, 256, 0, s>>>(psi, w, d, buf, buf + bytesA, E, Big, redo);
+  k_rho8_digits<<<4 * d.nib, 256, 0, s>>>(psi, w, d, buf, buf + bytesA, E, rows, redo);
   allow_smem(k_rho8_tc, R8_SMEM);
   k_rho8_tc<<<(unsigned)std::min<int64_t>(ntiles, sm_count()), R8_T, R8_SMEM, s>>>(buf, buf + bytesA, E, d, ntiles, rho,
                                                                                   redo);
-  nk += 2 + launch_rho_fix(psi, n, B, w + 64, E, Big, redo, rho, s);
+  nk += 2 + launch_rho_fix(psi, n, B, w + 64, E, rows, redo, rho, s);
   const qc_status st = check_launch("density matrix (tensor cores)", nk);
   cudaFreeAsync(buf, s);
   return st;
