@@ -212,7 +212,7 @@ __global__ void __launch_bounds__(R8_T, 1) k_rho8_tc(const unsigned char* __rest
   // the loading thread's next chunk, over all of this CTA's tiles
   R8Tile ld{0, 0, 0, 0}, cur{0, 0, 0, 0};
   int ld_kc = 0;
-  uint32_t loaded = 0, q = 0;  // chunks loaded, multiplied
+  uint32_t loaded = 0, q = 0, issued = 0;  // chunks loaded, multiplied; those whose products were issued
   ld.at(blockIdx.x, d);
   auto load = [&]() {
     if (ld.t >= ntiles) return;
@@ -255,6 +255,7 @@ __global__ void __launch_bounds__(R8_T, 1) k_rho8_tc(const unsigned char* __rest
           asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(
                            bar_free + 8 * st)
                        : "memory");
+          ++issued;
           // the chunk three ahead takes the stage of the chunk before this one
           if (q >= 1) ok = tc5_mbar_wait(bar_free + 8 * ((q - 1) % R8_NST), ((q - 1) / R8_NST) & 1u, R8_SPIN);
           if (!ok) break;
@@ -277,7 +278,7 @@ __global__ void __launch_bounds__(R8_T, 1) k_rho8_tc(const unsigned char* __rest
     // after a wait that gave up: what is still in flight (bounded once more)
     if (lane == 0 && !ok) {
       for (uint32_t c = q; c < loaded; ++c) tc5_mbar_wait(bar_full + 8 * (c % R8_NST), (c / R8_NST) & 1u, R8_SPIN);
-      for (uint32_t c = q >= R8_NST ? q - R8_NST : 0; c < q; ++c)
+      for (uint32_t c = issued >= R8_NST ? issued - R8_NST : 0; c < issued; ++c)
         tc5_mbar_wait(bar_free + 8 * (c % R8_NST), (c / R8_NST) & 1u, R8_SPIN);
     }
   } else {
